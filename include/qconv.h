@@ -267,6 +267,38 @@ int qconv_np_destroy(qconv_np_handle* h);
 int qmaxpool_i8(const int8_t* d_x, int N, int H, int W, int C, int R, int S, int stride, int pad,
                 int8_t* d_y, void* cuda_stream);
 
+/* A pass over a network as one call: the steps are run in order, asynchronously on cuda_stream, exactly as the
+ * calls they stand for (the first error ends the pass).
+ *   QNET_CONV      qconv_run(handle, d_x, d_residual, d_y, n)
+ *   QNET_CONV_F32  qconv_run_f32(handle, input, e_x, d_residual, d_y, n)
+ *   QNET_QUANTIZE  qquantize_f32(input, count, e_x, n_bits, d_y)
+ *   QNET_MAXPOOL   qmaxpool_i8(d_x, n, H, W, C, R, R, stride, pad, d_y)
+ * where input = d_input + input_offset bytes.  The steps are read during the call only. */
+enum { QNET_CONV = 0, QNET_CONV_F32 = 1, QNET_QUANTIZE = 2, QNET_MAXPOOL = 3 };
+typedef struct {
+  int op, n, e_x, n_bits;
+  qconv_handle* handle;
+  const int8_t* d_x;
+  const int8_t* d_residual;
+  int8_t* d_y;
+  size_t input_offset, count;
+  int H, W, C, R, stride, pad;
+} qnet_step;
+int qnet_run(const qnet_step* steps, int count, const float* d_input, void* cuda_stream);
+
+/* Replays of a captured graph on an input that is read where it lies.  Between qgraph_record_begin and
+ * qgraph_record_end the calling thread captures a pass whose float input is [d_input, d_input + bytes); the
+ * kernels that read it (qconv_run_f32, qquantize_f32) are noted.  qgraph_set_input then makes the LATER launches of
+ * an executable graph instantiated from that capture read d_input (same shape, same alignment modulo 16 bytes)
+ * instead; launches already enqueued are not affected.  The captured cudaGraph_t must outlive the object.
+ * qgraph_record_end fails with UNSUPPORTED_SHAPE when it cannot name every reader of the input (copy the input to
+ * the recorded buffer then).  One thread at a time. */
+typedef struct qgraph_inputs qgraph_inputs;
+int qgraph_record_begin(const float* d_input, size_t bytes);
+int qgraph_record_end(qgraph_inputs** out);
+int qgraph_set_input(qgraph_inputs* g, void* graph_exec /* cudaGraphExec_t */, const float* d_input);
+int qgraph_inputs_destroy(qgraph_inputs* g);
+
 /* Stand-alone eltwise addition layer with per-input scales (Eq. 10, widths per Eq. 12-13):
  *   wide[j] = sum_i x_i[j] << lshift[i]      (lshift[i] = e_i - min_j e_j >= 0: exact at the finest scale)
  *   y[j]    = saturate(round(relu?(wide[j]) / 2^rshift))       (rshift = e_z - min_j e_j in [0, 31],

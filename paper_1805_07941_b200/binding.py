@@ -58,6 +58,17 @@ class qcalib_stats(ctypes.Structure):
                 ("hist", ctypes.POINTER(ctypes.c_uint64))]
 
 
+class qnet_step(ctypes.Structure):
+    _fields_ = [("op", ctypes.c_int), ("n", ctypes.c_int), ("e_x", ctypes.c_int), ("n_bits", ctypes.c_int),
+                ("handle", ctypes.c_void_p), ("d_x", ctypes.c_void_p), ("d_residual", ctypes.c_void_p),
+                ("d_y", ctypes.c_void_p), ("input_offset", ctypes.c_size_t), ("count", ctypes.c_size_t),
+                ("H", ctypes.c_int), ("W", ctypes.c_int), ("C", ctypes.c_int), ("R", ctypes.c_int),
+                ("stride", ctypes.c_int), ("pad", ctypes.c_int)]
+
+
+NET_CONV, NET_CONV_F32, NET_QUANTIZE, NET_MAXPOOL = 0, 1, 2, 3
+
+
 def sources():
     return [os.path.join(_CSRC, f) for f in sorted(os.listdir(_CSRC)) if f.endswith((".cu", ".cuh"))] + \
         [HEADER_PATH]
@@ -146,6 +157,13 @@ def lib():
         L.qconv_create_packed.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(qconv_desc), vp, vp, vp, vp, vp]
         for name in ("qpack_weights", "qunpack_weights", "qconv_create_packed"):
             getattr(L, name).restype = ci
+        L.qnet_run.argtypes = [vp, ci, vp, vp]
+        L.qgraph_record_begin.argtypes = [vp, sz]
+        L.qgraph_record_end.argtypes = [ctypes.POINTER(vp)]
+        L.qgraph_set_input.argtypes = [vp, vp, vp]
+        L.qgraph_inputs_destroy.argtypes = [vp]
+        for name in ("qnet_run", "qgraph_record_begin", "qgraph_record_end", "qgraph_set_input", "qgraph_inputs_destroy"):
+            getattr(L, name).restype = ci
         L.qconv_checked_faults.argtypes = [ctypes.POINTER(ci)]
         L.qconv_checked_faults.restype = ci
         L.qconv_last_error_string.restype = ctypes.c_char_p
@@ -169,13 +187,22 @@ def _host(a, dtype):
     return a, ctypes.c_void_p(a.ctypes.data)
 
 
+_raw_stream = _current_device = None
+
+
 def _stream():
-    import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current CUDA stream as an integer.  (The accessors behind torch.cuda.current_stream(), without the Stream
+    object it builds: 0.2 against 3.5 us, most of what a small layer's call cost the host.)"""
+    global _raw_stream, _current_device
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()                          # initialises CUDA
+        _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    return _raw_stream(_current_device())
 
 
 def _dev(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 class plan_hints:
@@ -220,6 +247,7 @@ class QConv:
             _check(lib().qconv_create(ctypes.byref(self.handle), ctypes.byref(self.desc),
                                       *[p for _, p in self._keep]))
         self._keep = None
+        self._run = lib().qconv_run
         dd = self.desc
         self.P = (dd.H + 2 * dd.pad_h - dd.R) // dd.stride_h + 1
         self.Q = (dd.W + 2 * dd.pad_w - dd.S) // dd.stride_w + 1
@@ -228,8 +256,10 @@ class QConv:
 
     def run(self, x, y, residual=None, n_run=None):
         """x, y, residual: torch CUDA tensors (contiguous).  Asynchronous on the current stream."""
-        n = x.shape[0] if n_run is None else n_run
-        _check(lib().qconv_run(self.handle, _dev(x), _dev(residual), _dev(y), int(n), _stream()))
+        rc = self._run(self.handle, x.data_ptr(), None if residual is None else residual.data_ptr(), y.data_ptr(),
+                       x.shape[0] if n_run is None else int(n_run), _stream())
+        if rc:
+            _check(rc)
         return y
 
     def run_f32(self, x_f32, e_x, y, residual=None, n_run=None):
@@ -272,13 +302,15 @@ class QConvNP:
         keep = [_host(w_codes, np.uint8), _host(bias, np.int32), _host(shift, np.int32)]
         self.handle = ctypes.c_void_p()
         _check(lib().qconv_np_create(ctypes.byref(self.handle), ctypes.byref(self.desc), *[p for _, p in keep]))
+        self._run = lib().qconv_np_run
         dd = self.desc
         self.P = (dd.H + 2 * dd.pad_h - dd.R) // dd.stride_h + 1
         self.Q = (dd.W + 2 * dd.pad_w - dd.S) // dd.stride_w + 1
 
     def run(self, x, y, n_run=None):
-        n = x.shape[0] if n_run is None else n_run
-        _check(lib().qconv_np_run(self.handle, _dev(x), _dev(y), int(n), _stream()))
+        rc = self._run(self.handle, x.data_ptr(), y.data_ptr(), x.shape[0] if n_run is None else int(n_run), _stream())
+        if rc:
+            _check(rc)
         return y
 
     def status(self):
@@ -297,6 +329,50 @@ class QConvNP:
     def __del__(self):
         try:
             self.destroy()
+        except Exception:
+            pass
+
+
+class Steps:
+    """A pass over a network as one native call (qnet_run): a list of qnet_step field dicts, addresses as integers."""
+
+    def __init__(self, steps):
+        self.array = (qnet_step * len(steps))(*[qnet_step(**s) for s in steps])
+        self._run = lib().qnet_run
+
+    def run(self, d_input):
+        rc = self._run(self.array, len(self.array), d_input, _stream())
+        if rc:
+            _check(rc)
+
+
+class GraphInputs:
+    """The readers of the float input in a pass that is captured inside the `with` block (qgraph_record_begin / end).
+    `found` says whether all of them are known; then set(graph_exec, address) points later launches at another input."""
+
+    def __init__(self, x):
+        self.x, self.found, self.handle = x, False, ctypes.c_void_p()
+
+    def __enter__(self):
+        _check(lib().qgraph_record_begin(self.x.data_ptr(), self.x.numel() * self.x.element_size()))
+        return self
+
+    def __exit__(self, *exc):
+        rc = lib().qgraph_record_end(ctypes.byref(self.handle))
+        self.found = rc == QCONV_OK
+        if rc not in (QCONV_OK, ERR_UNSUPPORTED_SHAPE) and exc[0] is None:
+            _check(rc)
+        return False
+
+    def set(self, graph_exec, address):
+        rc = lib().qgraph_set_input(self.handle, graph_exec, address)
+        if rc:
+            _check(rc)
+
+    def __del__(self):
+        try:
+            if self.handle:
+                lib().qgraph_inputs_destroy(self.handle)
         except Exception:
             pass
 

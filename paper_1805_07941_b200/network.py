@@ -29,6 +29,28 @@ def _stages(nodes):
     return runs
 
 
+class _NetGraph:
+    """A captured pass whose input may be any buffer of the input's shape: `replay` reads the network's own x_static,
+    `replay_on` the given address (the graph's input kernels are pointed at it; nothing is copied)."""
+
+    def __init__(self, graph, inputs):
+        self.graph, self.inputs = graph, inputs
+        self.exec = graph.raw_cuda_graph_exec()
+        self.own = self.at = inputs.x.data_ptr()
+
+    def takes(self, address):
+        return address == self.own or (self.inputs.found and (address ^ self.own) % 16 == 0)
+
+    def replay_on(self, address):
+        if address != self.at:
+            self.inputs.set(self.exec, address)
+            self.at = address
+        self.graph.replay()
+
+    def replay(self):
+        self.replay_on(self.own)
+
+
 class QNetwork:
     def __init__(self, net, weights, n_bits=8, rounding=0, device="cuda", fuse_pool=True):
         """net: description from workloads.py; weights: {conv name: (w [K,R,S,C/g] float32, bias [K])}."""
@@ -44,6 +66,7 @@ class QNetwork:
         self.handles = {}
         self.bufs = {}
         self.graph = None
+        self._programs = {}
         self.stages = _stages(net["nodes"])
         for name, (h, w, pitch) in net["buffers"].items():
             if name == "input":
@@ -188,10 +211,16 @@ class QNetwork:
                 hnd.run(self.bufs[nd["src"]], self._conv_dst(nd), self._residual(nd), n_run=n)
             self.e_buf[nd0["dst"]] = e_z
         torch.cuda.synchronize()
+        self._forget_plans()
+        return self
+
+    def _forget_plans(self):
+        """New layer handles: drop what was made from the old ones."""
         self.graph = None
+        self._programs = {}
+        self._drop_parts()
         if hasattr(self, "_fused_name"):
             del self._fused_name
-        return self
 
     def load_params(self, params, e_buf):
         """Build the int8 handles from parameters chosen elsewhere (same keys as self.params)."""
@@ -201,9 +230,7 @@ class QNetwork:
             if nd["op"] != "conv":
                 continue
             self.handles[nd["name"]] = self._make_handle(nd)
-        self.graph = None
-        if hasattr(self, "_fused_name"):
-            del self._fused_name
+        self._forget_plans()
         return self
 
     # ------------------------------------------------------------------ inference
@@ -241,9 +268,43 @@ class QNetwork:
         else:
             h.run(self.bufs[nd["src"]][sl], dst, res, n_run=n)
 
-    def _forward_layers(self, n):
+    def _program(self, sl, handles=None):
+        """The pass over the images of slice sl on one stream, as one native call (binding.Steps)."""
+        def at(buf):
+            t = self.bufs[buf]
+            return t.data_ptr() + sl.start * t.stride(0) * t.element_size()
+
+        n, steps, fused = sl.stop - sl.start, [], self._fused_input()
+        image = self.x_static.stride(0)
+        src = dict(input_offset=sl.start * image * 4, e_x=self.e_buf["input"])
+        if fused is None:
+            steps.append(dict(op=binding.NET_QUANTIZE, count=n * image, n_bits=self.n_bits, d_y=at("input"), **src))
         for nd in self.net["nodes"]:
-            self._run_node(nd, slice(0, n))
+            if nd["op"] == "maxpool":
+                if nd["name"] not in self._pooled:
+                    assert nd["R"] == nd["S"]
+                    C = self.bufs[nd["src"]].shape[3]
+                    steps.append(dict(op=binding.NET_MAXPOOL, n=n, d_x=at(nd["src"]), d_y=at(nd["dst"]), H=nd["H"],
+                                      W=nd["W"], C=C, R=nd["R"], stride=nd["stride"], pad=nd["pad"]))
+                continue
+            if nd["residual"]:
+                self._residual(nd)
+            pool = self._pool_after.get(nd["name"])
+            dst = pool["dst"] if pool is not None and pool["name"] in self._pooled else nd["dst"]
+            step = dict(n=n, handle=(self.handles if handles is None else handles)[nd["name"]].handle, d_y=at(dst),
+                        d_residual=at(nd["residual"]) if nd["residual"] else None)
+            if nd["name"] == fused:
+                steps.append(dict(step, op=binding.NET_CONV_F32, **src))
+            else:
+                steps.append(dict(step, op=binding.NET_CONV, d_x=at(nd["src"])))
+        return binding.Steps(steps)
+
+    def _run_program(self, n, address):
+        if n not in self._programs:
+            if len(self._programs) >= 64:                    # (a list of addresses per batch size: a few KB each)
+                self._programs.clear()
+            self._programs[n] = self._program(slice(0, n))
+        self._programs[n].run(address)
 
     def _dependencies(self):
         """For every node, the earlier nodes it must follow: writers of what it reads (input or
@@ -356,9 +417,7 @@ class QNetwork:
             if k:
                 st.wait_event(start)
             with torch.cuda.stream(st):
-                self._convert_input(sl)
-                for nd in self.net["nodes"]:
-                    self._run_node(nd, sl, sets[k])
+                self._program(sl, sets[k]).run(self.x_static.data_ptr())
                 if k:
                     ev = torch.cuda.Event()
                     ev.record(st)
@@ -370,8 +429,7 @@ class QNetwork:
     def forward_static(self, n=None):
         """Input conversion + every layer on self.x_static[:n]; asynchronous on the current stream."""
         n = self.N if n is None else n
-        self._convert_input(slice(0, n))
-        self._forward_layers(n)
+        self._run_program(n, self.x_static.data_ptr())
         return self.bufs[self.last][:n]
 
     def _capture_one(self, how):
@@ -383,10 +441,12 @@ class QNetwork:
             fwd()                                       # warm-up outside capture: tensor maps get cached
         torch.cuda.current_stream().wait_stream(s)
         torch.cuda.synchronize()
-        g = torch.cuda.CUDAGraph()
-        with torch.cuda.graph(g):
-            fwd()
-        return g
+        g = torch.cuda.CUDAGraph(keep_graph=True)           # (its nodes are addressed later, to change the input)
+        with binding.GraphInputs(self.x_static) as inputs:
+            with torch.cuda.graph(g):
+                fwd()
+        g.instantiate()
+        return _NetGraph(g, inputs)
 
     def capture(self, how=None):
         """Record one pass over the full batch into a CUDA graph (launch overhead of the few dozen
@@ -423,13 +483,20 @@ class QNetwork:
         return self.graph
 
     def run(self, x):
-        """x: float32 [n, H, W, C] CUDA tensor.  Returns the int8 output buffer (a view)."""
+        """x: float32 [n, H, W, C] CUDA tensor.  Returns the int8 output buffer (a view).  A contiguous x is read where
+        it lies; anything else is first copied to x_static."""
         n = x.shape[0]
-        self.x_static[:n].copy_(x)
-        if self.graph is not None and n == self.N:
-            self.graph.replay()
+        replay = self.graph is not None and n == self.N
+        address = x.data_ptr()
+        if x.dtype != torch.float32 or x.device != self.x_static.device or x.shape[1:] != self.x_static.shape[1:] or \
+                not x.is_contiguous() or not 0 < n <= self.N or (replay and not self.graph.takes(address)):
+            self.x_static[:n].copy_(x)
+            address = self.x_static.data_ptr()
+        if replay:
+            self.graph.replay_on(address)
             return self.bufs[self.last]
-        return self.forward_static(n)
+        self._run_program(n, address)
+        return self.bufs[self.last][:n]
 
     def run_pipelined(self, host_batches, host_outputs):
         """End-to-end inference of a sequence of batches that live in pinned host memory.
@@ -460,10 +527,13 @@ class QNetwork:
                 in_ready[s] = torch.cuda.Event()
                 in_ready[s].record(pp["h2d"])
             comp.wait_event(in_ready[s])
-            self.x_static.copy_(pp["xin"][s], non_blocking=True)
+            if self.graph.takes(pp["xin"][s].data_ptr()):
+                self.graph.replay_on(pp["xin"][s].data_ptr())    # the copied batch is read where it lies
+            else:
+                self.x_static.copy_(pp["xin"][s], non_blocking=True)
+                self.graph.replay()
             in_free[s] = torch.cuda.Event()
             in_free[s].record(comp)
-            self.graph.replay()
             if out_free[s] is not None:
                 comp.wait_event(out_free[s])
             pp["yout"][s].copy_(self.bufs[self.last], non_blocking=True)
@@ -499,6 +569,10 @@ class QNetwork:
         for h in self.handles.values():
             h.destroy()
         self.handles = {}
+        self._programs = {}
+        self._drop_parts()
+
+    def _drop_parts(self):
         for sets in getattr(self, "_parts", {}).values():
             for hs in sets:
                 for h in hs.values():
