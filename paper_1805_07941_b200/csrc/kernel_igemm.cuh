@@ -69,6 +69,10 @@ struct IgemmParams {
   int out_c_offset, out_c_pitch;
   int tmem_cols;                   // power of two >= max(32, BN)
   int vec_store;                   // 1: 16-byte stores/loads of int8 rows are aligned
+  int gen_simple;                  // general int8 epilogue: the accumulator bound leaves room for the single-pass rounding
+  int gen_vec_y, gen_vec_res;      // general epilogues: widest power of two (<= 16) of bytes at which every row piece of the
+                                   //    output / the residual is aligned (set per run from the pointers)
+  uint32_t gen_stage_bytes;        // general epilogues: shared memory of the warps' staging rows (0 for the fast ones)
   int fast_epilogue;               // 1: int8 out, nearest-even, K % 16 == 0, aligned rows, and the
                                    //    accumulator bound leaves room for the rounding constant
   uint32_t a_stage_bytes, b_stage_bytes;   // shared-memory footprint per stage (1024-aligned)
@@ -301,8 +305,9 @@ __device__ __forceinline__ uint32_t make_idesc_i8(int bn) {
 // Per-channel epilogue constants, one 16-byte entry per output channel, prepared on the host:
 //   x = bias, y = right shift s, and
 //   int8 output:  z = 2^(s-1) - 1 (0 when s = 0), w = (s > 0) | 2^t << 1 with t the residual left shift;
-//                 they serve the single-pass nearest-even rounding  (v + z + ((v >> s) & w & 1)) >> s;
-//   float output: w = bit pattern of the float 2^(e_x + e_w[k]).
+//                 they serve the single-pass nearest-even rounding  (v + z + ((v >> s) & w & 1)) >> s
+//                 (other rounding modes: see general_round);
+//   wide output:  z = 2^t, and for float output w = bit pattern of the float 2^(e_x + e_w[k]).
 
 struct IgemmShared {
   uint64_t full[kMaxStages];
@@ -388,7 +393,8 @@ struct TileWalker {
 // (these kernels are short; instruction fetch of unused paths is measurable):
 //   FAST_I8 / FAST_I8_RES: int8 output, nearest-even, 8-bit saturation, K % 16 == 0, aligned rows,
 //                          accumulator bound leaves room for the rounding constant; without / with residual
-//   I8: any rounding mode, bit width, alignment;  I32, F32: wide or float output
+//   I8: any rounding mode, bit width, alignment;  I32, F32: wide or float output;  MAX: the largest |float output|
+//                          alone, nothing is stored (general_tile below)
 //   FAST_I8_U / FAST_I8_RES_U: the same with one shift for all channels (per-layer scales): only the
 //                          bias is per channel, everything else sits in kernel parameters
 //   FLT_I8*:               the four fast variants again for layers whose wide value provably stays below
@@ -400,10 +406,11 @@ struct TileWalker {
 //                          value sits in the low mantissa byte; ReLU and the clamps are integer min/max
 //                          on the bit patterns (positive floats order like integers).
 enum : int { EPI_FAST_I8 = 0, EPI_FAST_I8_RES = 1, EPI_I8 = 2, EPI_I32 = 3, EPI_F32 = 4, EPI_FAST_I8_U = 5,
-             EPI_FAST_I8_RES_U = 6, EPI_FLT_I8 = 7, EPI_FLT_I8_RES = 8, EPI_FLT_I8_U = 9, EPI_FLT_I8_RES_U = 10 };
+             EPI_FAST_I8_RES_U = 6, EPI_FLT_I8 = 7, EPI_FLT_I8_RES = 8, EPI_FLT_I8_U = 9, EPI_FLT_I8_RES_U = 10,
+             EPI_MAX = 11 };
 
 template <int EPI> struct EpiTraits {
-  static constexpr bool flt = EPI >= EPI_FLT_I8;
+  static constexpr bool flt = EPI >= EPI_FLT_I8 && EPI <= EPI_FLT_I8_RES_U;
   static constexpr bool fast = EPI == EPI_FAST_I8 || EPI == EPI_FAST_I8_RES || EPI == EPI_FAST_I8_U ||
                                EPI == EPI_FAST_I8_RES_U || flt;
   static constexpr bool res = EPI == EPI_FAST_I8_RES || EPI == EPI_FAST_I8_RES_U || EPI == EPI_FLT_I8_RES ||
@@ -504,48 +511,133 @@ __device__ __forceinline__ void convert_16(const uint32_t* acc, uint32_t cst_g, 
 template <int EPI, int RELU, int RSTG>
 __device__ __forceinline__ void epilogue_16(const uint32_t (&acc)[16], uint32_t cst, int col, int k,
                                             size_t pix, const IgemmParams& prm, const EpilogueParams& ep,
-                                            const int8_t* __restrict__ res, const uint4& res16,
-                                            void* __restrict__ y, uint32_t stage_row) {
-  const size_t o = pix * prm.out_c_pitch + prm.out_c_offset + k;
-  const bool relu = RELU == 2 ? ep.relu != 0 : RELU == 1;
-  if (EpiTraits<EPI>::fast) {
-    uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};         // residual bytes, fetched ahead
-    uint32_t stage_addr = 0;
-    if (prm.out_stage_bytes) {
-      // position of these 16 bytes in the staged tile (row-major, 16-byte chunks swizzled as the tensor
-      // maps of the output and the residual expect)
-      const uint32_t off = stage_row + static_cast<uint32_t>(col);
-      stage_addr = off ^ (((off >> 7) & prm.out_swz_mask) << 4);
-      if (EpiTraits<EPI>::res && RSTG == 1) {
-        // the residual tile was brought there by TMA; the result overwrites it in place
-        const int4 r4 = lds_int4(stage_addr);
-        rw[0] = r4.x; rw[1] = r4.y; rw[2] = r4.z; rw[3] = r4.w;
+                                            const uint4& res16, void* __restrict__ y, uint32_t stage_row) {
+  static_assert(EpiTraits<EPI>::fast, "16-byte-store variants; the others go through general_tile");
+  uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};           // residual bytes, fetched ahead
+  uint32_t stage_addr = 0;
+  if (prm.out_stage_bytes) {
+    // position of these 16 bytes in the staged tile (row-major, 16-byte chunks swizzled as the tensor
+    // maps of the output and the residual expect)
+    const uint32_t off = stage_row + static_cast<uint32_t>(col);
+    stage_addr = off ^ (((off >> 7) & prm.out_swz_mask) << 4);
+    if (EpiTraits<EPI>::res && RSTG == 1) {
+      // the residual tile was brought there by TMA; the result overwrites it in place
+      const int4 r4 = lds_int4(stage_addr);
+      rw[0] = r4.x; rw[1] = r4.y; rw[2] = r4.z; rw[3] = r4.w;
+    }
+  }
+  uint32_t wds[4];
+  convert_16<EPI, RELU>(acc, cst + static_cast<uint32_t>(col) * (EpiTraits<EPI>::uni ? 4u : 16u), rw, ep, wds);
+  if (prm.out_stage_bytes) {
+    ptx::sts_uint4(stage_addr, wds[0], wds[1], wds[2], wds[3]);
+  } else {
+    *reinterpret_cast<uint4*>(static_cast<int8_t*>(y) + pix * prm.out_c_pitch + prm.out_c_offset + k) =
+        make_uint4(wds[0], wds[1], wds[2], wds[3]);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// General epilogue: any rounding mode, bit width and alignment, K not a multiple of 16, int32 / float output, and
+// the maximum of the float output.
+//
+// A thread holds one pixel's 16 channels at a time, but rows of K bytes at any alignment can only be stored 1 to 8
+// bytes at a time, and 32 lanes storing bytes of 32 different rows touch 32 sectors per instruction.  So every warp
+// turns its part of the tile (32 rows x up to 64 bytes) around in its own rows of shared memory: conversion writes
+// 16 bytes per thread, then consecutive lanes store consecutive pieces of a row, as wide as the alignment allows; the
+// residual comes in the same way.  Only the warp itself is involved (no block barrier).  kGenPitch = 64 bytes of data
+// + 16: 16-byte accesses of 8 consecutive rows fall into different banks.
+// 13 x 35 x 27 x 96 -> 200, 3x3, residual, round-half-away: 58 -> 13 us with the byte stores gone.
+constexpr int kGenPitch = 80;
+constexpr int kGenWarpBytes = 32 * kGenPitch;
+
+template <int V> struct GenVec;
+template <> struct GenVec<1> { using T = uint8_t; };
+template <> struct GenVec<2> { using T = uint16_t; };
+template <> struct GenVec<4> { using T = uint32_t; };
+template <> struct GenVec<8> { using T = uint2; };
+template <> struct GenVec<16> { using T = uint4; };
+
+// Moves a warp's rows between its staging rows and global memory: row r's `bytes` first bytes, at
+// base + row_off(lane r) in global memory; rows whose lane passes ok == false are left out.
+template <int V, bool STORE>
+__device__ __forceinline__ void gen_copy_rows(uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
+  using T = typename GenVec<V>::T;
+  constexpr int kLanes = V == 1 ? 32 : 64 / V;              // lanes side by side on a row (64 bytes of it; 32 for bytes)
+  constexpr int kRows = 32 / kLanes;
+  const unsigned okmask = __ballot_sync(0xffffffffu, ok);
+#pragma unroll 4
+  for (int r0 = 0; r0 < 32; r0 += kRows) {
+    const int r = r0 + lane / kLanes;
+    const long long off = __shfl_sync(0xffffffffu, row_off, r);
+#pragma unroll
+    for (int c0 = 0; c0 < 64; c0 += kLanes * V) {
+      const int c = c0 + (lane % kLanes) * V;
+      if (((okmask >> r) & 1u) && c < bytes) {
+        T* sp = reinterpret_cast<T*>(stage + r * kGenPitch + c);
+        T* gp = reinterpret_cast<T*>(base + off + c);
+        if (STORE) *gp = *sp; else *sp = __ldg(gp);
       }
     }
-    uint32_t wds[4];
-    convert_16<EPI, RELU>(acc, cst + static_cast<uint32_t>(col) * (EpiTraits<EPI>::uni ? 4u : 16u), rw, ep, wds);
-    if (prm.out_stage_bytes) {
-      ptx::sts_uint4(stage_addr, wds[0], wds[1], wds[2], wds[3]);
-    } else {
-      *reinterpret_cast<uint4*>(static_cast<int8_t*>(y) + o) = make_uint4(wds[0], wds[1], wds[2], wds[3]);
-    }
-    return;
   }
-  const int8_t* rp = res ? res + pix * prm.K + k : nullptr;
+}
+
+template <bool STORE>
+__device__ __forceinline__ void gen_copy(int vec, uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
+  switch (vec) {
+    case 16: gen_copy_rows<16, STORE>(stage, base, row_off, ok, bytes, lane); break;
+    case 8: gen_copy_rows<8, STORE>(stage, base, row_off, ok, bytes, lane); break;
+    case 4: gen_copy_rows<4, STORE>(stage, base, row_off, ok, bytes, lane); break;
+    case 2: gen_copy_rows<2, STORE>(stage, base, row_off, ok, bytes, lane); break;
+    default: gen_copy_rows<1, STORE>(stage, base, row_off, ok, bytes, lane); break;
+  }
+}
+
+// v / 2^s rounded in the descriptor's mode, in one pass: (v + z + (cond & w & 1)) >> s with the addend z and the mask
+// bit of w made by the host (s = 0: both 0):
+//   nearest-even: z = 2^(s-1) - 1, cond = lowest bit of the truncated quotient;  half away: the same z, cond = v > 0;
+//   half up: z = 2^(s-1);  floor: z = 0  (mask bit 0).
+__device__ __forceinline__ int32_t general_round(int32_t v, const int4& c, int rounding) {
+  const int32_t cond = rounding == 0 ? v >> c.y : (v > 0 ? 1 : 0);
+  return (v + c.z + (cond & c.w & 1)) >> c.y;
+}
+
+// One group of 16 columns.  rw: the residual bytes (zero without).  int8: 16 codes to the staging row; int32 / float:
+// 16 words to it; MAX: into *mx.
+template <int EPI>
+__device__ __forceinline__ void general_16(const uint32_t (&acc)[16], uint32_t cst_g, const uint4& res16, int ncols, bool row_ok,
+                                           const IgemmParams& prm, const EpilogueParams& ep, uint32_t stage, float* mx) {
+  const uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (k + j >= prm.K) break;
-    const int4 c = lds_int4(cst + static_cast<uint32_t>(col + j) * 16u);
-    const int32_t rv = rp ? static_cast<int32_t>(rp[j]) : 0;
-    const int t = rp ? ep.res_lshift[k + j] : 0;
-    const int32_t wide = wide_value(static_cast<int32_t>(acc[j]), c.x, rv, t, relu);
-    if (EPI == EPI_I8)
-      static_cast<int8_t*>(y)[o + j] = static_cast<int8_t>(requantize(wide, c.y, ep.rounding, ep.lo, ep.hi));
-    else if (EPI == EPI_I32)
-      static_cast<int32_t*>(y)[o + j] = wide;
-    else
-      // beta -> float: c.w holds the bits of 2^(e_x + e_w[k]); the product is exact (power of two)
-      static_cast<float*>(y)[o + j] = __int2float_rn(wide) * __int_as_float(c.w);
+  for (int g = 0; g < 4; ++g) {
+    uint32_t o[4];
+    const int32_t rv[4] = {sign_extend_byte<0>(rw[g]), sign_extend_byte<1>(rw[g]), sign_extend_byte<2>(rw[g]), sign_extend_byte<3>(rw[g])};
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int j = g * 4 + b;
+      const int4 c = lds_int4(cst_g + static_cast<uint32_t>(j * 16));
+      int32_t v = static_cast<int32_t>(acc[j]) + c.x + rv[b] * (EPI == EPI_I8 ? c.w >> 1 : c.z);
+      if (ep.relu) v = max(v, 0);
+      if (EPI == EPI_I8) {
+        const int32_t q = prm.gen_simple ? general_round(v, c, ep.rounding) : round_shift(v, c.y, ep.rounding);
+        o[b] = static_cast<uint32_t>(min(max(q, ep.lo), ep.hi));
+      } else if (EPI == EPI_I32) {
+        o[b] = static_cast<uint32_t>(v);
+      } else {
+        // beta -> float: c.w holds the bits of 2^(e_x + e_w[k]); the product is exact (power of two)
+        const float f = __int2float_rn(v) * __int_as_float(c.w);
+        if (EPI == EPI_MAX) {
+          if (row_ok && j < ncols) *mx = fmaxf(*mx, fabsf(f));
+        } else {
+          o[b] = __float_as_uint(f);
+        }
+      }
+    }
+    if (EPI == EPI_I8) {
+      const uint32_t lo2 = __byte_perm(o[0], o[1], 0x0040), hi2 = __byte_perm(o[2], o[3], 0x0040);
+      asm volatile("st.shared.b32 [%0], %1;" ::"r"(stage + g * 4u), "r"(__byte_perm(lo2, hi2, 0x5410)) : "memory");
+    } else if (EPI != EPI_MAX) {
+      ptx::sts_uint4(stage + g * 16u, o[0], o[1], o[2], o[3]);
+    }
   }
 }
 
@@ -634,7 +726,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
   const int num_kb_all = prm.R * prm.S * prm.nchunks;
   const uint32_t b_res_off = static_cast<uint32_t>(prm.stages) * stage_bytes;
   uint8_t* out_stage = tiles + b_res_off + (prm.b_resident ? static_cast<uint32_t>(num_kb_all) * prm.b_stage_bytes : 0u);   // staged output tiles
-  IgemmShared* sh = reinterpret_cast<IgemmShared*>(out_stage + static_cast<uint32_t>(prm.out_stage_bufs) * prm.out_stage_bytes);
+  IgemmShared* sh = reinterpret_cast<IgemmShared*>(out_stage + static_cast<uint32_t>(prm.out_stage_bufs) * prm.out_stage_bytes +
+                                                   prm.gen_stage_bytes);
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -915,6 +1008,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       }
       asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
     }
+    uint8_t* gen_stage = out_stage + ew * kGenWarpBytes;     // (general epilogues)
+    float gen_max = 0.0f;
     TileWalker walk;
     walk.init(prm, blockIdx.x);
     // the residual may come from the previous kernel (the constants above never do)
@@ -997,6 +1092,19 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             rres[i] = __ldg(reinterpret_cast<const uint4*>(res + pix * prm.K + k));
         }
       }
+      // general epilogues: this warp's columns of the tile, and its residual rows by way of the staging rows
+      const int gen_k0 = tc.k0 + g_begin * 16;
+      const int gen_cols = max(0, min((g_end - g_begin) * 16, prm.K - gen_k0));
+      if (!EpiTraits<EPI>::fast && res != nullptr) {
+        __syncwarp();
+        gen_copy<false>(prm.gen_vec_res, gen_stage, const_cast<int8_t*>(res) + gen_k0, static_cast<long long>(pix) * prm.K, row_ok,
+                        gen_cols, lane);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kGroupsPerWarp; ++i)
+          if (i * 16 < gen_cols) rres[i] = *reinterpret_cast<const uint4*>(gen_stage + lane * kGenPitch + i * 16);
+        __syncwarp();
+      }
       ok = wait_bounded<64, kHint>(ptx::smem_u32(&sh->acc_full[buf]), use & 1u, wait_limit, sh, status);
       if (res_staged && ok) {
         ok = wait_bounded<32, kHint>(ptx::smem_u32(&sh->res_full[sbuf]), (res_phase >> sbuf) & 1u, wait_limit, sh, status);
@@ -1028,6 +1136,20 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         };
         const uint32_t stage_row = stage_base + static_cast<uint32_t>(row * prm.BN);
         uint32_t acc_a[16], acc_b[16];
+        // general epilogues: group i of this warp; words leave group by group (64 bytes a row), bytes after the last
+        [[maybe_unused]] auto gen_group = [&](const uint32_t (&acc)[16], int i, const uint4& r16) {
+          if (i * 16 >= gen_cols) return;
+          const uint32_t st_row = ptx::smem_u32(gen_stage) + static_cast<uint32_t>(lane * kGenPitch);
+          const int ncols = gen_cols - i * 16;
+          general_16<EPI>(acc, chan + static_cast<uint32_t>((g_begin + i) * 256), r16, ncols, row_ok, prm, ep,
+                          st_row + (EPI == EPI_I8 ? static_cast<uint32_t>(i * 16) : 0u), &gen_max);
+          if (EPI == EPI_I32 || EPI == EPI_F32) {
+            __syncwarp();
+            gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + 4ll * (prm.out_c_offset + gen_k0 + i * 16),
+                           4ll * static_cast<long long>(pix) * prm.out_c_pitch, row_ok, 4 * min(16, ncols), lane);
+            __syncwarp();
+          }
+        };
         if (kLeanOk && lean) {
           // loads one group ahead of the arithmetic, as below, without the bookkeeping
           const uint32_t t0 = t_addr + lean_col0;
@@ -1073,21 +1195,31 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             if constexpr (kPool) {
               if (tc.k0 + g0 * 16 < prm.K)
                 epilogue_pool_16<EPI, RELU>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pooled_pix, row_ok, lane, prm.pool_bit, prm, ep, y);
+            } else if constexpr (!EpiTraits<EPI>::fast) {
+              gen_group(acc_a, i, rres[i & (kGroupsPerWarp - 1)]);
             } else if (row_ok && tc.k0 + g0 * 16 < prm.K)
-              epilogue_16<EPI, RELU, RSTG>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, prm, ep, res, rres[i & (kGroupsPerWarp - 1)], y, stage_row);
+              epilogue_16<EPI, RELU, RSTG>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, prm, ep, rres[i & (kGroupsPerWarp - 1)], y, stage_row);
             if (g1 < g_end) {
               ptx::tmem_ld_wait();
               if (g2 < g_end && i + 2 < GPW) ptx::tmem_ld_32x16(t_addr + g2 * 16, acc_a); else release();
               if constexpr (kPool) {
                 if (tc.k0 + g1 * 16 < prm.K)
                   epilogue_pool_16<EPI, RELU>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pooled_pix, row_ok, lane, prm.pool_bit, prm, ep, y);
+              } else if constexpr (!EpiTraits<EPI>::fast) {
+                gen_group(acc_b, i + 1, rres[(i + 1) & (kGroupsPerWarp - 1)]);
               } else if (row_ok && tc.k0 + g1 * 16 < prm.K)
-                epilogue_16<EPI, RELU, RSTG>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, prm, ep, res, rres[(i + 1) & (kGroupsPerWarp - 1)], y, stage_row);
+                epilogue_16<EPI, RELU, RSTG>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, prm, ep, rres[(i + 1) & (kGroupsPerWarp - 1)], y, stage_row);
               if (g2 < g_end && i + 2 < GPW) ptx::tmem_ld_wait();
             }
           }
         }
         if (g_begin >= g_end) release();                     // a warp without columns still hands back
+        if (EPI == EPI_I8) {
+          __syncwarp();
+          gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + prm.out_c_offset + gen_k0,
+                         static_cast<long long>(pix) * prm.out_c_pitch, row_ok, gen_cols, lane);
+          __syncwarp();
+        }
         }
       }
       if (staged) {
@@ -1105,6 +1237,11 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         }
         sbuf = sbuf == 2 ? 0 : sbuf + 1;
       }
+    }
+    if (EPI == EPI_MAX) {
+      // non-negative floats order like their bit patterns; y is the running maximum's word
+      const unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(gen_max));
+      if (lane == 0 && m) atomicMax(static_cast<unsigned int*>(y), m);
     }
     if (EpiTraits<EPI>::fast && prm.out_stage_bytes && etid == 0) {
       ptx::bulk_wait_all();

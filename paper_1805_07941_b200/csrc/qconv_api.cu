@@ -502,11 +502,15 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
                      d.n_out == 8 &&
                      h->acc_bound + round_room <= 2147483647ll) ? 1 : 0;
   if (hint.fast_epilogue == 0) p.fast_epilogue = 0;
+  // rounding adds at most 2^(s-1) before the shift: in one pass when the accumulator bound leaves that room
+  p.gen_simple = h->acc_bound + round_room <= 2147483647ll ? 1 : 0;
+  p.gen_stage_bytes = p.fast_epilogue ? 0u : static_cast<uint32_t>(qc::kEpilogueWarps * qc::kGenWarpBytes);
   // Shared memory: the operand ring, plus -- for the fast epilogues of short contractions, where the
   // epilogue and not the operand ring sets the pace -- staged output tiles that leave by TMA stores:
   // two of them, or three when the residual tile is also brought into them by TMA one tile ahead
   // (as long as the ring keeps enough stages beside them).
-  const int full_budget = (h->ctas_per_sm == 2 ? 113 : 226) * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared));
+  const int full_budget = (h->ctas_per_sm == 2 ? 113 : 226) * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared)) -
+                          static_cast<int>(p.gen_stage_bytes);
   const int out_tile = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM) * p.BN, 1024));
   auto ring_stages = [&](int bkc, int staged_tiles) {
     const int a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * bkc, 1024)) * (group ? tps : 1);
@@ -572,7 +576,7 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
   p.stages = stages;
   h->smem_bytes = 1024 + static_cast<size_t>(stages) * (p.a_stage_bytes + (p.b_resident ? 0 : p.b_stage_bytes)) +
                   (p.b_resident ? static_cast<size_t>(num_kb_plan) * p.b_stage_bytes : 0) +
-                  static_cast<size_t>(staged_tiles) * p.out_stage_bytes + sizeof(qc::IgemmShared);
+                  static_cast<size_t>(staged_tiles) * p.out_stage_bytes + p.gen_stage_bytes + sizeof(qc::IgemmShared);
   p.stride_h = p.stride_w = 1;
   p.pad_h = p.pad_w = 0;
   if (h->mode == MODE_FLAT || h->mode == MODE_STEM) {
@@ -666,6 +670,11 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
     const int t = (d.has_residual && res_lshift_host) ? res_lshift_host[k] : 0;
     chan[k] = make_int4(bias_host ? bias_host[k] : 0, sft, sft > 0 ? (1 << (sft - 1)) - 1 : 0,
                         (sft > 0 ? 1 : 0) | ((1 << t) << 1));
+    if (d.rounding >= QCONV_ROUND_HALF_UP) {                   // (general_round: no condition, another addend)
+      chan[k].z = (d.rounding == QCONV_ROUND_HALF_UP && sft > 0) ? 1 << (sft - 1) : 0;
+      chan[k].w &= ~1;
+    }
+    if (d.out_mode != QCONV_OUT_INT8) chan[k].z = 1 << t;
     if (h->flt_epilogue && p.fast_epilogue) {
       // r = (M + v) * 2^-s + M * (1 - 2^-s) with M = 1.5 * 2^23: both constants are exact in binary32
       // for s <= 22; beyond that |v| < 2^22 always rounds to 0, which scale 0 and addend M give
@@ -1374,6 +1383,13 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
     }
     int rc = prepare_a_map(h, a_ptr, n_run);
     if (rc) return rc;
+    if (!h->prm.fast_epilogue) {
+      // bytes at which every row piece of the output and the residual is aligned
+      auto widest = [](uintptr_t bits) { return bits & 1 ? 1 : bits & 2 ? 2 : bits & 4 ? 4 : bits & 8 ? 8 : 16; };
+      const uintptr_t es = d.out_mode == QCONV_OUT_INT8 ? 1 : 4;
+      h->prm.gen_vec_y = widest(reinterpret_cast<uintptr_t>(d_y) | es * d.out_c_pitch | es * d.out_c_offset | es * d.K);
+      h->prm.gen_vec_res = widest(reinterpret_cast<uintptr_t>(d_residual) | static_cast<uintptr_t>(d.K));
+    }
     if (h->prm.out_stage_bytes) {
       rc = prepare_y_map(h, d_y, n_run);
       if (rc) return rc;
