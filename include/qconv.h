@@ -154,6 +154,12 @@ int qconv_run(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
 int qconv_run_f32(qconv_handle* h, const float* d_x_f32, int e_x, const int8_t* d_residual, void* d_y,
                   int n_run, void* cuda_stream);
 
+/* Largest |y| of a layer with float output (QCONV_OUT_FLOAT), without writing the output: the maximum Section 3
+ * takes as the default threshold of an activation tensor, found in the layer's own epilogue.  Equals the maximum of
+ * qconv_run's output, bit for bit.  Synchronous: *maxabs_out is complete on return.  Errors: as qconv_run, and TIMEOUT. */
+int qconv_run_maxabs(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, int n_run, float* maxabs_out,
+                     void* cuda_stream);
+
 /* Synchronise the stream of the last qconv_run and return its device status (QCONV_OK or
  * QCONV_ERR_TIMEOUT), clearing it. */
 int qconv_status(qconv_handle* h);
@@ -378,6 +384,15 @@ int qjoin_exponent(const int32_t* e_own_host, const int32_t* const* acc_exp_host
  * exponents. */
 int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layout,
                       int per_channel, int n, int8_t* wq_host, int32_t* e_w_host);
+
+/* qquantize_weights on several layers at once (in parallel on the host's cores; same results). */
+typedef struct {
+  const float* w_host;
+  int8_t* wq_host;
+  int32_t* e_w_host;
+  int K, R, S, Cg, layout, per_channel, n;
+} qweights_job;
+int qquantize_weights_list(const qweights_job* jobs, int count);
 
 /* Packed storage of n-bit weights (Section 4.3 takes the weights down to 5 bits): value i is the n-bit
  * two's-complement field at bits [i*n, (i+1)*n) of a little-endian bit stream of ceil(count*n/8) bytes.

@@ -66,6 +66,11 @@ class qnet_step(ctypes.Structure):
                 ("stride", ctypes.c_int), ("pad", ctypes.c_int)]
 
 
+class qweights_job(ctypes.Structure):
+    _fields_ = [("w_host", ctypes.c_void_p), ("wq_host", ctypes.c_void_p), ("e_w_host", ctypes.c_void_p)] + \
+        [(n, ctypes.c_int) for n in ("K", "R", "S", "Cg", "layout", "per_channel", "n")]
+
+
 NET_CONV, NET_CONV_F32, NET_QUANTIZE, NET_MAXPOOL = 0, 1, 2, 3
 
 
@@ -157,6 +162,10 @@ def lib():
         L.qconv_create_packed.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(qconv_desc), vp, vp, vp, vp, vp]
         for name in ("qpack_weights", "qunpack_weights", "qconv_create_packed"):
             getattr(L, name).restype = ci
+        L.qconv_run_maxabs.argtypes = [vp, vp, vp, ci, ctypes.POINTER(ctypes.c_float), vp]
+        L.qconv_run_maxabs.restype = ci
+        L.qquantize_weights_list.argtypes = [ctypes.POINTER(qweights_job), ci]
+        L.qquantize_weights_list.restype = ci
         L.qnet_run.argtypes = [vp, ci, vp, vp]
         L.qgraph_record_begin.argtypes = [vp, sz]
         L.qgraph_record_end.argtypes = [ctypes.POINTER(vp)]
@@ -267,6 +276,13 @@ class QConv:
         n = x_f32.shape[0] if n_run is None else n_run
         _check(lib().qconv_run_f32(self.handle, _dev(x_f32), int(e_x), _dev(residual), _dev(y), int(n), _stream()))
         return y
+
+    def run_maxabs(self, x, residual=None, n_run=None):
+        """Largest |y| of a float-out layer, without the tensor; synchronous."""
+        n = x.shape[0] if n_run is None else n_run
+        out = ctypes.c_float(0)
+        _check(lib().qconv_run_maxabs(self.handle, _dev(x), _dev(residual), int(n), ctypes.byref(out), _stream()))
+        return np.float32(out.value)
 
     def status(self):
         return lib().qconv_status(self.handle)
@@ -545,6 +561,22 @@ def qquantize_weights(w, K, R, S, Cg, layout=0, per_channel=1, n=8):
     _check(lib().qquantize_weights(wp, K, R, S, Cg, layout, per_channel, n,
                                    ctypes.c_void_p(wq.ctypes.data), ctypes.c_void_p(e_w.ctypes.data)))
     return wq, e_w
+
+
+def qquantize_weights_list(layers, n=8):
+    """layers: list of (w [K][R][S][Cg] float32, K, R, S, Cg, per_channel).  Returns [(wq, e_w)] as qquantize_weights does."""
+    keep, out = [], []
+    jobs = (qweights_job * len(layers))()
+    for job, (w, K, R, S, Cg, per_channel) in zip(jobs, layers):
+        w, wp = _host(w, np.float32)
+        assert w.size == K * R * S * Cg
+        wq, e_w = np.empty(w.shape, dtype=np.int8), np.empty(K, dtype=np.int32)
+        keep.append(w)
+        out.append((wq, e_w))
+        job.w_host, job.wq_host, job.e_w_host = wp, wq.ctypes.data, e_w.ctypes.data
+        job.K, job.R, job.S, job.Cg, job.layout, job.per_channel, job.n = K, R, S, Cg, 0, per_channel, n
+    _check(lib().qquantize_weights_list(jobs, len(layers)))
+    return out
 
 
 def qquantize_bias(b, e_x, e_w):

@@ -23,6 +23,8 @@ __device__ __forceinline__ bool checked_in(unsigned long long idx, unsigned long
 #define QC_IN(idx, extent) true
 #endif
 
+constexpr int kOutMaxAbs = 3;  // out_mode of a run that keeps only the largest |float output|
+
 struct EpilogueParams {
   const int32_t* bias;        // [K] or nullptr
   const int32_t* shift;       // [K]
@@ -31,7 +33,7 @@ struct EpilogueParams {
   int relu;
   int rounding;
   int lo, hi;                 // saturation bounds of the output beta
-  int out_mode;               // 0 int8, 1 int32, 2 float
+  int out_mode;               // 0 int8, 1 int32, 2 float, kOutMaxAbs
   // when every channel has the same shifts: s, 2^(s-1) - 1, and (s > 0) | 2^t << 1
   int uni_shift, uni_z, uni_w;
   float uni_c1;               // 2^-s, for the float-rounding epilogue (0 when s > 22)
@@ -68,6 +70,12 @@ __device__ __forceinline__ int32_t requantize(int32_t v, int s, int mode, int lo
 // beta -> float: integer to binary32 (nearest even), then exact scaling by 2^e.
 __device__ __forceinline__ float dequantize(int32_t v, int e) {
   return ldexpf(__int2float_rn(v), e);
+}
+
+// Every thread's running maximum into the word at `y` (non-negative floats order like their bit patterns).
+__device__ __forceinline__ void flush_maxabs(float mx, void* y) {
+  const unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(static_cast<unsigned int*>(y), m);
 }
 
 }  // namespace qc

@@ -1239,9 +1239,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       }
     }
     if (EPI == EPI_MAX) {
-      // non-negative floats order like their bit patterns; y is the running maximum's word
-      const unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(gen_max));
-      if (lane == 0 && m) atomicMax(static_cast<unsigned int*>(y), m);
+      __syncwarp();
+      flush_maxabs(gen_max, y);
     }
     if (EpiTraits<EPI>::fast && prm.out_stage_bytes && etid == 0) {
       ptx::bulk_wait_all();

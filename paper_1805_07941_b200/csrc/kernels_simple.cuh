@@ -541,10 +541,13 @@ struct ConvGeom {
   int out_c_offset, out_c_pitch;
 };
 
+// mx: the thread's running maximum (out_mode kOutMaxAbs; y is then the word it goes to at the end).
 __device__ __forceinline__ void store_out(void* y, size_t idx, size_t extent, int32_t wide, int k,
-                                          const EpilogueParams& ep) {
+                                          const EpilogueParams& ep, float& mx) {
   if (!QC_IN(idx, extent)) return;
-  if (ep.out_mode == 0) {
+  if (ep.out_mode == kOutMaxAbs) {
+    mx = fmaxf(mx, fabsf(dequantize(wide, ep.acc_exp[k])));
+  } else if (ep.out_mode == 0) {
     int32_t v = requantize(wide, ep.shift[k], ep.rounding, ep.lo, ep.hi);
     static_cast<int8_t*>(y)[idx] = static_cast<int8_t>(v);
   } else if (ep.out_mode == 1) {
@@ -561,6 +564,7 @@ direct_conv_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ w_rs
   const int Cg = g.C / g.groups;
   const int Kg = g.K / g.groups;
   const size_t total = static_cast<size_t>(g.N) * g.P * g.Q * g.K;
+  float mx = 0.0f;
   for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
     int k = static_cast<int>(idx % g.K);
@@ -588,7 +592,11 @@ direct_conv_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ w_rs
     int32_t rv = (res && QC_IN(pix * g.K + k, static_cast<size_t>(g.N) * g.P * g.Q * g.K)) ? static_cast<int32_t>(res[pix * g.K + k]) : 0;
     int t = ep.res_lshift ? ep.res_lshift[k] : 0;
     int32_t wide = wide_value(acc, ep.bias ? ep.bias[k] : 0, rv, t, ep.relu);
-    store_out(y, pix * g.out_c_pitch + g.out_c_offset + k, static_cast<size_t>(g.N) * g.P * g.Q * g.out_c_pitch, wide, k, ep);
+    store_out(y, pix * g.out_c_pitch + g.out_c_offset + k, static_cast<size_t>(g.N) * g.P * g.Q * g.out_c_pitch, wide, k, ep, mx);
+  }
+  if (ep.out_mode == kOutMaxAbs) {
+    __syncwarp();
+    flush_maxabs(mx, y);
   }
 }
 
@@ -610,6 +618,7 @@ depthwise3x3_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ w_r
   const size_t total = static_cast<size_t>(g.N) * g.P * qt * cw;
   const uint32_t* x32 = reinterpret_cast<const uint32_t*>(x);
   const uint32_t* w32 = reinterpret_cast<const uint32_t*>(w_rsc);
+  float mx = 0.0f;
   for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
     int c4 = static_cast<int>(idx % cw);
@@ -680,6 +689,9 @@ depthwise3x3_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ w_r
           wd |= (static_cast<uint32_t>(requantize(wide[l], sh[l], ep.rounding, ep.lo, ep.hi)) & 0xFFu)
                 << (8 * l);
         *reinterpret_cast<uint32_t*>(static_cast<int8_t*>(y) + o) = wd;
+      } else if (ep.out_mode == kOutMaxAbs) {
+#pragma unroll
+        for (int l = 0; l < 4; ++l) mx = fmaxf(mx, fabsf(dequantize(wide[l], ae[l])));
       } else if (ep.out_mode == 1) {
 #pragma unroll
         for (int l = 0; l < 4; ++l) static_cast<int32_t*>(y)[o + l] = wide[l];
@@ -688,6 +700,10 @@ depthwise3x3_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ w_r
         for (int l = 0; l < 4; ++l) static_cast<float*>(y)[o + l] = dequantize(wide[l], ae[l]);
       }
     }
+  }
+  if (ep.out_mode == kOutMaxAbs) {
+    __syncwarp();
+    flush_maxabs(mx, y);
   }
 }
 

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -11,11 +12,14 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "../../include/qconv.h"
 #include "epilogue.cuh"
 #include "graph_inputs.cuh"
+#include "host_weights.cuh"
 #include "kernel_igemm.cuh"
 #include "kernel_dw_tma.cuh"
 #include "kernel_igemm_pair.cuh"
@@ -109,7 +113,8 @@ struct qconv_handle {
   int P, Q, Cg, Kg;
   int algo;                      // resolved QCONV_ALGO_*
   int lo, hi;
-  // device copies
+  // device copies, all of them parts of one allocation
+  void* d_block = nullptr;
   int8_t* d_w = nullptr;         // direct: [R][S][Cg][K]; depthwise: [R*S][C]; igemm: [Kpad][Kg_total]
   int32_t* d_bias = nullptr;
   int32_t* d_shift = nullptr;
@@ -169,17 +174,41 @@ namespace {
 
 void free_handle(qconv_handle* h) {
   if (!h) return;
-  cudaFree(h->d_w);
-  cudaFree(h->d_bias);
-  cudaFree(h->d_shift);
-  cudaFree(h->d_lshift);
-  cudaFree(h->d_accexp);
-  cudaFree(h->d_status);
-  cudaFree(h->d_chan);
+  cudaFree(h->d_block);
   cudaFree(h->d_pack);
-  cudaFree(h->d_dw_tap);
   delete h;
 }
+
+// A handle's host tables on their way to the device: one allocation for all of them, the small ones in one copy.
+// (One allocation and one copy per table cost 7 + 7 runtime calls per layer, most of the time of building it.)
+class DeviceParts {
+ public:
+  // `bytes` bytes of `src` (NULL: zeros), which stays valid until upload(); *dst receives the device address.
+  template <typename T>
+  void add(T** dst, const void* src, size_t bytes) { parts_.push_back({reinterpret_cast<void**>(dst), src, bytes, 0}); }
+  int upload(void** block) {
+    constexpr size_t kDirect = 128 * 1024;                 // larger parts are not worth copying into the image first
+    size_t image = 0;
+    for (Part& p : parts_)
+      if (p.bytes < kDirect) { p.at = image; image = align_up(image + p.bytes, 256); }
+    size_t total = image;
+    for (Part& p : parts_)
+      if (p.bytes >= kDirect) { p.at = total; total = align_up(total + p.bytes, 256); }
+    CUDA_TRY(cudaMalloc(block, std::max<size_t>(total, 256)));
+    std::vector<uint8_t> host(image, 0);
+    for (const Part& p : parts_) {
+      *p.dst = static_cast<uint8_t*>(*block) + p.at;
+      if (p.bytes >= kDirect) CUDA_TRY(cudaMemcpy(*p.dst, p.src, p.bytes, cudaMemcpyHostToDevice));
+      else if (p.src) std::memcpy(host.data() + p.at, p.src, p.bytes);
+    }
+    if (image) CUDA_TRY(cudaMemcpy(*block, host.data(), image, cudaMemcpyHostToDevice));
+    return QCONV_OK;
+  }
+
+ private:
+  struct Part { void** dst; const void* src; size_t bytes, at; };
+  std::vector<Part> parts_;
+};
 
 // Multiplier and shift for the kernel's divisions by d (1 <= d < 2^31), checked against plain division.
 qc::FastDiv make_fastdiv(int d_in) {
@@ -283,12 +312,12 @@ typedef void (*IgemmKernel)(const CUtensorMap, const CUtensorMap, const CUtensor
                             const qc::EpilogueParams,
                             const int4*, const int8_t*, void*, int*, unsigned int);
 
-IgemmKernel igemm_kernel_for(const qconv_handle* h);
+IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs = false);
 typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const qc::PairParams, const qc::IgemmParams,
                            const qc::EpilogueParams, const int4*, void*, int*, unsigned int);
 PairKernel pair_kernel_for(const qconv_handle* h);
 
-int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, const int32_t* bias_host,
+int plan_igemm(qconv_handle* h, DeviceParts& parts, const int8_t* w_krsc /* host [K][R][S][Cg] */, const int32_t* bias_host,
                const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host) {
   const qconv_desc& d = h->d;
   const qconv_plan_hints& hint = h->hints;
@@ -605,10 +634,12 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
   p.b_res_tx_bytes = static_cast<uint32_t>(num_kb_plan * tps * p.BN * p.BKC);
   p.res_tx_bytes = static_cast<uint32_t>(p.tq * p.tp * p.tn * p.BN);
 
-  // weights -> [kpad][kg_total], K-major rows, zero padded
-  std::vector<int8_t> wp(static_cast<size_t>(h->kpad) * h->kg_total, 0);
+  // weights -> [kpad][kg_total], K-major rows, zero padded (already in that form when nothing is padded or folded)
+  const size_t w_bytes = static_cast<size_t>(h->kpad) * h->kg_total;
+  const bool as_is = h->fold == 1 && !is_window_mode(h->mode) && h->mode != MODE_STEM && h->kpad == d.K && p.nchunks * p.BKC == d.C;
+  std::vector<int8_t> wp(as_is ? 0 : w_bytes, 0);
   std::vector<int8_t> row(static_cast<size_t>(std::max(c_row, 1)), 0);
-  for (int k = 0; k < d.K; ++k) {
+  for (int k = 0; k < d.K && !as_is; ++k) {
     const int8_t* src = w_krsc + static_cast<size_t>(k) * d.R * d.S * h->Cg;
     if (h->fold > 1 && !is_window_mode(h->mode)) {
       // one pixel's row as the unfolded GEMM would see it, then once per folded pixel on the diagonal
@@ -662,8 +693,7 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
         std::memcpy(dst + static_cast<size_t>(t) * p.nchunks * p.BKC, src + static_cast<size_t>(t) * d.C, d.C);
     }
   }
-  CUDA_TRY(cudaMalloc(&h->d_w, wp.size()));
-  CUDA_TRY(cudaMemcpy(h->d_w, wp.data(), wp.size(), cudaMemcpyHostToDevice));
+  parts.add(&h->d_w, as_is ? w_krsc : wp.data(), w_bytes);
   std::vector<int4> chan(h->kpad, make_int4(0, 0, 0, 0));
   for (int k = 0; k < d.K; ++k) {
     const int sft = shift_host ? shift_host[k] : 0;
@@ -691,12 +721,13 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
   }
   for (int j = 1; j < h->fold; ++j)
     for (int k = 0; k < d.K; ++k) chan[static_cast<size_t>(j) * d.K + k] = chan[k];
-  CUDA_TRY(cudaMalloc(&h->d_chan, sizeof(int4) * chan.size()));
-  CUDA_TRY(cudaMemcpy(h->d_chan, chan.data(), sizeof(int4) * chan.size(), cudaMemcpyHostToDevice));
+  parts.add(&h->d_chan, chan.data(), sizeof(int4) * chan.size());
+  int rc = parts.upload(&h->d_block);
+  if (rc) return rc;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->kg_total), static_cast<cuuint64_t>(h->kpad)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->kg_total)};
   cuuint32_t box[2] = {static_cast<cuuint32_t>(p.BKC), static_cast<cuuint32_t>(h->pair ? p.BN / 2 : p.BN)};
-  int rc = encode_map(&h->tmap_b, h->d_w, 2, dims, strides, box, p.BKC);
+  rc = encode_map(&h->tmap_b, h->d_w, 2, dims, strides, box, p.BKC);
   if (rc) return rc;
   if (is_window_mode(h->mode)) {
     const size_t bytes = static_cast<size_t>(d.N) * h->s2d_h * h->s2d_wp * h->win_pb;
@@ -736,7 +767,8 @@ int plan_igemm(qconv_handle* h, const int8_t* w_krsc /* host [K][R][S][Cg] */, c
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8, 2, 0, qc::kGroupsPerWarpWide>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I8>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I32>),
-                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_F32>)}) {
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_F32>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_MAX>)}) {
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
       if (e != cudaSuccess) attr_err = e;
     }
@@ -765,7 +797,8 @@ PairKernel pair_kernel_for(const qconv_handle* h) {
   return uni ? qc::igemm_i8_pair_kernel<qc::EPI_FAST_I8_U, 2> : qc::igemm_i8_pair_kernel<qc::EPI_FAST_I8, 2>;
 }
 
-IgemmKernel igemm_kernel_for(const qconv_handle* h) {
+IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
+  if (maxabs) return qc::igemm_i8_kernel<qc::EPI_MAX>;
   if (h->d.out_mode == QCONV_OUT_INT32) return qc::igemm_i8_kernel<qc::EPI_I32>;
   if (h->d.out_mode == QCONV_OUT_FLOAT) return qc::igemm_i8_kernel<qc::EPI_F32>;
   if (!h->prm.fast_epilogue) return qc::igemm_i8_kernel<qc::EPI_I8>;
@@ -1086,28 +1119,28 @@ int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
 
   // weights to [K][R][S][Cg] on the host
   const size_t wcount = static_cast<size_t>(d.K) * d.R * d.S * Cg;
-  std::vector<int8_t> w_krsc(wcount);
-  if (d.weight_layout == 0) {
-    std::memcpy(w_krsc.data(), w_host, wcount);
-  } else {
+  std::vector<int8_t> w_turned;
+  const int8_t* w_krsc = w_host;
+  if (d.weight_layout != 0) {
+    w_turned.resize(wcount);
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
     for (int k = 0; k < d.K; ++k)
-      for (size_t j = 0; j < per_k; ++j) w_krsc[k * per_k + j] = w_host[j * d.K + k];
+      for (size_t j = 0; j < per_k; ++j) w_turned[k * per_k + j] = w_host[j * d.K + k];
+    w_krsc = w_turned.data();
   }
 
   // Weight-aware bound of the wide value: 2^(n_in-1) * sum|w[k,.]| + |bias[k]| + 128 * 2^t[k].  Below 2^22 the
   // tensor-core epilogue may round in fp32 (exactly).
-  {
+  if (d.out_mode == QCONV_OUT_INT8 && d.groups == 1 && h->hints.float_rounding != 0) {
     long long worst = 0;
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
-    for (int k = 0; k < d.K; ++k) {
-      long long sw = 0;
-      for (size_t j = 0; j < per_k; ++j) sw += std::abs(static_cast<int>(w_krsc[k * per_k + j]));
-      long long bnd = sw * (1ll << (d.n_in - 1)) + (bias_host ? std::llabs(static_cast<long long>(bias_host[k])) : 0) +
-                      (d.has_residual ? (128ll << res_lshift_host[k]) : 0);
+    for (int k = 0; k < d.K && worst < (1ll << 22); ++k) {
+      const long long bnd = qc::host_abs_sum(w_krsc + k * per_k, per_k) * (1ll << (d.n_in - 1)) +
+                            (bias_host ? std::llabs(static_cast<long long>(bias_host[k])) : 0) +
+                            (d.has_residual ? (128ll << res_lshift_host[k]) : 0);
       worst = std::max(worst, bnd);
     }
-    h->flt_epilogue = (worst < (1ll << 22)) && h->hints.float_rounding != 0;
+    h->flt_epilogue = worst < (1ll << 22);
   }
 
   // choose the algorithm
@@ -1147,62 +1180,48 @@ int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
   h->algo = algo;
   h->mode = mode;
 
-  auto upload_i32 = [&](int32_t** dst, const int32_t* src, int32_t fill) -> int {
-    std::vector<int32_t> tmp(d.K, fill);
-    if (src) std::memcpy(tmp.data(), src, sizeof(int32_t) * d.K);
-    CUDA_TRY(cudaMalloc(dst, sizeof(int32_t) * d.K));
-    CUDA_TRY(cudaMemcpy(*dst, tmp.data(), sizeof(int32_t) * d.K, cudaMemcpyHostToDevice));
-    return QCONV_OK;
-  };
+  DeviceParts parts;
+  parts.add(&h->d_status, nullptr, 2 * sizeof(int));       // status word, maximum of qconv_run_maxabs
   int rc = QCONV_OK;
-  if (bias_host) rc = upload_i32(&h->d_bias, bias_host, 0);
-  if (!rc) rc = upload_i32(&h->d_shift, shift_host, 0);
-  if (!rc && d.has_residual) rc = upload_i32(&h->d_lshift, res_lshift_host, 0);
-  if (!rc) rc = upload_i32(&h->d_accexp, acc_exp_host, 0);
-  if (!rc) {
-    cudaError_t e = cudaMalloc(&h->d_status, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
-    if (e != cudaSuccess) rc = fail(QCONV_ERR_CUDA, "status word: %s", cudaGetErrorString(e));
-  }
-  if (!rc) {
-    if (algo == QCONV_ALGO_IGEMM) {
-      rc = plan_igemm(h, w_krsc.data(), bias_host, shift_host, res_lshift_host, acc_exp_host);
-    } else {
-      std::vector<int8_t> wp(wcount);
-      const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
-      // [R][S][Cg][K]; for depthwise Cg == 1 this is [R*S][C]
-      for (int k = 0; k < d.K; ++k)
-        for (size_t j = 0; j < per_k; ++j) wp[j * d.K + k] = w_krsc[k * per_k + j];
-      cudaError_t e = cudaMalloc(&h->d_w, wcount);
-      if (e == cudaSuccess) e = cudaMemcpy(h->d_w, wp.data(), wcount, cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) rc = fail(QCONV_ERR_CUDA, "weights: %s", cudaGetErrorString(e));
-      // Depthwise fast path (tap-packed dp4a with float-magic requantization, exact while
-      // |bias| + 9 * 128 * 128 < 2^22): int8 output, nearest-even, 8-bit saturation, no residual.
-      if (!rc && algo == QCONV_ALGO_DEPTHWISE && d.out_mode == QCONV_OUT_INT8 && d.n_out == 8 &&
-          d.rounding == QCONV_ROUND_NEAREST_EVEN && !d.has_residual && max_bias <= 4000000 &&
-          h->hints.depthwise_form != 0) {
-        std::vector<uint32_t> t(static_cast<size_t>(6) * d.C);
-        for (int c = 0; c < d.C; ++c) {
-          for (int r = 0; r < 3; ++r) {
-            uint32_t word = 0;
-            for (int sx = 0; sx < 3; ++sx)
-              word |= static_cast<uint32_t>(static_cast<uint8_t>(wp[static_cast<size_t>(r * 3 + sx) * d.C + c])) << (8 * sx);
-            t[static_cast<size_t>(r) * d.C + c] = word;
-          }
-          t[static_cast<size_t>(3) * d.C + c] = static_cast<uint32_t>((bias_host ? bias_host[c] : 0) + 0x4B400000);
-          const int sh_c = shift_host ? shift_host[c] : 0;
-          const float sc = sh_c <= 22 ? std::ldexp(1.0f, -sh_c) : 0.0f;
-          const float off = static_cast<float>(12582912.0 * (1.0 - static_cast<double>(sc)));   // exact for s <= 22
-          std::memcpy(&t[static_cast<size_t>(4) * d.C + c], &sc, 4);
-          std::memcpy(&t[static_cast<size_t>(5) * d.C + c], &off, 4);
+  if (algo == QCONV_ALGO_IGEMM) {
+    rc = plan_igemm(h, parts, w_krsc, bias_host, shift_host, res_lshift_host, acc_exp_host);
+  } else {
+    if (bias_host) parts.add(&h->d_bias, bias_host, sizeof(int32_t) * d.K);
+    parts.add(&h->d_shift, shift_host, sizeof(int32_t) * d.K);
+    if (d.has_residual) parts.add(&h->d_lshift, res_lshift_host, sizeof(int32_t) * d.K);
+    parts.add(&h->d_accexp, acc_exp_host, sizeof(int32_t) * d.K);
+    std::vector<int8_t> wp(wcount);
+    const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
+    // [R][S][Cg][K]; for depthwise Cg == 1 this is [R*S][C]
+    for (int k = 0; k < d.K; ++k)
+      for (size_t j = 0; j < per_k; ++j) wp[j * d.K + k] = w_krsc[k * per_k + j];
+    parts.add(&h->d_w, wp.data(), wcount);
+    // Depthwise fast path (tap-packed dp4a with float-magic requantization, exact while
+    // |bias| + 9 * 128 * 128 < 2^22): int8 output, nearest-even, 8-bit saturation, no residual.
+    std::vector<uint32_t> t;
+    if (algo == QCONV_ALGO_DEPTHWISE && d.out_mode == QCONV_OUT_INT8 && d.n_out == 8 &&
+        d.rounding == QCONV_ROUND_NEAREST_EVEN && !d.has_residual && max_bias <= 4000000 &&
+        h->hints.depthwise_form != 0) {
+      t.resize(static_cast<size_t>(6) * d.C);
+      for (int c = 0; c < d.C; ++c) {
+        for (int r = 0; r < 3; ++r) {
+          uint32_t word = 0;
+          for (int sx = 0; sx < 3; ++sx)
+            word |= static_cast<uint32_t>(static_cast<uint8_t>(wp[static_cast<size_t>(r * 3 + sx) * d.C + c])) << (8 * sx);
+          t[static_cast<size_t>(r) * d.C + c] = word;
         }
-        e = cudaMalloc(&h->d_dw_tap, t.size() * 4);
-        if (e == cudaSuccess) e = cudaMemcpy(h->d_dw_tap, t.data(), t.size() * 4, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) rc = fail(QCONV_ERR_CUDA, "depthwise tables: %s", cudaGetErrorString(e));
-        h->dw_tap = 1;
-        if (!rc && d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
+        t[static_cast<size_t>(3) * d.C + c] = static_cast<uint32_t>((bias_host ? bias_host[c] : 0) + 0x4B400000);
+        const int sh_c = shift_host ? shift_host[c] : 0;
+        const float sc = sh_c <= 22 ? std::ldexp(1.0f, -sh_c) : 0.0f;
+        const float off = static_cast<float>(12582912.0 * (1.0 - static_cast<double>(sc)));   // exact for s <= 22
+        std::memcpy(&t[static_cast<size_t>(4) * d.C + c], &sc, 4);
+        std::memcpy(&t[static_cast<size_t>(5) * d.C + c], &off, 4);
       }
+      parts.add(&h->d_dw_tap, t.data(), t.size() * 4);
+      h->dw_tap = 1;
+      if (d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
     }
+    rc = parts.upload(&h->d_block);
   }
   if (rc) {
     free_handle(h);
@@ -1239,9 +1258,10 @@ cudaError_t launch_row_pack(const qconv_handle* h, const void* src, bool f32, in
 }
 
 // One layer launch.  input_is_packed: d_x is the handle's own space-to-depth scratch, already filled
-// (qconv_run_f32 converts and packs in one kernel).
+// (qconv_run_f32 converts and packs in one kernel).  maxabs: d_y is the word of a running maximum (float bits of the
+// largest |float output|) and nothing else is written.
 int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void* d_y, int n_run,
-              void* cuda_stream, bool input_is_packed) {
+              void* cuda_stream, bool input_is_packed, bool maxabs = false) {
   if (!h || !d_x || !d_y) return fail(QCONV_ERR_BAD_ARG, "NULL handle or tensor pointer");
   const qconv_desc& d = h->d;
   if (n_run <= 0 || n_run > d.N) return fail(QCONV_ERR_BAD_ARG, "n_run %d outside [1, %d]", n_run, d.N);
@@ -1251,7 +1271,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
   h->last_stream = st;
   const float uni_c1 = h->uni_s <= 22 ? std::ldexp(1.0f, -h->uni_s) : 0.0f;
   qc::EpilogueParams ep{h->d_bias, h->d_shift, h->d_lshift, h->d_accexp, d.relu, d.rounding,
-                        h->lo, h->hi, d.out_mode, h->uni_s, h->uni_s > 0 ? (1 << (h->uni_s - 1)) - 1 : 0,
+                        h->lo, h->hi, maxabs ? qc::kOutMaxAbs : d.out_mode, h->uni_s, h->uni_s > 0 ? (1 << (h->uni_s - 1)) - 1 : 0,
                         (h->uni_s > 0 ? 1 : 0) | ((1 << h->uni_t) << 1), uni_c1,
                         static_cast<float>(12582912.0 * (1.0 - static_cast<double>(uni_c1)))};
   qc::ConvGeom g{n_run, d.H, d.W, d.C, d.K, d.R, d.S, d.stride_h, d.stride_w, d.pad_h, d.pad_w,
@@ -1310,7 +1330,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
   } else {
     if (reinterpret_cast<uintptr_t>(d_x) & 15)
       return fail(QCONV_ERR_ALIGNMENT, "d_x must be 16-byte aligned");
-    if (h->prm.vec_store && ((reinterpret_cast<uintptr_t>(d_y) | reinterpret_cast<uintptr_t>(d_residual)) & 15))
+    if (h->prm.vec_store && !maxabs && ((reinterpret_cast<uintptr_t>(d_y) | reinterpret_cast<uintptr_t>(d_residual)) & 15))
       return fail(QCONV_ERR_ALIGNMENT, "d_y and d_residual must be 16-byte aligned");
     const int8_t* a_ptr = d_x;
     if (h->mode == MODE_STEM) {
@@ -1463,7 +1483,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const int4* chan_ptr = h->d_chan;
-    cudaError_t le = cudaLaunchKernelEx(&cfg, igemm_kernel_for(h), h->tmap_a, h->tmap_b,
+    cudaError_t le = cudaLaunchKernelEx(&cfg, igemm_kernel_for(h, maxabs), h->tmap_a, h->tmap_b,
                                         p.out_stage_bytes ? h->tmap_y : h->tmap_a,
                                         (p.out_stage_bytes && p.out_stage_bufs == 3) ? h->tmap_r : h->tmap_a, p, ep, chan_ptr, d_residual,
                                         d_y, h->d_status, h->wait_limit);
@@ -1480,6 +1500,26 @@ extern "C" {
 int qconv_run(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void* d_y, int n_run,
               void* cuda_stream) {
   return run_layer(h, d_x, d_residual, d_y, n_run, cuda_stream, false);
+}
+
+int qconv_run_maxabs(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, int n_run, float* maxabs_out,
+                     void* cuda_stream) {
+  if (!h || !maxabs_out) return fail(QCONV_ERR_BAD_ARG, "NULL handle or result pointer");
+  if (h->d.out_mode != QCONV_OUT_FLOAT) return fail(QCONV_ERR_BAD_ARG, "qconv_run_maxabs serves layers with float output");
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  int* word = h->d_status + 1;
+  CUDA_TRY(cudaMemsetAsync(word, 0, sizeof(int), st));
+  int rc = run_layer(h, d_x, d_residual, word, n_run, cuda_stream, false, true);
+  if (rc) return rc;
+  int host[2] = {0, 0};                                    // status and maximum in one read
+  CUDA_TRY(cudaMemcpyAsync(host, h->d_status, sizeof(host), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
+  if (host[0]) {
+    CUDA_TRY(cudaMemset(h->d_status, 0, sizeof(int)));
+    return fail(host[0], "a bounded device-side wait expired (status %d)", host[0]);
+  }
+  std::memcpy(maxabs_out, &host[1], sizeof(float));
+  return QCONV_OK;
 }
 
 int qconv_run_f32(qconv_handle* h, const float* d_x_f32, int e_x, const int8_t* d_residual, void* d_y, int n_run,
@@ -2227,25 +2267,25 @@ int qconv_create_packed(qconv_handle** out, const qconv_desc* desc, const uint8_
   return qconv_create(out, desc, w.data(), bias_host, shift_host, res_lshift_host, acc_exp_host);
 }
 
-namespace {
-int8_t host_quantize_one(float v, int e, int n) {
-  const float bmax = static_cast<float>((1 << (n - 1)) - 1);
-  if (std::isnan(v)) return 0;
-  const float gam = std::ldexp(bmax, e);
-  v = std::fmin(std::fmax(v, -gam), gam);
-  float r = std::nearbyint(std::ldexp(v, -e));
-  r = std::fmin(std::fmax(r, -bmax), bmax);
-  return static_cast<int8_t>(r);
-}
-}  // namespace
-
 int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layout, int per_channel, int n,
                       int8_t* wq_host, int32_t* e_w_host) {
   if (!w_host || !wq_host || !e_w_host) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
   if (K <= 0 || R <= 0 || S <= 0 || Cg <= 0 || n < 2 || n > 8 || layout < 0 || layout > 1)
     return fail(QCONV_ERR_BAD_ARG, "bad weight geometry");
   const size_t per_k = static_cast<size_t>(R) * S * Cg;
-  auto at = [&](int k, size_t j) { return layout == 0 ? k * per_k + j : j * K + k; };
+  if (layout == 0) {                                       // a channel's values are contiguous
+    float gall = per_channel ? 0.0f : qc::host_max_abs(w_host, per_k * K);
+    for (int k = 0; k < K; ++k) {
+      const float* row = w_host + k * per_k;
+      int e;
+      qscale_exponent(per_channel ? qc::host_max_abs(row, per_k) : gall, n, &e);
+      e_w_host[k] = e;
+      if (per_channel) qc::host_quantize(row, per_k, e, n, wq_host + k * per_k);
+    }
+    if (!per_channel) qc::host_quantize(w_host, per_k * K, e_w_host[0], n, wq_host);
+    return QCONV_OK;
+  }
+  auto at = [&](int k, size_t j) { return j * K + k; };
   float gall = 0.0f;
   std::vector<float> gk(K, 0.0f);
   for (int k = 0; k < K; ++k) {
@@ -2261,8 +2301,39 @@ int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layo
     int e;
     qscale_exponent(per_channel ? gk[k] : gall, n, &e);
     e_w_host[k] = e;
-    for (size_t j = 0; j < per_k; ++j) wq_host[at(k, j)] = host_quantize_one(w_host[at(k, j)], e, n);
+    for (size_t j = 0; j < per_k; ++j) wq_host[at(k, j)] = qc::host_quantize_one(w_host[at(k, j)], e, n);
   }
+  return QCONV_OK;
+}
+
+// Layers are independent: the largest first over up to eight threads.  (The conversion reads 5 bytes per value from
+// memory twice; beyond eight threads the memory, not the arithmetic, sets the pace.)
+int qquantize_weights_list(const qweights_job* jobs, int count) {
+  if (!jobs || count < 0) return fail(QCONV_ERR_BAD_ARG, "NULL jobs or negative count");
+  std::vector<int> order(count), rc(count, QCONV_OK);
+  for (int i = 0; i < count; ++i) order[i] = i;
+  auto size = [&](int i) { return static_cast<long long>(jobs[i].K) * jobs[i].R * jobs[i].S * jobs[i].Cg; };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return size(a) > size(b); });
+  std::atomic<int> next{0};
+  auto work = [&] {
+    for (int i; (i = next.fetch_add(1)) < count;) {
+      const qweights_job& j = jobs[order[i]];
+      rc[order[i]] = qquantize_weights(j.w_host, j.K, j.R, j.S, j.Cg, j.layout, j.per_channel, j.n, j.wq_host, j.e_w_host);
+    }
+  };
+  long long total = 0;
+  for (int i = 0; i < count; ++i) total += size(i);
+  // (a thread costs some 20 us to start: worth it from about 2^18 values each)
+  const int want = static_cast<int>(std::min<long long>({8, count, total >> 18, std::max(1u, std::thread::hardware_concurrency())}));
+  std::vector<std::thread> threads;
+  try {
+    for (int t = 1; t < want; ++t) threads.emplace_back(work);
+  } catch (const std::system_error&) {                     // no more threads: the ones there are (this one at least) do it
+  }
+  work();
+  for (std::thread& t : threads) t.join();
+  for (int i = 0; i < count; ++i)
+    if (rc[i]) return fail(rc[i], "weights %d: NULL argument or bad geometry", i);
   return QCONV_OK;
 }
 

@@ -164,6 +164,13 @@ class QNetwork:
             self.stats["input"] = st
         self.e_buf["input"] = binding.qscale_exponent(gamma_of(st), self.n_bits)
         binding.qquantize_f32(x_calib, self.e_buf["input"], self.n_bits, out=self.bufs["input"][:n])
+        convs = [nd for nd in self.net["nodes"] if nd["op"] == "conv"]
+        # the weights depend on nothing that is measured here: all layers at once, in parallel on the host
+        quantized = dict(zip([nd["name"] for nd in convs], binding.qquantize_weights_list(
+            [(self.weights[nd["name"]][0], nd["K"], nd["R"], nd["S"], nd["C"] // nd["groups"], self.net["per_channel"])
+             for nd in convs], self.n_bits)))
+        # where only the maximum is wanted, the layer finds it itself and its float output is never written
+        only_max = threshold is None and not keep_stats and not sync
         fbuf = None
         for stage in self.stages:
             nd0 = stage[0]
@@ -175,25 +182,26 @@ class QNetwork:
                 continue
             cands = []
             for nd in stage:
-                w, b = self.weights[nd["name"]]
-                cg = nd["C"] // nd["groups"]
-                wq, e_w = binding.qquantize_weights(w, nd["K"], nd["R"], nd["S"], cg, 0,
-                                                    self.net["per_channel"], self.n_bits)
+                wq, e_w = quantized[nd["name"]]
+                b = self.weights[nd["name"]][1]
                 e_x = self.e_buf[nd["src"]]
                 bias_q = binding.qquantize_bias(b, e_x, e_w)
                 acc_exp = binding.qacc_exponents(e_x, e_w)
                 res_lshift = None
                 if nd["residual"]:
                     res_lshift = binding.qresidual_shifts(self.e_buf[nd["residual"]], acc_exp)
-                need = n * nd["P"] * nd["Q"] * nd["K"]
-                if fbuf is None or fbuf.numel() < need:
-                    fbuf = None
-                    fbuf = torch.empty(need, dtype=torch.float32, device=self.device)
                 fl = binding.QConv(wq, bias_q, None, res_lshift, acc_exp, out_mode=binding.OUT_FLOAT,
                                    has_residual=int(res_lshift is not None), **self._geom(nd))
                 res = self._residual(nd)
-                fl.run(self.bufs[nd["src"]], fbuf, None if res is None else res, n_run=n)
-                st = collect(fbuf[:need])
+                if only_max:
+                    st = dict(maxabs=fl.run_maxabs(self.bufs[nd["src"]], res, n_run=n))
+                else:
+                    need = n * nd["P"] * nd["Q"] * nd["K"]
+                    if fbuf is None or fbuf.numel() < need:
+                        fbuf = None
+                        fbuf = torch.empty(need, dtype=torch.float32, device=self.device)
+                    fl.run(self.bufs[nd["src"]], fbuf, res, n_run=n)
+                    st = collect(fbuf[:need])
                 fl.destroy()
                 if keep_stats:
                     self.stats[nd["name"]] = st

@@ -45,3 +45,33 @@ def test_shifts_at_the_ends_of_their_range(rounding, shift):
     kw = dict(R=1, S=1, rounding=rounding, n_out=5)
     got, desc = gpu_conv(x, w, bias, s, **kw)
     assert (got == oracle_conv(x, w, bias, s, **kw)).all(), desc
+
+
+MAX_CASES = [  # N, H, W, C, K, R, groups, stride, n_run: every kernel that can run a float-out layer
+    (3, 9, 7, 32, 40, 3, 1, 1, 3), (3, 9, 7, 32, 40, 3, 1, 1, 2), (2, 14, 14, 64, 64, 3, 1, 1, 2), (5, 6, 5, 16, 17, 1, 1, 1, 5),
+    (2, 17, 15, 3, 24, 3, 1, 2, 2), (2, 12, 12, 32, 32, 3, 32, 1, 2), (2, 13, 11, 24, 24, 3, 24, 2, 1), (2, 8, 8, 20, 12, 3, 2, 1, 2)]
+
+
+@pytest.mark.parametrize("case", MAX_CASES)
+@pytest.mark.parametrize("with_res", [0, 1])
+def test_maximum_of_the_float_output_without_the_output(case, with_res):
+    import torch
+    from oracle import ref
+    from paper_1805_07941_b200 import binding
+    N, H, W, C, K, R, groups, stride, n_run = case
+    rng = np.random.default_rng(sum(case))
+    x, w, bias, _, res, t = rand_layer(rng, N, H, W, C, K, R, R, groups=groups, with_res=bool(with_res), stride=(stride, stride),
+                                       pad=(R // 2, R // 2))
+    acc_exp = rng.integers(-20, -8, K).astype(np.int32)
+    for relu in (0, 1):
+        want = ref.qconv(x, w, bias, None, res, t, acc_exp, R=R, S=R, stride=(stride, stride), pad=(R // 2, R // 2), groups=groups,
+                         relu=relu, out_mode=2)
+        conv = binding.QConv(w, bias, None, t, acc_exp, N=N, H=H, W=W, C=C, K=K, R=R, S=R, stride_h=stride, stride_w=stride,
+                             pad_h=R // 2, pad_w=R // 2, groups=groups, relu=relu, out_mode=2, has_residual=with_res)
+        rd = torch.from_numpy(res).cuda() if with_res else None
+        for _ in range(2):                                 # the word is cleared by every call
+            assert conv.run_maxabs(torch.from_numpy(x).cuda(), rd, n_run=n_run) == np.abs(want[:n_run]).max(), conv.describe()
+        conv.destroy()
+    with pytest.raises(binding.QconvError):
+        binding.QConv(w, bias, None, t, None, N=N, H=H, W=W, C=C, K=K, R=R, S=R, stride_h=stride, stride_w=stride, pad_h=R // 2,
+                      pad_w=R // 2, groups=groups, has_residual=with_res).run_maxabs(torch.from_numpy(x).cuda(), rd)
