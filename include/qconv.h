@@ -122,12 +122,22 @@ int qconv_set_plan_hints(const qconv_plan_hints* hints);
  *   shift_host      K right shifts s[k] = e_z - e_x - e_w[k] in [0, 31], or NULL for all zero
  *   res_lshift_host K left shifts t[k] = e_res - e_x - e_w[k] in [0, 23]; required iff has_residual
  *   acc_exp_host    K exponents e_x + e_w[k] in [-126, 96]; read only by QCONV_OUT_FLOAT; NULL means 0
+ * The tables' device memory comes from a pool that keeps up to 64 MB of what destroyed handles gave back, until the
+ * last handle of the device is gone.
  * Errors: BAD_ARG, UNSUPPORTED_SHAPE, OVERFLOW_RISK when
  *   (R*S*C/groups) * 2^(n_in-1) * 2^(n_w-1) + max|bias| + 2^(7 + max t) > 2^31 - 1,
  * BAD_SHIFT, RESIDUAL_SCALE, ALIGNMENT, CUDA.  On error *out is NULL. */
 int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host,
                  const int32_t* bias_host, const int32_t* shift_host,
                  const int32_t* res_lshift_host, const int32_t* acc_exp_host);
+
+/* qconv_create for a second handle of the SAME weights (another output mode, other shifts or biases): when both plans
+ * lay the weights out alike, the handle uses the device copy that `weights_of` holds instead of making its own (the
+ * copy lives until the last handle that uses it is destroyed, in any order).  w_host is needed all the same;
+ * weights_of may be NULL. */
+int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host, const int32_t* bias_host,
+                         const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
+                         const qconv_handle* weights_of);
 
 /* Run the layer on n_run <= desc.N images, asynchronously on cuda_stream.
  *   d_x        int8 [n_run][H][W][C], 16-byte aligned

@@ -113,6 +113,8 @@ def lib():
         L = ctypes.CDLL(LIB_PATH)
         vp, ci, sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
         L.qconv_create.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(qconv_desc), vp, vp, vp, vp, vp]
+        L.qconv_create_sharing.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(qconv_desc), vp, vp, vp, vp, vp, vp]
+        L.qconv_create_sharing.restype = ci
         L.qconv_run.argtypes = [vp, vp, vp, vp, ci, vp]
         L.qconv_run_f32.argtypes = [vp, vp, ci, vp, vp, ci, vp]
         L.qconv_run_f32.restype = ci
@@ -238,8 +240,9 @@ class plan_hints:
 class QConv:
     """One layer handle (qconv_create / qconv_run / qconv_status / qconv_destroy)."""
 
-    def __init__(self, w, bias=None, shift=None, res_lshift=None, acc_exp=None, packed=False, **desc):
-        """packed=True: w is the packed n_w-bit stream of qpack_weights (qconv_create_packed)."""
+    def __init__(self, w, bias=None, shift=None, res_lshift=None, acc_exp=None, packed=False, weights_of=None, **desc):
+        """packed=True: w is the packed n_w-bit stream of qpack_weights (qconv_create_packed).  weights_of: a QConv made
+        from the same w whose device copy of it may be shared (qconv_create_sharing)."""
         d = dict(stride_h=1, stride_w=1, pad_h=0, pad_w=0, groups=1, n_in=8, n_w=8, n_out=8,
                  symmetric=1, relu=0, rounding=0, out_mode=0, out_c_offset=0, out_c_pitch=0,
                  has_residual=0, weight_layout=0, algo=0, pool=0)
@@ -253,8 +256,8 @@ class QConv:
             _check(lib().qconv_create_packed(ctypes.byref(self.handle), ctypes.byref(self.desc),
                                              *[p for _, p in self._keep]))
         else:
-            _check(lib().qconv_create(ctypes.byref(self.handle), ctypes.byref(self.desc),
-                                      *[p for _, p in self._keep]))
+            _check(lib().qconv_create_sharing(ctypes.byref(self.handle), ctypes.byref(self.desc),
+                                              *[p for _, p in self._keep], weights_of.handle if weights_of else None))
         self._keep = None
         self._run = lib().qconv_run
         dd = self.desc

@@ -104,6 +104,80 @@ inline bool is_window_mode(int m) { return m == MODE_S2D || m == MODE_WROW; }
 
 }  // namespace
 
+// Device memory of the handles' tables.  A network's calibration builds and destroys two handles per layer; cudaMalloc and
+// cudaFree took two thirds of that time.  Blocks given back are kept for the next handle, at most kKeep bytes per
+// device, and all of them are freed when the last block in use is given back.  Any thread, any stream: a block is only
+// given back after the device is idle, so whoever takes it next may overwrite it at once.
+class DevicePool {
+ public:
+  struct Block {
+    void* ptr = nullptr;
+    size_t bytes = 0;
+    int device = 0;
+    Block() = default;
+    Block(const Block&) = delete;
+    Block& operator=(const Block&) = delete;
+    ~Block() { if (ptr) pool().give(*this); }
+  };
+  static DevicePool& pool() {
+    static DevicePool* p = new DevicePool;                 // never destroyed: handles may outlive static destructors
+    return *p;
+  }
+  cudaError_t take(Block* b, size_t bytes) {
+    bytes = (std::max<size_t>(bytes, 1) + 4095) / 4096 * 4096;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    b->device = dev;
+    std::lock_guard<std::mutex> lock(mu_);
+    PerDevice& d = per_device_[dev & 63];
+    size_t best = d.free.size();
+    for (size_t i = 0; i < d.free.size(); ++i)
+      if (d.free[i].second >= bytes && d.free[i].second <= 2 * bytes && (best == d.free.size() || d.free[i].second < d.free[best].second))
+        best = i;
+    if (best < d.free.size()) {
+      b->ptr = d.free[best].first;
+      b->bytes = d.free[best].second;
+      d.kept -= b->bytes;
+      d.free.erase(d.free.begin() + static_cast<long>(best));
+    } else {
+      e = cudaMalloc(&b->ptr, bytes);
+      if (e != cudaSuccess) { b->ptr = nullptr; return e; }
+      b->bytes = bytes;
+    }
+    ++d.live;
+    return cudaSuccess;
+  }
+
+ private:
+  static constexpr size_t kKeep = 64u << 20;
+  struct PerDevice {
+    std::vector<std::pair<void*, size_t>> free;            // oldest first
+    size_t kept = 0, live = 0;
+  };
+  std::mutex mu_;
+  PerDevice per_device_[64];
+
+  void give(Block& b) {
+    int dev = 0;
+    const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != b.device && cudaSetDevice(b.device) == cudaSuccess;
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    std::vector<void*> drop;
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      PerDevice& d = per_device_[b.device & 63];
+      --d.live;
+      if (idle) { d.free.emplace_back(b.ptr, b.bytes); d.kept += b.bytes; } else { drop.push_back(b.ptr); }
+      size_t n = 0;
+      while (n < d.free.size() && (d.live == 0 || d.kept > kKeep)) { drop.push_back(d.free[n].first); d.kept -= d.free[n].second; ++n; }
+      d.free.erase(d.free.begin(), d.free.begin() + static_cast<long>(n));
+    }
+    for (void* p : drop) cudaFree(p);
+    if (other) cudaSetDevice(dev);
+    b.ptr = nullptr;
+  }
+};
+
 struct qgraph_inputs {
   qc::GraphInputRecord rec;
 };
@@ -113,8 +187,10 @@ struct qconv_handle {
   int P, Q, Cg, Kg;
   int algo;                      // resolved QCONV_ALGO_*
   int lo, hi;
-  // device copies, all of them parts of one allocation
-  void* d_block = nullptr;
+  // device copies: the small tables in one block, large weights in a second one that handles of the same weights share
+  DevicePool::Block block;
+  std::shared_ptr<DevicePool::Block> weights;
+  bool weights_as_is = false;    // those weights lie as the host handed them over ([K][R][S][C])
   int8_t* d_w = nullptr;         // direct: [R][S][Cg][K]; depthwise: [R*S][C]; igemm: [Kpad][Kg_total]
   int32_t* d_bias = nullptr;
   int32_t* d_shift = nullptr;
@@ -174,41 +250,55 @@ namespace {
 
 void free_handle(qconv_handle* h) {
   if (!h) return;
-  cudaFree(h->d_block);
   cudaFree(h->d_pack);
   delete h;
 }
 
-// A handle's host tables on their way to the device: one allocation for all of them, the small ones in one copy.
-// (One allocation and one copy per table cost 7 + 7 runtime calls per layer, most of the time of building it.)
+// A handle's small host tables on their way to the device, in one block and one copy.
 class DeviceParts {
  public:
   // `bytes` bytes of `src` (NULL: zeros), which stays valid until upload(); *dst receives the device address.
   template <typename T>
-  void add(T** dst, const void* src, size_t bytes) { parts_.push_back({reinterpret_cast<void**>(dst), src, bytes, 0}); }
-  int upload(void** block) {
-    constexpr size_t kDirect = 128 * 1024;                 // larger parts are not worth copying into the image first
-    size_t image = 0;
-    for (Part& p : parts_)
-      if (p.bytes < kDirect) { p.at = image; image = align_up(image + p.bytes, 256); }
-    size_t total = image;
-    for (Part& p : parts_)
-      if (p.bytes >= kDirect) { p.at = total; total = align_up(total + p.bytes, 256); }
-    CUDA_TRY(cudaMalloc(block, std::max<size_t>(total, 256)));
-    std::vector<uint8_t> host(image, 0);
+  void add(T** dst, const void* src, size_t bytes) {
+    parts_.push_back({reinterpret_cast<void**>(dst), src, bytes, total_});
+    total_ = align_up(total_ + bytes, 256);
+  }
+  int upload(DevicePool::Block* block) {
+    CUDA_TRY(DevicePool::pool().take(block, total_));
+    std::vector<uint8_t> host(total_, 0);
     for (const Part& p : parts_) {
-      *p.dst = static_cast<uint8_t*>(*block) + p.at;
-      if (p.bytes >= kDirect) CUDA_TRY(cudaMemcpy(*p.dst, p.src, p.bytes, cudaMemcpyHostToDevice));
-      else if (p.src) std::memcpy(host.data() + p.at, p.src, p.bytes);
+      *p.dst = static_cast<uint8_t*>(block->ptr) + p.at;
+      if (p.src) std::memcpy(host.data() + p.at, p.src, p.bytes);
     }
-    if (image) CUDA_TRY(cudaMemcpy(*block, host.data(), image, cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(block->ptr, host.data(), total_, cudaMemcpyHostToDevice));
     return QCONV_OK;
   }
 
  private:
   struct Part { void** dst; const void* src; size_t bytes, at; };
   std::vector<Part> parts_;
+  size_t total_ = 0;
 };
+
+// The layer's weights: a part of the handle's block, or (from 64 KB) a block of their own that a second handle of the
+// same weights can use too.  `from`: the handle they may be shared with, or NULL.
+int place_weights(qconv_handle* h, DeviceParts& parts, const int8_t* w, size_t bytes, bool as_is, const qconv_handle* from) {
+  h->weights_as_is = as_is;
+  if (bytes < 64 * 1024) {
+    parts.add(&h->d_w, w, bytes);
+    return QCONV_OK;
+  }
+  if (as_is && from && from->weights && from->weights_as_is && from->device == h->device && from->d.K == h->d.K &&
+      from->d.R == h->d.R && from->d.S == h->d.S && from->d.C == h->d.C && from->algo == h->algo) {
+    h->weights = from->weights;
+  } else {
+    h->weights = std::make_shared<DevicePool::Block>();
+    CUDA_TRY(DevicePool::pool().take(h->weights.get(), bytes));
+    CUDA_TRY(cudaMemcpy(h->weights->ptr, w, bytes, cudaMemcpyHostToDevice));
+  }
+  h->d_w = static_cast<int8_t*>(h->weights->ptr);
+  return QCONV_OK;
+}
 
 // Multiplier and shift for the kernel's divisions by d (1 <= d < 2^31), checked against plain division.
 qc::FastDiv make_fastdiv(int d_in) {
@@ -317,8 +407,8 @@ typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const qc::PairP
                            const qc::EpilogueParams, const int4*, void*, int*, unsigned int);
 PairKernel pair_kernel_for(const qconv_handle* h);
 
-int plan_igemm(qconv_handle* h, DeviceParts& parts, const int8_t* w_krsc /* host [K][R][S][Cg] */, const int32_t* bias_host,
-               const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host) {
+int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_of, const int8_t* w_krsc /* host [K][R][S][Cg] */,
+               const int32_t* bias_host, const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host) {
   const qconv_desc& d = h->d;
   const qconv_plan_hints& hint = h->hints;
   qc::IgemmParams& p = h->prm;
@@ -693,7 +783,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const int8_t* w_krsc /* host
         std::memcpy(dst + static_cast<size_t>(t) * p.nchunks * p.BKC, src + static_cast<size_t>(t) * d.C, d.C);
     }
   }
-  parts.add(&h->d_w, as_is ? w_krsc : wp.data(), w_bytes);
+  int rc = place_weights(h, parts, as_is ? w_krsc : wp.data(), w_bytes, as_is, weights_of);
+  if (rc) return rc;
   std::vector<int4> chan(h->kpad, make_int4(0, 0, 0, 0));
   for (int k = 0; k < d.K; ++k) {
     const int sft = shift_host ? shift_host[k] : 0;
@@ -722,7 +813,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const int8_t* w_krsc /* host
   for (int j = 1; j < h->fold; ++j)
     for (int k = 0; k < d.K; ++k) chan[static_cast<size_t>(j) * d.K + k] = chan[k];
   parts.add(&h->d_chan, chan.data(), sizeof(int4) * chan.size());
-  int rc = parts.upload(&h->d_block);
+  rc = parts.upload(&h->block);
   if (rc) return rc;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->kg_total), static_cast<cuuint64_t>(h->kpad)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->kg_total)};
@@ -1048,6 +1139,12 @@ int qconv_set_plan_hints(const qconv_plan_hints* hints) {
 int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host,
                  const int32_t* bias_host, const int32_t* shift_host,
                  const int32_t* res_lshift_host, const int32_t* acc_exp_host) {
+  return qconv_create_sharing(out, desc, w_host, bias_host, shift_host, res_lshift_host, acc_exp_host, nullptr);
+}
+
+int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host, const int32_t* bias_host,
+                         const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
+                         const qconv_handle* weights_of) {
   if (!out) return fail(QCONV_ERR_BAD_ARG, "out is NULL");
   *out = nullptr;
   if (!desc || !w_host) return fail(QCONV_ERR_BAD_ARG, "desc or w_host is NULL");
@@ -1184,7 +1281,7 @@ int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
   parts.add(&h->d_status, nullptr, 2 * sizeof(int));       // status word, maximum of qconv_run_maxabs
   int rc = QCONV_OK;
   if (algo == QCONV_ALGO_IGEMM) {
-    rc = plan_igemm(h, parts, w_krsc, bias_host, shift_host, res_lshift_host, acc_exp_host);
+    rc = plan_igemm(h, parts, weights_of, w_krsc, bias_host, shift_host, res_lshift_host, acc_exp_host);
   } else {
     if (bias_host) parts.add(&h->d_bias, bias_host, sizeof(int32_t) * d.K);
     parts.add(&h->d_shift, shift_host, sizeof(int32_t) * d.K);
@@ -1195,7 +1292,7 @@ int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
     // [R][S][Cg][K]; for depthwise Cg == 1 this is [R*S][C]
     for (int k = 0; k < d.K; ++k)
       for (size_t j = 0; j < per_k; ++j) wp[j * d.K + k] = w_krsc[k * per_k + j];
-    parts.add(&h->d_w, wp.data(), wcount);
+    rc = place_weights(h, parts, wp.data(), wcount, false, nullptr);
     // Depthwise fast path (tap-packed dp4a with float-magic requantization, exact while
     // |bias| + 9 * 128 * 128 < 2^22): int8 output, nearest-even, 8-bit saturation, no residual.
     std::vector<uint32_t> t;
@@ -1221,7 +1318,7 @@ int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       h->dw_tap = 1;
       if (d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
     }
-    rc = parts.upload(&h->d_block);
+    if (!rc) rc = parts.upload(&h->block);
   }
   if (rc) {
     free_handle(h);

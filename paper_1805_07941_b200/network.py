@@ -98,11 +98,13 @@ class QNetwork:
                     groups=nd["groups"], relu=nd["relu"], n_in=self.n_bits, n_w=self.n_bits,
                     n_out=self.n_bits, rounding=self.rounding)
 
-    def _make_handle(self, nd, N=None, register=True):
+    def _make_handle(self, nd, N=None, register=True, weights_of=None):
         """The int8 handle of a convolution from self.params; with a fusable pool behind it, the handle that pools
-        inside the layer and writes the pool's buffer (when the library takes the shape)."""
+        inside the layer and writes the pool's buffer (when the library takes the shape).  weights_of: a handle of the
+        same weights."""
         p = self.params[nd["name"]]
-        common = dict(symmetric=nd["symmetric"], has_residual=int(p["res_lshift"] is not None), **self._geom(nd, N))
+        common = dict(symmetric=nd["symmetric"], has_residual=int(p["res_lshift"] is not None), weights_of=weights_of,
+                      **self._geom(nd, N))
         args = (p["wq"], p["bias_q"], p["shift"], p["res_lshift"], None)
         pool = self._pool_after.get(nd["name"]) if self.fuse_pool else None
         if pool is not None:
@@ -180,7 +182,7 @@ class QNetwork:
                                         out=self.bufs[nd0["dst"]][:n])
                 self.e_buf[nd0["dst"]] = self.e_buf[nd0["src"]]
                 continue
-            cands = []
+            cands, floats = [], {}
             for nd in stage:
                 wq, e_w = quantized[nd["name"]]
                 b = self.weights[nd["name"]][1]
@@ -202,7 +204,7 @@ class QNetwork:
                         fbuf = torch.empty(need, dtype=torch.float32, device=self.device)
                     fl.run(self.bufs[nd["src"]], fbuf, res, n_run=n)
                     st = collect(fbuf[:need])
-                fl.destroy()
+                floats[nd["name"]] = fl
                 if keep_stats:
                     self.stats[nd["name"]] = st
                 cands.append(binding.qscale_exponent(gamma_of(st), self.n_bits))
@@ -214,7 +216,8 @@ class QNetwork:
                 p["shift"] = binding.qrequant_shifts(e_z, p["acc_exp"])
                 if nd["name"] in self.handles:
                     self.handles[nd["name"]].destroy()
-                hnd = self._make_handle(nd)
+                hnd = self._make_handle(nd, weights_of=floats[nd["name"]])
+                floats[nd["name"]].destroy()
                 self.handles[nd["name"]] = hnd
                 hnd.run(self.bufs[nd["src"]], self._conv_dst(nd), self._residual(nd), n_run=n)
             self.e_buf[nd0["dst"]] = e_z
@@ -398,7 +401,7 @@ class QNetwork:
                 for nd in self.net["nodes"]:
                     if nd["op"] != "conv":
                         continue
-                    hs[nd["name"]] = self._make_handle(nd, n_sub, register=False)
+                    hs[nd["name"]] = self._make_handle(nd, n_sub, register=False, weights_of=self.handles[nd["name"]])
                 sets.append(hs)
             self._parts[parts] = sets
         return self._parts[parts]

@@ -59,3 +59,32 @@ def test_step_list_reports_the_first_error():
     with pytest.raises(binding.QconvError) as e:
         binding.Steps([dict(op=binding.NET_QUANTIZE, count=16, n_bits=8)]).run(None)
     assert e.value.code == binding.ERR_BAD_ARG
+
+
+@pytest.mark.parametrize("K,C", [(16, 32), (64, 128), (128, 512), (96, 512), (100, 512)])
+def test_handles_of_the_same_weights_share_them_in_any_order_of_destruction(K, C):
+    """Below and above the size from which weights have a block of their own; layouts that agree and that do not."""
+    import torch
+    from oracle import ref
+    rng = np.random.default_rng(K)
+    x = rng.integers(-128, 128, (2, 6, 5, C), dtype=np.int8)
+    w = rng.integers(-8, 8, (K, 3, 3, C), dtype=np.int8)
+    acc_exp, shift = np.full(K, -10, np.int32), np.full(K, 9, np.int32)
+    geom = dict(N=2, H=6, W=5, C=C, K=K, R=3, S=3, pad_h=1, pad_w=1)
+    want_f = ref.qconv(x, w, None, None, None, None, acc_exp, R=3, S=3, pad=(1, 1), out_mode=2)
+    want = ref.qconv(x, w, None, shift, R=3, S=3, pad=(1, 1))
+    xd = torch.from_numpy(x).cuda()
+    for first_gone in (0, 1):
+        fl = binding.QConv(w, None, None, None, acc_exp, out_mode=binding.OUT_FLOAT, **geom)
+        q8 = binding.QConv(w, None, shift, weights_of=fl, **geom)
+        other = binding.QConv(np.zeros_like(w), None, shift, **geom)
+        (fl, q8)[first_gone].destroy()
+        junk = [binding.QConv(rng.integers(-8, 8, w.shape, dtype=np.int8), None, shift, **geom) for _ in range(3)]   # reuses what was given back
+        if first_gone == 0:
+            y = torch.empty(want.shape, dtype=torch.int8, device="cuda")
+            assert (q8.run(xd, y).cpu().numpy() == want).all(), q8.describe()
+        else:
+            y = torch.empty(want.shape, dtype=torch.float32, device="cuda")
+            assert (fl.run(xd, y).cpu().numpy() == want_f).all(), fl.describe()
+        for h in [fl, q8, other] + junk:
+            h.destroy()
