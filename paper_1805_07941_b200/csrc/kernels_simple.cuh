@@ -31,7 +31,7 @@ __device__ __forceinline__ int quantize_one(float v, float gam, float inv_alpha,
   return __float2int_rn(r);
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 quantize_f32_kernel(const float* __restrict__ x, int8_t* __restrict__ y, size_t count, int e, int n,
                     int vec_ok) {
   chain_sync();
@@ -41,29 +41,22 @@ quantize_f32_kernel(const float* __restrict__ x, int8_t* __restrict__ y, size_t 
   const float inv_alpha = use_mul ? ldexpf(1.0f, -e) : 0.0f;
   const size_t tid = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
   const size_t nthreads = static_cast<size_t>(gridDim.x) * blockDim.x;
-  size_t nvec = vec_ok ? count / 16 : 0;
+  // consecutive threads take consecutive words, four loads in flight each
+  const size_t nvec = vec_ok ? count / 4 : 0;
   const float4* x4 = reinterpret_cast<const float4*>(x);
-  uint4* y16 = reinterpret_cast<uint4*>(y);
-  for (size_t i = tid; i < nvec; i += nthreads) {
-    if (!QC_IN(16 * i + 15, count)) continue;
-    float4 a = __ldg(x4 + 4 * i), b = __ldg(x4 + 4 * i + 1), c = __ldg(x4 + 4 * i + 2),
-           d = __ldg(x4 + 4 * i + 3);
-    float f[16] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
-    uint32_t wds[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      uint32_t wd = 0;
-#pragma unroll
-      for (int b8 = 0; b8 < 4; ++b8) {
-        int q = quantize_one(f[4 * j + b8], gam, inv_alpha, e, use_mul, bmax);
-        wd |= (static_cast<uint32_t>(q) & 0xFFu) << (8 * b8);
-      }
-      wds[j] = wd;
-    }
-    y16[i] = make_uint4(wds[0], wds[1], wds[2], wds[3]);
+  uint32_t* y4 = reinterpret_cast<uint32_t*>(y);
+  auto one = [&](float v) { return static_cast<uint32_t>(quantize_one(v, gam, inv_alpha, e, use_mul, bmax)) & 0xFFu; };
+  auto word = [&](const float4& v) { return one(v.x) | (one(v.y) << 8) | (one(v.z) << 16) | (one(v.w) << 24); };
+  size_t i = tid;
+  for (; i + 3 * nthreads < nvec; i += 4 * nthreads) {
+    if (!QC_IN(4 * (i + 3 * nthreads) + 3, count)) continue;
+    const float4 a = __ldg(x4 + i), b = __ldg(x4 + i + nthreads), c = __ldg(x4 + i + 2 * nthreads), d = __ldg(x4 + i + 3 * nthreads);
+    y4[i] = word(a); y4[i + nthreads] = word(b); y4[i + 2 * nthreads] = word(c); y4[i + 3 * nthreads] = word(d);
   }
-  for (size_t i = nvec * 16 + tid; i < count; i += nthreads)
-    y[i] = static_cast<int8_t>(quantize_one(x[i], gam, inv_alpha, e, use_mul, bmax));
+  for (; i < nvec; i += nthreads)
+    if (QC_IN(4 * i + 3, count)) y4[i] = word(__ldg(x4 + i));
+  for (size_t j = nvec * 4 + tid; j < count; j += nthreads)
+    y[j] = static_cast<int8_t>(quantize_one(x[j], gam, inv_alpha, e, use_mul, bmax));
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1763,26 +1763,34 @@ int qconv_destroy(qconv_handle* h) {
 static __device__ __align__(256) unsigned char g_calib_static_scratch[sizeof(qc::CalibScratch)];
 
 namespace {
-std::mutex g_calib_mu;
-qc::CalibScratch* g_calib_scratch[64] = {nullptr};       // cudaMalloc'ed on first use, per device
-qc::CalibScratch* g_calib_static_ptr[64] = {nullptr};    // device address of the built-in array, per device
+// Device scratch of qcalib_collect and pinned memory its results land in, both made on first use per device and kept.
+struct CalibDevice {
+  std::mutex mu;                                           // one collection at a time on a device's scratch
+  qc::CalibScratch* scratch = nullptr;
+  qc::CalibScratch* built_in = nullptr;                    // device address of the array in the library image
+  qc::CalibResult* landing = nullptr;
+};
+CalibDevice g_calib[64];
 
-// The statistics pass shared by both entry points: clear, maximum + sums, finalize, histogram, copy
-// back.  `sc` is device scratch the caller provides (it still holds the previous call's counters).
+// The statistics passes shared by both entry points: maximum + sums, histogram, results.  `sc` is device scratch whose
+// accumulators are zero (every collection leaves them so); `landing`: pinned host memory the second pass writes the
+// results to, or NULL to copy them to pageable memory.
 int calib_run(const float* d_x, size_t count, int nbins, float range_hi, qcalib_stats* host_out,
-              cudaStream_t st, qc::CalibScratch* sc) {
+              cudaStream_t st, qc::CalibScratch* sc, qc::CalibResult* landing) {
   const int vec_ok = (reinterpret_cast<uintptr_t>(d_x) & 15) == 0;
-  const int blocks = grid_for((count + 3) / 4, 256, 148 * 8);
-  CUDA_TRY(cudaMemsetAsync(sc, 0, offsetof(qc::CalibScratch, part_sum), st));
-  qc::calib_pass1_kernel<<<blocks, 256, 0, st>>>(d_x, count, sc, vec_ok);
-  qc::calib_finalize_kernel<<<1, 256, 0, st>>>(sc, blocks, static_cast<unsigned long long>(count));
-  qc::calib_hist_kernel<<<blocks, 256, nbins * sizeof(unsigned int), st>>>(d_x, count, sc, nbins, range_hi, vec_ok);
-  CUDA_TRY(cudaGetLastError());
-  struct { unsigned int maxabs_bits, pad; unsigned long long finite, nonfinite; double sum, sumsq; } head;
-  CUDA_TRY(cudaMemcpyAsync(&head, sc, sizeof(head), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(host_out->hist, reinterpret_cast<const unsigned char*>(sc) + offsetof(qc::CalibScratch, hist),
-                           sizeof(uint64_t) * nbins, cudaMemcpyDeviceToHost, st));
+  const size_t vecs = (count + 3) / 4;
+  CUDA_TRY(launch_chained(qc::calib_pass1_kernel, dim3(grid_for(vecs, 256, 148 * qc::kCalibBlocksPerSm)), dim3(256), 0, st, d_x, count, sc,
+                          nbins, vec_ok));
+  CUDA_TRY(launch_chained(qc::calib_hist_kernel, dim3(grid_for(vecs, qc::kCalibHistThreads, 148 * 2)), dim3(qc::kCalibHistThreads),
+                          nbins * sizeof(unsigned int), st, d_x, count, sc, nbins, range_hi, vec_ok, landing));
+  qc::CalibResult pageable;
+  if (!landing) {
+    CUDA_TRY(cudaMemcpyAsync(&pageable, &sc->res, offsetof(qc::CalibResult, hist) + sizeof(uint64_t) * nbins, cudaMemcpyDeviceToHost, st));
+    landing = &pageable;
+  }
   CUDA_TRY(cudaStreamSynchronize(st));
+  const qc::CalibHead head = landing->head;
+  std::memcpy(host_out->hist, landing->hist, sizeof(uint64_t) * nbins);
   std::memcpy(&host_out->maxabs, &head.maxabs_bits, sizeof(float));
   host_out->range_hi = range_hi > 0.0f ? range_hi : host_out->maxabs;
   host_out->count = head.finite;
@@ -1804,13 +1812,21 @@ int qcalib_collect(const float* d_x, size_t count, int nbins, float range_hi, qc
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(QCONV_ERR_CUDA, "device index %d out of range", dev);
-  qc::CalibScratch* sc;
-  {
-    std::lock_guard<std::mutex> lock(g_calib_mu);
-    if (!g_calib_scratch[dev]) CUDA_TRY(cudaMalloc(&g_calib_scratch[dev], sizeof(qc::CalibScratch)));
-    sc = g_calib_scratch[dev];
+  CalibDevice& d = g_calib[dev];
+  std::lock_guard<std::mutex> lock(d.mu);
+  if (!d.landing) CUDA_TRY(cudaHostAlloc(&d.landing, sizeof(qc::CalibResult), cudaHostAllocPortable));
+  if (!d.scratch) {
+    qc::CalibScratch* sc = nullptr;
+    CUDA_TRY(cudaMalloc(&sc, sizeof(qc::CalibScratch)));
+    const cudaError_t e = cudaMemset(sc, 0, sizeof(qc::CalibScratch));
+    if (e != cudaSuccess) {
+      cudaFree(sc);
+      return fail(QCONV_ERR_CUDA, "calibration scratch: %s", cudaGetErrorString(e));
+    }
+    d.scratch = sc;
+    CUDA_TRY(cudaDeviceSynchronize());                     // (the caller's stream may not wait for the legacy stream)
   }
-  return calib_run(d_x, count, nbins, range_hi, host_out, static_cast<cudaStream_t>(cuda_stream), sc);
+  return calib_run(d_x, count, nbins, range_hi, host_out, static_cast<cudaStream_t>(cuda_stream), d.scratch, d.landing);
 }
 
 // ----------------------------------------------------------- calibration without allocation
@@ -1827,21 +1843,20 @@ int qcalib_collect_static(const float* d_x, size_t count, int nbins, float range
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(QCONV_ERR_CUDA, "device index %d out of range", dev);
-  qc::CalibScratch* sc;
+  CalibDevice& d = g_calib[dev];
   {
     // first call on this device: translate the symbol into this device's address (no allocation)
-    std::lock_guard<std::mutex> lock(g_calib_mu);
-    if (!g_calib_static_ptr[dev]) {
+    std::lock_guard<std::mutex> lock(d.mu);
+    if (!d.built_in) {
       void* ptr = nullptr;
       cudaError_t e = cudaGetSymbolAddress(&ptr, g_calib_static_scratch);
       if (e != cudaSuccess || !ptr)
         return fail(QCONV_ERR_CUDA, "cudaGetSymbolAddress(built-in calibration scratch): %s", cudaGetErrorString(e));
-      g_calib_static_ptr[dev] = static_cast<qc::CalibScratch*>(ptr);
+      d.built_in = static_cast<qc::CalibScratch*>(ptr);
     }
-    sc = g_calib_static_ptr[dev];
   }
-  // the array still holds the previous call's counters: calib_run clears everything that accumulates
-  return calib_run(d_x, count, nbins, range_hi, host_out, static_cast<cudaStream_t>(cuda_stream), sc);
+  // the array starts out zero with the library image, and every collection leaves its accumulators so
+  return calib_run(d_x, count, nbins, range_hi, host_out, static_cast<cudaStream_t>(cuda_stream), d.built_in, nullptr);
 }
 
 int qquantize_f32(const float* d_x, size_t count, int e, int n, int8_t* d_y, void* cuda_stream) {
@@ -1849,7 +1864,7 @@ int qquantize_f32(const float* d_x, size_t count, int e, int n, int8_t* d_y, voi
   if (n < 2 || n > 8 || e < -126 || e > 126) return fail(QCONV_ERR_BAD_ARG, "n in [2, 8], e in [-126, 126]");
   if (count == 0) return QCONV_OK;
   const int vec_ok = ((reinterpret_cast<uintptr_t>(d_x) | reinterpret_cast<uintptr_t>(d_y)) & 15) == 0;
-  CUDA_TRY(launch_input(qc::quantize_f32_kernel, dim3(grid_for((count + 15) / 16, 256, 148 * 16)), dim3(256),
+  CUDA_TRY(launch_input(qc::quantize_f32_kernel, dim3(grid_for((count + 3) / 4, 256, 148 * 6)), dim3(256),
                         static_cast<cudaStream_t>(cuda_stream), d_x, d_y, count, e, n, vec_ok));
   CUDA_TRY(cudaGetLastError());
   return QCONV_OK;
@@ -1925,11 +1940,19 @@ namespace {
 int make_format(int n, int p, int e, qc::DynFloatFormat* f) {
   if (n < 2 || n > 8 || p < 0 || p > n - 1) return fail(QCONV_ERR_BAD_ARG, "need 2 <= n <= 8 and 0 <= p <= n-1");
   if (e < -126 || e > 126) return fail(QCONV_ERR_BAD_ARG, "scale exponent %d outside [-126, 126]", e);
-  f->n = n; f->p = p; f->e = e;
-  f->e_max = (p == n - 1) ? 0 : (1 << (n - p - 1)) - 1;
+  f->n = n; f->p = p;
+  f->scale = std::ldexp(1.0f, -e);                         // normal for every e allowed here
+  f->ke_min = static_cast<uint32_t>(127 + p) << 23;
+  f->ke_up = static_cast<uint32_t>(23 - p) << 23;
+  f->ke_off = f->ke_up + (static_cast<uint32_t>(127 + p) << p);
+  // decoding reads the pattern as a binary32 number 2^(126 + p) too small; 2^(126 + p + e) may not be a binary32 number,
+  // so the factor is split (the first product is exact, and what overflows on the way overflows in the end)
+  f->up0 = std::ldexp(1.0f, 126);
+  f->up1 = std::ldexp(1.0f, (p + e) / 2);
+  f->up2 = std::ldexp(1.0f, p + e - (p + e) / 2);
   // Eq. 5 with equality: every pattern is a number
   f->beta_max = (p == n - 1) ? static_cast<float>((1 << (n - 1)) - 1)
-                             : std::ldexp(static_cast<float>((2 << p) - 1), f->e_max - 1);
+                             : std::ldexp(static_cast<float>((2 << p) - 1), (1 << (n - p - 1)) - 2);
   return QCONV_OK;
 }
 }  // namespace
@@ -1941,8 +1964,10 @@ int qquantize_f32_np(const float* d_x, size_t count, int e, int n, int p, uint8_
   if (rc) return rc;
   if (count == 0) return QCONV_OK;
   const int vec_ok = ((reinterpret_cast<uintptr_t>(d_x) | reinterpret_cast<uintptr_t>(d_code)) & 15) == 0;
-  qc::dynfloat_encode_kernel<<<grid_for((count + 15) / 16, 256, 148 * 16), 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      d_x, d_code, count, f, vec_ok);
+  const int grid = grid_for((count + 3) / 4, 256, 148 * 6);
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  if (p == 0) qc::dynfloat_encode_kernel<true><<<grid, 256, 0, st>>>(d_x, d_code, count, f, vec_ok);
+  else qc::dynfloat_encode_kernel<false><<<grid, 256, 0, st>>>(d_x, d_code, count, f, vec_ok);
   CUDA_TRY(cudaGetLastError());
   return QCONV_OK;
 }
@@ -1954,7 +1979,7 @@ int qdequantize_np(const uint8_t* d_code, size_t count, int e, int n, int p, flo
   if (rc) return rc;
   if (count == 0) return QCONV_OK;
   const int vec_ok = ((reinterpret_cast<uintptr_t>(d_y) | reinterpret_cast<uintptr_t>(d_code)) & 15) == 0;
-  qc::dynfloat_decode_kernel<<<grid_for((count + 15) / 16, 256, 148 * 16), 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+  qc::dynfloat_decode_kernel<<<grid_for((count + 3) / 4, 256, 148 * 6), 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
       d_code, d_y, count, f, vec_ok);
   CUDA_TRY(cudaGetLastError());
   return QCONV_OK;
@@ -2165,40 +2190,68 @@ int qthreshold_search(const uint64_t* hist_host, int nbins, float range_hi, int 
   if (rc != QCONV_OK) return rc;
 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // device scratch sized for the largest histogram, allocated once per device and kept
-  const size_t off_cdf = sizeof(uint64_t) * qc::kThrMaxBins;
-  const size_t off_fp = off_cdf + sizeof(double) * qc::kThrMaxBins;
-  const size_t off_del = off_fp + sizeof(double) * qc::kThrMaxLevels;
-  const size_t off_best = off_del + sizeof(double) * (qc::kThrMaxBins + 1);
-  static std::mutex mu;
-  static unsigned char* scratch[64] = {nullptr};
+  // device scratch sized for the largest histogram and pinned memory the operands leave from, made once per device and
+  // kept; [counts | grid] go up in one copy
+  struct Device {
+    std::mutex mu;                                         // calls on one device share the scratch: serialised
+    unsigned char* scratch = nullptr;
+    unsigned char* pinned = nullptr;
+    bool configured = false;                               // shared-memory limits of the kernels raised
+  };
+  static Device devices[64];
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(QCONV_ERR_CUDA, "device index %d out of range", dev);
-  std::lock_guard<std::mutex> lock(mu);                    // calls on one device share the scratch: serialised
-  if (!scratch[dev]) CUDA_TRY(cudaMalloc(&scratch[dev], off_best + sizeof(qc::ThresholdBest)));
-  unsigned char* d = scratch[dev];
-  auto* d_hist = reinterpret_cast<unsigned long long*>(d);
-  auto* d_cdf = reinterpret_cast<double*>(d + off_cdf);
-  auto* d_fp = reinterpret_cast<double*>(d + off_fp);
+  Device& dv = devices[dev];
+  const size_t off_fp = sizeof(uint64_t) * qc::kThrMaxBins;
+  const size_t off_del = off_fp + sizeof(double) * qc::kThrMaxLevels;
+  const size_t off_ticket = off_del + sizeof(double) * (qc::kThrMaxBins + 1);
+  std::lock_guard<std::mutex> lock(dv.mu);
+  if (!dv.pinned) CUDA_TRY(cudaHostAlloc(&dv.pinned, off_del + sizeof(qc::ThresholdBest), cudaHostAllocPortable));
+  if (!dv.scratch) {
+    unsigned char* sc = nullptr;
+    CUDA_TRY(cudaMalloc(&sc, off_ticket + sizeof(unsigned int)));
+    cudaError_t me = cudaMemset(sc, 0, off_ticket + sizeof(unsigned int));
+    if (me == cudaSuccess) me = cudaDeviceSynchronize();
+    if (me != cudaSuccess) {
+      cudaFree(sc);
+      return fail(QCONV_ERR_CUDA, "threshold scratch: %s", cudaGetErrorString(me));
+    }
+    dv.scratch = sc;
+  }
+  unsigned char* d = dv.scratch;
+  // the levels follow the bins in memory, so that the copy is as short as the histogram
+  const size_t at_fp = sizeof(uint64_t) * nbins;
+  std::memcpy(dv.pinned, hist_host, at_fp);
+  std::memcpy(dv.pinned + at_fp, fp_host, sizeof(double) * levels);
   auto* d_del = reinterpret_cast<double*>(d + off_del);
-  auto* d_best = reinterpret_cast<qc::ThresholdBest*>(d + off_best);
-  qc::ThresholdBest best = {};
-  cudaError_t e = cudaMemcpyAsync(d_hist, hist_host, sizeof(uint64_t) * nbins, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_fp, fp_host, sizeof(double) * levels, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_del, 0xFF, sizeof(double) * (nbins + 1), st);   // NaN outside the loop's range
+  // (pinned memory is mapped at the same address on the device; the kernel writes its answer there)
+  qc::ThresholdBest* best_host = reinterpret_cast<qc::ThresholdBest*>(dv.pinned + off_del);
+  const double top = p == n - 1 ? levels - 1.0 : std::ldexp(static_cast<double>((2 << p) - 1), (1 << (n - p - 1)) - 2);   // beta_max
+  cudaError_t e = cudaMemcpyAsync(d, dv.pinned, at_fp + sizeof(double) * levels, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && deltas_host) e = cudaMemsetAsync(d_del, 0xFF, sizeof(double) * (nbins + 1), st);   // NaN outside the loop's range
   if (e == cudaSuccess) {
-    qc::threshold_cdf_kernel<<<1, 1024, 0, st>>>(d_hist, nbins, d_cdf);
-    qc::threshold_candidates_kernel<<<nbins - first + 1, qc::kThrThreads, 0, st>>>(d_cdf, d_fp, nbins, levels, first,
-                                                                                  measure, std::ldexp(1.0, -52), d_del);
-    qc::threshold_argmin_kernel<<<1, qc::kThrThreads, 0, st>>>(d_del, first, nbins, d_best);
+    using Kernel = decltype(&qc::threshold_search_kernel<0>);
+    static const Kernel kernels[4] = {qc::threshold_search_kernel<qc::kMeasureL1>, qc::threshold_search_kernel<qc::kMeasureKS>,
+                                      qc::threshold_search_kernel<qc::kMeasureCvM>, qc::threshold_search_kernel<qc::kMeasureKL>};
+    if (!dv.configured) {
+      for (Kernel k : kernels) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(qc::threshold_smem(qc::kThrMaxBins)));
+        if (e != cudaSuccess) return fail(QCONV_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+      }
+      dv.configured = true;
+    }
+    kernels[measure]<<<ceil_div(nbins - first + 1, qc::kThrCandidates), qc::kThrThreads, qc::threshold_smem(nbins), st>>>(
+        reinterpret_cast<const unsigned long long*>(d), reinterpret_cast<const double*>(d + at_fp), nbins, levels, p,
+        p == n - 1 ? 1 : 0, static_cast<float>(top), first, std::ldexp(1.0, -52), d_del,
+        reinterpret_cast<unsigned int*>(d + off_ticket), best_host);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&best, d_best, sizeof(best), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && deltas_host)
     e = cudaMemcpyAsync(deltas_host, d_del, sizeof(double) * (nbins + 1), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(QCONV_ERR_CUDA, "qthreshold_search: %s", cudaGetErrorString(e));
+  const qc::ThresholdBest best = *best_host;
   *index_out = best.index;
   *delta_out = best.delta;
   // bin_edges[i] of nbins equal bins on [0, range_hi]; the last edge is range_hi itself
