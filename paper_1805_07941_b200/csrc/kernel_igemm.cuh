@@ -30,6 +30,7 @@ constexpr int kGroupsPerWarp = 4;     // 16-column groups per epilogue warp: BN 
 constexpr int kGroupsPerWarpWide = 8; // the instantiations for 256-wide tiles (one CTA per SM)
 constexpr int kIgemmThreads = 64 + 32 * kEpilogueWarps;
 constexpr int kMaxStages = 12;
+constexpr int kNpMaxProducts = 6;     // digit products of two operands of up to three digits
 constexpr int kTileM = 128;
 
 // Division of a non-negative 31-bit integer by a divisor fixed for the launch: q = umulhi(n, mul) >> shr with
@@ -96,6 +97,15 @@ struct IgemmParams {
   int b_resident;                  // 1: the CTA's weight tile (all chunks) is loaded once and stays in shared memory;
                                    //    the ring then carries activations only and the CTA keeps one channel tile
   uint32_t b_res_tx_bytes;         // bytes of that weight tile
+  int acc_bufs;                    // accumulator buffers in tensor memory: 2, or 1 when the products of EPI_NP leave no room
+  // EPI_NP, floating-point operands: the chunks of a tap are those of np_products digit products one after the other, each
+  // accumulated in BN columns of its own (np_cpp chunks per product)
+  int np_products, np_cpp;
+  FastDiv fd_np_cpp;
+  int np_a[kNpMaxProducts];        // plane of the activations that product m multiplies
+  int np_coef[kNpMaxProducts];     // weight of its accumulator in the 64-bit sum
+  int np_n, np_p;                  // output type
+  float np_top;                    // its beta_max
 };
 
 // Error codes written to the status word.
@@ -394,7 +404,8 @@ struct TileWalker {
 //   FAST_I8 / FAST_I8_RES: int8 output, nearest-even, 8-bit saturation, K % 16 == 0, aligned rows,
 //                          accumulator bound leaves room for the rounding constant; without / with residual
 //   I8: any rounding mode, bit width, alignment;  I32, F32: wide or float output;  MAX: the largest |float output|
-//                          alone, nothing is stored (general_tile below)
+//                          alone, nothing is stored
+//   NP: digit products of floating-point operands recombined in 64 bits and converted to the (n, p) output type
 //   FAST_I8_U / FAST_I8_RES_U: the same with one shift for all channels (per-layer scales): only the
 //                          bias is per channel, everything else sits in kernel parameters
 //   FLT_I8*:               the four fast variants again for layers whose wide value provably stays below
@@ -407,7 +418,7 @@ struct TileWalker {
 //                          on the bit patterns (positive floats order like integers).
 enum : int { EPI_FAST_I8 = 0, EPI_FAST_I8_RES = 1, EPI_I8 = 2, EPI_I32 = 3, EPI_F32 = 4, EPI_FAST_I8_U = 5,
              EPI_FAST_I8_RES_U = 6, EPI_FLT_I8 = 7, EPI_FLT_I8_RES = 8, EPI_FLT_I8_U = 9, EPI_FLT_I8_RES_U = 10,
-             EPI_MAX = 11 };
+             EPI_MAX = 11, EPI_NP = 12 };
 
 template <int EPI> struct EpiTraits {
   static constexpr bool flt = EPI >= EPI_FLT_I8 && EPI <= EPI_FLT_I8_RES_U;
@@ -592,6 +603,35 @@ __device__ __forceinline__ void gen_copy(int vec, uint8_t* stage, int8_t* base, 
   }
 }
 
+// v / 2^s -> pattern of the nearest value of an (n, p) type; ties to the even pattern; saturation at beta_max;
+// a zero magnitude is pattern 0.  The magnitude is first made a binary32 number with its last bit sticky (round to odd:
+// 24 bits hold at least two more than any of these types, so rounding again is exact), then a float addition rounds it
+// to the type's grid: see dynfloat_mag, whose constants these are.
+struct NpEncode {
+  uint32_t ke_min, ke_up, ke_off;
+  int p, sign_bit;
+  float top;
+};
+__device__ __forceinline__ uint32_t np_encode(long long v, int s, const NpEncode& f) {
+  const unsigned long long mag = v < 0 ? 0ull - static_cast<unsigned long long>(v) : static_cast<unsigned long long>(v);
+  const int lz = __clzll(static_cast<long long>(mag));
+  const unsigned long long m = mag << (lz & 63);
+  const uint32_t hi = static_cast<uint32_t>(m >> 32), lo = static_cast<uint32_t>(m);
+  const uint32_t sig = (hi >> 8) | (((hi & 0xFFu) | lo) != 0u ? 1u : 0u);   // 24 bits, the first one set
+  // value = sig * 2^(40 - lz - s); exponent field minus the implicit bit that sig carries
+  const float exact = __uint_as_float((static_cast<uint32_t>(63 - lz - s + 126) << 23) + sig);
+  const float a = fminf(mag ? exact : 0.0f, f.top);
+  const uint32_t ke = max(__float_as_uint(a) & 0x7F800000u, f.ke_min);
+  const float t = __uint_as_float(ke + f.ke_up) + a;
+  uint32_t code = (ke >> (23 - f.p)) + __float_as_uint(t) - ke - f.ke_off;
+  if (f.p == 0) {
+    // bare powers of two: the tie at 1.5 * 2^k goes to the even exponent field, the one at 1/2 to 0
+    const uint32_t fr = __float_as_uint(a) & 0x7FFFFFu, E = (__float_as_uint(a) >> 23) - 126u;
+    code = a >= 1.0f ? E + (fr + (E & 1u) > 0x400000u ? 1u : 0u) : (a > 0.5f ? 1u : 0u);
+  }
+  return code | ((v < 0 && code) ? 1u << f.sign_bit : 0u);
+}
+
 // v / 2^s rounded in the descriptor's mode, in one pass: (v + z + (cond & w & 1)) >> s with the addend z and the mask
 // bit of w made by the host (s = 0: both 0):
 //   nearest-even: z = 2^(s-1) - 1, cond = lowest bit of the truncated quotient;  half away: the same z, cond = v > 0;
@@ -712,7 +752,7 @@ __device__ __forceinline__ void epilogue_pool_16(const uint32_t (&acc)[16], uint
 // carries twice the tensor work per byte fetched and per instruction of the issuing thread; both
 // accumulator buffers together fill the tensor memory, hence one CTA per SM).
 template <int EPI, int RELU = 2, int RSTG = 0, int GPW = kGroupsPerWarp>
-__global__ void __launch_bounds__(kIgemmThreads, GPW > kGroupsPerWarp ? 1 : 2)
+__global__ void __launch_bounds__(kIgemmThreads, (GPW > kGroupsPerWarp || EPI == EPI_NP) ? 1 : 2)
 igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                 const __grid_constant__ CUtensorMap tmap_y, const __grid_constant__ CUtensorMap tmap_r,
                 const IgemmParams prm, const EpilogueParams ep, const int4* __restrict__ chan_table,
@@ -758,7 +798,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     if (EpiTraits<EPI>::res && RSTG == 1) ptx::prefetch_tmap(&tmap_r);
   }
   if (warp == 1) {
-    ptx::tmem_alloc(ptx::smem_u32(&sh->tmem_base), static_cast<uint32_t>(2 * prm.tmem_cols));
+    ptx::tmem_alloc(ptx::smem_u32(&sh->tmem_base), static_cast<uint32_t>(prm.acc_bufs * prm.tmem_cols));
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
@@ -794,6 +834,12 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       const uint32_t full = ptx::smem_u32(&sh->full[slot]);
       const uint32_t a_dst = tiles_addr + static_cast<uint32_t>(slot) * stage_bytes;
       const int w0 = tc.q0 * prm.stride_w - prm.pad_w + sx, h0 = tc.p0 * prm.stride_h - prm.pad_h + r;
+      int a_ci = ci;                                         // channel chunk of the activations
+      if (EPI == EPI_NP) {
+        int in_plane;
+        const int product = prm.fd_np_cpp.divmod(ci, &in_plane);
+        a_ci = prm.np_a[product] * prm.np_cpp + in_plane;
+      }
       if (doit) {
         ptx::mbar_expect_tx(full, prm.tx_bytes);
         if (!prm.b_resident) {
@@ -806,10 +852,10 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           }
         }
         if (first) ptx::grid_dependency_wait();
-        ptx::tma_load_4d(a_dst, &tmap_a, full, ci * prm.BKC, w0, h0, tc.n0);
+        ptx::tma_load_4d(a_dst, &tmap_a, full, a_ci * prm.BKC, w0, h0, tc.n0);
         if (prm.tap_boxes)
           for (int hs = 1; hs < prm.halo_s; ++hs)           // the filter row's other taps, each a box of its own
-            ptx::tma_load_4d(a_dst + static_cast<uint32_t>(hs) * prm.a_tap_bytes, &tmap_a, full, ci * prm.BKC, w0 + hs, h0, tc.n0);
+            ptx::tma_load_4d(a_dst + static_cast<uint32_t>(hs) * prm.a_tap_bytes, &tmap_a, full, a_ci * prm.BKC, w0 + hs, h0, tc.n0);
       }
     };
     // stages this CTA issues in all, and how many of them make up the first pass
@@ -929,13 +975,15 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       uint32_t phase = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++it) {
-        const int buf = it & 1;
-        const uint32_t use = static_cast<uint32_t>(it >> 1);
+        const int buf = (EPI == EPI_NP && prm.acc_bufs == 1) ? 0 : it & 1;
+        const uint32_t use = static_cast<uint32_t>((EPI == EPI_NP && prm.acc_bufs == 1) ? it : it >> 1);
         // the epilogue must have drained this accumulator buffer (two tiles ago)
         ok = wait_bounded<0, kHint>(ptx::smem_u32(&sh->acc_empty[buf]), (use & 1u) ^ 1u, wait_limit, sh, status);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * prm.tmem_cols);
+        uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * prm.tmem_cols);
+        const uint32_t d_tmem0 = d_tmem;
+        int np_chunk = 0, np_product = 0;                    // EPI_NP: position inside the tap's chunks
         uint32_t accumulate = 0;
         if (bres) {
           if (it == 0) {
@@ -975,6 +1023,15 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             ptx::mma_commit(empty0 + 8u * stage);             // stage free once these MMAs retire
           }
           accumulate = 1;
+          if (EPI == EPI_NP) {
+            // the next product starts its own columns, cleared by its first chunk of the first tap
+            if (++np_chunk == prm.np_cpp) {
+              np_chunk = 0;
+              if (++np_product == prm.np_products) np_product = 0;
+              d_tmem = d_tmem0 + static_cast<uint32_t>(np_product * prm.BN);
+              accumulate = kb + 1 < prm.nchunks ? 0u : 1u;
+            }
+          }
           if (++stage == prm.stages) { stage = 0; phase ^= 1u; a_desc = a_desc0; if (!bres) b_desc = b_desc0; }
           else { a_desc += desc_step; if (!bres) b_desc += b_step; }
           if (bres) b_desc += b_step;
@@ -1049,8 +1106,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     // it carries `ok == false` to the next barrier, which doubles as a vote, and all leave together.
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it, walk.next(prm)) {
       const TileCoord tc = walk.coord(prm);
-      const int buf = it & 1;
-      const uint32_t use = static_cast<uint32_t>(it >> 1);
+      const int buf = (EPI == EPI_NP && prm.acc_bufs == 1) ? 0 : it & 1;
+      const uint32_t use = static_cast<uint32_t>((EPI == EPI_NP && prm.acc_bufs == 1) ? it : it >> 1);
       if (res_staged) {
         walk_next.next(prm);
         if (etid == 0 && tile + static_cast<int>(gridDim.x) < total_tiles) {
@@ -1150,7 +1207,49 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             __syncwarp();
           }
         };
-        if (kLeanOk && lean) {
+        if constexpr (EPI == EPI_NP) {
+          const NpEncode f = {static_cast<uint32_t>(127 + prm.np_p) << 23, static_cast<uint32_t>(23 - prm.np_p) << 23,
+                              (static_cast<uint32_t>(23 - prm.np_p) << 23) + (static_cast<uint32_t>(127 + prm.np_p) << prm.np_p),
+                              prm.np_p, prm.np_n - 1, prm.np_top};
+          for (int i = 0; i * 16 < gen_cols; ++i) {
+            const uint32_t col = static_cast<uint32_t>(g_begin + i) * 16u;
+            long long v[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = lds_int4(chan + (col + j) * 16u).x;      // bias
+            ptx::tmem_ld_32x16(t_addr + col, acc_a);
+            for (int m = 0; m < prm.np_products; m += 2) {
+              ptx::tmem_ld_wait();
+              if (m + 1 < prm.np_products) ptx::tmem_ld_32x16(t_addr + static_cast<uint32_t>((m + 1) * prm.BN) + col, acc_b);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) v[j] += static_cast<long long>(static_cast<int32_t>(acc_a[j])) * prm.np_coef[m];
+              if (m + 1 < prm.np_products) {
+                ptx::tmem_ld_wait();
+                if (m + 2 < prm.np_products) ptx::tmem_ld_32x16(t_addr + static_cast<uint32_t>((m + 2) * prm.BN) + col, acc_a);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += static_cast<long long>(static_cast<int32_t>(acc_b[j])) * prm.np_coef[m + 1];
+              }
+            }
+            if ((i + 1) * 16 >= gen_cols) release();
+            uint32_t wds[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              uint32_t o[4];
+#pragma unroll
+              for (int b = 0; b < 4; ++b) {
+                const long long w = v[g * 4 + b];
+                const int s = lds_int4(chan + (col + g * 4 + b) * 16u).y;
+                o[b] = np_encode(ep.relu && w < 0 ? 0ll : w, s, f);
+              }
+              wds[g] = __byte_perm(__byte_perm(o[0], o[1], 0x0040), __byte_perm(o[2], o[3], 0x0040), 0x5410);
+            }
+            ptx::sts_uint4(ptx::smem_u32(gen_stage) + static_cast<uint32_t>(lane * kGenPitch + i * 16), wds[0], wds[1], wds[2], wds[3]);
+          }
+          if (gen_cols <= 0) release();
+          __syncwarp();
+          gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + prm.out_c_offset + gen_k0,
+                         static_cast<long long>(pix) * prm.out_c_pitch, row_ok, gen_cols, lane);
+          __syncwarp();
+        } else if (kLeanOk && lean) {
           // loads one group ahead of the arithmetic, as below, without the bookkeeping
           const uint32_t t0 = t_addr + lean_col0;
           const uint32_t c0 = chan + lean_col0 * (EpiTraits<EPI>::uni ? 4u : 16u);
@@ -1257,7 +1356,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
   __syncthreads();
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, static_cast<uint32_t>(2 * prm.tmem_cols));
+    ptx::tmem_dealloc(tmem_base, static_cast<uint32_t>(prm.acc_bufs * prm.tmem_cols));
   }
 }
 

@@ -3,11 +3,13 @@
 // 245760 for (8, 3)), so the sum of Eq. 6 is an exact integer sum -- but its terms do not fit the int8
 // operands of the MMA.  Each beta is therefore written in base 128 with balanced digits,
 //   beta = d_0 + 128 d_1 + 128^2 d_2,   d_0, d_1 in [-64, 63], the last digit whatever is left (<= 127),
-// the digit planes of the input are laid side by side along the channel axis, and the weights are
-// arranged so that output column group g collects every digit product of weight 128^g:
-//   acc_g = sum_i x_plane_i * w_plane_(g-i).
-// One int8 GEMM (int32 accumulators, exact) produces all groups; the kernel below adds them up in 64
-// bits, sum_g acc_g << 7g, adds the bias, applies ReLU and converts to the output type.
+// and the product of two betas is taken from products of single digits and of sums of two digits (Karatsuba; see
+// np_products in qconv_api.cu).  The kernel below writes the digit combinations of the input that these products need
+// as planes side by side along the channel axis.  One tensor-core layer (igemm_i8_kernel<EPI_NP>) then accumulates every
+// product in columns of its own (int32, exact), adds them up in 64 bits with their weights, adds the bias, applies ReLU
+// and converts to the output type in its epilogue.
+// 32 x 28 x 28 x 128 -> 128, 3x3, (8, 4): 115 -> 32 us against one GEMM over all digit pairs with its int32 sums
+// written out and combined by a third kernel.
 #pragma once
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -16,9 +18,10 @@
 
 namespace qc {
 
-struct NpFormat {
-  int n, p;
-  long long beta_max;
+// Digit combinations of the input: bit i of a mask takes digit i into the plane's sum.
+struct NpPlanes {
+  int count = 0;
+  int mask[6] = {0, 0, 0, 0, 0, 0};
 };
 
 // Pattern (without sign) -> beta (Eq. 2 with the exponent field of Eq. 4).
@@ -28,93 +31,65 @@ __device__ __forceinline__ int np_decode_mag(int c, int n, int p) {
   return E == 0 ? m : ((1 << p) + m) << (E - 1);
 }
 
-// Value on the type's grid -> pattern (without sign).
-__device__ __forceinline__ int np_code_of(unsigned long long v, int p) {
-  if (v < (2ull << p)) return static_cast<int>(v);          // subnormals and the first binade: the pattern is the value
-  const int L = 63 - __clzll(static_cast<long long>(v));
-  const int E = L - p + 1;
-  return (E << p) | static_cast<int>((v >> (E - 1)) - (1ull << p));
-}
-
-// acc / 2^s -> pattern of the nearest (n, p) value; ties to the even pattern; beyond beta_max saturates;
-// a zero magnitude is pattern 0 (Section 3 conversion, applied to an exact rational).
-__device__ __forceinline__ uint8_t np_encode_i64(long long acc, int s, NpFormat f) {
-  const unsigned long long mag = acc < 0 ? 0ull - static_cast<unsigned long long>(acc) : static_cast<unsigned long long>(acc);
-  if (mag == 0) return 0;
-  int code;
-  if (mag >= (static_cast<unsigned long long>(f.beta_max) << s)) {
-    code = (1 << (f.n - 1)) - 1;
-  } else {
-    const int L = 63 - __clzll(static_cast<long long>(mag));
-    const int k = L - s;                                    // acc / 2^s lies in [2^k, 2^(k+1)); k < 0: below 1
-    const int sp = k > f.p ? k - f.p : 0;                   // grid spacing 2^sp in that binade
-    const int sh = s + sp;
-    const unsigned long long q = sh < 64 ? mag >> sh : 0ull;
-    const unsigned long long lo = q << sp, hi = (q + 1) << sp;   // neighbours on the grid (hi may open the next binade)
-    const unsigned long long rem = mag - (q << sh);
-    const unsigned long long half = sh > 0 ? 1ull << (sh - 1) : 0ull;
-    const int c_lo = np_code_of(lo, f.p), c_hi = np_code_of(hi, f.p);
-    if (sh == 0 || rem < half) code = c_lo;
-    else if (rem > half) code = c_hi;
-    else code = (c_hi & 1) ? c_lo : c_hi;
-  }
-  return static_cast<uint8_t>(code | ((acc < 0 && code != 0) ? 1 << (f.n - 1) : 0));
-}
-
-// codes [pixels][C] -> digit planes [pixels][planes * C] (plane-major inside a pixel), 16 codes per thread.
+// codes [pixels][C] -> planes [pixels][planes][c_pad], 16 codes per thread.  Decoding, splitting and summing digits take
+// some forty instructions per code, so every block first makes a table of what each of the 256 patterns contributes to
+// the planes (a byte per plane), and a code costs a lookup and its share of a byte transpose.
 __global__ void __launch_bounds__(256)
-np_split_kernel(const uint8_t* __restrict__ codes, int8_t* __restrict__ planes, size_t pixels, int C, int n, int p,
-                int nplanes) {
+np_split_kernel(const uint8_t* __restrict__ codes, int8_t* __restrict__ planes, size_t pixels, int C, int c_pad, int n, int p,
+                int digits, NpPlanes pl) {
+  __shared__ uint32_t table[2][256];                       // planes 0-3, planes 4-5
+  {
+    const int c = threadIdx.x;
+    int beta = np_decode_mag(c & ((1 << (n - 1)) - 1), n, p);
+    if ((c >> (n - 1)) & 1) beta = -beta;
+    int dig[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (i < digits) {
+        // balanced digit in [-64, 63]; the last one keeps what is left
+        dig[i] = i + 1 < digits ? ((beta + 64) & 127) - 64 : beta;
+        beta = (beta - dig[i]) >> 7;
+      }
+    }
+    uint32_t w[2] = {0u, 0u};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      // a sum of at most two digits, which stays inside an int8
+      const int sum = ((pl.mask[k] & 1) ? dig[0] : 0) + ((pl.mask[k] & 2) ? dig[1] : 0) + ((pl.mask[k] & 4) ? dig[2] : 0);
+      w[k >> 2] |= static_cast<uint32_t>(sum & 0xFF) << (8 * (k & 3));
+    }
+    table[0][c] = w[0];
+    table[1][c] = w[1];
+  }
+  __syncthreads();
   chain_sync();
   const int cv = C / 16;
   const size_t total = pixels * cv;
   for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < total;
        idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
     const size_t pix = idx / cv;
-    const int c0 = static_cast<int>(idx % cv) * 16;
+    const int c0 = static_cast<int>(idx - pix * cv) * 16;
     if (!QC_IN(pix * C + c0 + 15, pixels * C)) continue;
     const uint4 raw = __ldg(reinterpret_cast<const uint4*>(codes + pix * C + c0));
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-    uint32_t out[3][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};
+    int8_t* dst = planes + pix * static_cast<size_t>(pl.count) * c_pad + c0;
+    for (int half = 0; half * 4 < pl.count; ++half) {
+      uint32_t o[4][4];                                    // [plane][word]
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = (w[j >> 2] >> (8 * (j & 3))) & 0xFF;
-      int beta = np_decode_mag(c & ((1 << (n - 1)) - 1), n, p);
-      if ((c >> (n - 1)) & 1) beta = -beta;
+      for (int j = 0; j < 4; ++j) {
+        uint32_t t[4];
+        transpose4x4(table[half][w[j] & 0xFFu], table[half][(w[j] >> 8) & 0xFFu], table[half][(w[j] >> 16) & 0xFFu],
+                     table[half][w[j] >> 24], t);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        if (i < nplanes) {
-          // balanced digit in [-64, 63]; the last plane keeps what is left
-          const int d = i + 1 < nplanes ? ((beta + 64) & 127) - 64 : beta;
-          beta = (beta - d) >> 7;
-          out[i][j >> 2] |= static_cast<uint32_t>(d & 0xFF) << (8 * (j & 3));
-        }
+        for (int k = 0; k < 4; ++k) o[k][j] = t[k];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int plane = 4 * half + k;
+        if (plane < pl.count && QC_IN(pix * pl.count * c_pad + static_cast<size_t>(plane) * c_pad + c0 + 15, pixels * pl.count * c_pad))
+          *reinterpret_cast<uint4*>(dst + static_cast<size_t>(plane) * c_pad) = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
       }
     }
-    int8_t* dst = planes + pix * static_cast<size_t>(nplanes) * C + c0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-      if (i < nplanes)
-        *reinterpret_cast<uint4*>(dst + static_cast<size_t>(i) * C) = make_uint4(out[i][0], out[i][1], out[i][2], out[i][3]);
-  }
-}
-
-// acc32 [pixels][groups * K] -> codes [pixels][K]: 64-bit recombination, bias, ReLU, conversion.
-__global__ void __launch_bounds__(256)
-np_combine_kernel(const int32_t* __restrict__ acc32, const int32_t* __restrict__ bias, const int32_t* __restrict__ shift,
-                  uint8_t* __restrict__ y, size_t pixels, int K, int groups, int relu, NpFormat fout) {
-  const size_t total = pixels * K;
-  for (size_t idx = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; idx < total;
-       idx += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const size_t pix = idx / K;
-    const int k = static_cast<int>(idx % K);
-    const int32_t* a = acc32 + pix * static_cast<size_t>(groups) * K + k;
-    long long v = bias ? static_cast<long long>(__ldg(bias + k)) : 0ll;
-    for (int g = 0; g < groups; ++g)
-      if (QC_IN(pix * static_cast<size_t>(groups) * K + k + static_cast<size_t>(g) * K, pixels * static_cast<size_t>(groups) * K))
-        v += static_cast<long long>(__ldg(a + static_cast<size_t>(g) * K)) << (7 * g);
-    if (relu && v < 0) v = 0;
-    y[idx] = np_encode_i64(v, __ldg(shift + k), fout);
   }
 }
 

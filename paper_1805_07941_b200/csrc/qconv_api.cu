@@ -182,6 +182,15 @@ struct qgraph_inputs {
   qc::GraphInputRecord rec;
 };
 
+// Digit products of a layer on floating-point operands (qconv_np_create): what the planner needs beyond the descriptor.
+struct NpSpec {
+  int products = 0, planes = 0;
+  int a_plane[qc::kNpMaxProducts], coef[qc::kNpMaxProducts];
+  int n_out, p_out;
+  float top;                                               // beta_max of the output type
+  const int8_t* w[qc::kNpMaxProducts];                     // per product: the weights' digit combination, [K][R][S][C]
+};
+
 struct qconv_handle {
   qconv_desc d;
   int P, Q, Cg, Kg;
@@ -190,6 +199,9 @@ struct qconv_handle {
   // device copies: the small tables in one block, large weights in a second one that handles of the same weights share
   DevicePool::Block block;
   std::shared_ptr<DevicePool::Block> weights;
+  int a_channels = 0;            // channels of the activation tensor (planes * padded C for floating-point operands)
+  const NpSpec* np = nullptr;    // set while the handle is built
+  int np_products = 0;
   bool weights_as_is = false;    // those weights lie as the host handed them over ([K][R][S][C])
   int8_t* d_w = nullptr;         // direct: [R][S][Cg][K]; depthwise: [R*S][C]; igemm: [Kpad][Kg_total]
   int32_t* d_bias = nullptr;
@@ -457,7 +469,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   h->fold = 1;
   // only with the 16-byte-store epilogues, which index nothing but the (replicated) channel table
   const long long fold_round_room = h->max_shift > 0 ? (1ll << (h->max_shift - 1)) : 0;
-  const bool fast_possible = d.out_mode == QCONV_OUT_INT8 && d.rounding == QCONV_ROUND_NEAREST_EVEN && d.n_out == 8 &&
+  const NpSpec* np = h->np;
+  const bool fast_possible = !np && d.out_mode == QCONV_OUT_INT8 && d.rounding == QCONV_ROUND_NEAREST_EVEN && d.n_out == 8 &&
                              h->acc_bound + fold_round_room <= 2147483647ll && hint.fast_epilogue != 0;
   if ((h->mode == MODE_FLAT || h->mode == MODE_STEM) && fast_possible && d.out_c_offset == 0 &&
       d.out_c_pitch == d.K && hint.fold != 0) {
@@ -511,6 +524,17 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   p.BKC = choose_bkc(c_eff);
   if (is_window_mode(h->mode)) p.BKC = c_eff <= 32 ? 32 : (c_eff <= 64 ? 64 : 128);   // a row is one chunk (two at most)
   p.nchunks = ceil_div(c_eff, p.BKC);
+  h->a_channels = d.C;
+  p.acc_bufs = 2;
+  p.np_products = p.np_cpp = 0;
+  if (np) {
+    p.np_products = h->np_products = np->products;
+    p.np_cpp = p.nchunks;
+    p.nchunks *= np->products;
+    h->a_channels = np->planes * p.np_cpp * p.BKC;
+    for (int m = 0; m < np->products; ++m) { p.np_a[m] = np->a_plane[m]; p.np_coef[m] = np->coef[m]; }
+    p.np_n = np->n_out; p.np_p = np->p_out; p.np_top = np->top;
+  }
   p.R = taps_r; p.S = taps_s;
   int bn_max = std::min(2 * qc::kGroupsPerWarp * 16, std::max(16, (hint.bn_max > 0 ? hint.bn_max : 128) / 16 * 16));
   cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -557,7 +581,14 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     }
     if (m_tiles * ceil_div(k_eff, 128) < h->num_sms) bn_max = 64;
   }
-  halo = halo_fits && (bn_max <= 64 || k_eff <= 64 || hint.halo == 1);
+  if (np) {
+    // Every product has accumulator columns of its own, side by side: two buffers of them fill the tensor memory as long
+    // as products * BN <= 256; five and six products take one buffer (their tiles are long, the epilogue is not).
+    const int cols = np->products <= 4 ? 256 : 512;
+    bn_max = std::min({bn_max, 128, cols / np->products / 16 * 16});
+    p.acc_bufs = np->products <= 4 ? 2 : 1;
+  }
+  halo = halo_fits && (bn_max <= 64 || k_eff <= 64 || (np && np->products >= 3) || hint.halo == 1);
   if (halo) {
     wide = false;
     h->pair = 0;
@@ -602,11 +633,11 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   p.out_c_offset = d.out_c_offset;
   p.out_c_pitch = h->fold > 1 ? k_eff : d.out_c_pitch;
   p.tmem_cols = 32;
-  while (p.tmem_cols < p.BN) p.tmem_cols *= 2;            // two such buffers are allocated
+  while (p.tmem_cols < p.BN * std::max(1, p.np_products)) p.tmem_cols *= 2;   // acc_bufs such buffers are allocated
   cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
   h->ctas_per_sm = hint.ctas_per_sm == 1 ? 1 : 2;
   h->use_pdl = hint.pdl != 0 ? 1 : 0;
-  if (2 * p.tmem_cols * h->ctas_per_sm > 512) h->ctas_per_sm = 1;
+  if (p.acc_bufs * p.tmem_cols * h->ctas_per_sm > 512 || np) h->ctas_per_sm = 1;
   if (halo) {
     // A halo-form layer with no more tiles than SMs runs one CTA per SM at most: give that CTA the whole
     // shared memory (its stages are large, and its one chain of stages is as fast as the ring is deep).
@@ -617,7 +648,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   }
   p.vec_store = (p.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && k_eff % 16 == 0) ? 1 : 0;
   const long long round_room = h->max_shift > 0 ? (1ll << (h->max_shift - 1)) : 0;
-  p.fast_epilogue = (d.out_mode == QCONV_OUT_INT8 && d.rounding == QCONV_ROUND_NEAREST_EVEN && p.vec_store &&
+  p.fast_epilogue = (!np && d.out_mode == QCONV_OUT_INT8 && d.rounding == QCONV_ROUND_NEAREST_EVEN && p.vec_store &&
                      d.n_out == 8 &&
                      h->acc_bound + round_room <= 2147483647ll) ? 1 : 0;
   if (hint.fast_epilogue == 0) p.fast_epilogue = 0;
@@ -726,10 +757,16 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
 
   // weights -> [kpad][kg_total], K-major rows, zero padded (already in that form when nothing is padded or folded)
   const size_t w_bytes = static_cast<size_t>(h->kpad) * h->kg_total;
-  const bool as_is = h->fold == 1 && !is_window_mode(h->mode) && h->mode != MODE_STEM && h->kpad == d.K && p.nchunks * p.BKC == d.C;
+  const bool as_is = h->fold == 1 && !is_window_mode(h->mode) && h->mode != MODE_STEM && h->kpad == d.K && p.nchunks * p.BKC == d.C &&
+                     !np;
   std::vector<int8_t> wp(as_is ? 0 : w_bytes, 0);
   std::vector<int8_t> row(static_cast<size_t>(std::max(c_row, 1)), 0);
-  for (int k = 0; k < d.K && !as_is; ++k) {
+  for (int m = 0; np && m < np->products; ++m)             // [product][chunk] inside a tap
+    for (int k = 0; k < d.K; ++k)
+      for (int t = 0; t < d.R * d.S; ++t)
+        std::memcpy(wp.data() + static_cast<size_t>(k) * h->kg_total + (static_cast<size_t>(t) * p.nchunks + m * p.np_cpp) * p.BKC,
+                    np->w[m] + (static_cast<size_t>(k) * d.R * d.S + t) * d.C, d.C);
+  for (int k = 0; k < d.K && !as_is && !np; ++k) {
     const int8_t* src = w_krsc + static_cast<size_t>(k) * d.R * d.S * h->Cg;
     if (h->fold > 1 && !is_window_mode(h->mode)) {
       // one pixel's row as the unfolded GEMM would see it, then once per folded pixel on the diagonal
@@ -789,8 +826,9 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   for (int k = 0; k < d.K; ++k) {
     const int sft = shift_host ? shift_host[k] : 0;
     const int t = (d.has_residual && res_lshift_host) ? res_lshift_host[k] : 0;
-    chan[k] = make_int4(bias_host ? bias_host[k] : 0, sft, sft > 0 ? (1 << (sft - 1)) - 1 : 0,
+    chan[k] = make_int4(bias_host ? bias_host[k] : 0, sft, sft > 0 ? (1 << ((sft - 1) & 31)) - 1 : 0,
                         (sft > 0 ? 1 : 0) | ((1 << t) << 1));
+    if (np) { chan[k].z = chan[k].w = 0; continue; }         // (shifts up to 40)
     if (d.rounding >= QCONV_ROUND_HALF_UP) {                   // (general_round: no condition, another addend)
       chan[k].z = (d.rounding == QCONV_ROUND_HALF_UP && sft > 0) ? 1 << (sft - 1) : 0;
       chan[k].w &= ~1;
@@ -859,7 +897,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I8>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I32>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_F32>),
-                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_MAX>)}) {
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_MAX>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_NP>)}) {
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
       if (e != cudaSuccess) attr_err = e;
     }
@@ -890,6 +929,7 @@ PairKernel pair_kernel_for(const qconv_handle* h) {
 
 IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
   if (maxabs) return qc::igemm_i8_kernel<qc::EPI_MAX>;
+  if (h->np_products) return qc::igemm_i8_kernel<qc::EPI_NP>;
   if (h->d.out_mode == QCONV_OUT_INT32) return qc::igemm_i8_kernel<qc::EPI_I32>;
   if (h->d.out_mode == QCONV_OUT_FLOAT) return qc::igemm_i8_kernel<qc::EPI_F32>;
   if (!h->prm.fast_epilogue) return qc::igemm_i8_kernel<qc::EPI_I8>;
@@ -934,12 +974,13 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
   if (h->a_key_ptr == a_ptr && h->a_key_n == n_run) return QCONV_OK;
   const qconv_desc& d = h->d;
   qc::IgemmParams& p = h->prm;
+  const cuuint64_t ac = static_cast<cuuint64_t>(h->a_channels);
   cuuint64_t dims[4], strides[3];
   cuuint32_t estr[4] = {1, 1, 1, 1};
   cuuint32_t box[4] = {static_cast<cuuint32_t>(p.BKC), static_cast<cuuint32_t>(p.tq),
                        static_cast<cuuint32_t>(p.tp), static_cast<cuuint32_t>(p.tn)};
   if (h->mode == MODE_FLAT || h->mode == MODE_STEM) {
-    const cuuint64_t c = static_cast<cuuint64_t>(h->mode == MODE_STEM ? h->kg_pad : d.C) * h->fold;
+    const cuuint64_t c = static_cast<cuuint64_t>(h->mode == MODE_STEM ? h->kg_pad : ac) * h->fold;
     const cuuint64_t m = static_cast<cuuint64_t>(n_run) * h->P * h->Q / h->fold;
     dims[0] = c; dims[1] = m; dims[2] = 1; dims[3] = 1;
     strides[0] = c; strides[1] = m * c; strides[2] = m * c;
@@ -954,16 +995,16 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
     strides[2] = pb * h->s2d_wp * h->s2d_h;
     p.Q = h->Q / h->fold; p.P = h->P; p.Nimg = n_run;
   } else if (h->mode == MODE_VIEW) {
-    dims[0] = d.C; dims[1] = h->Q; dims[2] = h->P; dims[3] = n_run;
-    strides[0] = static_cast<cuuint64_t>(d.stride_w) * d.C;
-    strides[1] = static_cast<cuuint64_t>(d.stride_h) * d.W * d.C;
-    strides[2] = static_cast<cuuint64_t>(d.H) * d.W * d.C;
+    dims[0] = ac; dims[1] = h->Q; dims[2] = h->P; dims[3] = n_run;
+    strides[0] = static_cast<cuuint64_t>(d.stride_w) * ac;
+    strides[1] = static_cast<cuuint64_t>(d.stride_h) * d.W * ac;
+    strides[2] = static_cast<cuuint64_t>(d.H) * d.W * ac;
     p.Q = h->Q; p.P = h->P; p.Nimg = n_run;
   } else {
-    dims[0] = d.C; dims[1] = d.W; dims[2] = d.H; dims[3] = n_run;
-    strides[0] = d.C;
-    strides[1] = static_cast<cuuint64_t>(d.W) * d.C;
-    strides[2] = static_cast<cuuint64_t>(d.H) * d.W * d.C;
+    dims[0] = ac; dims[1] = d.W; dims[2] = d.H; dims[3] = n_run;
+    strides[0] = ac;
+    strides[1] = static_cast<cuuint64_t>(d.W) * ac;
+    strides[2] = static_cast<cuuint64_t>(d.H) * d.W * ac;
     p.Q = h->Q; p.P = h->P; p.Nimg = n_run;
     // strided filters: the box spans (t - 1) * stride + 1 input pixels per axis and the copy engine keeps
     // every stride-th one (traversal strides of the tensor map), so the tile still has tq x tp rows
@@ -979,6 +1020,7 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
   p.fd_tiles_k = make_fastdiv(p.tiles_k); p.fd_tiles_q = make_fastdiv(p.tiles_q); p.fd_tiles_p = make_fastdiv(p.tiles_p);
   p.fd_tq = make_fastdiv(p.tq); p.fd_tp = make_fastdiv(p.tp);
   p.fd_nchunks = make_fastdiv(p.nchunks); p.fd_S = make_fastdiv(p.S);
+  p.fd_np_cpp = make_fastdiv(std::max(1, p.np_cpp));
   if (!p.fd_tiles_k.d || !p.fd_tiles_q.d || !p.fd_tiles_p.d || !p.fd_tq.d || !p.fd_tp.d || !p.fd_nchunks.d || !p.fd_S.d)
     return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: division constants failed their check");
   int rc = encode_map(&h->tmap_a, a_ptr, 4, dims, strides, box, p.BKC, estr);
@@ -1112,6 +1154,12 @@ int grid_for(size_t work_items, int threads, int max_blocks) {
 
 }  // namespace
 
+namespace {
+int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host, const int32_t* bias_host,
+                 const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
+                 const qconv_handle* weights_of, const NpSpec* np);
+}
+
 extern "C" {
 
 const char* qconv_last_error_string(void) { return g_err; }
@@ -1145,6 +1193,16 @@ int qconv_create(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
 int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host, const int32_t* bias_host,
                          const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
                          const qconv_handle* weights_of) {
+  return create_layer(out, desc, w_host, bias_host, shift_host, res_lshift_host, acc_exp_host, weights_of, nullptr);
+}
+
+}  // extern "C"
+
+namespace {
+// np: the layer runs on the digit planes of floating-point operands (w_host is then only a placeholder for the checks).
+int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_host, const int32_t* bias_host,
+                 const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
+                 const qconv_handle* weights_of, const NpSpec* np) {
   if (!out) return fail(QCONV_ERR_BAD_ARG, "out is NULL");
   *out = nullptr;
   if (!desc || !w_host) return fail(QCONV_ERR_BAD_ARG, "desc or w_host is NULL");
@@ -1179,7 +1237,7 @@ int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_
   int max_t = 0;
   int64_t max_bias = 0;
   for (int k = 0; k < d.K; ++k) {
-    if (shift_host && (shift_host[k] < 0 || shift_host[k] > 31))
+    if (shift_host && !np && (shift_host[k] < 0 || shift_host[k] > 31))
       return fail(QCONV_ERR_BAD_SHIFT, "shift[%d] = %d outside [0, 31]", k, shift_host[k]);
     if (d.has_residual) {
       if (res_lshift_host[k] < 0 || res_lshift_host[k] > 23)
@@ -1193,7 +1251,7 @@ int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_
   // Eq. 9 / Eq. 13: the longest sum must fit a 32-bit two's-complement accumulator.
   const int64_t bound = static_cast<int64_t>(d.R) * d.S * Cg * (1ll << (d.n_in - 1)) * (1ll << (d.n_w - 1)) +
                         max_bias + (d.has_residual ? (128ll << max_t) : 0);
-  if (bound > 2147483647ll)
+  if (bound > 2147483647ll + (np ? max_bias : 0))          // (with digit products the bias meets the 64-bit sum)
     return fail(QCONV_ERR_OVERFLOW_RISK, "worst-case |accumulator| %lld exceeds 2^31 - 1", (long long)bound);
 
   qconv_handle* h = new qconv_handle();
@@ -1228,7 +1286,8 @@ int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_
 
   // Weight-aware bound of the wide value: 2^(n_in-1) * sum|w[k,.]| + |bias[k]| + 128 * 2^t[k].  Below 2^22 the
   // tensor-core epilogue may round in fp32 (exactly).
-  if (d.out_mode == QCONV_OUT_INT8 && d.groups == 1 && h->hints.float_rounding != 0) {
+  h->np = np;
+  if (d.out_mode == QCONV_OUT_INT8 && d.groups == 1 && h->hints.float_rounding != 0 && !np) {
     long long worst = 0;
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
     for (int k = 0; k < d.K && worst < (1ll << 22); ++k) {
@@ -1251,7 +1310,7 @@ int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_
     if (d.C % 16 == 0 && is_1x1 && s1) mode = MODE_FLAT;
     else if (d.C % 16 == 0 && is_1x1) mode = MODE_VIEW;
     else if (d.C % 16 == 0 && s1 && d.C <= 64 && d.S >= 4 && d.S * d.C <= 1024 &&
-             static_cast<long long>(d.N) * d.H * d.W * d.C <= (64ll << 20) && h->hints.window_rows != 0 && d.pool == 0) mode = MODE_WROW;
+             static_cast<long long>(d.N) * d.H * d.W * d.C <= (64ll << 20) && h->hints.window_rows != 0 && d.pool == 0 && !np) mode = MODE_WROW;
     else if (d.C % 16 == 0 && d.stride_h <= 2 && d.stride_w <= 2) mode = MODE_BOX;   // (strides: see prepare_a_map)
     else if (d.C <= 4 && d.stride_h == 2 && d.stride_w == 2 && d.S + 1 <= 16 && d.R * d.S * d.C <= 1024 &&
              h->hints.space_to_depth != 0) mode = MODE_S2D;
@@ -1324,13 +1383,11 @@ int qconv_create_sharing(qconv_handle** out, const qconv_desc* desc, const int8_
     free_handle(h);
     return rc;
   }
+  h->np = nullptr;
   *out = h;
   return QCONV_OK;
 }
 
-}  // extern "C"
-
-namespace {
 // Padded, widened copy of a stride-1 layer's input on at most 4 channels (from int8 or from float).
 template <int C, int PB>
 cudaError_t launch_row_pack_c(const qconv_handle* h, const void* src, bool f32, int e_x, int n_run, cudaStream_t st) {
@@ -1427,7 +1484,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
   } else {
     if (reinterpret_cast<uintptr_t>(d_x) & 15)
       return fail(QCONV_ERR_ALIGNMENT, "d_x must be 16-byte aligned");
-    if (h->prm.vec_store && !maxabs && ((reinterpret_cast<uintptr_t>(d_y) | reinterpret_cast<uintptr_t>(d_residual)) & 15))
+    if (h->prm.vec_store && !maxabs && !h->np_products && ((reinterpret_cast<uintptr_t>(d_y) | reinterpret_cast<uintptr_t>(d_residual)) & 15))
       return fail(QCONV_ERR_ALIGNMENT, "d_y and d_residual must be 16-byte aligned");
     const int8_t* a_ptr = d_x;
     if (h->mode == MODE_STEM) {
@@ -1990,14 +2047,12 @@ int qdequantize_np(const uint8_t* d_code, size_t count, int e, int n, int p, flo
 
 struct qconv_np_handle {
   qconv_np_desc d;
-  qconv_handle* gemm = nullptr;      // int8 GEMM on the digit planes, raw int32 accumulators out
-  int planes_x = 1, planes_w = 1, groups = 1;
+  qconv_handle* gemm = nullptr;      // tensor-core layer over the digit products, straight to the output patterns
+  int digits_x = 1, digits_w = 1;
+  qc::NpPlanes planes{};             // digit combinations of the input the products need
+  int c_pad = 0;                     // channels of a plane (a whole number of ring-stage chunks)
   int P = 0, Q = 0;
-  int8_t* d_planes = nullptr;        // [N][H][W][planes_x * C]
-  int32_t* d_acc = nullptr;          // [N][P][Q][groups * K]
-  int32_t* d_bias = nullptr;
-  int32_t* d_shift = nullptr;
-  qc::NpFormat fout{};
+  int8_t* d_planes = nullptr;        // [N][H][W][planes][c_pad]
 };
 
 namespace {
@@ -2029,10 +2084,31 @@ void free_np(qconv_np_handle* h) {
   if (!h) return;
   if (h->gemm) free_handle(h->gemm);
   cudaFree(h->d_planes);
-  cudaFree(h->d_acc);
-  cudaFree(h->d_bias);
-  cudaFree(h->d_shift);
   delete h;
+}
+
+// The digit products of x = sum x_i 128^i and w = sum w_j 128^j that give x w with the fewest multiplications
+// (Karatsuba): with P_S = (sum of x_i, i in S) (sum of w_i, i in S) over single digits and pairs,
+//   x_i w_j + x_j w_i = P_ij - P_ii - P_jj,
+// three products for two digits and six for three, where the digit-by-digit schoolbook form takes four and nine.  The
+// balanced digits (-64 ... 63, the last one at most 31) leave room for a sum of two in an int8.  Operands of different
+// lengths are padded with zero digits, and products with a zero factor drop out.
+struct NpProduct { int mask; long long coef; };
+std::vector<NpProduct> np_products(int digits_x, int digits_w) {
+  const int n = std::max(digits_x, digits_w);
+  std::vector<NpProduct> all;
+  for (int i = 0; i < n; ++i) {
+    long long c = 1ll << (14 * i);
+    for (int j = 0; j < n; ++j)
+      if (j != i) c -= 1ll << (7 * (i + j));
+    all.push_back({1 << i, c});
+  }
+  for (int i = 0; i < n; ++i)
+    for (int j = i + 1; j < n; ++j) all.push_back({(1 << i) | (1 << j), 1ll << (7 * (i + j))});
+  std::vector<NpProduct> kept;
+  for (const NpProduct& p : all)
+    if ((p.mask & ((1 << digits_x) - 1)) && (p.mask & ((1 << digits_w) - 1))) kept.push_back(p);
+  return kept;
 }
 }  // namespace
 
@@ -2071,43 +2147,52 @@ int qconv_np_create(qconv_np_handle** out, const qconv_np_desc* desc, const uint
   const long double worst = static_cast<long double>(d.R) * d.S * d.C * static_cast<long double>(bmax[0]) * bmax[1] + max_bias;
   if (worst >= 4.6e18L / 2)
     return fail(QCONV_ERR_OVERFLOW_RISK, "worst-case |sum| exceeds 2^62 (Eq. 9 with b = beta_max)");
-  const int groups = px + pw - 1;
-  const size_t acc_elems = static_cast<size_t>(d.N) * P * Q * groups * d.K;
-  if (acc_elems >= (1ull << 38)) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "tensor too large");
+  if (static_cast<long long>(d.R) * d.S * d.C * 128 * 128 > 2147483647ll)
+    return fail(QCONV_ERR_OVERFLOW_RISK, "a digit product's sum of %lld terms does not fit a 32-bit accumulator", static_cast<long long>(d.R) * d.S * d.C);
+  if (static_cast<size_t>(d.N) * P * Q * d.K >= (1ull << 38)) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "tensor too large");
 
-  // weights: digit planes arranged so that column group g sums x_plane_i * w_plane_(g - i)
-  const int Cp = px * d.C, Kp = groups * d.K;
-  std::vector<int8_t> wp(static_cast<size_t>(Kp) * d.R * d.S * Cp, 0);
-  const size_t taps = static_cast<size_t>(d.R) * d.S;
-  for (int k = 0; k < d.K; ++k)
-    for (size_t t = 0; t < taps; ++t)
-      for (int c = 0; c < d.C; ++c) {
-        int beta = np_host_decode(w_codes_host[(static_cast<size_t>(k) * taps + t) * d.C + c], d.n_w, d.p_w);
-        for (int j = 0; j < pw; ++j) {
-          const int dig = j + 1 < pw ? ((beta + 64) & 127) - 64 : beta;
-          beta = (beta - dig) >> 7;
-          for (int i = 0; i < px; ++i)
-            wp[((static_cast<size_t>(i + j) * d.K + k) * taps + t) * Cp + static_cast<size_t>(i) * d.C + c] = static_cast<int8_t>(dig);
-        }
-      }
   qconv_np_handle* h = new qconv_np_handle();
-  h->d = d; h->planes_x = px; h->planes_w = pw; h->groups = groups; h->P = P; h->Q = Q;
-  h->fout = qc::NpFormat{d.n_out, d.p_out, bmax[2]};
+  h->d = d; h->digits_x = px; h->digits_w = pw; h->P = P; h->Q = Q;
+  const std::vector<NpProduct> products = np_products(px, pw);
+  const size_t count = static_cast<size_t>(d.K) * d.R * d.S * d.C;
+  std::vector<std::vector<int8_t>> w(products.size());
+  NpSpec spec;
+  spec.products = static_cast<int>(products.size());
+  spec.n_out = d.n_out; spec.p_out = d.p_out; spec.top = static_cast<float>(bmax[2]);
+  for (size_t m = 0; m < products.size(); ++m) {
+    // the input's digit combination: one plane for each that differs
+    const int x_mask = products[m].mask & ((1 << px) - 1), w_mask = products[m].mask & ((1 << pw) - 1);
+    int plane = 0;
+    while (plane < h->planes.count && h->planes.mask[plane] != x_mask) ++plane;
+    if (plane == h->planes.count) h->planes.mask[h->planes.count++] = x_mask;
+    spec.a_plane[m] = plane;
+    spec.coef[m] = static_cast<int>(products[m].coef);
+    w[m].resize(count);
+    // one table of 256 patterns per product instead of decoding every weight
+    int8_t table[256];
+    for (int c = 0; c < 256; ++c) {
+      int beta = np_host_decode(c, d.n_w, d.p_w), sum = 0;
+      for (int j = 0; j < pw; ++j) {
+        const int dig = j + 1 < pw ? ((beta + 64) & 127) - 64 : beta;
+        beta = (beta - dig) >> 7;
+        if ((w_mask >> j) & 1) sum += dig;
+      }
+      table[c] = static_cast<int8_t>(sum);
+    }
+    for (size_t i = 0; i < count; ++i) w[m][i] = table[w_codes_host[i]];
+    spec.w[m] = w[m].data();
+  }
+  spec.planes = h->planes.count;
   qconv_desc g = {};
-  g.N = d.N; g.H = d.H; g.W = d.W; g.C = Cp; g.K = Kp; g.R = d.R; g.S = d.S;
+  g.N = d.N; g.H = d.H; g.W = d.W; g.C = d.C; g.K = d.K; g.R = d.R; g.S = d.S;
   g.stride_h = d.stride_h; g.stride_w = d.stride_w; g.pad_h = d.pad_h; g.pad_w = d.pad_w; g.groups = 1;
-  g.n_in = 8; g.n_w = 8; g.n_out = 8; g.symmetric = 1; g.out_mode = QCONV_OUT_INT32;
-  int rc = qconv_create(&h->gemm, &g, wp.data(), nullptr, nullptr, nullptr, nullptr);
+  g.n_in = 8; g.n_w = 8; g.n_out = 8; g.symmetric = 1; g.out_mode = QCONV_OUT_INT8; g.relu = d.relu; g.algo = QCONV_ALGO_IGEMM;
+  int rc = create_layer(&h->gemm, &g, w[0].data(), bias_host, shift_host, nullptr, nullptr, nullptr, &spec);
   if (rc) { free_np(h); return rc; }
-  std::vector<int32_t> sh(d.K, 0), bi(d.K, 0);
-  if (shift_host) std::memcpy(sh.data(), shift_host, sizeof(int32_t) * d.K);
-  if (bias_host) std::memcpy(bi.data(), bias_host, sizeof(int32_t) * d.K);
-  cudaError_t e = cudaMalloc(&h->d_planes, static_cast<size_t>(d.N) * d.H * d.W * Cp);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_acc, acc_elems * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_bias, sizeof(int32_t) * d.K);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_shift, sizeof(int32_t) * d.K);
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_bias, bi.data(), sizeof(int32_t) * d.K, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_shift, sh.data(), sizeof(int32_t) * d.K, cudaMemcpyHostToDevice);
+  h->c_pad = h->gemm->a_channels / spec.planes;
+  const size_t bytes = static_cast<size_t>(d.N) * d.H * d.W * h->gemm->a_channels;
+  cudaError_t e = cudaMalloc(&h->d_planes, bytes);
+  if (e == cudaSuccess && h->c_pad != d.C) e = cudaMemset(h->d_planes, 0, bytes);   // the padding channels stay zero
   if (e != cudaSuccess) {
     free_np(h);
     return fail(QCONV_ERR_CUDA, "qconv_np_create: %s", cudaGetErrorString(e));
@@ -2122,15 +2207,10 @@ int qconv_np_run(qconv_np_handle* h, const uint8_t* d_x_codes, uint8_t* d_y_code
   if (n_run <= 0 || n_run > d.N) return fail(QCONV_ERR_BAD_ARG, "n_run %d outside [1, %d]", n_run, d.N);
   if (reinterpret_cast<uintptr_t>(d_x_codes) & 15) return fail(QCONV_ERR_ALIGNMENT, "d_x_codes must be 16-byte aligned");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const size_t in_pix = static_cast<size_t>(n_run) * d.H * d.W, out_pix = static_cast<size_t>(n_run) * h->P * h->Q;
-  CUDA_TRY(launch_chained(qc::np_split_kernel, dim3(grid_for(in_pix * (d.C / 16), 256, 148 * 16)), dim3(256), 0, st,
-                          d_x_codes, h->d_planes, in_pix, d.C, d.n_in, d.p_in, h->planes_x));
-  int rc = qconv_run(h->gemm, h->d_planes, nullptr, h->d_acc, n_run, cuda_stream);
-  if (rc) return rc;
-  qc::np_combine_kernel<<<grid_for(out_pix * d.K, 256, 148 * 16), 256, 0, st>>>(h->d_acc, h->d_bias, h->d_shift, d_y_codes,
-                                                                                  out_pix, d.K, h->groups, d.relu, h->fout);
-  CUDA_TRY(cudaGetLastError());
-  return QCONV_OK;
+  const size_t in_pix = static_cast<size_t>(n_run) * d.H * d.W;
+  CUDA_TRY(launch_chained(qc::np_split_kernel, dim3(grid_for(in_pix * (d.C / 16), 256, 148 * 8)), dim3(256), 0, st,
+                          d_x_codes, h->d_planes, in_pix, d.C, h->c_pad, d.n_in, d.p_in, h->digits_x, h->planes));
+  return run_layer(h->gemm, h->d_planes, nullptr, d_y_codes, n_run, cuda_stream, false);
 }
 
 int qconv_np_status(qconv_np_handle* h) {
@@ -2142,7 +2222,7 @@ int qconv_np_describe(const qconv_np_handle* h, char* buf, size_t buf_len) {
   if (!h || !buf || buf_len == 0) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
   char inner[256];
   qconv_describe(h->gemm, inner, sizeof(inner));
-  snprintf(buf, buf_len, "np planes_x=%d planes_w=%d groups=%d | %s", h->planes_x, h->planes_w, h->groups, inner);
+  snprintf(buf, buf_len, "np digits_x=%d digits_w=%d products=%d | %s", h->digits_x, h->digits_w, h->gemm->np_products, inner);
   return QCONV_OK;
 }
 

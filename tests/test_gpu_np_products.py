@@ -1,0 +1,49 @@
+"""The digit products of the floating-point layers against the oracle at the sizes where their plan changes: one to six
+products (operands of one to three digits, mixed), one and two accumulator buffers, channel counts below / at / above a
+ring-stage chunk, partial batches, output rows at every alignment, and every input pattern of a type."""
+import numpy as np
+import pytest
+
+from oracle import fpconv_ref
+from paper_1805_07941_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+FMT = {1: (8, 7), 2: (8, 4), 3: (8, 3)}                    # types whose betas have that many base-128 digits
+PRODUCTS = {(1, 1): 1, (1, 2): 2, (2, 1): 2, (1, 3): 3, (3, 1): 3, (2, 2): 3, (2, 3): 5, (3, 2): 5, (3, 3): 6}
+CASES = [  # N, n_run, H, W, C, K, R, stride
+    (2, 2, 9, 7, 16, 17, 3, 1), (3, 2, 6, 5, 48, 80, 1, 1), (1, 1, 14, 14, 128, 100, 3, 1), (2, 2, 13, 11, 144, 33, 3, 2),
+    (9, 9, 8, 8, 64, 256, 1, 2)]
+
+
+@pytest.mark.parametrize("digits", sorted(PRODUCTS))
+@pytest.mark.parametrize("case", CASES)
+def test_products_match_the_oracle(digits, case):
+    import torch
+    N, n_run, H, W, C, K, R, stride = case
+    fi, fw, fo = FMT[digits[0]], FMT[digits[1]], FMT[2 if digits[0] != 2 else 3]
+    rng = np.random.default_rng(sum(case) + 10 * digits[0] + digits[1])
+    x = rng.integers(0, 256, (N, H, W, C)).astype(np.uint8)           # every pattern, the largest magnitudes included
+    x.reshape(-1)[:256] = np.arange(256, dtype=np.uint8)
+    x[(x & 0x7F) == 0] = 0                                            # (patterns have no negative zero)
+    w = rng.integers(0, 256, (K, R, R, C)).astype(np.uint8)
+    w[(w & 0x7F) == 0] = 0
+    bias = rng.integers(-2**31 + 1, 2**31 - 1, K).astype(np.int32)
+    pad, st = (R // 2, R // 2), (stride, stride)
+    acc = fpconv_ref.wide_value(x[:1], w, bias, fi, fw, R=R, S=R, stride=st, pad=pad)
+    base = np.log2(max(1.0, float(np.abs(acc).mean()) * 3 / fpconv_ref.magnitudes(*fo)[-1]))
+    shift = (int(base) + rng.integers(-2, 3, K)).clip(0, 40).astype(np.int32)
+    for relu in (0, 1):
+        want = fpconv_ref.qconv_np(x[:n_run], w, bias, shift, fi, fw, fo, R=R, S=R, stride=st, pad=pad, relu=relu)
+        conv = binding.QConvNP(w, bias, shift, N=N, H=H, W=W, C=C, K=K, R=R, S=R, stride_h=stride, stride_w=stride, pad_h=R // 2,
+                               pad_w=R // 2, n_in=fi[0], p_in=fi[1], n_w=fw[0], p_w=fw[1], n_out=fo[0], p_out=fo[1], relu=relu)
+        assert "products=%d " % PRODUCTS[digits] in conv.describe()
+        flat = torch.full((N * conv.P * conv.Q * K + 1,), 0x55, dtype=torch.uint8, device="cuda")
+        for offset in (0, 1):                                         # aligned rows, and rows one byte off
+            y = flat[offset:offset + N * conv.P * conv.Q * K].view(N, conv.P, conv.Q, K)
+            y.fill_(0x55)
+            conv.run(torch.from_numpy(x[:n_run]).cuda(), y)
+            assert conv.status() == 0
+            got = y.cpu().numpy()
+            assert (got[:n_run] == want).all() and (got[n_run:] == 0x55).all(), conv.describe()
+        conv.destroy()
