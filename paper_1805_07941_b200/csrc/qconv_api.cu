@@ -95,7 +95,7 @@ long ceil_div_l(long a, long b) { return (a + b - 1) / b; }
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Plan overrides of the calling thread (qconv_set_plan_hints); -1 / 0 = the planner decides.
-constexpr qconv_plan_hints kNoHints = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, 0};
+constexpr qconv_plan_hints kNoHints = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, 0};
 thread_local qconv_plan_hints g_hints = kNoHints;
 
 enum IgemmMode { MODE_FLAT = 0, MODE_VIEW = 1, MODE_BOX = 2, MODE_STEM = 3, MODE_S2D = 4, MODE_WROW = 5 };
@@ -526,6 +526,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   p.nchunks = ceil_div(c_eff, p.BKC);
   h->a_channels = d.C;
   p.acc_bufs = 2;
+  p.ksplit = 1;
   p.np_products = p.np_cpp = 0;
   if (np) {
     p.np_products = h->np_products = np->products;
@@ -898,7 +899,15 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I32>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_F32>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_MAX>),
-                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_NP>)}) {
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_NP>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_RES_U, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_RES, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_U, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES_U, 2, 4>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES, 2, 4>)}) {
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
       if (e != cudaSuccess) attr_err = e;
     }
@@ -967,6 +976,33 @@ IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
   if (uni)
     return h->d.has_residual ? qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES_U> : qc::igemm_i8_kernel<qc::EPI_FAST_I8_U>;
   return h->d.has_residual ? qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES> : qc::igemm_i8_kernel<qc::EPI_FAST_I8>;
+}
+
+// CTAs that share a tile's contraction in this run (1: none).
+int choose_ksplit(const qconv_handle* h, long tiles) {
+  const qc::IgemmParams& p = h->prm;
+  const int num_kb = p.R * p.S * p.nchunks, groups = p.BN / 16, want = h->hints.split_k;
+  if (!p.fast_epilogue || h->d.pool || p.b_resident || h->pair || p.BN > 128 || want == 0) return 1;
+  auto fits = [&](int ks) { return groups % ks == 0 && tiles * ks <= h->num_sms && num_kb >= ks; };
+  if (want > 0) return (want == 2 || want == 4) && fits(want) ? want : 1;
+  // A stage of a chain costs a quarter of a microsecond, one of three taps 0.4, the exchange about one.  In these units (2
+  // and 3 a stage) halves pay from 18 on (6 three-tap stages: 4.6 -> 4.3 us; 8 single ones: 4.0 either way), quarters from
+  // 16 on while the clusters fill half of the SMs at most: with more, the next kernel's CTAs find no room to set up beside
+  // them (14 x 14 x 256 3 x 3 on 16 tiles 4.6 -> 4.0, on 28 tiles 4.7 -> 5.1).
+  const int work = num_kb * (p.halo_s ? 3 : 2);
+  if (work >= 16 && fits(4) && tiles * 8 <= h->num_sms) return 4;
+  if (work >= 18 && fits(2)) return 2;
+  return 1;
+}
+
+IgemmKernel split_kernel_for(const qconv_handle* h) {
+  const bool uni = h->uniform_shift && h->hints.uniform_shift != 0, res = h->d.has_residual != 0;
+  if (h->flt_epilogue) {
+    if (uni) return res ? qc::igemm_i8_kernel<qc::EPI_FLT_I8_RES_U, 2, 4> : qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 2, 4>;
+    return res ? qc::igemm_i8_kernel<qc::EPI_FLT_I8_RES, 2, 4> : qc::igemm_i8_kernel<qc::EPI_FLT_I8, 2, 4>;
+  }
+  if (uni) return res ? qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES_U, 2, 4> : qc::igemm_i8_kernel<qc::EPI_FAST_I8_U, 2, 4>;
+  return res ? qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES, 2, 4> : qc::igemm_i8_kernel<qc::EPI_FAST_I8, 2, 4>;
 }
 
 // Activation tensor map and tile counts for this run (depends on the pointer and n_run).
@@ -1608,6 +1644,33 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
     }
     const long tiles = static_cast<long>(p.tiles_q) * p.tiles_p * p.tiles_n * p.tiles_k;
     if (tiles <= 0 || tiles > 2147483647l) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "tile count out of range");
+    const int ksplit = maxabs ? 1 : choose_ksplit(h, tiles);
+    if (ksplit > 1) {
+      qc::IgemmParams q = h->prm;
+      const int num_kb = p.R * p.S * p.nchunks, own = p.BN / 16 / ksplit;
+      q.ksplit = ksplit;
+      q.out_stage_bytes = 0;
+      q.gen_stage_bytes = static_cast<uint32_t>(own * (ksplit - 1) * 4 * 128 * 16);       // exchange area
+      const size_t fixed = 1024 + q.gen_stage_bytes + sizeof(qc::IgemmShared), stage = p.a_stage_bytes + p.b_stage_bytes;
+      q.stages = std::min<int>({ceil_div(num_kb, ksplit), qc::kMaxStages, static_cast<int>((226 * 1024 - fixed) / stage)});
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(static_cast<unsigned int>(tiles * ksplit));
+      cfg.blockDim = dim3(qc::kIgemmThreads);
+      cfg.dynamicSmemBytes = fixed + q.stages * stage;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[2];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned int>(ksplit); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = h->use_pdl;
+      cfg.attrs = attr;
+      cfg.numAttrs = 2;
+      const int4* chan_ptr = h->d_chan;
+      cudaError_t le = cudaLaunchKernelEx(&cfg, split_kernel_for(h), h->tmap_a, h->tmap_b, h->tmap_a, h->tmap_a, q, ep, chan_ptr, d_residual,
+                                          d_y, h->d_status, h->wait_limit);
+      if (le != cudaSuccess) return fail(QCONV_ERR_CUDA, "kernel launch (split contraction): %s", cudaGetErrorString(le));
+      return QCONV_OK;
+    }
     long grid = std::min<long>(tiles, static_cast<long>(h->num_sms) * h->ctas_per_sm);
     // with resident weights a CTA must stay on one channel tile: the stride over tiles is a multiple of tiles_k
     if (p.b_resident && p.tiles_k > 1) grid = std::max<long>(p.tiles_k, grid / p.tiles_k * p.tiles_k);
