@@ -71,8 +71,8 @@ struct IgemmParams {
   int tmem_cols;                   // power of two >= max(32, BN)
   int vec_store;                   // 1: 16-byte stores/loads of int8 rows are aligned
   int gen_simple;                  // general int8 epilogue: the accumulator bound leaves room for the single-pass rounding
-  int gen_vec_y, gen_vec_res;      // general epilogues: widest power of two (<= 16) of bytes at which every row piece of the
-                                   //    output / the residual is aligned (set per run from the pointers)
+  int gen_vec_y, gen_vec_res;      // general epilogues: 16 or 8 if every row piece of the output / the residual is aligned to
+                                   //    so many bytes, else 0 (set per run from the pointers)
   uint32_t gen_stage_bytes;        // general epilogues: shared memory of the warps' staging rows (0 for the fast ones)
   int fast_epilogue;               // 1: int8 out, nearest-even, K % 16 == 0, aligned rows, and the
                                    //    accumulator bound leaves room for the rounding constant
@@ -570,20 +570,19 @@ __device__ __forceinline__ void epilogue_16(const uint32_t (&acc)[16], uint32_t 
 // General epilogue: any rounding mode, bit width and alignment, K not a multiple of 16, int32 / float output, and
 // the maximum of the float output.
 //
-// A thread holds one pixel's 16 channels at a time, but rows of K bytes at any alignment can only be stored 1 to 8
-// bytes at a time, and 32 lanes storing bytes of 32 different rows touch 32 sectors per instruction.  So every warp
-// turns its part of the tile (32 rows x up to 64 bytes) around in its own rows of shared memory: conversion writes
-// 16 bytes per thread, then consecutive lanes store consecutive pieces of a row, as wide as the alignment allows; the
-// residual comes in the same way.  Only the warp itself is involved (no block barrier).  kGenPitch = 64 bytes of data
-// + 16: 16-byte accesses of 8 consecutive rows fall into different banks.
+// A thread holds one pixel's 16 channels at a time, but 32 lanes storing pieces of 32 different rows touch 32 sectors per
+// instruction, and rows of K bytes may start at any address.  So every warp turns its part of the tile (32 rows x up to
+// 64 bytes) around in its own rows of shared memory: conversion writes 16 bytes per thread, then consecutive lanes store
+// consecutive pieces of a row; the residual comes in the same way.  Only the warp itself is involved (no block barrier).
+// kGenPitch = 64 bytes of data + 16: 16-byte accesses of 8 consecutive rows fall into different banks.
+//  - rows aligned to 16 or 8 bytes: pieces of that size (gen_copy_rows);
+//  - any other alignment: the 4-byte words of global memory that the rows cover, shifted into place by a funnel shift,
+//    a row's first and last partial word byte by byte (gen_copy_words).
 // 13 x 35 x 27 x 96 -> 200, 3x3, residual, round-half-away: 58 -> 13 us with the byte stores gone.
 constexpr int kGenPitch = 80;
 constexpr int kGenWarpBytes = 32 * kGenPitch;
 
 template <int V> struct GenVec;
-template <> struct GenVec<1> { using T = uint8_t; };
-template <> struct GenVec<2> { using T = uint16_t; };
-template <> struct GenVec<4> { using T = uint32_t; };
 template <> struct GenVec<8> { using T = uint2; };
 template <> struct GenVec<16> { using T = uint4; };
 
@@ -592,34 +591,69 @@ template <> struct GenVec<16> { using T = uint4; };
 template <int V, bool STORE>
 __device__ __forceinline__ void gen_copy_rows(uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
   using T = typename GenVec<V>::T;
-  constexpr int kLanes = V == 1 ? 32 : 64 / V;              // lanes side by side on a row (64 bytes of it; 32 for bytes)
-  constexpr int kRows = 32 / kLanes;
+  constexpr int kLanes = 64 / V;                            // lanes side by side on a row
   const unsigned okmask = __ballot_sync(0xffffffffu, ok);
-#pragma unroll 4
-  for (int r0 = 0; r0 < 32; r0 += kRows) {
+  const int c = (lane % kLanes) * V;
+#pragma unroll
+  for (int r0 = 0; r0 < 32; r0 += 32 / kLanes) {
     const int r = r0 + lane / kLanes;
     const long long off = __shfl_sync(0xffffffffu, row_off, r);
-#pragma unroll
-    for (int c0 = 0; c0 < 64; c0 += kLanes * V) {
-      const int c = c0 + (lane % kLanes) * V;
-      if (((okmask >> r) & 1u) && c < bytes) {
-        T* sp = reinterpret_cast<T*>(stage + r * kGenPitch + c);
-        T* gp = reinterpret_cast<T*>(base + off + c);
-        if (STORE) *gp = *sp; else *sp = __ldg(gp);
-      }
+    if (((okmask >> r) & 1u) && c < bytes) {
+      T* sp = reinterpret_cast<T*>(stage + r * kGenPitch + c);
+      T* gp = reinterpret_cast<T*>(base + off + c);
+      if (STORE) *gp = *sp; else *sp = __ldg(gp);
+    }
+  }
+}
+
+// The same for any alignment: the aligned words that hold the rows.  A loaded row stays where its words were: its first
+// byte sits at its address modulo 4 (gen_row_words reads it).
+template <bool STORE>
+__device__ __forceinline__ void gen_copy_words(uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
+  const unsigned okmask = __ballot_sync(0xffffffffu, ok);
+  const int words = (bytes + 6) >> 2;                       // at most, wherever the row starts (<= 17)
+  const uint32_t inv = 65536u / static_cast<uint32_t>(words) + 1u;   // idx / words = (idx * inv) >> 16 for idx < 32 * 17
+#pragma unroll 4
+  for (int it = 0; it < words; ++it) {
+    const int idx = it * 32 + lane;
+    const int r = static_cast<int>((static_cast<uint32_t>(idx) * inv) >> 16), w = idx - r * words;
+    int8_t* row = base + __shfl_sync(0xffffffffu, row_off, r);
+    const int m = static_cast<int>(reinterpret_cast<uintptr_t>(row) & 3u), first = 4 * w - m;   // the word's first byte in the row
+    if (!((okmask >> r) & 1u) || first >= bytes) continue;
+    uint32_t* sp = reinterpret_cast<uint32_t*>(stage + r * kGenPitch) + w;
+    const bool whole = first >= 0 && first + 4 <= bytes;
+    if (STORE) {
+      const uint32_t lo = w ? sp[-1] : 0u;                  // (w <= 16: the row's 17th word is inside its pitch)
+      const uint32_t v = __funnelshift_l(lo, sp[0], 8 * m);
+      if (whole) *reinterpret_cast<uint32_t*>(row + first) = v;
+      else
+        for (int j = 0; j < 4; ++j)
+          if (first + j >= 0 && first + j < bytes) row[first + j] = static_cast<int8_t>(v >> (8 * j));
+    } else {
+      uint32_t v = 0u;
+      if (whole) v = __ldg(reinterpret_cast<const uint32_t*>(row + first));
+      else
+        for (int j = 0; j < 4; ++j)
+          if (first + j >= 0 && first + j < bytes) v |= static_cast<uint32_t>(static_cast<uint8_t>(__ldg(row + first + j))) << (8 * j);
+      *sp = v;
     }
   }
 }
 
 template <bool STORE>
 __device__ __forceinline__ void gen_copy(int vec, uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
-  switch (vec) {
-    case 16: gen_copy_rows<16, STORE>(stage, base, row_off, ok, bytes, lane); break;
-    case 8: gen_copy_rows<8, STORE>(stage, base, row_off, ok, bytes, lane); break;
-    case 4: gen_copy_rows<4, STORE>(stage, base, row_off, ok, bytes, lane); break;
-    case 2: gen_copy_rows<2, STORE>(stage, base, row_off, ok, bytes, lane); break;
-    default: gen_copy_rows<1, STORE>(stage, base, row_off, ok, bytes, lane); break;
-  }
+  if (bytes <= 0) return;
+  if (vec == 16) gen_copy_rows<16, STORE>(stage, base, row_off, ok, bytes, lane);
+  else if (vec == 8) gen_copy_rows<8, STORE>(stage, base, row_off, ok, bytes, lane);
+  else gen_copy_words<STORE>(stage, base, row_off, ok, bytes, lane);
+}
+
+// Bytes 16 i ... of this lane's loaded row, which starts `m` bytes into its staging row.
+__device__ __forceinline__ uint4 gen_row_words(const uint8_t* stage_row, int i, int m) {
+  const uint4 a = *reinterpret_cast<const uint4*>(stage_row + 16 * i);
+  const uint32_t next = *reinterpret_cast<const uint32_t*>(stage_row + 16 * i + 16);
+  return make_uint4(__funnelshift_r(a.x, a.y, 8 * m), __funnelshift_r(a.y, a.z, 8 * m), __funnelshift_r(a.z, a.w, 8 * m),
+                    __funnelshift_r(a.w, next, 8 * m));
 }
 
 // v / 2^s -> pattern of the nearest value of an (n, p) type; ties to the even pattern; saturation at beta_max;
@@ -1191,14 +1225,16 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       // general epilogues: this warp's columns of the tile, and its residual rows by way of the staging rows
       const int gen_k0 = tc.k0 + g_begin * 16;
       const int gen_cols = max(0, min((g_end - g_begin) * 16, prm.K - gen_k0));
-      if (!EpiTraits<EPI>::fast && res != nullptr) {
+      // (int8 results overwrite it in place, group by group; words have rows of their own behind it)
+      const bool gen_res = !EpiTraits<EPI>::fast && EPI != EPI_NP && res != nullptr;
+      uint8_t* gen_out = (EPI == EPI_I32 || EPI == EPI_F32) && gen_res ? gen_stage + kEpilogueWarps * kGenWarpBytes : gen_stage;
+      int gen_m = 0;
+      if (gen_res) {
+        int8_t* base = const_cast<int8_t*>(res) + gen_k0;
+        const long long off = static_cast<long long>(pix) * prm.K;
+        gen_m = static_cast<int>(reinterpret_cast<uintptr_t>(base + off) & 3u);
         __syncwarp();
-        gen_copy<false>(prm.gen_vec_res, gen_stage, const_cast<int8_t*>(res) + gen_k0, static_cast<long long>(pix) * prm.K, row_ok,
-                        gen_cols, lane);
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < kGroupsPerWarp; ++i)
-          if (i * 16 < gen_cols) rres[i] = *reinterpret_cast<const uint4*>(gen_stage + lane * kGenPitch + i * 16);
+        gen_copy<false>(prm.gen_vec_res, gen_stage, base, off, row_ok, gen_cols, lane);
         __syncwarp();
       }
       ok = wait_bounded<64, kHint>(ptx::smem_u32(&sh->acc_full[buf]), use & 1u, wait_limit, sh, status);
@@ -1279,15 +1315,16 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         const uint32_t stage_row = stage_base + static_cast<uint32_t>(row * prm.BN);
         uint32_t acc_a[16], acc_b[16];
         // general epilogues: group i of this warp; words leave group by group (64 bytes a row), bytes after the last
-        [[maybe_unused]] auto gen_group = [&](const uint32_t (&acc)[16], int i, const uint4& r16) {
+        [[maybe_unused]] auto gen_group = [&](const uint32_t (&acc)[16], int i) {
           if (i * 16 >= gen_cols) return;
-          const uint32_t st_row = ptx::smem_u32(gen_stage) + static_cast<uint32_t>(lane * kGenPitch);
+          const uint32_t st_row = ptx::smem_u32(gen_out) + static_cast<uint32_t>(lane * kGenPitch);
+          const uint4 r16 = gen_res ? gen_row_words(gen_stage + lane * kGenPitch, i, gen_m) : make_uint4(0u, 0u, 0u, 0u);
           const int ncols = gen_cols - i * 16;
           general_16<EPI>(acc, chan + static_cast<uint32_t>((g_begin + i) * 256), r16, ncols, row_ok, prm, ep,
                           st_row + (EPI == EPI_I8 ? static_cast<uint32_t>(i * 16) : 0u), &gen_max);
           if (EPI == EPI_I32 || EPI == EPI_F32) {
             __syncwarp();
-            gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + 4ll * (prm.out_c_offset + gen_k0 + i * 16),
+            gen_copy<true>(prm.gen_vec_y, gen_out, static_cast<int8_t*>(y) + 4ll * (prm.out_c_offset + gen_k0 + i * 16),
                            4ll * static_cast<long long>(pix) * prm.out_c_pitch, row_ok, 4 * min(16, ncols), lane);
             __syncwarp();
           }
@@ -1380,7 +1417,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
               if (tc.k0 + g0 * 16 < prm.K)
                 epilogue_pool_16<EPI, RELU>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pooled_pix, row_ok, lane, prm.pool_bit, prm, ep, y);
             } else if constexpr (!EpiTraits<EPI>::fast) {
-              gen_group(acc_a, i, rres[i & (kGroupsPerWarp - 1)]);
+              gen_group(acc_a, i);
             } else if (row_ok && tc.k0 + g0 * 16 < prm.K)
               epilogue_16<EPI, RELU, RSTG>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, prm, ep, rres[i & (kGroupsPerWarp - 1)], y, stage_row);
             if (g1 < g_end) {
@@ -1390,7 +1427,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                 if (tc.k0 + g1 * 16 < prm.K)
                   epilogue_pool_16<EPI, RELU>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pooled_pix, row_ok, lane, prm.pool_bit, prm, ep, y);
               } else if constexpr (!EpiTraits<EPI>::fast) {
-                gen_group(acc_b, i + 1, rres[(i + 1) & (kGroupsPerWarp - 1)]);
+                gen_group(acc_b, i + 1);
               } else if (row_ok && tc.k0 + g1 * 16 < prm.K)
                 epilogue_16<EPI, RELU, RSTG>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, prm, ep, rres[(i + 1) & (kGroupsPerWarp - 1)], y, stage_row);
               if (g2 < g_end && i + 2 < GPW) ptx::tmem_ld_wait();

@@ -312,7 +312,9 @@ int place_weights(qconv_handle* h, DeviceParts& parts, const int8_t* w, size_t b
   return QCONV_OK;
 }
 
-// Multiplier and shift for the kernel's divisions by d (1 <= d < 2^31), checked against plain division.
+// Multiplier and shift for the kernel's divisions by d (1 <= d < 2^31) of n < 2^31.  With 2^shr < d <= 2^(shr+1) and
+// mul = ceil(2^(32+shr) / d), e = mul d - 2^(32+shr) lies in [0, d), so n e < 2^31 2^(shr+1) = 2^(32+shr): the quotient
+// n mul / 2^(32+shr) exceeds n / d by less than 1 / d and has the same whole part.
 qc::FastDiv make_fastdiv(int d_in) {
   qc::FastDiv f = {0u, 0u, static_cast<uint32_t>(std::max(1, d_in))};
   if (f.d > 1u) {
@@ -320,15 +322,6 @@ qc::FastDiv make_fastdiv(int d_in) {
     while ((1ull << lg) < f.d) ++lg;                       // ceil(log2 d) >= 1
     f.shr = lg - 1;
     f.mul = static_cast<uint32_t>(((1ull << (32 + f.shr)) + f.d - 1) / f.d);
-    auto apply = [&](uint32_t n) { return static_cast<uint32_t>((static_cast<unsigned long long>(n) * f.mul) >> 32) >> f.shr; };
-    uint32_t probe = 2463534242u;
-    for (int i = 0; i < 512; ++i) {
-      probe ^= probe << 13; probe ^= probe >> 17; probe ^= probe << 5;
-      const uint32_t ns[6] = {static_cast<uint32_t>(i), i * f.d, i * f.d + f.d - 1, probe & 0x7fffffffu, 0x7fffffffu - static_cast<uint32_t>(i),
-                              (probe % (1u << 20))};
-      for (uint32_t n : ns)
-        if (n <= 0x7fffffffu && apply(n) != n / f.d) { f.mul = 0; f.shr = 0; f.d = 0; return f; }   // (never seen; the caller refuses)
-    }
   }
   return f;
 }
@@ -655,7 +648,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   if (hint.fast_epilogue == 0) p.fast_epilogue = 0;
   // rounding adds at most 2^(s-1) before the shift: in one pass when the accumulator bound leaves that room
   p.gen_simple = h->acc_bound + round_room <= 2147483647ll ? 1 : 0;
-  p.gen_stage_bytes = p.fast_epilogue ? 0u : static_cast<uint32_t>(qc::kEpilogueWarps * qc::kGenWarpBytes);
+  p.gen_stage_bytes = p.fast_epilogue ? 0u : static_cast<uint32_t>((d.has_residual && d.out_mode != QCONV_OUT_INT8 ? 2 : 1) *
+                                                                   qc::kEpilogueWarps * qc::kGenWarpBytes);
   // Shared memory: the operand ring, plus -- for the fast epilogues of short contractions, where the
   // epilogue and not the operand ring sets the pace -- staged output tiles that leave by TMA stores:
   // two of them, or three when the residual tile is also brought into them by TMA one tile ahead
@@ -1057,8 +1051,6 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
   p.fd_tq = make_fastdiv(p.tq); p.fd_tp = make_fastdiv(p.tp);
   p.fd_nchunks = make_fastdiv(p.nchunks); p.fd_S = make_fastdiv(p.S);
   p.fd_np_cpp = make_fastdiv(std::max(1, p.np_cpp));
-  if (!p.fd_tiles_k.d || !p.fd_tiles_q.d || !p.fd_tiles_p.d || !p.fd_tq.d || !p.fd_tp.d || !p.fd_nchunks.d || !p.fd_S.d)
-    return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: division constants failed their check");
   int rc = encode_map(&h->tmap_a, a_ptr, 4, dims, strides, box, p.BKC, estr);
   if (rc) return rc;
   h->a_key_ptr = a_ptr;
@@ -1134,7 +1126,6 @@ void plan_dw_tma(qconv_handle* h) {
   while ((1 << bp.cwb_log2) < bp.cwb) ++bp.cwb_log2;
   while ((1 << bp.cwb_box_log2) < bp.cwb_box) ++bp.cwb_box_log2;
   bp.fd_q_blocks = make_fastdiv(bp.q_blocks);
-  if (!bp.fd_q_blocks.d) return;
   h->dw_prm = bp;
   h->dw_tma = 1;
 }
@@ -1595,7 +1586,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
     if (rc) return rc;
     if (!h->prm.fast_epilogue) {
       // bytes at which every row piece of the output and the residual is aligned
-      auto widest = [](uintptr_t bits) { return bits & 1 ? 1 : bits & 2 ? 2 : bits & 4 ? 4 : bits & 8 ? 8 : 16; };
+      auto widest = [](uintptr_t bits) { return bits & 7 ? 0 : bits & 8 ? 8 : 16; };
       const uintptr_t es = d.out_mode == QCONV_OUT_INT8 ? 1 : 4;
       h->prm.gen_vec_y = widest(reinterpret_cast<uintptr_t>(d_y) | es * d.out_c_pitch | es * d.out_c_offset | es * d.K);
       h->prm.gen_vec_res = widest(reinterpret_cast<uintptr_t>(d_residual) | static_cast<uintptr_t>(d.K));
@@ -1683,7 +1674,6 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
       pw.walk_dq = static_cast<int>(m % p.tiles_q); m /= p.tiles_q;
       pw.walk_dp = static_cast<int>(m % p.tiles_p); pw.walk_dn = static_cast<int>(m / p.tiles_p);
       pw.fd_grid = make_fastdiv(static_cast<int>(grid));
-      if (!pw.fd_grid.d) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: division constants failed their check");
       h->walk_grid = grid;
       }
     }
