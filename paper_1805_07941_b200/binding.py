@@ -42,7 +42,7 @@ class qconv_plan_hints(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int) for n in (
         "halo", "window_rows", "space_to_depth", "resident_weights", "fold", "fast_epilogue",
         "float_rounding", "uniform_shift", "tma_store", "tma_residual", "depthwise_form", "pdl",
-        "group_taps", "pair_tiles", "split_k", "bn_max", "ctas_per_sm")]
+        "group_taps", "pair_tiles", "split_k", "patch_halo", "bn_max", "ctas_per_sm")]
 
 
 class qconv_np_desc(ctypes.Structure):
@@ -299,8 +299,8 @@ class QConv:
         _check(lib().qconv_set_wait_limit(self.handle, int(polls)))
 
     def describe(self):
-        buf = ctypes.create_string_buffer(256)
-        _check(lib().qconv_describe(self.handle, buf, 256))
+        buf = ctypes.create_string_buffer(400)
+        _check(lib().qconv_describe(self.handle, buf, 400))
         return buf.value.decode()
 
     def destroy(self):

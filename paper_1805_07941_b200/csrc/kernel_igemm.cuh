@@ -86,6 +86,10 @@ struct IgemmParams {
                                    //    per image row) that serves the S horizontal taps of a filter row -- the same rows of
                                    //    shared memory, the operand's start advanced by one pixel per tap; the stage then
                                    //    carries S weight chunks, and the kernel sees R x 1 taps
+  int halo_w;                      // taps of a stage that share a row of the box: halo_s, or 3 of 9 in the patch form, where the
+                                   //    box also has tp + 2 rows and serves all taps of a 3 x 3 filter
+  int store_rows;                  // patch form, staged tiles: image rows of a tile, each stored as a box of its own (the halo's
+                                   //    columns stay behind); 0 otherwise
   uint32_t b_chunk_bytes;          // halo form: footprint of one of those weight chunks
   int tap_boxes;                   // 1: the halo_s taps of a stage are separate activation boxes, a_tap_bytes apart
                                    //    (grouped taps: no halo, no shifted reads; only the stage is shared)
@@ -909,6 +913,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         const int product = prm.fd_np_cpp.divmod(ci, &in_plane);
         a_ci = prm.np_a[product] * prm.np_cpp + in_plane;
       }
+      const int a_c = a_ci * prm.BKC;
       if (doit) {
         ptx::mbar_expect_tx(full, prm.tx_bytes);
         if (!prm.b_resident) {
@@ -921,10 +926,10 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           }
         }
         if (first) ptx::grid_dependency_wait();
-        ptx::tma_load_4d(a_dst, &tmap_a, full, a_ci * prm.BKC, w0, h0, tc.n0);
+        ptx::tma_load_4d(a_dst, &tmap_a, full, a_c, w0, h0, tc.n0);
         if (prm.tap_boxes)
           for (int hs = 1; hs < prm.halo_s; ++hs)           // the filter row's other taps, each a box of its own
-            ptx::tma_load_4d(a_dst + static_cast<uint32_t>(hs) * prm.a_tap_bytes, &tmap_a, full, a_ci * prm.BKC, w0 + hs, h0, tc.n0);
+            ptx::tma_load_4d(a_dst + static_cast<uint32_t>(hs) * prm.a_tap_bytes, &tmap_a, full, a_c, w0 + hs, h0, tc.n0);
       }
     };
     // stages this CTA issues in all, and how many of them make up the first pass
@@ -1040,6 +1045,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       // taps of one stage: one pixel row further on in the same box (halo form) or the next box (grouped taps)
       const uint64_t halo_row = static_cast<uint64_t>(prm.tap_boxes ? prm.a_tap_bytes : static_cast<uint32_t>(prm.BKC)) >> 4;
       const uint64_t halo_bchunk = prm.b_chunk_bytes >> 4;
+      // patch form: from a filter row's last tap to the next row's first one
+      const uint64_t halo_next_row = static_cast<uint64_t>((prm.tq - prm.halo_w + 1) * prm.BKC) >> 4;
       const uint32_t full0 = ptx::smem_u32(&sh->full[0]), empty0 = ptx::smem_u32(&sh->empty[0]);
       int stage = 0, it = 0;
       uint32_t phase = 0;
@@ -1080,9 +1087,11 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             // halo form: the other horizontal taps are the same activation rows one pixel (one row of BKC
             // bytes) further on -- start address advanced by a row, the descriptor's base offset telling the
             // swizzle phase of the new first row -- against the next weight chunk of the stage
-            for (int hs = 1; hs < prm.halo_s; ++hs) {
-              const uint64_t ah = a_desc + static_cast<uint64_t>(hs) * halo_row;
-              const uint64_t bh = b_desc + static_cast<uint64_t>(hs) * halo_bchunk;
+            uint64_t ah = a_desc, bh = b_desc;
+            for (int hs = 1, hw = 1; hs < prm.halo_s; ++hs, ++hw) {
+              if (hw == prm.halo_w) { ah += halo_next_row; hw = 0; }
+              else ah += halo_row;
+              bh += halo_bchunk;
               ptx::mma_i8(d_tmem, ah, bh, idesc, 1u);
               if (mma_per_stage > 1) ptx::mma_i8(d_tmem, ah + 2u, bh + 2u, idesc, 1u);
               if (mma_per_stage > 2) {
@@ -1453,7 +1462,12 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         ptx::fence_async_smem();
         if (epilogue_vote(!ok)) { ok = false; break; }
         if (etid == 0) {
-          ptx::tma_store_4d(&tmap_y, stage_base, tc.k0, tc.q0, tc.p0, tc.n0);
+          if (prm.store_rows) {
+            for (int p = 0; p < prm.store_rows && tc.p0 + p < prm.P; ++p)
+              ptx::tma_store_4d(&tmap_y, stage_base + static_cast<uint32_t>(p * prm.tq * prm.BN), tc.k0, tc.q0, tc.p0 + p, tc.n0);
+          } else {
+            ptx::tma_store_4d(&tmap_y, stage_base, tc.k0, tc.q0, tc.p0, tc.n0);
+          }
           ptx::bulk_commit();
         }
         sbuf = sbuf == 2 ? 0 : sbuf + 1;

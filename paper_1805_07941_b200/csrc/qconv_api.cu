@@ -95,7 +95,7 @@ long ceil_div_l(long a, long b) { return (a + b - 1) / b; }
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Plan overrides of the calling thread (qconv_set_plan_hints); -1 / 0 = the planner decides.
-constexpr qconv_plan_hints kNoHints = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, 0};
+constexpr qconv_plan_hints kNoHints = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, 0, 0};
 thread_local qconv_plan_hints g_hints = kNoHints;
 
 enum IgemmMode { MODE_FLAT = 0, MODE_VIEW = 1, MODE_BOX = 2, MODE_STEM = 3, MODE_S2D = 4, MODE_WROW = 5 };
@@ -221,6 +221,7 @@ struct qconv_handle {
   int use_pdl = 1;
   uint32_t* d_dw_tap = nullptr;  // tap-packed form: weight rows [3][C], bias + magic [C], 2^-s [C], rounding offset [C] (float bits)
   int dw_tap = 0;
+  int patch = 0;                 // 1: patch form (one activation box of 16 x (tp + 2) pixels serves all nine taps)
   int pair = 0;                  // 1: tiles of 256 pixels x 256 channels on pairs of SMs (kernel_igemm_pair.cuh)
   int fold = 1;                  // flat GEMMs with few output channels: this many pixels form one GEMM row
   int dw_tma = 0;                // rows staged by TMA (C % 32 == 0)
@@ -412,6 +413,20 @@ typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const qc::PairP
                            const qc::EpilogueParams, const int4*, void*, int*, unsigned int);
 PairKernel pair_kernel_for(const qconv_handle* h);
 
+// Tile of the patch form: 16 accumulator rows per image row, 14 of them outputs (the other two are the halo's columns),
+// so that image rows start at multiples of 16 rows; up to eight image rows.
+struct PatchTile { int q_step, segs, tp, rows; };
+PatchTile patch_tile(int Q, int P, bool pool) {
+  PatchTile t;
+  t.segs = ceil_div(Q, 14);
+  t.q_step = ceil_div(Q, t.segs);
+  if (pool) t.q_step += t.q_step & 1;                      // (a 2 x 2 window stays inside a tile)
+  t.rows = ceil_div(P, 8);
+  t.tp = ceil_div(P, t.rows);
+  if (pool) t.tp += t.tp & 1;
+  return t;
+}
+
 int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_of, const int8_t* w_krsc /* host [K][R][S][Cg] */,
                const int32_t* bias_host, const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host) {
   const qconv_desc& d = h->d;
@@ -590,11 +605,37 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     taps_s = 1;                                            // what the kernel's stage loop sees
     p.S = 1;
   }
+  // Patch form of a 3 x 3 / stride 1 layer on one chunk of channels: ONE box of (tp + 2) x 16 pixels serves all nine taps
+  // (row and column shifts of the same shared-memory rows), against resident weights.  A box per filter row reads every
+  // activation three times, a box per tap nine times; where that traffic and not the tensor pipe is the bound (up to 128
+  // channels), this is what limits the layer.  us: 64 x 224 x 224 x 64 -> 64 with its pool 167 -> 129, 64 x 112 x 112 x 64
+  // -> 128 72 -> 60, x 128 -> 128 with its pool 102 -> 84, 128 x 28 x 28 x 96 -> 128 20.0 -> 14.8, 128 x 14 x 14 x 112 -> 224
+  // 14.8 -> 9.1; at one wave of tiles (32 x 28 x 28 x 128 -> 128: 7.2 -> 6.8) it is about even.
+  const PatchTile pt = patch_tile(h->Q, h->P, d.pool != 0);
+  const bool patch_fits = h->mode == MODE_BOX && d.R == 3 && d.S == 3 && d.stride_h == 1 && d.stride_w == 1 && d.pad_h == 1 && d.pad_w == 1 &&
+                          p.nchunks == 1 && p.BKC >= 64 && fast_possible && d.K % 16 == 0 && d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0;
+  bool patch = false;
+  if (patch_fits && hint.patch_halo != 0 && hint.bn_max <= 0 && hint.halo != 1 && hint.group_taps != 1 && hint.pair_tiles != 1) {
+    const long tiles = static_cast<long>(pt.segs) * pt.rows * d.N * ceil_div(k_eff, 128);
+    const double used = static_cast<double>(h->Q) * h->P / (static_cast<double>(pt.segs) * pt.rows * 128);
+    // from a wave of tiles on, as long as most accumulator rows are outputs and the activations are read for two channel
+    // tiles at most
+    patch = hint.patch_halo == 1 || (tiles >= h->num_sms && used >= 0.75 && k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0);
+  }
+  if (patch) {
+    wide = false;
+    halo = false;
+    h->pair = 0;
+    bn_max = 128;
+    taps_r = taps_s = 1;
+    p.R = p.S = 1;
+  }
+  h->patch = patch ? 1 : 0;
   // Grouped taps: on few channels (rows of at most 64 bytes) a ring stage of ONE tap carries one or two
   // MMAs, far less tensor work than the few hundred cycles of instructions a stage costs the issuing
   // thread.  The S taps of a filter row then share a stage -- S activation boxes side by side, S weight
   // chunks -- and the stage loop runs over filter rows only.
-  bool group = !halo && !wide && h->mode == MODE_BOX && d.S >= 2 && d.S <= 4 && p.nchunks == 1 && p.BKC <= 64 &&
+  bool group = !halo && !wide && !patch && h->mode == MODE_BOX && d.S >= 2 && d.S <= 4 && p.nchunks == 1 && p.BKC <= 64 &&
                hint.group_taps != 0;
   if (group && hint.group_taps != 1) {
     // ... as long as the fatter stages still form a ring of three, or the weights can stay resident beside
@@ -616,13 +657,16 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     taps_s = 1;
     p.S = 1;
   }
-  const int tps = halo ? 3 : (group ? d.S : 1);            // taps (weight chunks) per ring stage
-  p.halo_s = (halo || group) ? tps : 0;
+  const int tps = patch ? 9 : halo ? 3 : (group ? d.S : 1);   // taps (weight chunks) per ring stage
+  p.halo_s = (halo || group || patch) ? tps : 0;
+  p.halo_w = patch ? 3 : std::max(1, tps);
+  p.store_rows = 0;
   p.tap_boxes = group ? 1 : 0;
   p.tiles_k = ceil_div(k_eff, bn_max);
   p.BN = static_cast<int>(align_up(ceil_div(k_eff, p.tiles_k), 16));
   h->kpad = p.tiles_k * p.BN;
-  h->kg_total = taps_r * taps_s_w * p.nchunks * p.BKC;
+  const int all_taps = patch ? 9 : taps_r * taps_s_w;
+  h->kg_total = all_taps * p.nchunks * p.BKC;
   p.K = k_eff;
   p.out_c_offset = d.out_c_offset;
   p.out_c_pitch = h->fold > 1 ? k_eff : d.out_c_pitch;
@@ -681,10 +725,33 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
       }
     }
   }
+  // (patch form: resident weights and at least two activation boxes; two CTAs per SM where they fit, staged tiles where
+  // they still do)
+  const int patch_a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + 2 * 16 + 8) * p.BKC, 1024));
+  if (patch) {
+    const int b_res = 9 * static_cast<int>(align_up(static_cast<size_t>(p.BN) * p.BKC, 1024));
+    const bool may_stage = p.fast_epilogue && hint.tma_store != 0 && (p.BN == 64 || p.BN == 128) && !d.pool && !d.has_residual;
+    bool placed = false;
+    p.out_stage_bytes = 0;
+    for (int ctas : {2, 1}) {
+      if (ctas == 2 && (hint.ctas_per_sm == 1 || 4 * p.tmem_cols > 512)) continue;
+      const int budget = (ctas == 2 ? 113 : 226) * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared)) - b_res;
+      for (int staged : {2, 0}) {
+        if (placed || (staged && !may_stage) || (budget - staged * out_tile) / patch_a < 2) continue;
+        placed = true;
+        h->ctas_per_sm = ctas;
+        p.out_stage_bytes = staged ? static_cast<uint32_t>(out_tile) : 0u;
+        p.out_stage_bufs = 2;
+      }
+    }
+    if (!placed || !p.fast_epilogue) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: the patch form does not fit");
+    p.store_rows = p.out_stage_bytes ? pt.tp : 0;
+  }
   const int staged_tiles = p.out_stage_bytes ? p.out_stage_bufs : 0;
-  h->kg_total = taps_r * taps_s_w * p.nchunks * p.BKC;
+  h->kg_total = all_taps * p.nchunks * p.BKC;
   // (halo form: the shifted operand reads up to two rows past the 128th, and a stage holds three weight chunks)
-  p.a_tap_bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * p.BKC, 1024));
+  p.a_tap_bytes = patch ? static_cast<uint32_t>(patch_a)
+                        : static_cast<uint32_t>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * p.BKC, 1024));
   p.a_stage_bytes = p.a_tap_bytes * (group ? static_cast<uint32_t>(tps) : 1u);
   p.b_chunk_bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(h->pair ? p.BN / 2 : p.BN) * p.BKC, 1024));
   p.b_stage_bytes = p.b_chunk_bytes * static_cast<uint32_t>(tps);
@@ -709,7 +776,11 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     const long grid_max = static_cast<long>(h->num_sms) * h->ctas_per_sm;
     const int b_res_bytes = num_kb_plan * static_cast<int>(p.b_stage_bytes);
     const int mode_env = hint.resident_weights;                      // 0: never, 1: whenever it fits
-    if (mode_env != 0 && !h->pair && (!(halo || group) || p.nchunks == 1) && b_res_bytes <= 72 * 1024 &&
+    if (patch) {
+      p.b_resident = 1;
+      const int budget = (h->ctas_per_sm == 2 ? 113 : 226) * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared));
+      stages = std::min((budget - staged_tiles * out_tile - b_res_bytes) / patch_a, qc::kMaxStages);
+    } else if (mode_env != 0 && !h->pair && (!(halo || group) || p.nchunks == 1) && b_res_bytes <= 72 * 1024 &&
         (m_tiles * p.tiles_k > grid_max || mode_env == 1)) {
       const int st = (full_budget - staged_tiles * out_tile - b_res_bytes) / static_cast<int>(p.a_stage_bytes);
       if (st >= std::min(num_kb_plan + 1, 2)) {
@@ -737,16 +808,18 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   } else {
     choose_box(h->Q, h->P, d.N, &p.tq, &p.tp, &p.tn, d.pool != 0, static_cast<long>(h->num_sms) * h->ctas_per_sm / p.tiles_k);
     if (halo) halo_box(&p.tq, &p.tp, &p.tn, &p.q_step);
+    if (patch) { p.tq = 16; p.tp = pt.tp; p.tn = 1; p.q_step = pt.q_step; }
     p.pad_h = d.pad_h; p.pad_w = d.pad_w;
     p.stride_h = d.stride_h; p.stride_w = d.stride_w;
   }
-  if (!halo) p.q_step = p.tq;
+  if (!halo && !patch) p.q_step = p.tq;
   p.pool_bit = d.pool ? p.tq : 0;
   if (d.pool && (!p.fast_epilogue || h->mode != MODE_BOX)) {
     return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "pool: needs the tensor-core path with per-tap boxes and an int8 output at 8 bits "
                 "with nearest-even rounding, K %% 16 == 0 and an accumulator bound below 2^31 - 2^(s-1)");
   }
   p.tx_bytes = static_cast<uint32_t>((group ? tps : 1) * p.tq * p.tp * p.tn * p.BKC + (p.b_resident ? 0 : tps * p.BN * p.BKC));
+  if (patch) p.tx_bytes = static_cast<uint32_t>(16 * (p.tp + 2) * p.BKC);
   p.b_res_tx_bytes = static_cast<uint32_t>(num_kb_plan * tps * p.BN * p.BKC);
   p.res_tx_bytes = static_cast<uint32_t>(p.tq * p.tp * p.tn * p.BN);
 
@@ -1042,6 +1115,7 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
     box[1] = static_cast<cuuint32_t>((p.tq - 1) * d.stride_w + 1);
     box[2] = static_cast<cuuint32_t>((p.tp - 1) * d.stride_h + 1);
     if (p.halo_s && !p.tap_boxes) box[1] = static_cast<cuuint32_t>(p.tq);
+    if (h->patch) box[2] = static_cast<cuuint32_t>(p.tp + 2);
   }
   p.tiles_q = ceil_div(p.Q, p.q_step);
   p.tiles_p = ceil_div(p.P, p.tp);
@@ -1070,6 +1144,7 @@ int prepare_y_map(qconv_handle* h, const void* y_ptr, int n_run) {
   cuuint64_t strides[3] = {pitch, pitch * p.Q, pitch * p.Q * p.P};
   cuuint32_t box[4] = {static_cast<cuuint32_t>(p.BN), static_cast<cuuint32_t>(p.tq), static_cast<cuuint32_t>(p.tp),
                        static_cast<cuuint32_t>(p.tn)};
+  if (p.store_rows) { box[1] = static_cast<cuuint32_t>(p.q_step); box[2] = 1; }
   const int swz = (p.BN == 128 || p.BN == 64 || p.BN == 32) ? p.BN : 0;
   int rc = encode_map(&h->tmap_y, static_cast<const int8_t*>(y_ptr) + p.out_c_offset, 4, dims, strides, box, swz);
   if (rc) return rc;
@@ -1847,10 +1922,10 @@ int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len) {
     static const char* names[] = {"flat", "view", "box", "stem", "s2d", "wrow"};
     const qc::IgemmParams& p = h->prm;
     snprintf(buf, buf_len, "igemm/%s box=%dx%dx%d BN=%d tiles_k=%d BKC=%d chunks=%d taps=%dx%d stages=%d smem=%zu "
-             "ctas/sm=%d fast=%d uni=%d flt=%d fold=%d tma_store=%d b_res=%d halo=%d grp=%d pair=%d pool=%d",
+             "ctas/sm=%d fast=%d uni=%d flt=%d fold=%d tma_store=%d b_res=%d halo=%d grp=%d pair=%d pool=%d%s",
              names[h->mode], p.tq, p.tp, p.tn, p.BN, p.tiles_k, p.BKC, p.nchunks, p.R, p.S, p.stages,
              h->smem_bytes, h->ctas_per_sm, p.fast_epilogue, h->uniform_shift, h->flt_epilogue && p.fast_epilogue, h->fold,
-             p.out_stage_bytes ? p.out_stage_bufs : 0, p.b_resident, p.tap_boxes ? 0 : p.halo_s, p.tap_boxes ? p.halo_s : 0, h->pair, h->d.pool);
+             p.out_stage_bytes ? p.out_stage_bufs : 0, p.b_resident, p.tap_boxes || h->patch ? 0 : p.halo_s, p.tap_boxes ? p.halo_s : 0, h->pair, h->d.pool, h->patch ? " patch=1" : "");
   } else {
     snprintf(buf, buf_len, "%s", h->algo == QCONV_ALGO_DEPTHWISE ? (h->dw_tma ? "depthwise3x3/tap-packed+tma" : h->dw_tap ? "depthwise3x3/tap-packed" : "depthwise3x3/dp4a")
                                                                   : "direct");

@@ -1,0 +1,47 @@
+"""The patch form of 3 x 3 layers (one activation box for all nine taps) against the oracle: images around the tile's
+14 x 8 outputs, channel counts that fill a chunk or not, one and several channel tiles, staged and direct stores,
+residual, concat window, pool, per-layer and per-channel shifts, both roundings' epilogues, several tiles per CTA."""
+import numpy as np
+import pytest
+
+from oracle import ref
+from tests.helpers import gpu_conv, oracle_conv, rand_layer
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # N, H, W, C, K
+    (2, 8, 14, 64, 64), (1, 7, 13, 64, 128), (3, 9, 15, 128, 128), (2, 16, 28, 48, 64), (1, 17, 29, 96, 208), (2, 5, 3, 128, 256),
+    (1, 1, 1, 64, 16), (2, 20, 43, 112, 80), (40, 28, 28, 64, 64), (30, 30, 30, 128, 128)]
+
+
+@pytest.mark.parametrize("case", CASES)
+@pytest.mark.parametrize("uniform", [0, 1])
+def test_patch_form_matches_the_oracle(case, uniform):
+    from paper_1805_07941_b200 import binding
+    N, H, W, C, K = case
+    for small in (0, 1):
+        for with_res in (0, 1):
+            rng = np.random.default_rng(sum(case) + uniform)
+            x, w, bias, shift, res, t = rand_layer(rng, N, H, W, C, K, 3, 3, with_res=bool(with_res), pad=(1, 1), per_channel_shift=not uniform)
+            if small:                                        # the float-rounding epilogue
+                w, shift = (w // 16).astype(np.int8), np.maximum(shift - 4, 0).astype(np.int32)
+                t = np.minimum(t, 5).astype(np.int32) if with_res else None
+            if with_res and uniform:
+                t = np.full(K, int(t[0]), np.int32)
+            kw = dict(R=3, S=3, pad=(1, 1), relu=small)
+            with binding.plan_hints(patch_halo=1):
+                got, desc = gpu_conv(x, w, bias, shift, res, t, **kw)
+                assert "patch=1" in desc and (got == oracle_conv(x, w, bias, shift, res, t, **kw)).all(), (desc, small, with_res)
+                if with_res:
+                    continue
+                win = dict(kw, out_c_offset=16, out_c_pitch=K + 48)
+                got, desc = gpu_conv(x, w, bias, shift, **win)
+                assert "patch=1" in desc and (got == oracle_conv(x, w, bias, shift, **win)).all(), desc
+                with binding.plan_hints(patch_halo=1, tma_store=0, ctas_per_sm=1):
+                    got, desc = gpu_conv(x, w, bias, shift, **kw)
+                want = oracle_conv(x, w, bias, shift, **kw)
+                assert "patch=1" in desc and (got == want).all(), desc
+                if H % 2 == 0 and W % 2 == 0:
+                    with binding.plan_hints(patch_halo=1):
+                        got, desc = gpu_conv(x, w, bias, shift, pool=2, **kw)
+                    assert "patch=1" in desc and (got == ref.maxpool_i8(want, 2, 2, 2, 0)).all(), desc
