@@ -351,16 +351,12 @@ struct IgemmShared {
   uint64_t b_full;                // resident weight tile landed
   uint32_t tmem_base;
   volatile int abort_flag;
-  // Epilogue constants.  When they fit, those of ALL output channels are staged once per CTA
-  // (kpad <= 512 entries, or kpad <= 2048 biases when the shift is per layer); otherwise the current
-  // and next tile's channels (at most 256 each) alternate in the two halves.
-  union {
-    int4 chan[512];
-    int32_t bias[2048];
-  } cst;
+  // Epilogue constants.  When they fit, those of ALL output channels are staged once per CTA; otherwise the current
+  // and next tile's channels (at most 256 each) alternate.
+  alignas(16) int32_t cst[2048];
 };
 
-constexpr int kChanAllMax = 512, kBiasAllMax = 2048;
+constexpr uint32_t kCstBytes = sizeof(int32_t) * 2048;
 
 // Bounded wait.  Returns false (and raises the CTA abort flag and the global status) if the
 // barrier did not flip within `limit` polls, or if another role already gave up.
@@ -451,7 +447,22 @@ template <int EPI> struct EpiTraits {
                               EPI == EPI_FLT_I8_RES_U;
   static constexpr bool uni = EPI == EPI_FAST_I8_U || EPI == EPI_FAST_I8_RES_U || EPI == EPI_FLT_I8_U ||
                               EPI == EPI_FLT_I8_RES_U;
+  // shared-memory form of the channel constants: 4 bytes a channel when only the biases differ; for the float rounding
+  // without residual 8, two channels side by side as {bias, bias, 2^-s, 2^-s}; else the table's 16
+  static constexpr bool paired = EPI == EPI_FLT_I8;
+  static constexpr uint32_t cst_bytes = uni ? 4u : paired ? 8u : 16u;
 };
+
+// Channel constant i of the table to its place in shared memory.
+template <int EPI>
+__device__ __forceinline__ void stage_constant(int32_t* cst, int i, const int4* __restrict__ entry) {
+  if (EpiTraits<EPI>::uni) cst[i] = __ldg(&entry->x);
+  else if (EpiTraits<EPI>::paired) {
+    const int2 v = __ldg(reinterpret_cast<const int2*>(entry));
+    cst[4 * (i >> 1) + (i & 1)] = v.x;
+    cst[4 * (i >> 1) + 2 + (i & 1)] = v.y;
+  } else reinterpret_cast<int4*>(cst)[i] = __ldg(entry);
+}
 
 constexpr int kMagicBits = 0x4B400000;        // bit pattern of 1.5 * 2^23 = 12582912.0f
 
@@ -487,12 +498,72 @@ __device__ __forceinline__ int4 lds_int4(uint32_t addr) {
 // RSTG: 1 when the residual tile has been brought into the staged tile by TMA (read there, overwritten
 // in place by the result).
 // The fast conversion of 16 accumulator columns to 16 int8 codes (four packed words): bias, residual << t, ReLU,
-// shift with nearest-even rounding, saturation.  cst_g: shared-memory address of the first column's constant
-// (4 bytes per column when only the biases differ, 16 otherwise); rw: the 16 residual bytes (ignored without).
+// shift with nearest-even rounding, saturation.  cst_g: shared-memory address of the first column's constant;
+// rw: the 16 residual bytes (ignored without).
+//
+// The epilogue's warps are bound by their own latency (two CTAs of eight warps per SM, nine cycles from one instruction of
+// a warp to its next), so what counts is instructions and exposed waits.  The constants of the first four columns come in
+// from the caller, who loads them before it waits for the accumulators, and those of the next four are loaded before the
+// current four's arithmetic.  Float rounding, per four outputs: four additions with the ReLU's maximum, two fused
+// multiply-adds on pairs, and the clamp on pairs of 16-bit halves (the host sees to it that |result| < 2^15 before the
+// clamp), which the byte packing needs anyway.
+template <int EPI> struct CstAhead { int4 v[EpiTraits<EPI>::paired ? 2 : 1]; };
+template <int EPI>
+__device__ __forceinline__ CstAhead<EPI> load_ahead(uint32_t cst_g, int g) {
+  CstAhead<EPI> a;
+  if (EpiTraits<EPI>::uni) a.v[0] = lds_int4(cst_g + static_cast<uint32_t>(g * 16));
+  if constexpr (EpiTraits<EPI>::paired) {
+    a.v[0] = lds_int4(cst_g + static_cast<uint32_t>(g * 32));
+    a.v[1] = lds_int4(cst_g + static_cast<uint32_t>(g * 32 + 16));
+  }
+  return a;
+}
+
+// (a.x * b.x + c.x, a.y * b.y + c.y), (a.x + b.x, a.y + b.y): one instruction each.
+__device__ __forceinline__ float2 fma_pair(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 add_pair(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
+// Four wide values + magic (as float bits, ReLU already applied) -> four codes.  scale: 2^-s per value; the addend is
+// M (1 - 2^-s), or is made from M where only 2^-s is at hand: (M + v) - M is exact, and M + v 2^-s rounds once.
+template <bool OWN_SCALE>
+__device__ __forceinline__ uint32_t round_pack_4(const int32_t (&fb)[4], float2 s01, float2 s23, float2 add, bool relu, int lo) {
+  constexpr float kM = 12582912.0f;
+  float2 a = make_float2(__int_as_float(fb[0]), __int_as_float(fb[1])), b = make_float2(__int_as_float(fb[2]), __int_as_float(fb[3]));
+  if (OWN_SCALE) {
+    a = add_pair(a, make_float2(-kM, -kM));
+    b = add_pair(b, make_float2(-kM, -kM));
+  }
+  const float2 r = fma_pair(a, s01, add), q = fma_pair(b, s23, add);
+  uint32_t h0 = __byte_perm(__float_as_uint(r.x), __float_as_uint(r.y), 0x5410), h1 = __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x5410);
+  h0 = __vmins2(h0, 0x007F007Fu);
+  h1 = __vmins2(h1, 0x007F007Fu);
+  if (!relu) {
+    const uint32_t lo2 = static_cast<uint32_t>(lo) * 0x10001u + (lo < 0 ? 0x10000u : 0u);   // lo in both halves
+    h0 = __vmaxs2(h0, lo2);
+    h1 = __vmaxs2(h1, lo2);
+  }
+  return __byte_perm(h0, h1, 0x6420);
+}
+
 template <int EPI, int RELU>
-__device__ __forceinline__ void convert_16(const uint32_t* acc, uint32_t cst_g, const uint32_t (&rw)[4],
+__device__ __forceinline__ void convert_16(const uint32_t* acc, uint32_t cst_g, CstAhead<EPI> ahead, const uint32_t (&rw)[4],
                                            const EpilogueParams& ep, uint32_t (&wds)[4]) {
   const bool relu = RELU == 2 ? ep.relu != 0 : RELU == 1;
+  const float2 uni_c1 = make_float2(ep.uni_c1, ep.uni_c1), uni_c2 = make_float2(ep.uni_c2, ep.uni_c2);
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
     int32_t q[4];
@@ -501,29 +572,41 @@ __device__ __forceinline__ void convert_16(const uint32_t* acc, uint32_t cst_g, 
       rv[0] = sign_extend_byte<0>(rw[g]); rv[1] = sign_extend_byte<1>(rw[g]);
       rv[2] = sign_extend_byte<2>(rw[g]); rv[3] = sign_extend_byte<3>(rw[g]);
     }
-    // with per-layer shifts only the biases differ per channel: four of them per shared-memory load
-    int4 bq = make_int4(0, 0, 0, 0);
-    if (EpiTraits<EPI>::uni) bq = lds_int4(cst_g + static_cast<uint32_t>(g * 16));
-    const int32_t bias4[4] = {bq.x, bq.y, bq.z, bq.w};
-    if (EpiTraits<EPI>::flt) {
+    const CstAhead<EPI> now = ahead;
+    if (g < 3) ahead = load_ahead<EPI>(cst_g, g + 1);
+    if constexpr (EpiTraits<EPI>::flt) {
+      // x = bias + magic bits; y = bits of 2^-s; z = bits of M * (1 - 2^-s); w >> 1 = 2^t
+      int32_t bias[4], mult[4];
+      float2 s01 = uni_c1, s23 = uni_c1, add = uni_c2;
+      if constexpr (EpiTraits<EPI>::uni) {
+        bias[0] = now.v[0].x; bias[1] = now.v[0].y; bias[2] = now.v[0].z; bias[3] = now.v[0].w;
+        mult[0] = mult[1] = mult[2] = mult[3] = ep.uni_w >> 1;
+      } else if constexpr (EpiTraits<EPI>::paired) {
+        bias[0] = now.v[0].x; bias[1] = now.v[0].y; bias[2] = now.v[1].x; bias[3] = now.v[1].y;
+        s01 = make_float2(__int_as_float(now.v[0].z), __int_as_float(now.v[0].w));
+        s23 = make_float2(__int_as_float(now.v[1].z), __int_as_float(now.v[1].w));
+        add = make_float2(12582912.0f, 12582912.0f);
+      } else {
+        int4 c[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          c[b] = lds_int4(cst_g + static_cast<uint32_t>((g * 4 + b) * 16));
+          bias[b] = c[b].x;
+          mult[b] = c[b].w >> 1;
+        }
+        s01 = make_float2(__int_as_float(c[0].y), __int_as_float(c[1].y));
+        s23 = make_float2(__int_as_float(c[2].y), __int_as_float(c[3].y));
+        add = make_float2(12582912.0f, 12582912.0f);
+      }
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
-        const int j = g * 4 + b;
-        // x = bias + magic bits; y = bits of 2^-s; z = bits of M * (1 - 2^-s); w >> 1 = 2^t
-        const int4 c = EpiTraits<EPI>::uni ? make_int4(bias4[b], __float_as_int(ep.uni_c1), __float_as_int(ep.uni_c2), ep.uni_w)
-                                           : lds_int4(cst_g + static_cast<uint32_t>(j * 16));
-        int32_t v = static_cast<int32_t>(acc[j]);
-        if (EpiTraits<EPI>::res) v += rv[b] * (c.w >> 1);
-        const int32_t fb = relu ? __viaddmax_s32(v, c.x, kMagicBits) : v + c.x;
-        const float r = fmaf(__int_as_float(fb), __int_as_float(c.y), __int_as_float(c.z));
-        int32_t rb = min(__float_as_int(r), kMagicBits + 127);
-        if (!relu) rb = max(rb, kMagicBits + ep.lo);
-        q[b] = rb;                                     // the int8 code is the low byte
+        int32_t v = static_cast<int32_t>(acc[g * 4 + b]);
+        if (EpiTraits<EPI>::res) v += rv[b] * mult[b];
+        q[b] = relu ? __viaddmax_s32(v, bias[b], kMagicBits) : v + bias[b];
       }
-      const uint32_t lo2 = __byte_perm(static_cast<uint32_t>(q[0]), static_cast<uint32_t>(q[1]), 0x0040);
-      const uint32_t hi2 = __byte_perm(static_cast<uint32_t>(q[2]), static_cast<uint32_t>(q[3]), 0x0040);
-      wds[g] = __byte_perm(lo2, hi2, 0x5410);
+      wds[g] = round_pack_4<!EpiTraits<EPI>::uni>(q, s01, s23, add, relu, ep.lo);
     } else {
+      const int32_t bias4[4] = {now.v[0].x, now.v[0].y, now.v[0].z, now.v[0].w};
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
         const int j = g * 4 + b;
@@ -561,7 +644,8 @@ __device__ __forceinline__ void epilogue_16(const uint32_t (&acc)[16], uint32_t 
     }
   }
   uint32_t wds[4];
-  convert_16<EPI, RELU>(acc, cst + static_cast<uint32_t>(col) * (EpiTraits<EPI>::uni ? 4u : 16u), rw, ep, wds);
+  const uint32_t cst_g = cst + static_cast<uint32_t>(col) * EpiTraits<EPI>::cst_bytes;
+  convert_16<EPI, RELU>(acc, cst_g, load_ahead<EPI>(cst_g, 0), rw, ep, wds);
   if (prm.out_stage_bytes) {
     ptx::sts_uint4(stage_addr, wds[0], wds[1], wds[2], wds[3]);
   } else {
@@ -767,34 +851,35 @@ __device__ __forceinline__ void epilogue_pool_16(const uint32_t (&acc)[16], uint
     v4[i] = max(keep, __shfl_xor_sync(0xffffffffu, send, vbit));
   }
   const int c0 = (odd_q ? 8 : 0) + (odd_p ? 4 : 0);              // this lane's 4 columns of the 16
-  int4 bq = make_int4(0, 0, 0, 0);
-  if (EpiTraits<EPI>::uni) bq = lds_int4(cst + static_cast<uint32_t>(col + c0) * 4u);
-  const int32_t bias4[4] = {bq.x, bq.y, bq.z, bq.w};
-  int32_t q[4];
+  const uint32_t cst_g = cst + static_cast<uint32_t>(col + c0) * EpiTraits<EPI>::cst_bytes;
+  uint32_t word;
+  if constexpr (EpiTraits<EPI>::flt) {
+    const CstAhead<EPI> k = load_ahead<EPI>(cst_g, 0);
+    int32_t q[4];
+    int32_t bias[4] = {k.v[0].x, k.v[0].y, k.v[0].z, k.v[0].w};
+    float2 s01 = make_float2(ep.uni_c1, ep.uni_c1), s23 = s01, add = make_float2(ep.uni_c2, ep.uni_c2);
+    if constexpr (EpiTraits<EPI>::paired) {
+      bias[2] = k.v[1].x; bias[3] = k.v[1].y;
+      s01 = make_float2(__int_as_float(k.v[0].z), __int_as_float(k.v[0].w));
+      s23 = make_float2(__int_as_float(k.v[1].z), __int_as_float(k.v[1].w));
+      add = make_float2(12582912.0f, 12582912.0f);
+    }
 #pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    if (EpiTraits<EPI>::flt) {
-      const int4 c = EpiTraits<EPI>::uni ? make_int4(bias4[b], __float_as_int(ep.uni_c1), __float_as_int(ep.uni_c2), ep.uni_w)
-                                         : lds_int4(cst + static_cast<uint32_t>(col + c0 + b) * 16u);
-      const int32_t fb = relu ? __viaddmax_s32(v4[b], c.x, kMagicBits) : v4[b] + c.x;
-      const float r = fmaf(__int_as_float(fb), __int_as_float(c.y), __int_as_float(c.z));
-      int32_t rb = min(__float_as_int(r), kMagicBits + 127);
-      if (!relu) rb = max(rb, kMagicBits + ep.lo);
-      q[b] = rb;
-    } else {
+    for (int b = 0; b < 4; ++b) q[b] = relu ? __viaddmax_s32(v4[b], bias[b], kMagicBits) : v4[b] + bias[b];
+    word = round_pack_4<!EpiTraits<EPI>::uni>(q, s01, s23, add, relu, ep.lo);
+  } else {
+    int4 bq = make_int4(0, 0, 0, 0);
+    if (EpiTraits<EPI>::uni) bq = lds_int4(cst_g);
+    const int32_t bias4[4] = {bq.x, bq.y, bq.z, bq.w};
+    int32_t q[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
       const int4 c = EpiTraits<EPI>::uni ? make_int4(bias4[b], ep.uni_shift, ep.uni_z, ep.uni_w)
-                                         : lds_int4(cst + static_cast<uint32_t>(col + c0 + b) * 16u);
+                                         : lds_int4(cst_g + static_cast<uint32_t>(b) * 16u);
       int32_t v = relu ? __viaddmax_s32(v4[b], c.x, 0) : v4[b] + c.x;
       v = (v + c.z + ((v >> c.y) & c.w & 1)) >> c.y;
       q[b] = relu ? v : max(v, ep.lo);
     }
-  }
-  uint32_t word;
-  if (EpiTraits<EPI>::flt) {
-    const uint32_t lo2 = __byte_perm(static_cast<uint32_t>(q[0]), static_cast<uint32_t>(q[1]), 0x0040);
-    const uint32_t hi2 = __byte_perm(static_cast<uint32_t>(q[2]), static_cast<uint32_t>(q[3]), 0x0040);
-    word = __byte_perm(lo2, hi2, 0x5410);
-  } else {
     word = pack_sat_s8(q[1], q[0], pack_sat_s8(q[3], q[2], 0u));
   }
   if (store_ok)
@@ -1138,11 +1223,10 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     int it = 0;
     bool ok = true;
     const int kpad = prm.tiles_k * prm.BN;
-    const bool cst_all = EpiTraits<EPI>::uni ? kpad <= kBiasAllMax : kpad <= kChanAllMax;
+    const bool cst_all = static_cast<uint32_t>(kpad) * EpiTraits<EPI>::cst_bytes <= kCstBytes;
     if (cst_all) {
       for (int i = etid; i < kpad; i += kEpilogueWarps * 32) {
-        if (EpiTraits<EPI>::uni) sh->cst.bias[i] = __ldg(&chan_table[i].x);
-        else sh->cst.chan[i] = __ldg(chan_table + i);
+        stage_constant<EPI>(sh->cst, i, chan_table + i);
       }
       asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
     }
@@ -1205,8 +1289,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       if (!cst_all) {
         // stage this tile's channel constants, then meet the other epilogue warps
         for (int i = etid; i < prm.BN; i += kEpilogueWarps * 32) {
-          if (EpiTraits<EPI>::uni) sh->cst.bias[buf * 256 + i] = __ldg(&chan_table[tc.k0 + i].x);
-          else sh->cst.chan[buf * 256 + i] = __ldg(chan_table + tc.k0 + i);
+          stage_constant<EPI>(sh->cst, buf * 256 + i, chan_table + tc.k0 + i);
         }
         if (epilogue_vote(!ok)) { ok = false; break; }
       }
@@ -1277,7 +1360,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         __syncwarp();
         ptx::cluster_sync_all();                             // every sender's groups are here
         if (ok) {
-          const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : 0) * (EpiTraits<EPI>::uni ? 4u : 16u);
+          const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : 0) * EpiTraits<EPI>::cst_bytes;
 #pragma unroll
           for (int i = 0; i < kGroupsPerWarp; ++i) {
             const int own = (ew >> 2) + 2 * i, g = own * ks + ks_rank;
@@ -1312,7 +1395,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                                 static_cast<uint32_t>(buf * prm.tmem_cols);
         // shared-memory address of this tile's first channel constant (16 bytes per channel, or 4 when
         // only the biases differ)
-        const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : buf * 256) * (EpiTraits<EPI>::uni ? 4u : 16u);
+        const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : buf * 256) * EpiTraits<EPI>::cst_bytes;
         // This warp's 16-column groups, up to kGroupsPerWarp of them.  Tensor-memory loads run one
         // group ahead of the arithmetic; after the warp's last load the accumulator buffer goes back
         // to the MMA warp.
@@ -1383,34 +1466,39 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         } else if (kLeanOk && lean) {
           // loads one group ahead of the arithmetic, as below, without the bookkeeping
           const uint32_t t0 = t_addr + lean_col0;
-          const uint32_t c0 = chan + lean_col0 * (EpiTraits<EPI>::uni ? 4u : 16u);
-          auto group = [&](const uint32_t (&acc)[16], int i) {
+          const uint32_t c0 = chan + lean_col0 * EpiTraits<EPI>::cst_bytes;
+          constexpr uint32_t kGroupCst = 16u * EpiTraits<EPI>::cst_bytes;
+          auto group = [&](const uint32_t (&acc)[16], int i, const CstAhead<EPI>& ahead) {
             const uint32_t addr = stage_base + lean_off[i];
             uint32_t rw[4] = {0u, 0u, 0u, 0u}, wds[4];
             if (EpiTraits<EPI>::res) {                       // the residual tile was brought there by TMA
               const int4 r4 = lds_int4(addr);
               rw[0] = r4.x; rw[1] = r4.y; rw[2] = r4.z; rw[3] = r4.w;
             }
-            convert_16<EPI, RELU>(acc, c0 + static_cast<uint32_t>(i) * (EpiTraits<EPI>::uni ? 64u : 256u), rw, ep, wds);
+            convert_16<EPI, RELU>(acc, c0 + static_cast<uint32_t>(i) * kGroupCst, ahead, rw, ep, wds);
             ptx::sts_uint4(addr, wds[0], wds[1], wds[2], wds[3]);
           };
           ptx::tmem_ld_32x16(t0, acc_a);
+          CstAhead<EPI> k0 = load_ahead<EPI>(c0, 0);
           ptx::tmem_ld_wait();
           ptx::tmem_ld_32x16(t0 + 16, acc_b);
-          group(acc_a, 0);
+          CstAhead<EPI> k1 = load_ahead<EPI>(c0 + kGroupCst, 0);
+          group(acc_a, 0, k0);
           ptx::tmem_ld_wait();
           if (prm.BN == 128) {
             ptx::tmem_ld_32x16(t0 + 32, acc_a);
-            group(acc_b, 1);
+            k0 = load_ahead<EPI>(c0 + 2 * kGroupCst, 0);
+            group(acc_b, 1, k1);
             ptx::tmem_ld_wait();
             ptx::tmem_ld_32x16(t0 + 48, acc_b);
-            group(acc_a, 2);
+            k1 = load_ahead<EPI>(c0 + 3 * kGroupCst, 0);
+            group(acc_a, 2, k0);
             ptx::tmem_ld_wait();
             release();
-            group(acc_b, 3);
+            group(acc_b, 3, k1);
           } else {                                            // 64 wide: two groups per warp
             release();
-            group(acc_b, 1);
+            group(acc_b, 1, k1);
           }
         } else {
         if (g_begin < g_end) {

@@ -253,11 +253,10 @@ igemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     const int groups16 = prm.BN / 16, g_split = (groups16 + 1) / 2;
     const int g_begin = (ew < 4) ? 0 : g_split, g_end = (ew < 4) ? g_split : groups16;
     const int kpad = prm.tiles_k * prm.BN;
-    const bool cst_all = EpiTraits<EPI>::uni ? kpad <= kBiasAllMax : kpad <= kChanAllMax;
+    const bool cst_all = static_cast<uint32_t>(kpad) * EpiTraits<EPI>::cst_bytes <= kCstBytes;
     if (cst_all) {
       for (int i = etid; i < kpad; i += kEpilogueWarps * 32) {
-        if (EpiTraits<EPI>::uni) sh->cst.bias[i] = __ldg(&chan_table[i].x);
-        else sh->cst.chan[i] = __ldg(chan_table + i);
+        stage_constant<EPI>(sh->cst, i, chan_table + i);
       }
       asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
     }
@@ -272,8 +271,7 @@ igemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       const uint32_t use = static_cast<uint32_t>(it >> 1);
       if (!cst_all) {
         for (int i = etid; i < prm.BN; i += kEpilogueWarps * 32) {
-          if (EpiTraits<EPI>::uni) sh->cst.bias[buf * 256 + i] = __ldg(&chan_table[tc.k0 + i].x);
-          else sh->cst.chan[buf * 256 + i] = __ldg(chan_table + tc.k0 + i);
+          stage_constant<EPI>(sh->cst, buf * 256 + i, chan_table + tc.k0 + i);
         }
         if (epilogue_vote(!ok)) { ok = false; break; }
       }
@@ -289,7 +287,7 @@ igemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       }
       ptx::tc_fence_after();
       const uint32_t t_addr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(buf * prm.tmem_cols);
-      const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : buf * 256) * (EpiTraits<EPI>::uni ? 4u : 16u);
+      const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : buf * 256) * EpiTraits<EPI>::cst_bytes;
       auto release = [&]() {
         ptx::tc_fence_before();
         __syncwarp();

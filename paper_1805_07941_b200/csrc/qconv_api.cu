@@ -1390,15 +1390,17 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
   // tensor-core epilogue may round in fp32 (exactly).
   h->np = np;
   if (d.out_mode == QCONV_OUT_INT8 && d.groups == 1 && h->hints.float_rounding != 0 && !np) {
-    long long worst = 0;
+    // ... and below 2^15 after the shift, where the clamp works on 16-bit halves.
+    long long worst = 0, worst_out = 0;
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
-    for (int k = 0; k < d.K && worst < (1ll << 22); ++k) {
+    for (int k = 0; k < d.K && worst < (1ll << 22) && worst_out < 32767; ++k) {
       const long long bnd = qc::host_abs_sum(w_krsc + k * per_k, per_k) * (1ll << (d.n_in - 1)) +
                             (bias_host ? std::llabs(static_cast<long long>(bias_host[k])) : 0) +
                             (d.has_residual ? (128ll << res_lshift_host[k]) : 0);
       worst = std::max(worst, bnd);
+      worst_out = std::max(worst_out, (bnd >> (shift_host ? shift_host[k] : 0)) + 1);
     }
-    h->flt_epilogue = worst < (1ll << 22);
+    h->flt_epilogue = worst < (1ll << 22) && worst_out < 32767;
   }
 
   // choose the algorithm
