@@ -126,8 +126,8 @@ int qconv_set_plan_hints(const qconv_plan_hints* hints);
  *   shift_host      K right shifts s[k] = e_z - e_x - e_w[k] in [0, 31], or NULL for all zero
  *   res_lshift_host K left shifts t[k] = e_res - e_x - e_w[k] in [0, 23]; required iff has_residual
  *   acc_exp_host    K exponents e_x + e_w[k] in [-126, 96]; read only by QCONV_OUT_FLOAT; NULL means 0
- * The tables' device memory comes from a pool that keeps up to 64 MB of what destroyed handles gave back, until the
- * last handle of the device is gone.
+ * Tables and scratch come from a pool of device memory that keeps up to 256 MB of what destroyed handles gave back,
+ * until the last handle of the device is gone.
  * Errors: BAD_ARG, UNSUPPORTED_SHAPE, OVERFLOW_RISK when
  *   (R*S*C/groups) * 2^(n_in-1) * 2^(n_w-1) + max|bias| + 2^(7 + max t) > 2^31 - 1,
  * BAD_SHIFT, RESIDUAL_SCALE, ALIGNMENT, CUDA.  On error *out is NULL. */

@@ -104,8 +104,8 @@ inline bool is_window_mode(int m) { return m == MODE_S2D || m == MODE_WROW; }
 
 }  // namespace
 
-// Device memory of the handles' tables.  A network's calibration builds and destroys two handles per layer; cudaMalloc and
-// cudaFree took two thirds of that time.  Blocks given back are kept for the next handle, at most kKeep bytes per
+// Device memory of the handles' tables and scratch.  A network's calibration builds and destroys two handles per layer;
+// cudaMalloc and cudaFree took two thirds of that time, and at times a hundred milliseconds for one call.  Blocks given back are kept for the next handle, at most kKeep bytes per
 // device, and all of them are freed when the last block in use is given back.  Any thread, any stream: a block is only
 // given back after the device is idle, so whoever takes it next may overwrite it at once.
 class DevicePool {
@@ -150,7 +150,7 @@ class DevicePool {
   }
 
  private:
-  static constexpr size_t kKeep = 64u << 20;
+  static constexpr size_t kKeep = 256u << 20;
   struct PerDevice {
     std::vector<std::pair<void*, size_t>> free;            // oldest first
     size_t kept = 0, live = 0;
@@ -197,7 +197,7 @@ struct qconv_handle {
   int algo;                      // resolved QCONV_ALGO_*
   int lo, hi;
   // device copies: the small tables in one block, large weights in a second one that handles of the same weights share
-  DevicePool::Block block;
+  DevicePool::Block block, pack;
   std::shared_ptr<DevicePool::Block> weights;
   int a_channels = 0;            // channels of the activation tensor (planes * padded C for floating-point operands)
   const NpSpec* np = nullptr;    // set while the handle is built
@@ -263,7 +263,6 @@ namespace {
 
 void free_handle(qconv_handle* h) {
   if (!h) return;
-  cudaFree(h->d_pack);
   delete h;
 }
 
@@ -926,15 +925,15 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   cuuint32_t box[2] = {static_cast<cuuint32_t>(p.BKC), static_cast<cuuint32_t>(h->pair ? p.BN / 2 : p.BN)};
   rc = encode_map(&h->tmap_b, h->d_w, 2, dims, strides, box, p.BKC);
   if (rc) return rc;
-  if (is_window_mode(h->mode)) {
-    const size_t bytes = static_cast<size_t>(d.N) * h->s2d_h * h->s2d_wp * h->win_pb;
-    CUDA_TRY(cudaMalloc(&h->d_pack, bytes));
-    CUDA_TRY(cudaMemset(h->d_pack, 0, bytes));             // padding pixels and ragged edges stay zero
-  }
-  if (h->mode == MODE_STEM) {
-    const size_t bytes = static_cast<size_t>(d.N) * h->P * h->Q * h->kg_pad;
-    CUDA_TRY(cudaMalloc(&h->d_pack, bytes));
-    CUDA_TRY(cudaMemset(h->d_pack, 0, bytes));             // padding bytes of each row stay zero
+  size_t pack_bytes = 0;
+  if (is_window_mode(h->mode)) pack_bytes = static_cast<size_t>(d.N) * h->s2d_h * h->s2d_wp * h->win_pb;
+  if (h->mode == MODE_STEM) pack_bytes = static_cast<size_t>(d.N) * h->P * h->Q * h->kg_pad;
+  if (pack_bytes) {
+    // cleared once: padding pixels, ragged edges and the padding bytes of each row stay zero
+    CUDA_TRY(DevicePool::pool().take(&h->pack, pack_bytes));
+    h->d_pack = static_cast<int8_t*>(h->pack.ptr);
+    CUDA_TRY(cudaMemsetAsync(h->d_pack, 0, pack_bytes, nullptr));
+    CUDA_TRY(cudaStreamSynchronize(nullptr));              // (the stream of the first run need not wait for this one)
   }
   // the attribute belongs to the current device: once per device, not once per process
   static std::once_flag attr_once[64];

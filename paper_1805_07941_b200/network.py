@@ -11,6 +11,8 @@ conversion -- runs inside the library.  The bookkeeping it does is the paper's:
   * a residual input enters the accumulator shifted left by e_res - (e_x + e_w[k]);
   * right shifts s[k] = e_z - e_x - e_w[k] are never negative (factors in (0, 1]).
 """
+import concurrent.futures
+
 import numpy as np
 import torch
 
@@ -167,10 +169,16 @@ class QNetwork:
         self.e_buf["input"] = binding.qscale_exponent(gamma_of(st), self.n_bits)
         binding.qquantize_f32(x_calib, self.e_buf["input"], self.n_bits, out=self.bufs["input"][:n])
         convs = [nd for nd in self.net["nodes"] if nd["op"] == "conv"]
-        # the weights depend on nothing that is measured here: all layers at once, in parallel on the host
-        quantized = dict(zip([nd["name"] for nd in convs], binding.qquantize_weights_list(
-            [(self.weights[nd["name"]][0], nd["K"], nd["R"], nd["S"], nd["C"] // nd["groups"], self.net["per_channel"])
-             for nd in convs], self.n_bits)))
+        # the weights depend on nothing that is measured here: converted in the background, a few layers ahead of the
+        # measuring, each group in parallel on the host's cores
+        jobs = [(self.weights[nd["name"]][0], nd["K"], nd["R"], nd["S"], nd["C"] // nd["groups"], self.net["per_channel"])
+                for nd in convs]
+        ahead = concurrent.futures.ThreadPoolExecutor(1)
+        quantized = {}
+        for i in range(0, len(convs), 8):
+            group_jobs = ahead.submit(binding.qquantize_weights_list, jobs[i:i + 8], self.n_bits)
+            quantized.update((nd["name"], (group_jobs, j)) for j, nd in enumerate(convs[i:i + 8]))
+        ahead.shutdown(wait=False)
         # where only the maximum is wanted, the layer finds it itself and its float output is never written
         only_max = threshold is None and not keep_stats and not sync
         fbuf = None
@@ -184,7 +192,8 @@ class QNetwork:
                 continue
             cands, floats = [], {}
             for nd in stage:
-                wq, e_w = quantized[nd["name"]]
+                pending, j = quantized[nd["name"]]
+                wq, e_w = pending.result()[j]
                 b = self.weights[nd["name"]][1]
                 e_x = self.e_buf[nd["src"]]
                 bias_q = binding.qquantize_bias(b, e_x, e_w)
