@@ -102,7 +102,8 @@ typedef struct {
   int uniform_shift;     /* the instantiation for one shift per layer: 0 = per-channel constants    */
   int tma_store;         /* output tiles staged in shared memory and stored by TMA: 0 never, 1 wherever they fit */
   int tma_residual;      /* residual tiles fetched by TMA into the staged tiles: 0 never            */
-  int depthwise_form;    /* 0: general dp4a kernel, 1: tap-packed kernel with register loads (no TMA rows) */
+  int depthwise_form;    /* 0: general dp4a kernel, 1: tap-packed kernel with register loads (no TMA rows),
+                            2: with TMA rows, 3: tensor cores wherever they fit                     */
   int pdl;               /* programmatic dependent launch: 0 off                                    */
   int group_taps;        /* 3x3-like layers on at most 64 channels, the taps of a filter row sharing
                             one ring stage: 0 never, 1 wherever the shape allows                    */

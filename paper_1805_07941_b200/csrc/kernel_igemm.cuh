@@ -895,6 +895,14 @@ __device__ __forceinline__ void epilogue_pool_16(const uint32_t (&acc)[16], uint
 // consecutive.  Per launch in a train: 7 x 7 x 512 3 x 3 6.9 -> 4.5 us, 7 x 7 x 2048 -> 512 6.2 -> 4.2, 14 x 14 x 256
 // 3 x 3 4.6 -> 4.0; ResNet-50 on one image 212 -> 199 us.
 //
+// Depthwise 3 x 3 (RSTG == 5).  A tile's BN channels are its contraction chunk too (BKC = BN bytes of a pixel), and only
+// the diagonal of a tap's matrix is not zero.  An MMA of N <= 96 takes 54 cycles whatever its width, so the chunk's MMAs
+// (32 bytes along K each) multiply a 32 x 32 block, each into accumulator columns of its own: 9 taps x BN / 32 MMAs a
+// tile, which leaves the CUDA cores the conversion alone (the tap-packed kernels spend 17 instructions an output).
+// Weights: [channel][tap][32], the tap's weight at position channel % 32.  Per launch, batch 256: 112 x 112 x 64 stride 2
+// 61 -> 49 us, 56 x 56 x 128 78 -> 71, stride 2 35 -> 28, 28 x 28 x 256 43 -> 37, stride 2 21 -> 14, 14 x 14 x 512
+// 26 -> 22, 7 x 7 x 1024 16.7 -> 14.2; a single image 6.4 -> 4.6.
+//
 // Persistent kernel: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...  The shared-memory
 // ring of operand stages runs on across tiles, and the accumulator is double-buffered in tensor
 // memory so the epilogue of one tile overlaps the loads and MMAs of the next.
@@ -924,6 +932,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
   const int lane = threadIdx.x & 31;
   constexpr bool kPool = RSTG == 2;              // 2 x 2 max-pool taken in the epilogue
   constexpr bool kSplit = RSTG == 4;             // this CTA's cluster shares one tile's contraction
+  constexpr bool kDw = RSTG == 5;                // depthwise
+  const int b_row = kDw ? 32 : prm.BKC;          // bytes of a weight row per stage and tap
   constexpr bool kHint = GPW > kGroupsPerWarp;   // one CTA per SM on long stages: waits use the suspend hint
   const int num_kb = prm.R * prm.S * prm.nchunks;
   const int total_tiles = prm.tiles_q * prm.tiles_p * prm.tiles_n * prm.tiles_k;
@@ -998,16 +1008,16 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
         const int product = prm.fd_np_cpp.divmod(ci, &in_plane);
         a_ci = prm.np_a[product] * prm.np_cpp + in_plane;
       }
-      const int a_c = a_ci * prm.BKC;
+      const int a_c = kDw ? tc.k0 : a_ci * prm.BKC;
       if (doit) {
         ptx::mbar_expect_tx(full, prm.tx_bytes);
         if (!prm.b_resident) {
           if (prm.halo_s) {
             for (int hs = 0; hs < prm.halo_s; ++hs)
               ptx::tma_load_2d(a_dst + prm.a_stage_bytes + static_cast<uint32_t>(hs) * prm.b_chunk_bytes, &tmap_b, full,
-                               ((r * prm.halo_s + hs) * prm.nchunks + ci) * prm.BKC, tc.k0);
+                               ((r * prm.halo_s + hs) * prm.nchunks + ci) * b_row, tc.k0);
           } else {
-            ptx::tma_load_2d(a_dst + prm.a_stage_bytes, &tmap_b, full, ((r * prm.S + sx) * prm.nchunks + ci) * prm.BKC, tc.k0);
+            ptx::tma_load_2d(a_dst + prm.a_stage_bytes, &tmap_b, full, ((r * prm.S + sx) * prm.nchunks + ci) * b_row, tc.k0);
           }
         }
         if (first) ptx::grid_dependency_wait();
@@ -1101,7 +1111,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     //    instructions, which is what bounds layers whose stages carry little tensor work.
     {
       const bool leader = ptx::elect_one();
-      const uint32_t idesc = make_idesc_i8(prm.BN);
+      const uint32_t idesc = make_idesc_i8(kDw ? 32 : prm.BN);
       const int mma_per_stage = prm.BKC / 32;
       const uint32_t tiles_addr = ptx::smem_u32(tiles);
       const bool bres = prm.b_resident != 0;
@@ -1118,11 +1128,11 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           for (int hs = 0; hs < per_stage; ++hs)
             ptx::tma_load_2d(tiles_addr + b_res_off + static_cast<uint32_t>(kb) * prm.b_stage_bytes +
                                  static_cast<uint32_t>(hs) * prm.b_chunk_bytes,
-                             &tmap_b, bar, (kb * per_stage + hs) * prm.BKC, k0);
+                             &tmap_b, bar, (kb * per_stage + hs) * b_row, k0);
       }
       __syncwarp();
       const uint64_t a_desc0 = make_kmajor_desc(tiles_addr, prm.BKC);
-      const uint64_t b_desc0 = make_kmajor_desc(tiles_addr + (bres ? b_res_off : prm.a_stage_bytes), prm.BKC);
+      const uint64_t b_desc0 = make_kmajor_desc(tiles_addr + (bres ? b_res_off : prm.a_stage_bytes), b_row);
       const uint64_t desc_step = stage_bytes >> 4;          // start-address field counts 16-byte units
       // resident weights: chunk kb of the tile sits at its own place, whatever the ring position
       const uint64_t b_step = bres ? (prm.b_stage_bytes >> 4) : desc_step;
@@ -1133,6 +1143,19 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       // patch form: from a filter row's last tap to the next row's first one
       const uint64_t halo_next_row = static_cast<uint64_t>((prm.tq - prm.halo_w + 1) * prm.BKC) >> 4;
       const uint32_t full0 = ptx::smem_u32(&sh->full[0]), empty0 = ptx::smem_u32(&sh->empty[0]);
+      // One tap's chunk: 32 bytes along K inside the swizzle span = +2 in the descriptor's 16-byte address units.
+      // (depthwise: 32 channels each, against their own 1 KB of weights, into their own columns)
+      auto tap_mmas = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+        constexpr uint32_t dn = kDw ? 32u : 0u;
+        constexpr uint64_t bk = kDw ? 64u : 2u;
+        const uint32_t later = kDw ? acc : 1u;
+        ptx::mma_i8(d, a, b, idesc, acc);
+        if (mma_per_stage > 1) ptx::mma_i8(d + dn, a + 2u, b + bk, idesc, later);
+        if (mma_per_stage > 2) {
+          ptx::mma_i8(d + 2u * dn, a + 4u, b + 2u * bk, idesc, later);
+          ptx::mma_i8(d + 3u * dn, a + 6u, b + 3u * bk, idesc, later);
+        }
+      };
       int stage = 0, it = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -1162,13 +1185,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           }
           ptx::tc_fence_after();
           if (leader) {
-            // 32 bytes along K inside the swizzle span = +2 in the descriptor's 16-byte address units
-            ptx::mma_i8(d_tmem, a_desc, b_desc, idesc, accumulate);
-            if (mma_per_stage > 1) ptx::mma_i8(d_tmem, a_desc + 2u, b_desc + 2u, idesc, 1u);
-            if (mma_per_stage > 2) {
-              ptx::mma_i8(d_tmem, a_desc + 4u, b_desc + 4u, idesc, 1u);
-              ptx::mma_i8(d_tmem, a_desc + 6u, b_desc + 6u, idesc, 1u);
-            }
+            tap_mmas(d_tmem, a_desc, b_desc, accumulate);
             // halo form: the other horizontal taps are the same activation rows one pixel (one row of BKC
             // bytes) further on -- start address advanced by a row, the descriptor's base offset telling the
             // swizzle phase of the new first row -- against the next weight chunk of the stage
@@ -1177,12 +1194,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
               if (hw == prm.halo_w) { ah += halo_next_row; hw = 0; }
               else ah += halo_row;
               bh += halo_bchunk;
-              ptx::mma_i8(d_tmem, ah, bh, idesc, 1u);
-              if (mma_per_stage > 1) ptx::mma_i8(d_tmem, ah + 2u, bh + 2u, idesc, 1u);
-              if (mma_per_stage > 2) {
-                ptx::mma_i8(d_tmem, ah + 4u, bh + 4u, idesc, 1u);
-                ptx::mma_i8(d_tmem, ah + 6u, bh + 6u, idesc, 1u);
-              }
+              tap_mmas(d_tmem, ah, bh, 1u);
             }
             ptx::mma_commit(empty0 + 8u * stage);             // stage free once these MMAs retire
           }

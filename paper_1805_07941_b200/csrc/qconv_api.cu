@@ -219,6 +219,8 @@ struct qconv_handle {
   int num_sms = 148;
   int ctas_per_sm = 2;
   int use_pdl = 1;
+  int dw_mma = 0;                // depthwise on the tensor cores (prm, mode and the maps are then its plan)
+  int8_t* d_w_mma = nullptr;     // its weights: [C][9][32]
   uint32_t* d_dw_tap = nullptr;  // tap-packed form: weight rows [3][C], bias + magic [C], 2^-s [C], rounding offset [C] (float bits)
   int dw_tap = 0;
   int patch = 0;                 // 1: patch form (one activation box of 16 x (tp + 2) pixels serves all nine taps)
@@ -432,6 +434,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const qconv_plan_hints& hint = h->hints;
   qc::IgemmParams& p = h->prm;
   int c_eff = d.C;                 // channels of the GEMM's activation operand
+  const bool dw = h->dw_mma != 0;
   int taps_r = d.R, taps_s = d.S;
   if (h->mode == MODE_STEM) {
     // packed patch row: either the R*S*C taps back to back, or (when a filter row is at most 28
@@ -516,7 +519,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const int taps_s_w = taps_s;                             // taps per filter row in the packed weights
   // It costs three weight chunks per stage, so it is used where tiles are 64 channels wide anyway (layers below
   // one wave, which sit at the fill rate), not for the wide tiles of the tensor-bound layers.
-  const bool halo_fits = h->mode == MODE_BOX && d.stride_h == 1 && d.stride_w == 1 && d.S == 3 && d.pad_w == 1 && (d.C == 64 || d.C % 128 == 0) &&
+  const bool halo_fits = h->mode == MODE_BOX && d.stride_h == 1 && d.stride_w == 1 && d.S == 3 && d.pad_w == 1 && (dw || d.C == 64 || d.C % 128 == 0) &&
                          hint.halo != 0 && d.pool == 0;
   bool halo = false;
   // Its tile: whole image rows with their halo, W + 2 accumulator rows per image row (two of them discarded);
@@ -528,9 +531,13 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     *tp = std::max(1, std::min(h->P, qc::kTileM / *tq));
     *tn = (halo_segs == 1 && *tp == h->P) ? std::max(1, std::min(d.N, qc::kTileM / (*tq * *tp))) : 1;
   };
+  const PatchTile pt = patch_tile(h->Q, h->P, d.pool != 0);
   p.BKC = choose_bkc(c_eff);
   if (is_window_mode(h->mode)) p.BKC = c_eff <= 32 ? 32 : (c_eff <= 64 ? 64 : 128);   // a row is one chunk (two at most)
-  p.nchunks = ceil_div(c_eff, p.BKC);
+  // (depthwise at stride 2: rows of 64 bytes, the three taps of a filter row sharing a stage)
+  if (dw) p.BKC = d.C % 128 == 0 && d.stride_h == 1 && !(hint.bn_max > 0 && hint.bn_max < 128) ? 128 : d.C % 64 == 0 ? 64 : 32;
+  p.nchunks = dw ? 1 : ceil_div(c_eff, p.BKC);
+  const int b_row = dw ? 32 : p.BKC;                       // bytes of a weight row per chunk
   h->a_channels = d.C;
   p.acc_bufs = 2;
   p.ksplit = 1;
@@ -564,7 +571,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
       m_tiles = static_cast<long>(ceil_div(h->Q, tq)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
     }
     const long contraction = static_cast<long>(taps_r) * taps_s * p.nchunks * p.BKC;
-    if (hint.bn_max > 128) wide = shape_ok;
+    if (dw) wide = false;
+    else if (hint.bn_max > 128) wide = shape_ok;
     else if (hint.bn_max <= 0)
       wide = shape_ok && k_eff >= 256 && contraction >= 2048 && m_tiles * ceil_div(k_eff, 256) >= h->num_sms;
     if (wide) bn_max = 2 * qc::kGroupsPerWarpWide * 16;
@@ -575,7 +583,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     h->pair = wide && hint.pair_tiles != 0 &&
               (hint.pair_tiles == 1 || ceil_div_l(m_tiles, 2) * ceil_div(k_eff, 256) >= 4L * (h->num_sms / 2));
   }
-  if (hint.bn_max <= 0 && k_eff > 64 && !wide) {
+  if (hint.bn_max <= 0 && k_eff > 64 && !wide && !dw) {
     // A layer with fewer 128-wide tiles than SMs leaves SMs idle while each busy one walks a long
     // chain of MMAs: halve the tile width to spread the work (measured: helps below one wave only).
     long m_tiles;
@@ -597,10 +605,18 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     p.acc_bufs = np->products <= 4 ? 2 : 1;
   }
   halo = halo_fits && (bn_max <= 64 || k_eff <= 64 || (np && np->products >= 3) || hint.halo == 1);
+  if (dw) {
+    // stride 1: the form (patch, or a box per filter row) whose tiles waste fewer accumulator rows
+    int tq, tp, tn, step;
+    halo_box(&tq, &tp, &tn, &step);
+    const long halo_tiles = static_cast<long>(ceil_div(h->Q, step)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
+    bn_max = p.BKC;
+    halo = halo_fits && halo_tiles < static_cast<long>(pt.segs) * pt.rows * d.N;
+  }
   if (halo) {
     wide = false;
     h->pair = 0;
-    if (!(hint.halo == 1 && hint.bn_max >= 128)) bn_max = std::min(bn_max, 64);   // three weight chunks per stage: keep the stage small
+    if (!dw && !(hint.halo == 1 && hint.bn_max >= 128)) bn_max = std::min(bn_max, 64);   // three weight chunks per stage: keep the stage small
     taps_s = 1;                                            // what the kernel's stage loop sees
     p.S = 1;
   }
@@ -610,7 +626,6 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   // channels), this is what limits the layer.  us: 64 x 224 x 224 x 64 -> 64 with its pool 167 -> 129, 64 x 112 x 112 x 64
   // -> 128 72 -> 60, x 128 -> 128 with its pool 102 -> 84, 128 x 28 x 28 x 96 -> 128 20.0 -> 14.8, 128 x 14 x 14 x 112 -> 224
   // 14.8 -> 9.1; at one wave of tiles (32 x 28 x 28 x 128 -> 128: 7.2 -> 6.8) it is about even.
-  const PatchTile pt = patch_tile(h->Q, h->P, d.pool != 0);
   const bool patch_fits = h->mode == MODE_BOX && d.R == 3 && d.S == 3 && d.stride_h == 1 && d.stride_w == 1 && d.pad_h == 1 && d.pad_w == 1 &&
                           p.nchunks == 1 && p.BKC >= 64 && fast_possible && d.K % 16 == 0 && d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0;
   bool patch = false;
@@ -621,11 +636,12 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // tiles at most
     patch = hint.patch_halo == 1 || (tiles >= h->num_sms && used >= 0.75 && k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0);
   }
+  if (dw) patch = !halo && halo_fits && hint.patch_halo != 0;
   if (patch) {
     wide = false;
     halo = false;
     h->pair = 0;
-    bn_max = 128;
+    bn_max = dw ? p.BKC : 128;
     taps_r = taps_s = 1;
     p.R = p.S = 1;
   }
@@ -642,7 +658,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     const int tk = ceil_div(k_eff, bn_max);
     const int bn = static_cast<int>(align_up(ceil_div(k_eff, tk), 16));
     const int a_tap = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM) * p.BKC, 1024));
-    const int b_chunk = static_cast<int>(align_up(static_cast<size_t>(bn) * p.BKC, 1024));
+    const int b_chunk = static_cast<int>(align_up(static_cast<size_t>(bn) * b_row, 1024));
     const int budget = 113 * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared));
     int tq, tp, tn;
     choose_box(h->Q, h->P, d.N, &tq, &tp, &tn, d.pool != 0);
@@ -665,7 +681,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   p.BN = static_cast<int>(align_up(ceil_div(k_eff, p.tiles_k), 16));
   h->kpad = p.tiles_k * p.BN;
   const int all_taps = patch ? 9 : taps_r * taps_s_w;
-  h->kg_total = all_taps * p.nchunks * p.BKC;
+  h->kg_total = all_taps * p.nchunks * b_row;
   p.K = k_eff;
   p.out_c_offset = d.out_c_offset;
   p.out_c_pitch = h->fold > 1 ? k_eff : d.out_c_pitch;
@@ -702,7 +718,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const int out_tile = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM) * p.BN, 1024));
   auto ring_stages = [&](int bkc, int staged_tiles) {
     const int a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * bkc, 1024)) * (group ? tps : 1);
-    const int b = static_cast<int>(align_up(static_cast<size_t>(h->pair ? p.BN / 2 : p.BN) * bkc, 1024)) * tps;
+    const int b = static_cast<int>(align_up(static_cast<size_t>(h->pair ? p.BN / 2 : p.BN) * (dw ? 32 : bkc), 1024)) * tps;
     return (full_budget - staged_tiles * out_tile) / (a + b);
   };
   const bool force_stage = hint.tma_store == 1;
@@ -728,7 +744,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   // they still do)
   const int patch_a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + 2 * 16 + 8) * p.BKC, 1024));
   if (patch) {
-    const int b_res = 9 * static_cast<int>(align_up(static_cast<size_t>(p.BN) * p.BKC, 1024));
+    const int b_res = 9 * static_cast<int>(align_up(static_cast<size_t>(p.BN) * b_row, 1024));
     const bool may_stage = p.fast_epilogue && hint.tma_store != 0 && (p.BN == 64 || p.BN == 128) && !d.pool && !d.has_residual;
     bool placed = false;
     p.out_stage_bytes = 0;
@@ -747,12 +763,12 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     p.store_rows = p.out_stage_bytes ? pt.tp : 0;
   }
   const int staged_tiles = p.out_stage_bytes ? p.out_stage_bufs : 0;
-  h->kg_total = all_taps * p.nchunks * p.BKC;
+  h->kg_total = all_taps * p.nchunks * b_row;
   // (halo form: the shifted operand reads up to two rows past the 128th, and a stage holds three weight chunks)
   p.a_tap_bytes = patch ? static_cast<uint32_t>(patch_a)
                         : static_cast<uint32_t>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * p.BKC, 1024));
   p.a_stage_bytes = p.a_tap_bytes * (group ? static_cast<uint32_t>(tps) : 1u);
-  p.b_chunk_bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(h->pair ? p.BN / 2 : p.BN) * p.BKC, 1024));
+  p.b_chunk_bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(h->pair ? p.BN / 2 : p.BN) * b_row, 1024));
   p.b_stage_bytes = p.b_chunk_bytes * static_cast<uint32_t>(tps);
   p.out_swz_mask = p.BN == 128 ? 7u : (p.BN == 64 ? 3u : (p.BN == 32 ? 1u : 0u));
   int stages = ring_stages(p.BKC, staged_tiles);
@@ -817,15 +833,15 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "pool: needs the tensor-core path with per-tap boxes and an int8 output at 8 bits "
                 "with nearest-even rounding, K %% 16 == 0 and an accumulator bound below 2^31 - 2^(s-1)");
   }
-  p.tx_bytes = static_cast<uint32_t>((group ? tps : 1) * p.tq * p.tp * p.tn * p.BKC + (p.b_resident ? 0 : tps * p.BN * p.BKC));
+  p.tx_bytes = static_cast<uint32_t>((group ? tps : 1) * p.tq * p.tp * p.tn * p.BKC + (p.b_resident ? 0 : tps * p.BN * b_row));
   if (patch) p.tx_bytes = static_cast<uint32_t>(16 * (p.tp + 2) * p.BKC);
-  p.b_res_tx_bytes = static_cast<uint32_t>(num_kb_plan * tps * p.BN * p.BKC);
+  p.b_res_tx_bytes = static_cast<uint32_t>(num_kb_plan * tps * p.BN * b_row);
   p.res_tx_bytes = static_cast<uint32_t>(p.tq * p.tp * p.tn * p.BN);
 
   // weights -> [kpad][kg_total], K-major rows, zero padded (already in that form when nothing is padded or folded)
   const size_t w_bytes = static_cast<size_t>(h->kpad) * h->kg_total;
   const bool as_is = h->fold == 1 && !is_window_mode(h->mode) && h->mode != MODE_STEM && h->kpad == d.K && p.nchunks * p.BKC == d.C &&
-                     !np;
+                     !np && !dw;
   std::vector<int8_t> wp(as_is ? 0 : w_bytes, 0);
   std::vector<int8_t> row(static_cast<size_t>(std::max(c_row, 1)), 0);
   for (int m = 0; np && m < np->products; ++m)             // [product][chunk] inside a tap
@@ -833,7 +849,9 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
       for (int t = 0; t < d.R * d.S; ++t)
         std::memcpy(wp.data() + static_cast<size_t>(k) * h->kg_total + (static_cast<size_t>(t) * p.nchunks + m * p.np_cpp) * p.BKC,
                     np->w[m] + (static_cast<size_t>(k) * d.R * d.S + t) * d.C, d.C);
-  for (int k = 0; k < d.K && !as_is && !np; ++k) {
+  for (int k = 0; k < d.K && dw; ++k)
+    for (int t = 0; t < 9; ++t) wp[static_cast<size_t>(k) * h->kg_total + t * 32 + k % 32] = w_krsc[static_cast<size_t>(k) * 9 + t];
+  for (int k = 0; k < d.K && !as_is && !np && !dw; ++k) {
     const int8_t* src = w_krsc + static_cast<size_t>(k) * d.R * d.S * h->Cg;
     if (h->fold > 1 && !is_window_mode(h->mode)) {
       // one pixel's row as the unfolded GEMM would see it, then once per folded pixel on the diagonal
@@ -887,7 +905,9 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
         std::memcpy(dst + static_cast<size_t>(t) * p.nchunks * p.BKC, src + static_cast<size_t>(t) * d.C, d.C);
     }
   }
-  int rc = place_weights(h, parts, as_is ? w_krsc : wp.data(), w_bytes, as_is, weights_of);
+  int rc = QCONV_OK;
+  if (dw) parts.add(&h->d_w_mma, wp.data(), w_bytes);      // (beside the tables of the kernels for other alignments)
+  else rc = place_weights(h, parts, as_is ? w_krsc : wp.data(), w_bytes, as_is, weights_of);
   if (rc) return rc;
   std::vector<int4> chan(h->kpad, make_int4(0, 0, 0, 0));
   for (int k = 0; k < d.K; ++k) {
@@ -922,8 +942,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   if (rc) return rc;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->kg_total), static_cast<cuuint64_t>(h->kpad)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->kg_total)};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(p.BKC), static_cast<cuuint32_t>(h->pair ? p.BN / 2 : p.BN)};
-  rc = encode_map(&h->tmap_b, h->d_w, 2, dims, strides, box, p.BKC);
+  cuuint32_t box[2] = {static_cast<cuuint32_t>(b_row), static_cast<cuuint32_t>(h->pair ? p.BN / 2 : p.BN)};
+  rc = encode_map(&h->tmap_b, dw ? h->d_w_mma : h->d_w, 2, dims, strides, box, b_row);
   if (rc) return rc;
   size_t pack_bytes = 0;
   if (is_window_mode(h->mode)) pack_bytes = static_cast<size_t>(d.N) * h->s2d_h * h->s2d_wp * h->win_pb;
@@ -983,7 +1003,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   if (h->pair) {
     PairKernel pk = pair_kernel_for(h);
     CUDA_TRY(cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  } else if (d.pool) {
+  } else if (d.pool || dw) {
     CUDA_TRY(cudaFuncSetAttribute(igemm_kernel_for(h), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   }
   return QCONV_OK;
@@ -1009,6 +1029,11 @@ IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
   if (h->d.out_mode == QCONV_OUT_FLOAT) return qc::igemm_i8_kernel<qc::EPI_F32>;
   if (!h->prm.fast_epilogue) return qc::igemm_i8_kernel<qc::EPI_I8>;
   const bool uni = h->uniform_shift && h->hints.uniform_shift != 0;
+  if (h->dw_mma) {
+    constexpr int G = qc::kGroupsPerWarp;
+    if (h->d.relu) return uni ? qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 1, 5, G> : qc::igemm_i8_kernel<qc::EPI_FLT_I8, 1, 5, G>;
+    return uni ? qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 0, 5, G> : qc::igemm_i8_kernel<qc::EPI_FLT_I8, 0, 5, G>;
+  }
   if (h->d.pool) {                                         // 2 x 2 max-pool in the epilogue (ReLU read at run time)
     constexpr int W = qc::kGroupsPerWarpWide;
     if (h->prm.BN > 128) {
@@ -1048,7 +1073,7 @@ IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
 int choose_ksplit(const qconv_handle* h, long tiles) {
   const qc::IgemmParams& p = h->prm;
   const int num_kb = p.R * p.S * p.nchunks, groups = p.BN / 16, want = h->hints.split_k;
-  if (!p.fast_epilogue || h->d.pool || p.b_resident || h->pair || p.BN > 128 || want == 0) return 1;
+  if (!p.fast_epilogue || h->d.pool || p.b_resident || h->pair || h->dw_mma || p.BN > 128 || want == 0) return 1;
   auto fits = [&](int ks) { return groups % ks == 0 && tiles * ks <= h->num_sms && num_kb >= ks; };
   if (want > 0) return (want == 2 || want == 4) && fits(want) ? want : 1;
   // A stage of a chain costs a quarter of a microsecond, one of three taps 0.4, the exchange about one.  In these units (2
@@ -1388,7 +1413,7 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
   // Weight-aware bound of the wide value: 2^(n_in-1) * sum|w[k,.]| + |bias[k]| + 128 * 2^t[k].  Below 2^22 the
   // tensor-core epilogue may round in fp32 (exactly).
   h->np = np;
-  if (d.out_mode == QCONV_OUT_INT8 && d.groups == 1 && h->hints.float_rounding != 0 && !np) {
+  if (d.out_mode == QCONV_OUT_INT8 && (d.groups == 1 || (Cg == 1 && d.C == d.K)) && h->hints.float_rounding != 0 && !np) {
     // ... and below 2^15 after the shift, where the clamp works on 16-bit halves.
     long long worst = 0, worst_out = 0;
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
@@ -1479,8 +1504,17 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       parts.add(&h->d_dw_tap, t.data(), t.size() * 4);
       h->dw_tap = 1;
       if (d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
+      // On the tensor cores where a pixel's channels fill rows of 64 or 128 bytes (with rows of 32 the per-tile work
+      // outweighs it: 112 x 112 x 32 at batch 256 76 -> 96 us).
+      h->dw_mma = h->flt_epilogue && d.pad_h == 1 && d.pad_w == 1 && d.C % (h->hints.depthwise_form == 3 ? 32 : 64) == 0 &&
+                  d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && (h->hints.depthwise_form < 0 || h->hints.depthwise_form == 3);
     }
-    if (!rc) rc = parts.upload(&h->block);
+    if (!rc && h->dw_mma) {
+      h->mode = MODE_BOX;
+      rc = plan_igemm(h, parts, nullptr, w_krsc, bias_host, shift_host, nullptr, nullptr);
+    } else if (!rc) {
+      rc = parts.upload(&h->block);
+    }
   }
   if (rc) {
     free_handle(h);
@@ -1537,7 +1571,8 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
   if (h->algo == QCONV_ALGO_DIRECT) {
     qc::direct_conv_kernel<<<grid_for(outs * d.K, 256, h->num_sms * 64), 256, 0, st>>>(d_x, h->d_w, d_residual, d_y,
                                                                                 g, ep);
-  } else if (h->algo == QCONV_ALGO_DEPTHWISE) {
+  } else if (h->algo == QCONV_ALGO_DEPTHWISE &&
+             !(h->dw_mma && ((reinterpret_cast<uintptr_t>(d_x) | reinterpret_cast<uintptr_t>(d_y)) & 15) == 0)) {
     if ((reinterpret_cast<uintptr_t>(d_x) | reinterpret_cast<uintptr_t>(d_y) |
          reinterpret_cast<uintptr_t>(d_residual)) & 3)
       return fail(QCONV_ERR_ALIGNMENT, "depthwise kernel needs 4-byte aligned tensors");
@@ -1919,12 +1954,12 @@ int qconv_set_wait_limit(qconv_handle* h, unsigned int polls) {
 
 int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len) {
   if (!h || !buf || buf_len == 0) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
-  if (h->algo == QCONV_ALGO_IGEMM) {
+  if (h->algo == QCONV_ALGO_IGEMM || h->dw_mma) {
     static const char* names[] = {"flat", "view", "box", "stem", "s2d", "wrow"};
     const qc::IgemmParams& p = h->prm;
-    snprintf(buf, buf_len, "igemm/%s box=%dx%dx%d BN=%d tiles_k=%d BKC=%d chunks=%d taps=%dx%d stages=%d smem=%zu "
+    snprintf(buf, buf_len, "%s/%s box=%dx%dx%d BN=%d tiles_k=%d BKC=%d chunks=%d taps=%dx%d stages=%d smem=%zu "
              "ctas/sm=%d fast=%d uni=%d flt=%d fold=%d tma_store=%d b_res=%d halo=%d grp=%d pair=%d pool=%d%s",
-             names[h->mode], p.tq, p.tp, p.tn, p.BN, p.tiles_k, p.BKC, p.nchunks, p.R, p.S, p.stages,
+             h->dw_mma ? "depthwise3x3/mma" : "igemm", names[h->mode], p.tq, p.tp, p.tn, p.BN, p.tiles_k, p.BKC, p.nchunks, p.R, p.S, p.stages,
              h->smem_bytes, h->ctas_per_sm, p.fast_epilogue, h->uniform_shift, h->flt_epilogue && p.fast_epilogue, h->fold,
              p.out_stage_bytes ? p.out_stage_bufs : 0, p.b_resident, p.tap_boxes || h->patch ? 0 : p.halo_s, p.tap_boxes ? p.halo_s : 0, h->pair, h->d.pool, h->patch ? " patch=1" : "");
   } else {

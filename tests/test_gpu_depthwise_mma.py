@@ -1,0 +1,48 @@
+"""The depthwise layers on the tensor cores against the oracle: rows of 32, 64 and 128 bytes, images around the tile, both
+strides, concat window, per-layer and per-channel shifts, and tensors too little aligned for it (the other kernels)."""
+import numpy as np
+import pytest
+import torch
+
+from tests.helpers import gpu_conv, oracle_conv, rand_layer
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # N, H, W, C, stride
+    (2, 9, 11, 32, 1), (1, 8, 14, 64, 1), (3, 7, 7, 128, 1), (2, 9, 15, 128, 1), (1, 1, 1, 64, 1), (2, 17, 130, 192, 1),
+    (2, 14, 14, 64, 2), (1, 13, 9, 128, 2), (5, 3, 2, 96, 2), (1, 30, 61, 32, 2), (40, 14, 14, 256, 1), (40, 14, 14, 256, 2)]
+
+
+@pytest.mark.parametrize("case", CASES)
+@pytest.mark.parametrize("uniform", [0, 1])
+def test_depthwise_on_tensor_cores_matches_the_oracle(case, uniform):
+    from paper_1805_07941_b200 import binding
+    N, H, W, C, st = case
+    rng = np.random.default_rng(sum(case))
+    x, w, bias, shift, _, _ = rand_layer(rng, N, H, W, C, C, 3, 3, groups=C, stride=(st, st), pad=(1, 1), per_channel_shift=not uniform)
+    shift = (shift - 1).clip(4, 31)
+    for relu in (0, 1):
+        kw = dict(R=3, S=3, stride=(st, st), pad=(1, 1), groups=C, relu=relu)
+        win = dict(kw, out_c_offset=16, out_c_pitch=C + 32)
+        want, want_win = oracle_conv(x, w, bias, shift, **kw), oracle_conv(x, w, bias, shift, **win)
+        for hints in (dict(), dict(bn_max=64), dict(patch_halo=0), dict(patch_halo=0, halo=0), dict(tma_store=1)):
+            with binding.plan_hints(depthwise_form=3, **hints):
+                got, desc = gpu_conv(x, w, bias, shift, **kw)
+                assert "depthwise3x3/mma" in desc and (got == want).all(), (hints, desc)
+                got, desc = gpu_conv(x, w, bias, shift, **win)
+                assert "depthwise3x3/mma" in desc and (got == want_win).all(), (hints, desc)
+
+
+def test_less_aligned_tensors_take_the_other_kernels():
+    from paper_1805_07941_b200 import binding
+    N, H, W, C = 2, 9, 11, 64
+    rng = np.random.default_rng(0)
+    x, w, bias, shift, _, _ = rand_layer(rng, N, H, W, C, C, 3, 3, groups=C, pad=(1, 1))
+    conv = binding.QConv(w, bias, shift, N=N, H=H, W=W, C=C, K=C, R=3, S=3, pad_h=1, pad_w=1, groups=C)
+    want = oracle_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1), groups=C)
+    for off in (0, 4):
+        xb, yb = (torch.zeros(x.size + 16, dtype=torch.int8, device="cuda") for _ in range(2))
+        xd, yd = (b[off:off + x.size].view(N, H, W, C) for b in (xb, yb))
+        xd.copy_(torch.from_numpy(x))
+        conv.run(xd, yd)
+        assert conv.status() == 0 and (yd.cpu().numpy() == want).all(), off
