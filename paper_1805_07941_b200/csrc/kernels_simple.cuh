@@ -96,24 +96,15 @@ maxpool_i8_vec_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, int 
 // of one output column and walks down a strip of output rows.  The horizontal maximum of an input
 // row is taken once and kept in registers for every output row whose window contains it, so a
 // 3x3 stride-1 pool loads 3 vectors per output instead of 9.  The maxima are taken on pairs of
-// sign-extended 16-bit lanes (one permute per pair, then the two-lane integer max the hardware
-// has; a four-lane byte max would be emulated) and narrowed back to bytes at the end.
-struct PoolRow { uint32_t w[8]; };            // 16 channels as 8 words of two 16-bit lanes
+// 16-bit lanes with the byte on top (the two-lane integer max the hardware has; a four-lane byte
+// max would be emulated) and the top bytes are put together at the end.
+struct PoolRow { uint32_t w[8]; };            // 16 channels as 8 words of two 16-bit lanes: bytes 0 and 2 of a word, then 1 and 3
 
-// bytes (0, 1) / (2, 3) of a word as two sign-extended 16-bit lanes
-__device__ __forceinline__ uint32_t widen_lo(uint32_t v) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, 0, 0x9180;" : "=r"(d) : "r"(v));
-  return d;
-}
-__device__ __forceinline__ uint32_t widen_hi(uint32_t v) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, 0, 0xB3A2;" : "=r"(d) : "r"(v));
-  return d;
-}
+// A word's bytes as 16-bit lanes with the byte on top: the even ones shifted there, the odd ones where they are.  What lies
+// below a byte only decides between equal bytes.
 __device__ __forceinline__ void pool_widen(const uint4& v, PoolRow& r) {
-  r.w[0] = widen_lo(v.x); r.w[1] = widen_hi(v.x); r.w[2] = widen_lo(v.y); r.w[3] = widen_hi(v.y);
-  r.w[4] = widen_lo(v.z); r.w[5] = widen_hi(v.z); r.w[6] = widen_lo(v.w); r.w[7] = widen_hi(v.w);
+  r.w[0] = v.x << 8; r.w[1] = v.x; r.w[2] = v.y << 8; r.w[3] = v.y;
+  r.w[4] = v.z << 8; r.w[5] = v.z; r.w[6] = v.w << 8; r.w[7] = v.w;
 }
 
 template <int R, int S, int ST>
@@ -136,11 +127,10 @@ maxpool_i8_strip_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, in
   const uint4 lowest = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
   const uint4* xin = reinterpret_cast<const uint4*>(x) + static_cast<size_t>(n) * H * W * cv + c;
   const int w0 = q * ST - pad;
-  // horizontal maximum of input row h over the window's columns (taps outside the image are ignored)
-  auto hmax = [&](int h, PoolRow& m) {
+  // input row h over the window's columns (taps outside the image are ignored)
+  auto load = [&](int h, uint4 (&v)[S]) {
     const bool row_in = h >= 0 && h < H;
     const uint4* row = xin + static_cast<size_t>(row_in ? h : 0) * W * cv;
-    uint4 v[S];
 #pragma unroll
     for (int sx = 0; sx < S; ++sx) {
       const int w = w0 + sx;
@@ -149,6 +139,9 @@ maxpool_i8_strip_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, in
                             static_cast<size_t>(N) * H * W * cv);
       v[sx] = in ? __ldg(row + static_cast<size_t>(w) * cv) : lowest;
     }
+  };
+  // its horizontal maximum
+  auto hmax = [&](const uint4 (&v)[S], PoolRow& m) {
     pool_widen(v[0], m);
     if (S == 3) {
       PoolRow a, b;
@@ -166,16 +159,36 @@ maxpool_i8_strip_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, in
       }
     }
   };
+  // The rows of a step are loaded a step ahead (the first ones with the rows above them): a strip is otherwise a chain of
+  // load latencies.  128 x 28 x 28 x 192, 3 x 3 stride 1: 14.9 -> 10.7 us; 128 x 14 x 14 x 512: 10.6 -> 8.5.
   constexpr int KEEP = R > ST ? R - ST : 0;       // rows shared by consecutive windows
+  constexpr int NEW = R - KEEP;
   PoolRow win[R];
+  uint4 ahead[NEW][S];
+  {
+    uint4 first[KEEP ? KEEP : 1][S];
 #pragma unroll
-  for (int i = 0; i < KEEP; ++i) hmax(p0 * ST - pad + i, win[i + (R - KEEP)]);
+    for (int i = 0; i < KEEP; ++i) load(p0 * ST - pad + i, first[i]);
+#pragma unroll
+    for (int i = 0; i < NEW; ++i) load(p0 * ST - pad + KEEP + i, ahead[i]);
+#pragma unroll
+    for (int i = 0; i < KEEP; ++i) hmax(first[i], win[i + (R - KEEP)]);
+  }
   uint4* yout = reinterpret_cast<uint4*>(y) + ((static_cast<size_t>(n) * P + p0) * Q + q) * cv + c;
   for (int p = p0; p < p1; ++p) {
+    uint4 now[NEW][S];
+#pragma unroll
+    for (int i = 0; i < NEW; ++i)
+#pragma unroll
+      for (int sx = 0; sx < S; ++sx) now[i][sx] = ahead[i][sx];
+    if (p + 1 < p1) {
+#pragma unroll
+      for (int i = 0; i < NEW; ++i) load((p + 1) * ST - pad + KEEP + i, ahead[i]);
+    }
 #pragma unroll
     for (int i = 0; i < KEEP; ++i) win[i] = win[i + (R - KEEP)];
 #pragma unroll
-    for (int i = KEEP; i < R; ++i) hmax(p * ST - pad + i, win[i]);
+    for (int i = KEEP; i < R; ++i) hmax(now[i - KEEP], win[i]);
     PoolRow m = win[0];
     if (R == 3) {
 #pragma unroll
@@ -186,10 +199,9 @@ maxpool_i8_strip_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, in
 #pragma unroll
         for (int j = 0; j < 8; ++j) m.w[j] = __vmaxs2(m.w[j], win[i].w[j]);
     }
-    // every lane holds a value in [-128, 127]: its low byte is the result
     if (QC_IN(((static_cast<size_t>(n) * P + p) * Q + q) * cv + c, static_cast<size_t>(N) * P * Q * cv))
-      *yout = make_uint4(__byte_perm(m.w[0], m.w[1], 0x6420), __byte_perm(m.w[2], m.w[3], 0x6420),
-                         __byte_perm(m.w[4], m.w[5], 0x6420), __byte_perm(m.w[6], m.w[7], 0x6420));
+      *yout = make_uint4(__byte_perm(m.w[0], m.w[1], 0x7351), __byte_perm(m.w[2], m.w[3], 0x7351),
+                         __byte_perm(m.w[4], m.w[5], 0x7351), __byte_perm(m.w[6], m.w[7], 0x7351));
     yout += static_cast<size_t>(Q) * cv;
   }
 }

@@ -2105,7 +2105,7 @@ int qmaxpool_i8(const int8_t* d_x, int N, int H, int W, int C, int R, int S, int
   if (strip_ok) {
     // strips as long as still leaves every SM several hundred threads
     int rows = 16;
-    while (rows > 2 && static_cast<size_t>(N) * ceil_div(P, rows) * Q * (C / 16) < 148u * 2048u) rows /= 2;
+    while (rows > 2 && static_cast<size_t>(N) * ceil_div(P, rows) * Q * (C / 16) < 148u * 1024u) rows /= 2;
     const int strips = ceil_div(P, rows);
     const size_t threads = static_cast<size_t>(N) * strips * Q * (C / 16);
     if (threads > 2147483647ull) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "pooling: tensor too large");
