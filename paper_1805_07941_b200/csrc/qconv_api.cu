@@ -178,6 +178,12 @@ class DevicePool {
   }
 };
 
+// What handles of the same weights share: the device copy, and per output channel the sum of the magnitudes.
+struct SharedWeights {
+  DevicePool::Block block;
+  std::vector<long long> abs_sum;
+};
+
 struct qgraph_inputs {
   qc::GraphInputRecord rec;
 };
@@ -198,7 +204,8 @@ struct qconv_handle {
   int lo, hi;
   // device copies: the small tables in one block, large weights in a second one that handles of the same weights share
   DevicePool::Block block, pack;
-  std::shared_ptr<DevicePool::Block> weights;
+  std::shared_ptr<SharedWeights> weights;
+  std::vector<long long> abs_sum;  // (while the handle is built)
   int a_channels = 0;            // channels of the activation tensor (planes * padded C for floating-point operands)
   const NpSpec* np = nullptr;    // set while the handle is built
   int np_products = 0;
@@ -268,6 +275,42 @@ void free_handle(qconv_handle* h) {
   delete h;
 }
 
+// Streams for the copies that build a handle: they neither wait for the kernels that other threads have queued on the
+// default stream nor hold them up (a network's calibration uploads weights in the background).  Kept for the next copy.
+class CopyStream {
+ public:
+  CopyStream() {
+    cudaGetDevice(&dev_);
+    std::lock_guard<std::mutex> lock(mu());
+    std::vector<cudaStream_t>& f = free_list(dev_);
+    if (!f.empty()) { st_ = f.back(); f.pop_back(); }
+  }
+  ~CopyStream() {
+    std::lock_guard<std::mutex> lock(mu());
+    if (st_) free_list(dev_).push_back(st_);
+  }
+  cudaError_t copy(void* dst, const void* src, size_t bytes) {
+    cudaError_t e = ready();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st_);
+    return e == cudaSuccess ? cudaStreamSynchronize(st_) : e;
+  }
+  cudaError_t clear(void* dst, size_t bytes) {
+    cudaError_t e = ready();
+    if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, bytes, st_);
+    return e == cudaSuccess ? cudaStreamSynchronize(st_) : e;
+  }
+
+ private:
+  int dev_ = 0;
+  cudaStream_t st_ = nullptr;
+  cudaError_t ready() { return st_ ? cudaSuccess : cudaStreamCreateWithFlags(&st_, cudaStreamNonBlocking); }
+  static std::mutex& mu() { static std::mutex* m = new std::mutex; return *m; }
+  static std::vector<cudaStream_t>& free_list(int dev) {
+    static std::vector<cudaStream_t>* lists = new std::vector<cudaStream_t>[64];
+    return lists[dev & 63];
+  }
+};
+
 // A handle's small host tables on their way to the device, in one block and one copy.
 class DeviceParts {
  public:
@@ -284,7 +327,7 @@ class DeviceParts {
       *p.dst = static_cast<uint8_t*>(block->ptr) + p.at;
       if (p.src) std::memcpy(host.data() + p.at, p.src, p.bytes);
     }
-    CUDA_TRY(cudaMemcpy(block->ptr, host.data(), total_, cudaMemcpyHostToDevice));
+    CUDA_TRY(CopyStream().copy(block->ptr, host.data(), total_));
     return QCONV_OK;
   }
 
@@ -296,21 +339,26 @@ class DeviceParts {
 
 // The layer's weights: a part of the handle's block, or (from 64 KB) a block of their own that a second handle of the
 // same weights can use too.  `from`: the handle they may be shared with, or NULL.
+bool same_weights(const qconv_handle* h, const qconv_handle* from) {
+  return from && from->weights && from->weights_as_is && from->device == h->device && from->d.K == h->d.K &&
+         from->d.R == h->d.R && from->d.S == h->d.S && from->d.C == h->d.C && from->d.groups == h->d.groups;
+}
+
 int place_weights(qconv_handle* h, DeviceParts& parts, const int8_t* w, size_t bytes, bool as_is, const qconv_handle* from) {
   h->weights_as_is = as_is;
   if (bytes < 64 * 1024) {
     parts.add(&h->d_w, w, bytes);
     return QCONV_OK;
   }
-  if (as_is && from && from->weights && from->weights_as_is && from->device == h->device && from->d.K == h->d.K &&
-      from->d.R == h->d.R && from->d.S == h->d.S && from->d.C == h->d.C && from->algo == h->algo) {
+  if (as_is && same_weights(h, from) && from->algo == h->algo) {
     h->weights = from->weights;
   } else {
-    h->weights = std::make_shared<DevicePool::Block>();
-    CUDA_TRY(DevicePool::pool().take(h->weights.get(), bytes));
-    CUDA_TRY(cudaMemcpy(h->weights->ptr, w, bytes, cudaMemcpyHostToDevice));
+    h->weights = std::make_shared<SharedWeights>();
+    CUDA_TRY(DevicePool::pool().take(&h->weights->block, bytes));
+    CUDA_TRY(CopyStream().copy(h->weights->block.ptr, w, bytes));
+    h->weights->abs_sum.swap(h->abs_sum);
   }
-  h->d_w = static_cast<int8_t*>(h->weights->ptr);
+  h->d_w = static_cast<int8_t*>(h->weights->block.ptr);
   return QCONV_OK;
 }
 
@@ -331,7 +379,7 @@ qc::FastDiv make_fastdiv(int d_in) {
 // Output-pixel box (tq x tp x tn <= 128) that wastes the fewest accumulator rows.
 // pool: the epilogue takes a 2 x 2 max-pool with warp shuffles, so a window's four pixels must be lanes of one
 // warp: tq a power of two up to 16 (rows run q fastest), tp even; Q and P are even.
-void choose_box(int Q, int P, int N, int* tq_o, int* tp_o, int* tn_o, bool pool = false, long slots = 0) {
+void search_box(int Q, int P, int N, int* tq_o, int* tp_o, int* tn_o, bool pool, long slots) {
   long best_tiles = -1;
   int btq = 1, btp = 1, btn = 1;
   if (pool) {
@@ -389,6 +437,16 @@ void choose_box(int Q, int P, int N, int* tq_o, int* tp_o, int* tn_o, bool pool 
     }
   }
   *tq_o = btq; *tp_o = btp; *tn_o = btn;
+}
+
+// (a layer's plan asks for the same box several times, a search of some thousand steps each)
+void choose_box(int Q, int P, int N, int* tq_o, int* tp_o, int* tn_o, bool pool = false, long slots = 0) {
+  static thread_local struct { int Q = -1, P, N; bool pool; long slots; int tq, tp, tn; } last[2];
+  for (const auto& l : last)
+    if (l.Q == Q && l.P == P && l.N == N && l.pool == pool && l.slots == slots) { *tq_o = l.tq; *tp_o = l.tp; *tn_o = l.tn; return; }
+  search_box(Q, P, N, tq_o, tp_o, tn_o, pool, slots);
+  last[1] = last[0];
+  last[0] = {Q, P, N, pool, slots, *tq_o, *tp_o, *tn_o};
 }
 
 // Bytes of the contraction axis per ring stage.  A stage costs about the same whether its rows are
@@ -637,11 +695,23 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     patch = hint.patch_halo == 1 || (tiles >= h->num_sms && used >= 0.75 && k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0);
   }
   if (dw) patch = !halo && halo_fits && hint.patch_halo != 0;
+  if (np && halo && d.R == 3 && d.pad_h == 1 && p.np_cpp == 1 && bn_max <= 64 && hint.patch_halo != 0 && hint.halo != 1) {
+    // Floating-point operands: a stage of a digit product is a patch and its nine weight chunks.  The layer runs at the rate
+    // its operands arrive, so the form with fewer bytes on the busiest SM wins.
+    int tq, tp, tn, step;
+    halo_box(&tq, &tp, &tn, &step);
+    auto busiest = [&](long boxes, long activations) {
+      return ceil_div_l(boxes * ceil_div(k_eff, bn_max), h->num_sms) * (activations + 9l * bn_max * p.BKC);
+    };
+    patch = hint.patch_halo == 1 ||
+            busiest(static_cast<long>(pt.segs) * pt.rows * d.N, 16l * (pt.tp + 2) * p.BKC) <
+                busiest(static_cast<long>(ceil_div(h->Q, step)) * ceil_div(h->P, tp) * ceil_div(d.N, tn), 3l * tq * tp * tn * p.BKC);
+  }
   if (patch) {
     wide = false;
     halo = false;
     h->pair = 0;
-    bn_max = dw ? p.BKC : 128;
+    bn_max = dw ? p.BKC : np ? bn_max : 128;
     taps_r = taps_s = 1;
     p.R = p.S = 1;
   }
@@ -716,8 +786,9 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const int full_budget = (h->ctas_per_sm == 2 ? 113 : 226) * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared)) -
                           static_cast<int>(p.gen_stage_bytes);
   const int out_tile = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM) * p.BN, 1024));
+  const int patch_a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + 2 * 16 + 8) * p.BKC, 1024));
   auto ring_stages = [&](int bkc, int staged_tiles) {
-    const int a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * bkc, 1024)) * (group ? tps : 1);
+    const int a = patch ? patch_a : static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + (halo ? 8 : 0)) * bkc, 1024)) * (group ? tps : 1);
     const int b = static_cast<int>(align_up(static_cast<size_t>(h->pair ? p.BN / 2 : p.BN) * (dw ? 32 : bkc), 1024)) * tps;
     return (full_budget - staged_tiles * out_tile) / (a + b);
   };
@@ -742,8 +813,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   }
   // (patch form: resident weights and at least two activation boxes; two CTAs per SM where they fit, staged tiles where
   // they still do)
-  const int patch_a = static_cast<int>(align_up(static_cast<size_t>(qc::kTileM + 2 * 16 + 8) * p.BKC, 1024));
-  if (patch) {
+  if (patch && !np) {
     const int b_res = 9 * static_cast<int>(align_up(static_cast<size_t>(p.BN) * b_row, 1024));
     const bool may_stage = p.fast_epilogue && hint.tma_store != 0 && (p.BN == 64 || p.BN == 128) && !d.pool && !d.has_residual;
     bool placed = false;
@@ -791,11 +861,11 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     const long grid_max = static_cast<long>(h->num_sms) * h->ctas_per_sm;
     const int b_res_bytes = num_kb_plan * static_cast<int>(p.b_stage_bytes);
     const int mode_env = hint.resident_weights;                      // 0: never, 1: whenever it fits
-    if (patch) {
+    if (patch && !np) {
       p.b_resident = 1;
       const int budget = (h->ctas_per_sm == 2 ? 113 : 226) * 1024 - 1024 - static_cast<int>(sizeof(qc::IgemmShared));
       stages = std::min((budget - staged_tiles * out_tile - b_res_bytes) / patch_a, qc::kMaxStages);
-    } else if (mode_env != 0 && !h->pair && (!(halo || group) || p.nchunks == 1) && b_res_bytes <= 72 * 1024 &&
+    } else if (mode_env != 0 && !patch && !h->pair && (!(halo || group) || p.nchunks == 1) && b_res_bytes <= 72 * 1024 &&
         (m_tiles * p.tiles_k > grid_max || mode_env == 1)) {
       const int st = (full_budget - staged_tiles * out_tile - b_res_bytes) / static_cast<int>(p.a_stage_bytes);
       if (st >= std::min(num_kb_plan + 1, 2)) {
@@ -834,7 +904,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                 "with nearest-even rounding, K %% 16 == 0 and an accumulator bound below 2^31 - 2^(s-1)");
   }
   p.tx_bytes = static_cast<uint32_t>((group ? tps : 1) * p.tq * p.tp * p.tn * p.BKC + (p.b_resident ? 0 : tps * p.BN * b_row));
-  if (patch) p.tx_bytes = static_cast<uint32_t>(16 * (p.tp + 2) * p.BKC);
+  if (patch) p.tx_bytes = static_cast<uint32_t>(16 * (p.tp + 2) * p.BKC + (p.b_resident ? 0 : tps * p.BN * b_row));
   p.b_res_tx_bytes = static_cast<uint32_t>(num_kb_plan * tps * p.BN * b_row);
   p.res_tx_bytes = static_cast<uint32_t>(p.tq * p.tp * p.tn * p.BN);
 
@@ -952,8 +1022,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // cleared once: padding pixels, ragged edges and the padding bytes of each row stay zero
     CUDA_TRY(DevicePool::pool().take(&h->pack, pack_bytes));
     h->d_pack = static_cast<int8_t*>(h->pack.ptr);
-    CUDA_TRY(cudaMemsetAsync(h->d_pack, 0, pack_bytes, nullptr));
-    CUDA_TRY(cudaStreamSynchronize(nullptr));              // (the stream of the first run need not wait for this one)
+    CUDA_TRY(CopyStream().clear(h->d_pack, pack_bytes));   // (the stream of the first run need not wait for this one)
   }
   // the attribute belongs to the current device: once per device, not once per process
   static std::once_flag attr_once[64];
@@ -1413,12 +1482,23 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
   // Weight-aware bound of the wide value: 2^(n_in-1) * sum|w[k,.]| + |bias[k]| + 128 * 2^t[k].  Below 2^22 the
   // tensor-core epilogue may round in fp32 (exactly).
   h->np = np;
+  if (d.out_mode == QCONV_OUT_FLOAT && d.groups == 1 && !np && wcount >= 64 * 1024 && !same_weights(h, weights_of)) {
+    const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;                  // (for the handles that will share the weights)
+    h->abs_sum.resize(d.K);
+    for (int k = 0; k < d.K; ++k) h->abs_sum[k] = qc::host_abs_sum(w_krsc + k * per_k, per_k);
+  }
   if (d.out_mode == QCONV_OUT_INT8 && (d.groups == 1 || (Cg == 1 && d.C == d.K)) && h->hints.float_rounding != 0 && !np) {
     // ... and below 2^15 after the shift, where the clamp works on 16-bit halves.
     long long worst = 0, worst_out = 0;
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
-    for (int k = 0; k < d.K && worst < (1ll << 22) && worst_out < 32767; ++k) {
-      const long long bnd = qc::host_abs_sum(w_krsc + k * per_k, per_k) * (1ll << (d.n_in - 1)) +
+    const std::vector<long long>* sums = same_weights(h, weights_of) && !weights_of->weights->abs_sum.empty() ? &weights_of->weights->abs_sum : nullptr;
+    if (!sums) {
+      h->abs_sum.resize(d.K);
+      for (int k = 0; k < d.K; ++k) h->abs_sum[k] = qc::host_abs_sum(w_krsc + k * per_k, per_k);
+      sums = &h->abs_sum;
+    }
+    for (int k = 0; k < d.K; ++k) {
+      const long long bnd = (*sums)[k] * (1ll << (d.n_in - 1)) +
                             (bias_host ? std::llabs(static_cast<long long>(bias_host[k])) : 0) +
                             (d.has_residual ? (128ll << res_lshift_host[k]) : 0);
       worst = std::max(worst, bnd);
@@ -1931,6 +2011,32 @@ int qgraph_set_input(qgraph_inputs* g, void* graph_exec, const float* d_input) {
 int qgraph_inputs_destroy(qgraph_inputs* g) {
   if (!g) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
   delete g;
+  return QCONV_OK;
+}
+
+int qconv_update_float(qconv_handle* h, const int32_t* bias_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
+                       void* cuda_stream) {
+  if (!h) return fail(QCONV_ERR_BAD_ARG, "NULL handle");
+  const qconv_desc& d = h->d;
+  if (h->algo != QCONV_ALGO_IGEMM || d.out_mode != QCONV_OUT_FLOAT || h->np_products)
+    return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "qconv_update_float serves tensor-core layers with float output");
+  if (d.has_residual && !res_lshift_host) return fail(QCONV_ERR_BAD_ARG, "has_residual needs res_lshift_host");
+  int max_t = 0;
+  long long max_bias = 0;
+  std::vector<int4> chan(h->kpad, make_int4(0, 0, 0, 0));
+  for (int k = 0; k < d.K; ++k) {
+    const int t = d.has_residual ? res_lshift_host[k] : 0, e = acc_exp_host ? acc_exp_host[k] : 0, b = bias_host ? bias_host[k] : 0;
+    if (t < 0 || t > 23) return fail(QCONV_ERR_RESIDUAL_SCALE, "res_lshift[%d] = %d outside [0, 23]", k, t);
+    if (e < -126 || e > 96) return fail(QCONV_ERR_BAD_ARG, "acc_exp[%d] = %d outside [-126, 96]", k, e);
+    max_t = std::max(max_t, t);
+    max_bias = std::max(max_bias, std::llabs(static_cast<long long>(b)));
+    chan[k] = make_int4(b, 0, 1 << t, (e + 127) << 23);
+  }
+  const long long bound = static_cast<long long>(d.R) * d.S * h->Cg * (1ll << (d.n_in - 1)) * (1ll << (d.n_w - 1)) + max_bias +
+                          (d.has_residual ? (128ll << max_t) : 0);
+  if (bound > 2147483647ll) return fail(QCONV_ERR_OVERFLOW_RISK, "worst-case |accumulator| %lld exceeds 2^31 - 1", bound);
+  h->acc_bound = bound;
+  CUDA_TRY(cudaMemcpyAsync(h->d_chan, chan.data(), sizeof(int4) * chan.size(), cudaMemcpyHostToDevice, static_cast<cudaStream_t>(cuda_stream)));
   return QCONV_OK;
 }
 
@@ -2700,32 +2806,73 @@ int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layo
   return QCONV_OK;
 }
 
-// Layers are independent: the largest first over up to eight threads.  (The conversion reads 5 bytes per value from
-// memory twice; beyond eight threads the memory, not the arithmetic, sets the pace.)
+// Every thread takes a share of the channels of every large layer (and whole small ones in turn), so that the few large
+// layers of a network do not leave one thread at work alone; where one exponent serves the whole layer the threads meet
+// between its maximum and its conversion, and each finds its share still in its own cache.
 int qquantize_weights_list(const qweights_job* jobs, int count) {
   if (!jobs || count < 0) return fail(QCONV_ERR_BAD_ARG, "NULL jobs or negative count");
-  std::vector<int> order(count), rc(count, QCONV_OK);
-  for (int i = 0; i < count; ++i) order[i] = i;
   auto size = [&](int i) { return static_cast<long long>(jobs[i].K) * jobs[i].R * jobs[i].S * jobs[i].Cg; };
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return size(a) > size(b); });
-  std::atomic<int> next{0};
-  auto work = [&] {
-    for (int i; (i = next.fetch_add(1)) < count;) {
-      const qweights_job& j = jobs[order[i]];
-      rc[order[i]] = qquantize_weights(j.w_host, j.K, j.R, j.S, j.Cg, j.layout, j.per_channel, j.n, j.wq_host, j.e_w_host);
+  long long total = 0;
+  std::vector<char> shared(count, 0);
+  std::vector<int> rc(count, QCONV_OK);
+  for (int i = 0; i < count; ++i) {
+    const qweights_job& j = jobs[i];
+    const bool sane = j.w_host && j.wq_host && j.e_w_host && j.K > 0 && j.R > 0 && j.S > 0 && j.Cg > 0 && j.n >= 2 && j.n <= 8;
+    total += sane ? size(i) : 0;
+    shared[i] = sane && j.layout == 0 && size(i) >= (1 << 17);
+  }
+  // (a thread costs some 20 us to start: worth it from about 2^18 values each)
+  int threads = static_cast<int>(std::min<long long>({8, total >> 18, std::thread::hardware_concurrency()}));
+  threads = std::max(1, threads);
+  std::vector<float> top(static_cast<size_t>(threads) * 16, 0.0f);     // a cache line per thread
+  std::atomic<int> arrived{0}, go{0};
+  auto work = [&](int t, int T) {
+    int met = 0;
+    auto meet = [&] {
+      ++met;
+      arrived.fetch_add(1);
+      while (arrived.load() < met * T) std::this_thread::yield();
+    };
+    for (int i = 0; i < count; ++i) {
+      const qweights_job& j = jobs[i];
+      if (!shared[i]) {
+        if (i % T == t) rc[i] = qquantize_weights(j.w_host, j.K, j.R, j.S, j.Cg, j.layout, j.per_channel, j.n, j.wq_host, j.e_w_host);
+        continue;
+      }
+      const size_t per_k = static_cast<size_t>(j.R) * j.S * j.Cg;
+      const int k0 = static_cast<int>(static_cast<long long>(j.K) * t / T), k1 = static_cast<int>(static_cast<long long>(j.K) * (t + 1) / T);
+      const float* w = j.w_host + k0 * per_k;
+      int8_t* q = j.wq_host + k0 * per_k;
+      if (j.per_channel) {
+        if (k1 > k0) qquantize_weights(w, k1 - k0, j.R, j.S, j.Cg, 0, 1, j.n, q, j.e_w_host + k0);
+        continue;
+      }
+      top[static_cast<size_t>(t) * 16] = qc::host_max_abs(w, per_k * (k1 - k0));
+      meet();
+      float g = 0.0f;
+      for (int u = 0; u < T; ++u) g = std::max(g, top[static_cast<size_t>(u) * 16]);
+      meet();                                              // everyone has read the maxima
+      int e;
+      qscale_exponent(g, j.n, &e);
+      for (int k = k0; k < k1; ++k) j.e_w_host[k] = e;
+      qc::host_quantize(w, per_k * (k1 - k0), e, j.n, q);
     }
   };
-  long long total = 0;
-  for (int i = 0; i < count; ++i) total += size(i);
-  // (a thread costs some 20 us to start: worth it from about 2^18 values each)
-  const int want = static_cast<int>(std::min<long long>({8, count, total >> 18, std::max(1u, std::thread::hardware_concurrency())}));
-  std::vector<std::thread> threads;
+  // The shares depend on how many threads there are, so they wait for that number.
+  std::vector<std::thread> pool;
   try {
-    for (int t = 1; t < want; ++t) threads.emplace_back(work);
+    for (int t = 1; t < threads; ++t)
+      pool.emplace_back([&, t] {
+        int T;
+        while ((T = go.load()) == 0) std::this_thread::yield();
+        work(t, T);
+      });
   } catch (const std::system_error&) {                     // no more threads: the ones there are (this one at least) do it
   }
-  work();
-  for (std::thread& t : threads) t.join();
+  const int have = static_cast<int>(pool.size()) + 1;
+  go.store(have);
+  work(0, have);
+  for (std::thread& t : pool) t.join();
   for (int i = 0; i < count; ++i)
     if (rc[i]) return fail(rc[i], "weights %d: NULL argument or bad geometry", i);
   return QCONV_OK;
@@ -2733,8 +2880,16 @@ int qquantize_weights_list(const qweights_job* jobs, int count) {
 
 int qquantize_bias(const float* b_host, int K, int e_x, const int32_t* e_w_host, int32_t* bias_q_host) {
   if (!b_host || !e_w_host || !bias_q_host || K <= 0) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
-  for (int k = 0; k < K; ++k) {
-    double r = std::nearbyint(std::ldexp(static_cast<double>(b_host[k]), -(e_x + e_w_host[k])));
+  int e = 0;
+  double scale = 1.0;                                      // 2^-e: the product is ldexp(b, -e) wherever that is a normal number,
+  for (int k = 0; k < K; ++k) {                            // and far below one half where it is not
+    const int ek = e_x + e_w_host[k];
+    if (ek != e) {
+      e = ek;
+      scale = std::ldexp(1.0, -e);
+    }
+    const bool plain = e >= -800 && e <= 800;
+    double r = std::nearbyint(plain ? static_cast<double>(b_host[k]) * scale : std::ldexp(static_cast<double>(b_host[k]), -e));
     if (std::isnan(r)) r = 0.0;
     r = std::min(2147483647.0, std::max(-2147483648.0, r));
     bias_q_host[k] = static_cast<int32_t>(r);
