@@ -175,12 +175,6 @@ int qconv_run_f32(qconv_handle* h, const float* d_x_f32, int e_x, const int8_t* 
 int qconv_run_maxabs(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, int n_run, float* maxabs_out,
                      void* cuda_stream);
 
-/* New biases, residual shifts and accumulator exponents (as at create, NULL for zeros) for a tensor-core layer with
- * float output, for the runs after this call on this stream: a layer can be built, and its weights copied, before the
- * exponent of its input is known.  Errors: as qconv_create for the tables; UNSUPPORTED_SHAPE for other layers. */
-int qconv_update_float(qconv_handle* h, const int32_t* bias_host, const int32_t* res_lshift_host,
-                       const int32_t* acc_exp_host, void* cuda_stream);
-
 /* Synchronise the stream of the last qconv_run and return its device status (QCONV_OK or
  * QCONV_ERR_TIMEOUT), clearing it. */
 int qconv_status(qconv_handle* h);

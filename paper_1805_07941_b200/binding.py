@@ -166,8 +166,6 @@ def lib():
             getattr(L, name).restype = ci
         L.qconv_run_maxabs.argtypes = [vp, vp, vp, ci, ctypes.POINTER(ctypes.c_float), vp]
         L.qconv_run_maxabs.restype = ci
-        L.qconv_update_float.argtypes = [vp, vp, vp, vp, vp]
-        L.qconv_update_float.restype = ci
         L.qquantize_weights_list.argtypes = [ctypes.POINTER(qweights_job), ci]
         L.qquantize_weights_list.restype = ci
         L.qnet_run.argtypes = [vp, ci, vp, vp]
@@ -293,11 +291,6 @@ class QConv:
         out = ctypes.c_float(0)
         _check(lib().qconv_run_maxabs(self.handle, _dev(x), _dev(residual), int(n), ctypes.byref(out), _stream()))
         return np.float32(out.value)
-
-    def update_float(self, bias=None, res_lshift=None, acc_exp=None):
-        """New tables for a tensor-core layer with float output, for the runs that follow on the current stream."""
-        keep = [_host(bias, np.int32), _host(res_lshift, np.int32), _host(acc_exp, np.int32)]
-        _check(lib().qconv_update_float(self.handle, *[p for _, p in keep], _stream()))
 
     def status(self):
         return lib().qconv_status(self.handle)

@@ -71,6 +71,7 @@ struct IgemmParams {
   int tmem_cols;                   // power of two >= max(32, BN)
   int vec_store;                   // 1: 16-byte stores/loads of int8 rows are aligned
   int gen_simple;                  // general int8 epilogue: the accumulator bound leaves room for the single-pass rounding
+  int gen_down, gen_away;          // EPI_GEN: round down (the table's bias then holds the mode's half), half away from zero by sign
   int gen_vec_y, gen_vec_res;      // general epilogues: 16 or 8 if every row piece of the output / the residual is aligned to
                                    //    so many bytes, else 0 (set per run from the pointers)
   uint32_t gen_stage_bytes;        // general epilogues: shared memory of the warps' staging rows (0 for the fast ones)
@@ -340,7 +341,7 @@ __device__ __forceinline__ uint32_t make_idesc_i8(int bn) {
 //   int8 output:  z = 2^(s-1) - 1 (0 when s = 0), w = (s > 0) | 2^t << 1 with t the residual left shift;
 //                 they serve the single-pass nearest-even rounding  (v + z + ((v >> s) & w & 1)) >> s
 //                 (other rounding modes: see general_round);
-//   wide output:  z = 2^t, and for float output w = bit pattern of the float 2^(e_x + e_w[k]).
+//   general int8: y = s | t << 8;  wide output: y = t, with the bit pattern of the float 2^(e_x + e_w[k]) for float output.
 
 struct IgemmShared {
   uint64_t full[kMaxStages];
@@ -424,6 +425,8 @@ struct TileWalker {
 //                          accumulator bound leaves room for the rounding constant; without / with residual
 //   I8: any rounding mode, bit width, alignment;  I32, F32: wide or float output;  MAX: the largest |float output|
 //                          alone, nothing is stored
+//   GEN, GEN_RES: I8 where the wide value stays below 2^22 as well (see FLT below): any rounding mode by the rounding of the
+//                          fused multiply-add; GEN_RES also serves the mode that needs the sign (half away, no ReLU)
 //   NP: digit products of floating-point operands recombined in 64 bits and converted to the (n, p) output type
 //   FAST_I8_U / FAST_I8_RES_U: the same with one shift for all channels (per-layer scales): only the
 //                          bias is per channel, everything else sits in kernel parameters
@@ -437,7 +440,7 @@ struct TileWalker {
 //                          on the bit patterns (positive floats order like integers).
 enum : int { EPI_FAST_I8 = 0, EPI_FAST_I8_RES = 1, EPI_I8 = 2, EPI_I32 = 3, EPI_F32 = 4, EPI_FAST_I8_U = 5,
              EPI_FAST_I8_RES_U = 6, EPI_FLT_I8 = 7, EPI_FLT_I8_RES = 8, EPI_FLT_I8_U = 9, EPI_FLT_I8_RES_U = 10,
-             EPI_MAX = 11, EPI_NP = 12 };
+             EPI_MAX = 11, EPI_NP = 12, EPI_GEN = 13, EPI_GEN_RES = 14 };
 
 template <int EPI> struct EpiTraits {
   static constexpr bool flt = EPI >= EPI_FLT_I8 && EPI <= EPI_FLT_I8_RES_U;
@@ -449,7 +452,8 @@ template <int EPI> struct EpiTraits {
                               EPI == EPI_FLT_I8_RES_U;
   // shared-memory form of the channel constants: 4 bytes a channel when only the biases differ; for the float rounding
   // without residual 8, two channels side by side as {bias, bias, 2^-s, 2^-s}; else the table's 16
-  static constexpr bool paired = EPI == EPI_FLT_I8;
+  static constexpr bool paired = EPI == EPI_FLT_I8 || EPI == EPI_GEN || EPI == EPI_I8 || EPI == EPI_I32 || EPI == EPI_F32 || EPI == EPI_MAX;
+  static constexpr bool gen = EPI == EPI_GEN || EPI == EPI_GEN_RES, bytes = EPI == EPI_I8 || gen;   // general int8
   static constexpr uint32_t cst_bytes = uni ? 4u : paired ? 8u : 16u;
 };
 
@@ -728,11 +732,48 @@ __device__ __forceinline__ void gen_copy_words(uint8_t* stage, int8_t* base, lon
   }
 }
 
+// Rows at any alignment to global memory in the aligned 8-byte units that hold them, shifted into place; a row's first and
+// last partial unit in pieces of 4, 2 and 1 bytes.  At least 16 bytes a row.
+__device__ __forceinline__ void gen_store_units(const uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
+  const unsigned okmask = __ballot_sync(0xffffffffu, ok);
+  const int units = (bytes + 14) >> 3;                      // at most, wherever the row starts (<= 9)
+  const uint32_t inv = 65536u / static_cast<uint32_t>(units) + 1u;   // idx / units = (idx * inv) >> 16 for idx < 32 * 9
+#pragma unroll 3
+  for (int it = 0; it < units; ++it) {
+    const int idx = it * 32 + lane;
+    const int r = static_cast<int>((static_cast<uint32_t>(idx) * inv) >> 16), u = idx - r * units;
+    int8_t* row = base + __shfl_sync(0xffffffffu, row_off, r);
+    const int m = static_cast<int>(reinterpret_cast<uintptr_t>(row) & 7u), first = 8 * u - m;   // the unit's first byte in the row
+    if (!((okmask >> r) & 1u) || first >= bytes) continue;
+    // (before a row's first byte: whatever lies there, never stored)
+    const uint32_t* sp = reinterpret_cast<const uint32_t*>(stage + r * kGenPitch) + (first >> 2);
+    const uint32_t w0 = sp[0], w1 = sp[1], w2 = sp[2];
+    const uint32_t lo = __funnelshift_r(w0, w1, 8 * (first & 3)), hi = __funnelshift_r(w1, w2, 8 * (first & 3));
+    int8_t* dst = row + first;
+    if (first >= 0 && first + 8 <= bytes) {
+      *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
+    } else if (first < 0) {                                 // bytes m ... 7 of the unit
+      if (m & 1) dst[m] = static_cast<int8_t>((m & 4 ? hi : lo) >> (8 * (m & 3)));
+      const int h = (m + 1) & ~1;                           // then from an even byte
+      if (h & 2) *reinterpret_cast<uint16_t*>(dst + h) = static_cast<uint16_t>((h & 4 ? hi : lo) >> 16);
+      if (h <= 4) *reinterpret_cast<uint32_t*>(dst + 4) = hi;
+    } else {                                                // bytes 0 ... t - 1
+      const int t = bytes - first;
+      if (t & 4) *reinterpret_cast<uint32_t*>(dst) = lo;
+      const uint32_t w = t & 4 ? hi : lo;
+      int8_t* at = dst + (t & 4);
+      if (t & 2) *reinterpret_cast<uint16_t*>(at) = static_cast<uint16_t>(w);
+      if (t & 1) at[t & 2] = static_cast<int8_t>(t & 2 ? w >> 16 : w);
+    }
+  }
+}
+
 template <bool STORE>
 __device__ __forceinline__ void gen_copy(int vec, uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
   if (bytes <= 0) return;
   if (vec == 16) gen_copy_rows<16, STORE>(stage, base, row_off, ok, bytes, lane);
   else if (vec == 8) gen_copy_rows<8, STORE>(stage, base, row_off, ok, bytes, lane);
+  else if (STORE && bytes >= 16) gen_store_units(stage, base, row_off, ok, bytes, lane);
   else gen_copy_words<STORE>(stage, base, row_off, ok, bytes, lane);
 }
 
@@ -773,39 +814,65 @@ __device__ __forceinline__ uint32_t np_encode(long long v, int s, const NpEncode
   return code | ((v < 0 && code) ? 1u << f.sign_bit : 0u);
 }
 
-// v / 2^s rounded in the descriptor's mode, in one pass: (v + z + (cond & w & 1)) >> s with the addend z and the mask
-// bit of w made by the host (s = 0: both 0):
-//   nearest-even: z = 2^(s-1) - 1, cond = lowest bit of the truncated quotient;  half away: the same z, cond = v > 0;
-//   half up: z = 2^(s-1);  floor: z = 0  (mask bit 0).
-__device__ __forceinline__ int32_t general_round(int32_t v, const int4& c, int rounding) {
-  const int32_t cond = rounding == 0 ? v >> c.y : (v > 0 ? 1 : 0);
-  return (v + c.z + (cond & c.w & 1)) >> c.y;
+// v / 2^s rounded in the descriptor's mode, in one pass: (v + z + cond) >> s, with m = 2^s - 1 (odd unless s = 0):
+//   nearest-even: z = m / 2, cond = lowest bit of the truncated quotient;  half away: z = m / 2, cond = v > 0;
+//   half up: z = (m + 1) / 2;  floor: z = 0;  no cond where s = 0.
+template <bool EVEN>
+__device__ __forceinline__ int32_t general_round(int32_t v, int s, int rounding) {
+  const int32_t m = static_cast<int32_t>((1u << s) - 1u);
+  if (EVEN) return (v + (m >> 1) + ((v >> s) & m & 1)) >> s;
+  const int32_t z = rounding == 1 ? (m >> 1) + ((v > 0 ? 1 : 0) & m) : rounding == 2 ? static_cast<int32_t>((static_cast<uint32_t>(m) + 1u) >> 1) : 0;
+  return (v + z) >> s;
 }
 
-// One group of 16 columns.  rw: the residual bytes (zero without).  int8: 16 codes to the staging row; int32 / float:
-// 16 words to it; MAX: into *mx.
+// One group of 16 columns of the integer general int8 epilogue -> 16 codes in the staging row.  Channel constants: the bias
+// and s | t << 8, 8 bytes a channel (with 16, reading them took as long as everything else).  A negative wide value never
+// rounds above zero, so a ReLU is the lower clamp.
+template <bool SIMPLE, bool EVEN>
+__device__ __forceinline__ void general_int8_16(const uint32_t (&acc)[16], uint32_t cst_g, const uint4& res16, const EpilogueParams& ep, uint32_t stage) {
+  const uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};
+  const int lo = ep.relu ? max(ep.lo, 0) : ep.lo;
+  uint32_t wds[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    const int4 a = lds_int4(cst_g + static_cast<uint32_t>(g * 32)), c = lds_int4(cst_g + static_cast<uint32_t>(g * 32 + 16));
+    const int32_t bias[4] = {a.x, a.y, c.x, c.y}, pk[4] = {a.z, a.w, c.z, c.w};
+    const int32_t rv[4] = {sign_extend_byte<0>(rw[g]), sign_extend_byte<1>(rw[g]), sign_extend_byte<2>(rw[g]), sign_extend_byte<3>(rw[g])};
+    int32_t q[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int sft = pk[b] & 31;
+      int32_t v = static_cast<int32_t>(acc[4 * g + b]) + bias[b] + static_cast<int32_t>(static_cast<uint32_t>(rv[b]) << (pk[b] >> 8));
+      if (!SIMPLE && ep.relu) v = max(v, 0);
+      q[b] = min(max(SIMPLE ? general_round<EVEN>(v, sft, ep.rounding) : round_shift(v, sft, ep.rounding), lo), ep.hi);
+    }
+    wds[g] = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+  }
+  ptx::sts_uint4(stage, wds[0], wds[1], wds[2], wds[3]);
+}
+
+// One group of 16 columns with wide output.  res16: the residual bytes (zero without).  int32 / float: 16 words to the staging
+// row; MAX: into *mx.
 template <int EPI>
 __device__ __forceinline__ void general_16(const uint32_t (&acc)[16], uint32_t cst_g, const uint4& res16, int ncols, bool row_ok,
                                            const IgemmParams& prm, const EpilogueParams& ep, uint32_t stage, float* mx) {
   const uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
+    const int4 k01 = lds_int4(cst_g + static_cast<uint32_t>(g * 32)), k23 = lds_int4(cst_g + static_cast<uint32_t>(g * 32 + 16));
+    const int32_t bias[4] = {k01.x, k01.y, k23.x, k23.y}, pk[4] = {k01.z, k01.w, k23.z, k23.w};
     uint32_t o[4];
     const int32_t rv[4] = {sign_extend_byte<0>(rw[g]), sign_extend_byte<1>(rw[g]), sign_extend_byte<2>(rw[g]), sign_extend_byte<3>(rw[g])};
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int j = g * 4 + b;
-      const int4 c = lds_int4(cst_g + static_cast<uint32_t>(j * 16));
-      int32_t v = static_cast<int32_t>(acc[j]) + c.x + rv[b] * (EPI == EPI_I8 ? c.w >> 1 : c.z);
+      int32_t v = static_cast<int32_t>(acc[j]) + bias[b] + static_cast<int32_t>(static_cast<uint32_t>(rv[b]) << (pk[b] & 31));
       if (ep.relu) v = max(v, 0);
-      if (EPI == EPI_I8) {
-        const int32_t q = prm.gen_simple ? general_round(v, c, ep.rounding) : round_shift(v, c.y, ep.rounding);
-        o[b] = static_cast<uint32_t>(min(max(q, ep.lo), ep.hi));
-      } else if (EPI == EPI_I32) {
+      if (EPI == EPI_I32) {
         o[b] = static_cast<uint32_t>(v);
       } else {
-        // beta -> float: c.w holds the bits of 2^(e_x + e_w[k]); the product is exact (power of two)
-        const float f = __int2float_rn(v) * __int_as_float(c.w);
+        // beta -> float: the bits of 2^(e_x + e_w[k]); the product is exact (power of two)
+        const float f = __int2float_rn(v) * __int_as_float(pk[b] & 0x7F800000);
         if (EPI == EPI_MAX) {
           if (row_ok && j < ncols) *mx = fmaxf(*mx, fabsf(f));
         } else {
@@ -813,13 +880,65 @@ __device__ __forceinline__ void general_16(const uint32_t (&acc)[16], uint32_t c
         }
       }
     }
-    if (EPI == EPI_I8) {
-      const uint32_t lo2 = __byte_perm(o[0], o[1], 0x0040), hi2 = __byte_perm(o[2], o[3], 0x0040);
-      asm volatile("st.shared.b32 [%0], %1;" ::"r"(stage + g * 4u), "r"(__byte_perm(lo2, hi2, 0x5410)) : "memory");
-    } else if (EPI != EPI_MAX) {
+    if (EPI != EPI_MAX) {
       ptx::sts_uint4(stage + g * 16u, o[0], o[1], o[2], o[3]);
     }
   }
+}
+
+// One group of 16 columns of the float-rounding general epilogues (EPI_GEN, EPI_GEN_RES) -> 16 codes in the staging row.
+// q = magic + v + h, an integer below 2^22 in magnitude; with h = 2^(s-1) and the multiply-add rounding down that is round
+// half up, with h = 0 floor, and rounding to nearest half to even.  Half away from zero is half up from zero on, and one
+// less below: the table's z = h - 1, plus one where v >= 0 (bit 22 of the float's pattern); with a ReLU it is half up.
+template <int EPI>
+__device__ __forceinline__ void gen_flt_16(const uint32_t (&acc)[16], uint32_t cst_g, const uint4& res16, const IgemmParams& prm,
+                                           const EpilogueParams& ep, uint32_t stage) {
+  constexpr float kM = 12582912.0f;
+  const uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};
+  const int lo = ep.relu ? 0 : ep.lo;
+  const uint32_t lo2 = __byte_perm(static_cast<uint32_t>(lo), 0u, 0x1010), hi2 = __byte_perm(static_cast<uint32_t>(ep.hi), 0u, 0x1010);
+  auto fma_down = [](float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "fma.rm.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+  };
+  uint32_t wds[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    int32_t q[4];
+    float2 s01, s23;
+    if constexpr (EpiTraits<EPI>::paired) {
+      const int4 a = lds_int4(cst_g + static_cast<uint32_t>(g * 32)), b = lds_int4(cst_g + static_cast<uint32_t>(g * 32 + 16));
+      q[0] = static_cast<int32_t>(acc[4 * g]) + a.x; q[1] = static_cast<int32_t>(acc[4 * g + 1]) + a.y;
+      q[2] = static_cast<int32_t>(acc[4 * g + 2]) + b.x; q[3] = static_cast<int32_t>(acc[4 * g + 3]) + b.y;
+      s01 = make_float2(__int_as_float(a.z), __int_as_float(a.w));
+      s23 = make_float2(__int_as_float(b.z), __int_as_float(b.w));
+    } else {
+      const int32_t rv[4] = {sign_extend_byte<0>(rw[g]), sign_extend_byte<1>(rw[g]), sign_extend_byte<2>(rw[g]), sign_extend_byte<3>(rw[g])};
+      float sc[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int4 c = lds_int4(cst_g + static_cast<uint32_t>((g * 4 + b) * 16));
+        q[b] = static_cast<int32_t>(acc[4 * g + b]) + c.x + rv[b] * (c.w >> 1);
+        if (prm.gen_away) q[b] += c.z + ((q[b] >> 22) & 1);
+        sc[b] = __int_as_float(c.y);
+      }
+      s01 = make_float2(sc[0], sc[1]);
+      s23 = make_float2(sc[2], sc[3]);
+    }
+    const float2 m = make_float2(kM, kM);
+    const float2 a = add_pair(make_float2(__int_as_float(q[0]), __int_as_float(q[1])), make_float2(-kM, -kM));
+    const float2 b = add_pair(make_float2(__int_as_float(q[2]), __int_as_float(q[3])), make_float2(-kM, -kM));
+    const float2 x = prm.gen_down ? fma_down(a, s01, m) : fma_pair(a, s01, m), y = prm.gen_down ? fma_down(b, s23, m) : fma_pair(b, s23, m);
+    uint32_t h0 = __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x5410), h1 = __byte_perm(__float_as_uint(y.x), __float_as_uint(y.y), 0x5410);
+    h0 = __vmaxs2(__vmins2(h0, hi2), lo2);
+    h1 = __vmaxs2(__vmins2(h1, hi2), lo2);
+    wds[g] = __byte_perm(h0, h1, 0x6420);
+  }
+  ptx::sts_uint4(stage, wds[0], wds[1], wds[2], wds[3]);
 }
 
 // 16 accumulator columns of one row with a 2 x 2 / stride 2 max-pool over pixels taken on the way.  The conversion
@@ -1424,8 +1543,14 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           const uint32_t st_row = ptx::smem_u32(gen_out) + static_cast<uint32_t>(lane * kGenPitch);
           const uint4 r16 = gen_res ? gen_row_words(gen_stage + lane * kGenPitch, i, gen_m) : make_uint4(0u, 0u, 0u, 0u);
           const int ncols = gen_cols - i * 16;
-          general_16<EPI>(acc, chan + static_cast<uint32_t>((g_begin + i) * 256), r16, ncols, row_ok, prm, ep,
-                          st_row + (EPI == EPI_I8 ? static_cast<uint32_t>(i * 16) : 0u), &gen_max);
+          const uint32_t cst_g = chan + static_cast<uint32_t>(g_begin + i) * 16u * EpiTraits<EPI>::cst_bytes;
+          const uint32_t at = st_row + (EpiTraits<EPI>::bytes ? static_cast<uint32_t>(i * 16) : 0u);
+          if constexpr (EPI == EPI_I8) {
+            if (!prm.gen_simple) general_int8_16<false, false>(acc, cst_g, r16, ep, at);
+            else if (ep.rounding == 0) general_int8_16<true, true>(acc, cst_g, r16, ep, at);
+            else general_int8_16<true, false>(acc, cst_g, r16, ep, at);
+          } else if constexpr (EpiTraits<EPI>::gen) gen_flt_16<EPI>(acc, cst_g, r16, prm, ep, at);
+          else general_16<EPI>(acc, cst_g, r16, ncols, row_ok, prm, ep, at, &gen_max);
           if (EPI == EPI_I32 || EPI == EPI_F32) {
             __syncwarp();
             gen_copy<true>(prm.gen_vec_y, gen_out, static_cast<int8_t*>(y) + 4ll * (prm.out_c_offset + gen_k0 + i * 16),
@@ -1544,7 +1669,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           }
         }
         if (g_begin >= g_end) release();                     // a warp without columns still hands back
-        if (EPI == EPI_I8) {
+        if (EpiTraits<EPI>::bytes) {
           __syncwarp();
           gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + prm.out_c_offset + gen_k0,
                          static_cast<long long>(pix) * prm.out_c_pitch, row_ok, gen_cols, lane);

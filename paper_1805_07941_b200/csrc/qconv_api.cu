@@ -178,12 +178,6 @@ class DevicePool {
   }
 };
 
-// What handles of the same weights share: the device copy, and per output channel the sum of the magnitudes.
-struct SharedWeights {
-  DevicePool::Block block;
-  std::vector<long long> abs_sum;
-};
-
 struct qgraph_inputs {
   qc::GraphInputRecord rec;
 };
@@ -204,8 +198,7 @@ struct qconv_handle {
   int lo, hi;
   // device copies: the small tables in one block, large weights in a second one that handles of the same weights share
   DevicePool::Block block, pack;
-  std::shared_ptr<SharedWeights> weights;
-  std::vector<long long> abs_sum;  // (while the handle is built)
+  std::shared_ptr<DevicePool::Block> weights;
   int a_channels = 0;            // channels of the activation tensor (planes * padded C for floating-point operands)
   const NpSpec* np = nullptr;    // set while the handle is built
   int np_products = 0;
@@ -220,6 +213,7 @@ struct qconv_handle {
   long long acc_bound = 0;       // worst-case |accumulator| (Eq. 9 / Eq. 13 bound)
   int max_shift = 0;
   long walk_grid = -1;             // grid size the tile-walk constants in prm were made for
+  int gen_flt = 0;               // 1: the same bound with the rounding mode's half: float rounding in the general epilogue
   int flt_epilogue = 0;          // 1: |wide value| < 2^22 for any input (weight-aware bound): float-rounding epilogue
   int uniform_shift = 0;         // 1: all channels share the right shift and the residual left shift
   int uni_s = 0, uni_t = 0;
@@ -275,42 +269,6 @@ void free_handle(qconv_handle* h) {
   delete h;
 }
 
-// Streams for the copies that build a handle: they neither wait for the kernels that other threads have queued on the
-// default stream nor hold them up (a network's calibration uploads weights in the background).  Kept for the next copy.
-class CopyStream {
- public:
-  CopyStream() {
-    cudaGetDevice(&dev_);
-    std::lock_guard<std::mutex> lock(mu());
-    std::vector<cudaStream_t>& f = free_list(dev_);
-    if (!f.empty()) { st_ = f.back(); f.pop_back(); }
-  }
-  ~CopyStream() {
-    std::lock_guard<std::mutex> lock(mu());
-    if (st_) free_list(dev_).push_back(st_);
-  }
-  cudaError_t copy(void* dst, const void* src, size_t bytes) {
-    cudaError_t e = ready();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st_);
-    return e == cudaSuccess ? cudaStreamSynchronize(st_) : e;
-  }
-  cudaError_t clear(void* dst, size_t bytes) {
-    cudaError_t e = ready();
-    if (e == cudaSuccess) e = cudaMemsetAsync(dst, 0, bytes, st_);
-    return e == cudaSuccess ? cudaStreamSynchronize(st_) : e;
-  }
-
- private:
-  int dev_ = 0;
-  cudaStream_t st_ = nullptr;
-  cudaError_t ready() { return st_ ? cudaSuccess : cudaStreamCreateWithFlags(&st_, cudaStreamNonBlocking); }
-  static std::mutex& mu() { static std::mutex* m = new std::mutex; return *m; }
-  static std::vector<cudaStream_t>& free_list(int dev) {
-    static std::vector<cudaStream_t>* lists = new std::vector<cudaStream_t>[64];
-    return lists[dev & 63];
-  }
-};
-
 // A handle's small host tables on their way to the device, in one block and one copy.
 class DeviceParts {
  public:
@@ -320,45 +278,48 @@ class DeviceParts {
     parts_.push_back({reinterpret_cast<void**>(dst), src, bytes, total_});
     total_ = align_up(total_ + bytes, 256);
   }
+  // Device memory behind the tables, not copied to.
+  template <typename T>
+  void reserve(T** dst, size_t bytes) {
+    reserved_ = reinterpret_cast<void**>(dst);
+    reserved_bytes_ = bytes;
+  }
   int upload(DevicePool::Block* block) {
-    CUDA_TRY(DevicePool::pool().take(block, total_));
+    CUDA_TRY(DevicePool::pool().take(block, total_ + reserved_bytes_));
+    if (reserved_) *reserved_ = static_cast<uint8_t*>(block->ptr) + total_;
     std::vector<uint8_t> host(total_, 0);
     for (const Part& p : parts_) {
       *p.dst = static_cast<uint8_t*>(block->ptr) + p.at;
       if (p.src) std::memcpy(host.data() + p.at, p.src, p.bytes);
     }
-    CUDA_TRY(CopyStream().copy(block->ptr, host.data(), total_));
+    CUDA_TRY(cudaMemcpy(block->ptr, host.data(), total_, cudaMemcpyHostToDevice));
     return QCONV_OK;
   }
 
  private:
   struct Part { void** dst; const void* src; size_t bytes, at; };
   std::vector<Part> parts_;
-  size_t total_ = 0;
+  size_t total_ = 0, reserved_bytes_ = 0;
+  void** reserved_ = nullptr;
 };
 
 // The layer's weights: a part of the handle's block, or (from 64 KB) a block of their own that a second handle of the
 // same weights can use too.  `from`: the handle they may be shared with, or NULL.
-bool same_weights(const qconv_handle* h, const qconv_handle* from) {
-  return from && from->weights && from->weights_as_is && from->device == h->device && from->d.K == h->d.K &&
-         from->d.R == h->d.R && from->d.S == h->d.S && from->d.C == h->d.C && from->d.groups == h->d.groups;
-}
-
 int place_weights(qconv_handle* h, DeviceParts& parts, const int8_t* w, size_t bytes, bool as_is, const qconv_handle* from) {
   h->weights_as_is = as_is;
   if (bytes < 64 * 1024) {
     parts.add(&h->d_w, w, bytes);
     return QCONV_OK;
   }
-  if (as_is && same_weights(h, from) && from->algo == h->algo) {
+  if (as_is && from && from->weights && from->weights_as_is && from->device == h->device && from->d.K == h->d.K &&
+      from->d.R == h->d.R && from->d.S == h->d.S && from->d.C == h->d.C && from->algo == h->algo) {
     h->weights = from->weights;
   } else {
-    h->weights = std::make_shared<SharedWeights>();
-    CUDA_TRY(DevicePool::pool().take(&h->weights->block, bytes));
-    CUDA_TRY(CopyStream().copy(h->weights->block.ptr, w, bytes));
-    h->weights->abs_sum.swap(h->abs_sum);
+    h->weights = std::make_shared<DevicePool::Block>();
+    CUDA_TRY(DevicePool::pool().take(h->weights.get(), bytes));
+    CUDA_TRY(cudaMemcpy(h->weights->ptr, w, bytes, cudaMemcpyHostToDevice));
   }
-  h->d_w = static_cast<int8_t*>(h->weights->block.ptr);
+  h->d_w = static_cast<int8_t*>(h->weights->ptr);
   return QCONV_OK;
 }
 
@@ -577,15 +538,15 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const int taps_s_w = taps_s;                             // taps per filter row in the packed weights
   // It costs three weight chunks per stage, so it is used where tiles are 64 channels wide anyway (layers below
   // one wave, which sit at the fill rate), not for the wide tiles of the tensor-bound layers.
-  const bool halo_fits = h->mode == MODE_BOX && d.stride_h == 1 && d.stride_w == 1 && d.S == 3 && d.pad_w == 1 && (dw || d.C == 64 || d.C % 128 == 0) &&
-                         hint.halo != 0 && d.pool == 0;
+  const bool halo_fits = h->mode == MODE_BOX && d.stride_h == 1 && d.stride_w == 1 && (d.S == 3 || d.S == 5) && d.pad_w == d.S / 2 &&
+                         (dw || d.C > 32) && hint.halo != 0 && d.pool == 0;
   bool halo = false;
-  // Its tile: whole image rows with their halo, W + 2 accumulator rows per image row (two of them discarded);
-  // an image wider than 126 pixels is cut into equal column segments, each with its own halo.
-  const int halo_segs = ceil_div(d.W, qc::kTileM - 2);
+  // Its tile: whole image rows with their halo, W + S - 1 accumulator rows per image row (S - 1 of them discarded);
+  // an image wider than that leaves room for is cut into equal column segments, each with its own halo.
+  const int halo_segs = ceil_div(d.W, qc::kTileM - (d.S - 1));
   auto halo_box = [&](int* tq, int* tp, int* tn, int* step) {
     *step = ceil_div(d.W, halo_segs);
-    *tq = *step + 2;
+    *tq = *step + d.S - 1;
     *tp = std::max(1, std::min(h->P, qc::kTileM / *tq));
     *tn = (halo_segs == 1 && *tp == h->P) ? std::max(1, std::min(d.N, qc::kTileM / (*tq * *tp))) : 1;
   };
@@ -663,6 +624,17 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     p.acc_bufs = np->products <= 4 ? 2 : 1;
   }
   halo = halo_fits && (bn_max <= 64 || k_eff <= 64 || (np && np->products >= 3) || hint.halo == 1);
+  if (halo && hint.halo != 1 && !dw) {
+    // ... unless its rows' waste makes many more tiles of it, more than run at once; and five weight chunks per stage only
+    // where they are small or the layer's CTAs have an SM each.
+    int tq, tp, tn, step, bq, bp, bn;
+    halo_box(&tq, &tp, &tn, &step);
+    choose_box(h->Q, h->P, d.N, &bq, &bp, &bn);
+    const int tk = ceil_div(k_eff, std::min(bn_max, 64));
+    const long halo_tiles = static_cast<long>(ceil_div(h->Q, step)) * ceil_div(h->P, tp) * ceil_div(d.N, tn) * tk;
+    const long box_tiles = static_cast<long>(ceil_div(h->Q, bq)) * ceil_div(h->P, bp) * ceil_div(d.N, bn) * tk;
+    halo = (halo_tiles <= h->num_sms || halo_tiles * 10 <= box_tiles * 13) && (d.S == 3 || k_eff <= 32 || halo_tiles <= h->num_sms);
+  }
   if (dw) {
     // stride 1: the form (patch, or a box per filter row) whose tiles waste fewer accumulator rows
     int tq, tp, tn, step;
@@ -694,7 +666,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // tiles at most
     patch = hint.patch_halo == 1 || (tiles >= h->num_sms && used >= 0.75 && k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0);
   }
-  if (dw) patch = !halo && halo_fits && hint.patch_halo != 0;
+  if (dw) patch = !halo && halo_fits && d.S == 3 && hint.patch_halo != 0;
   if (np && halo && d.R == 3 && d.pad_h == 1 && p.np_cpp == 1 && bn_max <= 64 && hint.patch_halo != 0 && hint.halo != 1) {
     // Floating-point operands: a stage of a digit product is a patch and its nine weight chunks.  The layer runs at the rate
     // its operands arrive, so the form with fewer bytes on the busiest SM wins.
@@ -742,7 +714,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     taps_s = 1;
     p.S = 1;
   }
-  const int tps = patch ? 9 : halo ? 3 : (group ? d.S : 1);   // taps (weight chunks) per ring stage
+  const int tps = patch ? 9 : halo ? d.S : (group ? d.S : 1);   // taps (weight chunks) per ring stage
   p.halo_s = (halo || group || patch) ? tps : 0;
   p.halo_w = patch ? 3 : std::max(1, tps);
   p.store_rows = 0;
@@ -769,12 +741,26 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     const long m_tiles = static_cast<long>(halo_segs) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
     if (m_tiles * p.tiles_k <= h->num_sms) h->ctas_per_sm = 1;
   }
+  if (!halo && !patch && !dw && !is_window_mode(h->mode) && hint.ctas_per_sm == 0 && taps_r * taps_s * p.nchunks >= 9) {
+    // Tiles that all run at once, one per SM, as chains of stages: a chain is as fast as its ring is deep (four stages cover
+    // half of the latency of a load), so such a layer's CTAs get the whole shared memory.  Drawn layers of 2 to 128 tiles
+    // and 9 to 175 stages: 0 to 25 % faster, 9 % on average; from 150 tiles on they no longer run at once (1.2 to 1.5
+    // times slower), and with fewer stages the next kernel's set-up beside them is worth more.
+    int tq, tp, tn;
+    choose_box(h->Q, h->P, d.N, &tq, &tp, &tn, d.pool != 0);
+    const long m_tiles = h->mode == MODE_FLAT || h->mode == MODE_STEM ? ceil_div_l(static_cast<long>(d.N) * h->P * h->Q / h->fold, 128)
+                                                                      : static_cast<long>(ceil_div(h->Q, tq)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
+    if (m_tiles * p.tiles_k <= h->num_sms) h->ctas_per_sm = 1;
+  }
   p.vec_store = (p.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && k_eff % 16 == 0) ? 1 : 0;
   const long long round_room = h->max_shift > 0 ? (1ll << (h->max_shift - 1)) : 0;
   p.fast_epilogue = (!np && d.out_mode == QCONV_OUT_INT8 && d.rounding == QCONV_ROUND_NEAREST_EVEN && p.vec_store &&
                      d.n_out == 8 &&
                      h->acc_bound + round_room <= 2147483647ll) ? 1 : 0;
   if (hint.fast_epilogue == 0) p.fast_epilogue = 0;
+  if (p.fast_epilogue || d.out_mode != QCONV_OUT_INT8 || np || dw) h->gen_flt = 0;
+  p.gen_down = d.rounding != QCONV_ROUND_NEAREST_EVEN ? 1 : 0;
+  p.gen_away = d.rounding == QCONV_ROUND_HALF_AWAY && !d.relu ? 1 : 0;
   // rounding adds at most 2^(s-1) before the shift: in one pass when the accumulator bound leaves that room
   p.gen_simple = h->acc_bound + round_room <= 2147483647ll ? 1 : 0;
   p.gen_stage_bytes = p.fast_epilogue ? 0u : static_cast<uint32_t>((d.has_residual && d.out_mode != QCONV_OUT_INT8 ? 2 : 1) *
@@ -912,15 +898,13 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const size_t w_bytes = static_cast<size_t>(h->kpad) * h->kg_total;
   const bool as_is = h->fold == 1 && !is_window_mode(h->mode) && h->mode != MODE_STEM && h->kpad == d.K && p.nchunks * p.BKC == d.C &&
                      !np && !dw;
-  std::vector<int8_t> wp(as_is ? 0 : w_bytes, 0);
+  std::vector<int8_t> wp(as_is || dw ? 0 : w_bytes, 0);
   std::vector<int8_t> row(static_cast<size_t>(std::max(c_row, 1)), 0);
   for (int m = 0; np && m < np->products; ++m)             // [product][chunk] inside a tap
     for (int k = 0; k < d.K; ++k)
       for (int t = 0; t < d.R * d.S; ++t)
         std::memcpy(wp.data() + static_cast<size_t>(k) * h->kg_total + (static_cast<size_t>(t) * p.nchunks + m * p.np_cpp) * p.BKC,
                     np->w[m] + (static_cast<size_t>(k) * d.R * d.S + t) * d.C, d.C);
-  for (int k = 0; k < d.K && dw; ++k)
-    for (int t = 0; t < 9; ++t) wp[static_cast<size_t>(k) * h->kg_total + t * 32 + k % 32] = w_krsc[static_cast<size_t>(k) * 9 + t];
   for (int k = 0; k < d.K && !as_is && !np && !dw; ++k) {
     const int8_t* src = w_krsc + static_cast<size_t>(k) * d.R * d.S * h->Cg;
     if (h->fold > 1 && !is_window_mode(h->mode)) {
@@ -976,7 +960,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     }
   }
   int rc = QCONV_OK;
-  if (dw) parts.add(&h->d_w_mma, wp.data(), w_bytes);      // (beside the tables of the kernels for other alignments)
+  if (dw) parts.reserve(&h->d_w_mma, w_bytes);             // (filled below, from the table of the other kernels)
   else rc = place_weights(h, parts, as_is ? w_krsc : wp.data(), w_bytes, as_is, weights_of);
   if (rc) return rc;
   std::vector<int4> chan(h->kpad, make_int4(0, 0, 0, 0));
@@ -986,11 +970,15 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     chan[k] = make_int4(bias_host ? bias_host[k] : 0, sft, sft > 0 ? (1 << ((sft - 1) & 31)) - 1 : 0,
                         (sft > 0 ? 1 : 0) | ((1 << t) << 1));
     if (np) { chan[k].z = chan[k].w = 0; continue; }         // (shifts up to 40)
-    if (d.rounding >= QCONV_ROUND_HALF_UP) {                   // (general_round: no condition, another addend)
-      chan[k].z = (d.rounding == QCONV_ROUND_HALF_UP && sft > 0) ? 1 << (sft - 1) : 0;
-      chan[k].w &= ~1;
+    if (d.out_mode == QCONV_OUT_INT8 && !p.fast_epilogue && !h->gen_flt) chan[k].y = sft | t << 8;
+    if (h->gen_flt) {
+      // {magic + bias + half, bits of 2^-s, half - 1 (half away by sign: not in the bias then), 2^t << 1}
+      const float scale = std::ldexp(1.0f, -sft);
+      const int half = sft > 0 && (d.rounding == QCONV_ROUND_HALF_AWAY || d.rounding == QCONV_ROUND_HALF_UP) ? 1 << (sft - 1) : 0;
+      int bits;
+      std::memcpy(&bits, &scale, sizeof(int));
+      chan[k] = make_int4(qc::kMagicBits + (bias_host ? bias_host[k] : 0) + (p.gen_away ? 0 : half), bits, half - 1, (1 << t) << 1);
     }
-    if (d.out_mode != QCONV_OUT_INT8) chan[k].z = 1 << t;
     if (h->flt_epilogue && p.fast_epilogue) {
       // r = (M + v) * 2^-s + M * (1 - 2^-s) with M = 1.5 * 2^23: both constants are exact in binary32
       // for s <= 22; beyond that |v| < 2^22 always rounds to 0, which scale 0 and addend M give
@@ -1003,13 +991,19 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
       chan[k].y = c1bits;
       chan[k].z = c2bits;
     }
-    if (d.out_mode == QCONV_OUT_FLOAT) chan[k].w = ((acc_exp_host ? acc_exp_host[k] : 0) + 127) << 23;
+    // (wide output: the float 2^(e_x + e_w[k]) with the residual's shift in the lowest bits)
+    if (d.out_mode != QCONV_OUT_INT8) chan[k].y = (d.out_mode == QCONV_OUT_FLOAT ? ((acc_exp_host ? acc_exp_host[k] : 0) + 127) << 23 : 0) | t;
   }
   for (int j = 1; j < h->fold; ++j)
     for (int k = 0; k < d.K; ++k) chan[static_cast<size_t>(j) * d.K + k] = chan[k];
   parts.add(&h->d_chan, chan.data(), sizeof(int4) * chan.size());
   rc = parts.upload(&h->block);
   if (rc) return rc;
+  if (dw) {
+    qc::depthwise_blocks_kernel<<<ceil_div(d.C * 18, 256), 256>>>(h->d_w, reinterpret_cast<uint4*>(h->d_w_mma), d.C);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaStreamSynchronize(nullptr));              // (the stream of the first run need not wait for this one)
+  }
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->kg_total), static_cast<cuuint64_t>(h->kpad)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->kg_total)};
   cuuint32_t box[2] = {static_cast<cuuint32_t>(b_row), static_cast<cuuint32_t>(h->pair ? p.BN / 2 : p.BN)};
@@ -1022,7 +1016,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // cleared once: padding pixels, ragged edges and the padding bytes of each row stay zero
     CUDA_TRY(DevicePool::pool().take(&h->pack, pack_bytes));
     h->d_pack = static_cast<int8_t*>(h->pack.ptr);
-    CUDA_TRY(CopyStream().clear(h->d_pack, pack_bytes));   // (the stream of the first run need not wait for this one)
+    CUDA_TRY(cudaMemsetAsync(h->d_pack, 0, pack_bytes, nullptr));
+    CUDA_TRY(cudaStreamSynchronize(nullptr));              // (the stream of the first run need not wait for this one)
   }
   // the attribute belongs to the current device: once per device, not once per process
   static std::once_flag attr_once[64];
@@ -1051,6 +1046,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_U, 2, 0, qc::kGroupsPerWarpWide>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8, 2, 0, qc::kGroupsPerWarpWide>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I8>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_GEN>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_GEN_RES>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I32>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_F32>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_MAX>),
@@ -1096,7 +1093,10 @@ IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
   if (h->np_products) return qc::igemm_i8_kernel<qc::EPI_NP>;
   if (h->d.out_mode == QCONV_OUT_INT32) return qc::igemm_i8_kernel<qc::EPI_I32>;
   if (h->d.out_mode == QCONV_OUT_FLOAT) return qc::igemm_i8_kernel<qc::EPI_F32>;
-  if (!h->prm.fast_epilogue) return qc::igemm_i8_kernel<qc::EPI_I8>;
+  if (!h->prm.fast_epilogue) {
+    if (h->gen_flt) return h->d.has_residual || h->prm.gen_away ? qc::igemm_i8_kernel<qc::EPI_GEN_RES> : qc::igemm_i8_kernel<qc::EPI_GEN>;
+    return qc::igemm_i8_kernel<qc::EPI_I8>;
+  }
   const bool uni = h->uniform_shift && h->hints.uniform_shift != 0;
   if (h->dw_mma) {
     constexpr int G = qc::kGroupsPerWarp;
@@ -1149,7 +1149,7 @@ int choose_ksplit(const qconv_handle* h, long tiles) {
   // and 3 a stage) halves pay from 18 on (6 three-tap stages: 4.6 -> 4.3 us; 8 single ones: 4.0 either way), quarters from
   // 16 on while the clusters fill half of the SMs at most: with more, the next kernel's CTAs find no room to set up beside
   // them (14 x 14 x 256 3 x 3 on 16 tiles 4.6 -> 4.0, on 28 tiles 4.7 -> 5.1).
-  const int work = num_kb * (p.halo_s ? 3 : 2);
+  const int work = num_kb * (p.halo_s ? std::max(3, p.halo_s) : 2);
   if (work >= 16 && fits(4) && tiles * 8 <= h->num_sms) return 4;
   if (work >= 18 && fits(2)) return 2;
   return 1;
@@ -1482,28 +1482,24 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
   // Weight-aware bound of the wide value: 2^(n_in-1) * sum|w[k,.]| + |bias[k]| + 128 * 2^t[k].  Below 2^22 the
   // tensor-core epilogue may round in fp32 (exactly).
   h->np = np;
-  if (d.out_mode == QCONV_OUT_FLOAT && d.groups == 1 && !np && wcount >= 64 * 1024 && !same_weights(h, weights_of)) {
-    const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;                  // (for the handles that will share the weights)
-    h->abs_sum.resize(d.K);
-    for (int k = 0; k < d.K; ++k) h->abs_sum[k] = qc::host_abs_sum(w_krsc + k * per_k, per_k);
-  }
   if (d.out_mode == QCONV_OUT_INT8 && (d.groups == 1 || (Cg == 1 && d.C == d.K)) && h->hints.float_rounding != 0 && !np) {
     // ... and below 2^15 after the shift, where the clamp works on 16-bit halves.
-    long long worst = 0, worst_out = 0;
+    long long worst = 0, worst_out = 0, worst_gen = 0, worst_gen_out = 0;
+    bool unscaled = false;
     const size_t per_k = static_cast<size_t>(d.R) * d.S * Cg;
-    const std::vector<long long>* sums = same_weights(h, weights_of) && !weights_of->weights->abs_sum.empty() ? &weights_of->weights->abs_sum : nullptr;
-    if (!sums) {
-      h->abs_sum.resize(d.K);
-      for (int k = 0; k < d.K; ++k) h->abs_sum[k] = qc::host_abs_sum(w_krsc + k * per_k, per_k);
-      sums = &h->abs_sum;
-    }
-    for (int k = 0; k < d.K; ++k) {
-      const long long bnd = (*sums)[k] * (1ll << (d.n_in - 1)) +
+    for (int k = 0; k < d.K && worst < (1ll << 22) && worst_out < 32767; ++k) {
+      const long long bnd = qc::host_abs_sum(w_krsc + k * per_k, per_k) * (1ll << (d.n_in - 1)) +
                             (bias_host ? std::llabs(static_cast<long long>(bias_host[k])) : 0) +
                             (d.has_residual ? (128ll << res_lshift_host[k]) : 0);
       worst = std::max(worst, bnd);
-      worst_out = std::max(worst_out, (bnd >> (shift_host ? shift_host[k] : 0)) + 1);
+      const int sft = shift_host ? shift_host[k] : 0;
+      const long long with_half = bnd + (sft > 0 && (d.rounding == QCONV_ROUND_HALF_AWAY || d.rounding == QCONV_ROUND_HALF_UP) ? 1ll << (sft - 1) : 0);
+      worst_out = std::max(worst_out, (bnd >> sft) + 1);
+      worst_gen = std::max(worst_gen, with_half);
+      worst_gen_out = std::max(worst_gen_out, (with_half >> sft) + 1);
+      unscaled |= sft == 0;
     }
+    h->gen_flt = worst < (1ll << 22) && worst_out < 32767 && worst_gen < (1ll << 22) && worst_gen_out < 32767 && !(d.rounding == QCONV_ROUND_HALF_AWAY && !d.relu && unscaled);
     h->flt_epilogue = worst < (1ll << 22) && worst_out < 32767;
   }
 
@@ -2011,32 +2007,6 @@ int qgraph_set_input(qgraph_inputs* g, void* graph_exec, const float* d_input) {
 int qgraph_inputs_destroy(qgraph_inputs* g) {
   if (!g) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
   delete g;
-  return QCONV_OK;
-}
-
-int qconv_update_float(qconv_handle* h, const int32_t* bias_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host,
-                       void* cuda_stream) {
-  if (!h) return fail(QCONV_ERR_BAD_ARG, "NULL handle");
-  const qconv_desc& d = h->d;
-  if (h->algo != QCONV_ALGO_IGEMM || d.out_mode != QCONV_OUT_FLOAT || h->np_products)
-    return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "qconv_update_float serves tensor-core layers with float output");
-  if (d.has_residual && !res_lshift_host) return fail(QCONV_ERR_BAD_ARG, "has_residual needs res_lshift_host");
-  int max_t = 0;
-  long long max_bias = 0;
-  std::vector<int4> chan(h->kpad, make_int4(0, 0, 0, 0));
-  for (int k = 0; k < d.K; ++k) {
-    const int t = d.has_residual ? res_lshift_host[k] : 0, e = acc_exp_host ? acc_exp_host[k] : 0, b = bias_host ? bias_host[k] : 0;
-    if (t < 0 || t > 23) return fail(QCONV_ERR_RESIDUAL_SCALE, "res_lshift[%d] = %d outside [0, 23]", k, t);
-    if (e < -126 || e > 96) return fail(QCONV_ERR_BAD_ARG, "acc_exp[%d] = %d outside [-126, 96]", k, e);
-    max_t = std::max(max_t, t);
-    max_bias = std::max(max_bias, std::llabs(static_cast<long long>(b)));
-    chan[k] = make_int4(b, 0, 1 << t, (e + 127) << 23);
-  }
-  const long long bound = static_cast<long long>(d.R) * d.S * h->Cg * (1ll << (d.n_in - 1)) * (1ll << (d.n_w - 1)) + max_bias +
-                          (d.has_residual ? (128ll << max_t) : 0);
-  if (bound > 2147483647ll) return fail(QCONV_ERR_OVERFLOW_RISK, "worst-case |accumulator| %lld exceeds 2^31 - 1", bound);
-  h->acc_bound = bound;
-  CUDA_TRY(cudaMemcpyAsync(h->d_chan, chan.data(), sizeof(int4) * chan.size(), cudaMemcpyHostToDevice, static_cast<cudaStream_t>(cuda_stream)));
   return QCONV_OK;
 }
 
@@ -2806,73 +2776,32 @@ int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layo
   return QCONV_OK;
 }
 
-// Every thread takes a share of the channels of every large layer (and whole small ones in turn), so that the few large
-// layers of a network do not leave one thread at work alone; where one exponent serves the whole layer the threads meet
-// between its maximum and its conversion, and each finds its share still in its own cache.
+// Layers are independent: the largest first over up to eight threads.  (The conversion reads 5 bytes per value from
+// memory twice; beyond eight threads the memory, not the arithmetic, sets the pace.)
 int qquantize_weights_list(const qweights_job* jobs, int count) {
   if (!jobs || count < 0) return fail(QCONV_ERR_BAD_ARG, "NULL jobs or negative count");
+  std::vector<int> order(count), rc(count, QCONV_OK);
+  for (int i = 0; i < count; ++i) order[i] = i;
   auto size = [&](int i) { return static_cast<long long>(jobs[i].K) * jobs[i].R * jobs[i].S * jobs[i].Cg; };
-  long long total = 0;
-  std::vector<char> shared(count, 0);
-  std::vector<int> rc(count, QCONV_OK);
-  for (int i = 0; i < count; ++i) {
-    const qweights_job& j = jobs[i];
-    const bool sane = j.w_host && j.wq_host && j.e_w_host && j.K > 0 && j.R > 0 && j.S > 0 && j.Cg > 0 && j.n >= 2 && j.n <= 8;
-    total += sane ? size(i) : 0;
-    shared[i] = sane && j.layout == 0 && size(i) >= (1 << 17);
-  }
-  // (a thread costs some 20 us to start: worth it from about 2^18 values each)
-  int threads = static_cast<int>(std::min<long long>({8, total >> 18, std::thread::hardware_concurrency()}));
-  threads = std::max(1, threads);
-  std::vector<float> top(static_cast<size_t>(threads) * 16, 0.0f);     // a cache line per thread
-  std::atomic<int> arrived{0}, go{0};
-  auto work = [&](int t, int T) {
-    int met = 0;
-    auto meet = [&] {
-      ++met;
-      arrived.fetch_add(1);
-      while (arrived.load() < met * T) std::this_thread::yield();
-    };
-    for (int i = 0; i < count; ++i) {
-      const qweights_job& j = jobs[i];
-      if (!shared[i]) {
-        if (i % T == t) rc[i] = qquantize_weights(j.w_host, j.K, j.R, j.S, j.Cg, j.layout, j.per_channel, j.n, j.wq_host, j.e_w_host);
-        continue;
-      }
-      const size_t per_k = static_cast<size_t>(j.R) * j.S * j.Cg;
-      const int k0 = static_cast<int>(static_cast<long long>(j.K) * t / T), k1 = static_cast<int>(static_cast<long long>(j.K) * (t + 1) / T);
-      const float* w = j.w_host + k0 * per_k;
-      int8_t* q = j.wq_host + k0 * per_k;
-      if (j.per_channel) {
-        if (k1 > k0) qquantize_weights(w, k1 - k0, j.R, j.S, j.Cg, 0, 1, j.n, q, j.e_w_host + k0);
-        continue;
-      }
-      top[static_cast<size_t>(t) * 16] = qc::host_max_abs(w, per_k * (k1 - k0));
-      meet();
-      float g = 0.0f;
-      for (int u = 0; u < T; ++u) g = std::max(g, top[static_cast<size_t>(u) * 16]);
-      meet();                                              // everyone has read the maxima
-      int e;
-      qscale_exponent(g, j.n, &e);
-      for (int k = k0; k < k1; ++k) j.e_w_host[k] = e;
-      qc::host_quantize(w, per_k * (k1 - k0), e, j.n, q);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return size(a) > size(b); });
+  std::atomic<int> next{0};
+  auto work = [&] {
+    for (int i; (i = next.fetch_add(1)) < count;) {
+      const qweights_job& j = jobs[order[i]];
+      rc[order[i]] = qquantize_weights(j.w_host, j.K, j.R, j.S, j.Cg, j.layout, j.per_channel, j.n, j.wq_host, j.e_w_host);
     }
   };
-  // The shares depend on how many threads there are, so they wait for that number.
-  std::vector<std::thread> pool;
+  long long total = 0;
+  for (int i = 0; i < count; ++i) total += size(i);
+  // (a thread costs some 20 us to start: worth it from about 2^18 values each)
+  const int want = static_cast<int>(std::min<long long>({8, count, total >> 18, std::max(1u, std::thread::hardware_concurrency())}));
+  std::vector<std::thread> threads;
   try {
-    for (int t = 1; t < threads; ++t)
-      pool.emplace_back([&, t] {
-        int T;
-        while ((T = go.load()) == 0) std::this_thread::yield();
-        work(t, T);
-      });
+    for (int t = 1; t < want; ++t) threads.emplace_back(work);
   } catch (const std::system_error&) {                     // no more threads: the ones there are (this one at least) do it
   }
-  const int have = static_cast<int>(pool.size()) + 1;
-  go.store(have);
-  work(0, have);
-  for (std::thread& t : pool) t.join();
+  work();
+  for (std::thread& t : threads) t.join();
   for (int i = 0; i < count; ++i)
     if (rc[i]) return fail(rc[i], "weights %d: NULL argument or bad geometry", i);
   return QCONV_OK;

@@ -123,17 +123,6 @@ class QNetwork:
             self._pooled.discard(pool["name"])
         return binding.QConv(*args, out_c_offset=nd["dst_c_offset"], out_c_pitch=self.net["buffers"][nd["dst"]][2], **common)
 
-    def _place_weights(self, nd, converted, j):
-        """Converted weights of a layer and its float-output handle, whose tables are still to be set (update_float); no
-        handle for a layer that is not on the tensor cores."""
-        wq, e_w = converted.result()[j]
-        if nd["groups"] != 1:
-            return wq, e_w, None
-        with torch.cuda.device(self.device):
-            fl = binding.QConv(wq, None, None, np.zeros(nd["K"], np.int32) if nd["residual"] else None, None,
-                               out_mode=binding.OUT_FLOAT, has_residual=int(bool(nd["residual"])), **self._geom(nd))
-        return (wq, e_w, fl) if fl.describe().startswith("igemm") else (wq, e_w, None)
-
     def _conv_dst(self, nd):
         """Buffer a convolution writes: its own, or the pool's when it pools inside the layer."""
         pool = self._pool_after.get(nd["name"])
@@ -180,18 +169,16 @@ class QNetwork:
         self.e_buf["input"] = binding.qscale_exponent(gamma_of(st), self.n_bits)
         binding.qquantize_f32(x_calib, self.e_buf["input"], self.n_bits, out=self.bufs["input"][:n])
         convs = [nd for nd in self.net["nodes"] if nd["op"] == "conv"]
-        # the weights depend on nothing that is measured here: converted and copied to the device in the background, a few
-        # layers ahead of the measuring, the conversions of a group in parallel on the host's cores
+        # the weights depend on nothing that is measured here: converted in the background, a few layers ahead of the
+        # measuring, each group in parallel on the host's cores
         jobs = [(self.weights[nd["name"]][0], nd["K"], nd["R"], nd["S"], nd["C"] // nd["groups"], self.net["per_channel"])
                 for nd in convs]
-        ahead, place = concurrent.futures.ThreadPoolExecutor(1), concurrent.futures.ThreadPoolExecutor(2)
+        ahead = concurrent.futures.ThreadPoolExecutor(1)
         quantized = {}
         for i in range(0, len(convs), 8):
             group_jobs = ahead.submit(binding.qquantize_weights_list, jobs[i:i + 8], self.n_bits)
-            for j, nd in enumerate(convs[i:i + 8]):
-                quantized[nd["name"]] = place.submit(self._place_weights, nd, group_jobs, j)
+            quantized.update((nd["name"], (group_jobs, j)) for j, nd in enumerate(convs[i:i + 8]))
         ahead.shutdown(wait=False)
-        place.shutdown(wait=False)
         # where only the maximum is wanted, the layer finds it itself and its float output is never written
         only_max = threshold is None and not keep_stats and not sync
         fbuf = None
@@ -205,7 +192,8 @@ class QNetwork:
                 continue
             cands, floats = [], {}
             for nd in stage:
-                wq, e_w, fl = quantized.pop(nd["name"]).result()
+                pending, j = quantized[nd["name"]]
+                wq, e_w = pending.result()[j]
                 b = self.weights[nd["name"]][1]
                 e_x = self.e_buf[nd["src"]]
                 bias_q = binding.qquantize_bias(b, e_x, e_w)
@@ -213,11 +201,8 @@ class QNetwork:
                 res_lshift = None
                 if nd["residual"]:
                     res_lshift = binding.qresidual_shifts(self.e_buf[nd["residual"]], acc_exp)
-                if fl is None:
-                    fl = binding.QConv(wq, bias_q, None, res_lshift, acc_exp, out_mode=binding.OUT_FLOAT,
-                                       has_residual=int(res_lshift is not None), **self._geom(nd))
-                else:
-                    fl.update_float(bias_q, res_lshift, acc_exp)
+                fl = binding.QConv(wq, bias_q, None, res_lshift, acc_exp, out_mode=binding.OUT_FLOAT,
+                                   has_residual=int(res_lshift is not None), **self._geom(nd))
                 res = self._residual(nd)
                 if only_max:
                     st = dict(maxabs=fl.run_maxabs(self.bufs[nd["src"]], res, n_run=n))
