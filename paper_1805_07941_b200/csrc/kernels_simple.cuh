@@ -98,17 +98,17 @@ maxpool_i8_vec_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, int 
 // 3x3 stride-1 pool loads 3 vectors per output instead of 9.  The maxima are taken on pairs of
 // 16-bit lanes with the byte on top (the two-lane integer max the hardware has; a four-lane byte
 // max would be emulated) and the top bytes are put together at the end.
-// Depthwise weights [9][C] as the tensor-core form wants them, [C][9][32] with the weight at position c % 32 and zeros
+// Depthwise weights [9][C] as the tensor-core form wants them, [rows][9][32] (rows past C are zero) with the weight at position c % 32 and zeros
 // beside it: 16 bytes a thread.  (Made here: the table is 32 times what has to be copied to the device.)
 __global__ void __launch_bounds__(256)
-depthwise_blocks_kernel(const int8_t* __restrict__ w, uint4* __restrict__ out, int C) {
+depthwise_blocks_kernel(const int8_t* __restrict__ w, uint4* __restrict__ out, int C, int rows) {
   const int i = blockIdx.x * 256 + threadIdx.x;
-  if (i >= C * 18) return;
+  if (i >= rows * 18) return;
   const int half = i & 1, tap = (i >> 1) % 9, c = (i >> 1) / 9, at = c % 32 - 16 * half;
   uint32_t v[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    if (at >= 0 && (at >> 2) == j) v[j] = static_cast<uint32_t>(static_cast<uint8_t>(w[tap * C + c])) << (8 * (at & 3));
+    if (c < C && at >= 0 && (at >> 2) == j) v[j] = static_cast<uint32_t>(static_cast<uint8_t>(w[tap * C + c])) << (8 * (at & 3));
   out[i] = make_uint4(v[0], v[1], v[2], v[3]);
 }
 

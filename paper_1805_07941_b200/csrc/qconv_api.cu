@@ -284,7 +284,10 @@ class DeviceParts {
     reserved_ = reinterpret_cast<void**>(dst);
     reserved_bytes_ = bytes;
   }
-  int upload(DevicePool::Block* block) {
+  // first: runs once the tables have their addresses, before they are copied (the copy is waited for, and so is what
+  // `first` puts on the default stream).
+  template <typename First>
+  int upload(DevicePool::Block* block, First first) {
     CUDA_TRY(DevicePool::pool().take(block, total_ + reserved_bytes_));
     if (reserved_) *reserved_ = static_cast<uint8_t*>(block->ptr) + total_;
     std::vector<uint8_t> host(total_, 0);
@@ -292,8 +295,17 @@ class DeviceParts {
       *p.dst = static_cast<uint8_t*>(block->ptr) + p.at;
       if (p.src) std::memcpy(host.data() + p.at, p.src, p.bytes);
     }
+    CUDA_TRY(first());
     CUDA_TRY(cudaMemcpy(block->ptr, host.data(), total_, cudaMemcpyHostToDevice));
     return QCONV_OK;
+  }
+  int upload(DevicePool::Block* block) { return upload(block, [] { return cudaSuccess; }); }
+  // The part of destination `dst` to the device at once (inside `first`).
+  template <typename T>
+  cudaError_t copy_now(T** dst) const {
+    for (const Part& p : parts_)
+      if (p.dst == reinterpret_cast<void**>(dst)) return cudaMemcpyAsync(*dst, p.src, p.bytes, cudaMemcpyHostToDevice, nullptr);
+    return cudaSuccess;                                    // (has a block of its own and is there already)
   }
 
  private:
@@ -554,7 +566,11 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   p.BKC = choose_bkc(c_eff);
   if (is_window_mode(h->mode)) p.BKC = c_eff <= 32 ? 32 : (c_eff <= 64 ? 64 : 128);   // a row is one chunk (two at most)
   // (depthwise at stride 2: rows of 64 bytes, the three taps of a filter row sharing a stage)
-  if (dw) p.BKC = d.C % 128 == 0 && d.stride_h == 1 && !(hint.bn_max > 0 && hint.bn_max < 128) ? 128 : d.C % 64 == 0 ? 64 : 32;
+  // (128 wide unless the last tile would be mostly padding)
+  if (dw) {
+    const bool wide_row = d.stride_h == 1 && !(hint.bn_max > 0 && hint.bn_max < 128) && align_up(d.C, 128) * 7 <= align_up(d.C, 64) * 8;
+    p.BKC = wide_row ? 128 : d.C > 32 ? 64 : 32;
+  }
   p.nchunks = dw ? 1 : ceil_div(c_eff, p.BKC);
   const int b_row = dw ? 32 : p.BKC;                       // bytes of a weight row per chunk
   h->a_channels = d.C;
@@ -622,6 +638,13 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     const int cols = np->products <= 4 ? 256 : 512;
     bn_max = std::min({bn_max, 128, cols / np->products / 16 * 16});
     p.acc_bufs = np->products <= 4 ? 2 : 1;
+    // Few tiles: an MMA of N <= 96 takes the same time whatever its width, so narrower tiles on idle SMs have less to load
+    // and less to convert each, for free.
+    int tq, tp, tn;
+    choose_box(h->Q, h->P, d.N, &tq, &tp, &tn);
+    const long m_tiles = h->mode == MODE_FLAT ? ceil_div_l(static_cast<long>(d.N) * h->P * h->Q, 128)
+                                              : static_cast<long>(ceil_div(h->Q, tq)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
+    for (int next; hint.bn_max <= 0 && bn_max > 16 && m_tiles * ceil_div(k_eff, next = std::max(16, bn_max / 32 * 16)) <= h->num_sms;) bn_max = next;
   }
   halo = halo_fits && (bn_max <= 64 || k_eff <= 64 || (np && np->products >= 3) || hint.halo == 1);
   if (halo && hint.halo != 1 && !dw) {
@@ -720,7 +743,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   p.store_rows = 0;
   p.tap_boxes = group ? 1 : 0;
   p.tiles_k = ceil_div(k_eff, bn_max);
-  p.BN = static_cast<int>(align_up(ceil_div(k_eff, p.tiles_k), 16));
+  p.BN = dw ? p.BKC : static_cast<int>(align_up(ceil_div(k_eff, p.tiles_k), 16));
   h->kpad = p.tiles_k * p.BN;
   const int all_taps = patch ? 9 : taps_r * taps_s_w;
   h->kg_total = all_taps * p.nchunks * b_row;
@@ -997,13 +1020,14 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   for (int j = 1; j < h->fold; ++j)
     for (int k = 0; k < d.K; ++k) chan[static_cast<size_t>(j) * d.K + k] = chan[k];
   parts.add(&h->d_chan, chan.data(), sizeof(int4) * chan.size());
-  rc = parts.upload(&h->block);
+  rc = parts.upload(&h->block, [&] {
+    if (!dw) return cudaSuccess;
+    const cudaError_t e = parts.copy_now(&h->d_w);
+    if (e != cudaSuccess) return e;
+    qc::depthwise_blocks_kernel<<<ceil_div(h->kpad * 18, 256), 256>>>(h->d_w, reinterpret_cast<uint4*>(h->d_w_mma), d.C, h->kpad);
+    return cudaGetLastError();
+  });
   if (rc) return rc;
-  if (dw) {
-    qc::depthwise_blocks_kernel<<<ceil_div(d.C * 18, 256), 256>>>(h->d_w, reinterpret_cast<uint4*>(h->d_w_mma), d.C);
-    CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaStreamSynchronize(nullptr));              // (the stream of the first run need not wait for this one)
-  }
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->kg_total), static_cast<cuuint64_t>(h->kpad)};
   cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->kg_total)};
   cuuint32_t box[2] = {static_cast<cuuint32_t>(b_row), static_cast<cuuint32_t>(h->pair ? p.BN / 2 : p.BN)};
@@ -1046,6 +1070,10 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_U, 2, 0, qc::kGroupsPerWarpWide>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8, 2, 0, qc::kGroupsPerWarpWide>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I8>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 0, 5>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8, 0, 5>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 1, 5>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8, 1, 5>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_GEN>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_GEN_RES>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_I32>),
@@ -1069,7 +1097,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   if (h->pair) {
     PairKernel pk = pair_kernel_for(h);
     CUDA_TRY(cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  } else if (d.pool || dw) {
+  } else if (d.pool) {
     CUDA_TRY(cudaFuncSetAttribute(igemm_kernel_for(h), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   }
   return QCONV_OK;
@@ -1580,9 +1608,11 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       parts.add(&h->d_dw_tap, t.data(), t.size() * 4);
       h->dw_tap = 1;
       if (d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
-      // On the tensor cores where a pixel's channels fill rows of 64 or 128 bytes (with rows of 32 the per-tile work
-      // outweighs it: 112 x 112 x 32 at batch 256 76 -> 96 us).
-      h->dw_mma = h->flt_epilogue && d.pad_h == 1 && d.pad_w == 1 && d.C % (h->hints.depthwise_form == 3 ? 32 : 64) == 0 &&
+      // On the tensor cores in rows of 64 or 128 channels, an eighth of padding at most (23 x 49 x 8 x 928, stride 2:
+      // 33 -> 8.4 us; a third of it costs: 64 x 56 x 56 x 144 27 -> 34; with rows of 32 the per-tile work outweighs the gain:
+      // 112 x 112 x 32 at batch 256 76 -> 96).
+      h->dw_mma = h->flt_epilogue && d.pad_h == 1 && d.pad_w == 1 && d.C % 16 == 0 &&
+                  (h->hints.depthwise_form == 3 || align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8) &&
                   d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && (h->hints.depthwise_form < 0 || h->hints.depthwise_form == 3);
     }
     if (!rc && h->dw_mma) {

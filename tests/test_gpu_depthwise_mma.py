@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = [  # N, H, W, C, stride
     (2, 9, 11, 32, 1), (1, 8, 14, 64, 1), (3, 7, 7, 128, 1), (2, 9, 15, 128, 1), (1, 1, 1, 64, 1), (2, 17, 130, 192, 1),
-    (2, 14, 14, 64, 2), (1, 13, 9, 128, 2), (5, 3, 2, 96, 2), (1, 30, 61, 32, 2), (40, 14, 14, 256, 1), (40, 14, 14, 256, 2)]
+    (2, 14, 14, 64, 2), (1, 13, 9, 128, 2), (2, 9, 17, 48, 1), (1, 20, 15, 208, 1), (2, 7, 31, 112, 2), (1, 5, 5, 16, 1), (5, 3, 2, 96, 2), (1, 30, 61, 32, 2), (40, 14, 14, 256, 1), (40, 14, 14, 256, 2)]
 
 
 @pytest.mark.parametrize("case", CASES)
