@@ -775,12 +775,51 @@ __device__ __forceinline__ void gen_store_units(const uint8_t* stage, int8_t* ba
   }
 }
 
+// The same way in.  A loaded row keeps its place relative to the words of memory: its first byte at its address modulo 4.
+__device__ __forceinline__ void gen_load_units(uint8_t* stage, const int8_t* base, long long row_off, bool ok, int bytes, int lane) {
+  const unsigned okmask = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+  for (int r0 = 0; r0 < 32; r0 += 4) {
+    const int r = r0 + (lane >> 3);
+    const int8_t* row = base + __shfl_sync(0xffffffffu, row_off, r);
+    const int head = static_cast<int>(-reinterpret_cast<uintptr_t>(row) & 7u), at = head + 8 * (lane & 7);
+    if (((okmask >> r) & 1u) && at + 8 <= bytes) {
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(row + at));
+      uint32_t* sp = reinterpret_cast<uint32_t*>(stage + r * kGenPitch + at + (reinterpret_cast<uintptr_t>(row) & 3u));
+      sp[0] = v.x;
+      sp[1] = v.y;
+    }
+  }
+  if (!ok) return;
+  const int8_t* row = base + row_off;
+  uint8_t* dst = stage + lane * kGenPitch + (reinterpret_cast<uintptr_t>(row) & 3u);
+  const int head = static_cast<int>(-reinterpret_cast<uintptr_t>(row) & 7u), tail = (bytes - head) & 7;
+  int pos = 0;
+  if (head & 1) { dst[0] = static_cast<uint8_t>(__ldg(row)); pos = 1; }
+  if (head & 2) {
+    *reinterpret_cast<uint16_t*>(dst + pos) = __ldg(reinterpret_cast<const uint16_t*>(row + pos));
+    pos += 2;
+  }
+  if (head & 4) *reinterpret_cast<uint32_t*>(dst + pos) = __ldg(reinterpret_cast<const uint32_t*>(row + pos));
+  pos = bytes - tail;
+  if (tail & 4) {
+    *reinterpret_cast<uint32_t*>(dst + pos) = __ldg(reinterpret_cast<const uint32_t*>(row + pos));
+    pos += 4;
+  }
+  if (tail & 2) {
+    *reinterpret_cast<uint16_t*>(dst + pos) = __ldg(reinterpret_cast<const uint16_t*>(row + pos));
+    pos += 2;
+  }
+  if (tail & 1) dst[pos] = static_cast<uint8_t>(__ldg(row + pos));
+}
+
 template <bool STORE>
 __device__ __forceinline__ void gen_copy(int vec, uint8_t* stage, int8_t* base, long long row_off, bool ok, int bytes, int lane) {
   if (bytes <= 0) return;
   if (vec == 16) gen_copy_rows<16, STORE>(stage, base, row_off, ok, bytes, lane);
   else if (vec == 8) gen_copy_rows<8, STORE>(stage, base, row_off, ok, bytes, lane);
   else if (STORE && bytes >= 16) gen_store_units(stage, base, row_off, ok, bytes, lane);
+  else if (bytes >= 16) gen_load_units(stage, base, row_off, ok, bytes, lane);
   else gen_copy_words<STORE>(stage, base, row_off, ok, bytes, lane);
 }
 
