@@ -1450,6 +1450,10 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       const TileCoord tc = walk.coord(prm);
       const int buf = (EPI == EPI_NP && prm.acc_bufs == 1) ? 0 : it & 1;
       const uint32_t use = static_cast<uint32_t>((EPI == EPI_NP && prm.acc_bufs == 1) ? it : it >> 1);
+      // Slot of the per-tile channel constants: by the tile's parity even where there is one accumulator buffer.  A warp that
+      // is done with a tile stages the next one's constants while slower warps still read theirs; past the vote behind the
+      // staging every warp is done with the tile before, whose slot the tile after may then overwrite.
+      const int cst_slot = it & 1;
       if (res_staged) {
         walk_next.next(prm);
         if (etid == 0 && tile + static_cast<int>(gridDim.x) < total_tiles) {
@@ -1466,7 +1470,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       if (!cst_all) {
         // stage this tile's channel constants, then meet the other epilogue warps
         for (int i = etid; i < prm.BN; i += kEpilogueWarps * 32) {
-          stage_constant<EPI>(sh->cst, buf * 256 + i, chan_table + tc.k0 + i);
+          stage_constant<EPI>(sh->cst, cst_slot * 256 + i, chan_table + tc.k0 + i);
         }
         if (epilogue_vote(!ok)) { ok = false; break; }
       }
@@ -1572,7 +1576,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                                 static_cast<uint32_t>(buf * prm.tmem_cols);
         // shared-memory address of this tile's first channel constant (16 bytes per channel, or 4 when
         // only the biases differ)
-        const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : buf * 256) * EpiTraits<EPI>::cst_bytes;
+        const uint32_t chan = cst_addr + static_cast<uint32_t>(cst_all ? tc.k0 : cst_slot * 256) * EpiTraits<EPI>::cst_bytes;
         // This warp's 16-column groups, up to kGroupsPerWarp of them.  Tensor-memory loads run one
         // group ahead of the arithmetic; after the warp's last load the accumulator buffer goes back
         // to the MMA warp.

@@ -47,3 +47,34 @@ def test_products_match_the_oracle(digits, case):
             got = y.cpu().numpy()
             assert (got[:n_run] == want).all() and (got[n_run:] == 0x55).all(), conv.describe()
         conv.destroy()
+
+
+@pytest.mark.parametrize("digits", [(2, 3), (3, 3), (2, 2)])
+@pytest.mark.parametrize("case", [(1, 1, 80, 80, 16, 512, 1, 1), (2, 2, 45, 43, 16, 1000, 1, 1), (1, 1, 131, 129, 16, 520, 1, 2)])
+def test_constants_of_many_channels_tile_by_tile(digits, case):
+    """More channels than shared memory holds constants for (512 of 16 bytes, padding included): every tile stages its own, and
+    a CTA walks several tiles of different channels, with one accumulator buffer (five and six products) and with two.  Shifts
+    and biases differ from channel to channel, so that a tile on another tile's constants is wrong."""
+    import torch
+    N, n_run, H, W, C, K, R, stride = case
+    fi, fw, fo = FMT[digits[0]], FMT[digits[1]], FMT[2]
+    rng = np.random.default_rng(sum(case) + 10 * digits[0] + digits[1])
+    x, w = (rng.integers(0, 256, s).astype(np.uint8) for s in ((N, H, W, C), (K, R, R, C)))
+    for a in (x, w):
+        a[(a & 0x7F) == 0] = 0
+    bias = rng.integers(-2**31 + 1, 2**31 - 1, K).astype(np.int32)
+    acc = fpconv_ref.wide_value(x[:1, :16], w, bias, fi, fw, R=R, S=R, stride=(stride, stride), pad=(0, 0))
+    base = np.log2(max(1.0, float(np.abs(acc).mean()) * 3 / fpconv_ref.magnitudes(*fo)[-1]))
+    shift = (int(base) + rng.integers(-3, 4, K)).clip(0, 40).astype(np.int32)
+    want = fpconv_ref.qconv_np(x, w, bias, shift, fi, fw, fo, R=R, S=R, stride=(stride, stride), pad=(0, 0))
+    conv = binding.QConvNP(w, bias, shift, N=N, H=H, W=W, C=C, K=K, R=R, S=R, stride_h=stride, stride_w=stride, n_in=fi[0],
+                           p_in=fi[1], n_w=fw[0], p_w=fw[1], n_out=fo[0], p_out=fo[1])
+    plan = dict(f.split("=") for f in conv.describe().split() if f.count("=") == 1)
+    m_tiles = -(-N * conv.P * conv.Q // 128)
+    assert int(plan["BN"]) * int(plan["tiles_k"]) > 512 and m_tiles * int(plan["tiles_k"]) > 148, plan
+    xd = torch.from_numpy(x).cuda()
+    for _ in range(3):
+        y = torch.full((N, conv.P, conv.Q, K), 0x55, dtype=torch.uint8, device="cuda")
+        conv.run(xd, y)
+        assert conv.status() == 0 and (y.cpu().numpy() == want).all(), conv.describe()
+    conv.destroy()
