@@ -2462,7 +2462,11 @@ int qconv_np_create(qconv_np_handle** out, const qconv_np_desc* desc, const uint
   h->c_pad = h->gemm->a_channels / spec.planes;
   const size_t bytes = static_cast<size_t>(d.N) * d.H * d.W * h->gemm->a_channels;
   cudaError_t e = cudaMalloc(&h->d_planes, bytes);
-  if (e == cudaSuccess && h->c_pad != d.C) e = cudaMemset(h->d_planes, 0, bytes);   // the padding channels stay zero
+  if (e == cudaSuccess && h->c_pad != d.C) {
+    // cleared once: the padding channels stay zero (waited for: the stream of the first run need not wait for this one)
+    e = cudaMemsetAsync(h->d_planes, 0, bytes, nullptr);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  }
   if (e != cudaSuccess) {
     free_np(h);
     return fail(QCONV_ERR_CUDA, "qconv_np_create: %s", cudaGetErrorString(e));

@@ -78,3 +78,30 @@ def test_constants_of_many_channels_tile_by_tile(digits, case):
         conv.run(xd, y)
         assert conv.status() == 0 and (y.cpu().numpy() == want).all(), conv.describe()
     conv.destroy()
+
+
+def test_first_run_on_another_stream_finds_the_padding_cleared():
+    """48 channels are padded to 64 in the digit planes (0.8 GB here), which creation clears; a run right behind it on a stream
+    that does not wait for the default one must not have its planes cleared under it."""
+    import torch
+    N, H, W, C, K = 256, 128, 128, 48, 16
+    rng = np.random.default_rng(1)
+    w = rng.integers(1, 127, (K, 1, 1, C)).astype(np.uint8)
+    shift = np.full(K, 14, np.int32)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(2)
+    x = torch.randint(1, 127, (N, H, W, C), generator=gen, device="cuda", dtype=torch.uint8)
+    y = torch.empty((N, H, W, K), dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        conv = binding.QConvNP(w, None, shift, N=N, H=H, W=W, C=C, K=K, R=1, S=1, n_in=8, p_in=4, n_w=8, p_w=4, n_out=8, p_out=4)
+        conv.run(x, y)
+    assert conv.status() == 0
+    first = y.clone()
+    conv.run(x, y)
+    assert conv.status() == 0 and torch.equal(first, y)
+    for n in (0, N // 2, N - 1):
+        want = fpconv_ref.qconv_np(x[n:n + 1].cpu().numpy(), w, None, shift, (8, 4), (8, 4), (8, 4), R=1, S=1)
+        assert (first[n:n + 1].cpu().numpy() == want).all()
+    conv.destroy()
