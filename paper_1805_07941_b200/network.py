@@ -12,6 +12,7 @@ conversion -- runs inside the library.  The bookkeeping it does is the paper's:
   * right shifts s[k] = e_z - e_x - e_w[k] are never negative (factors in (0, 1]).
 """
 import concurrent.futures
+import operator
 
 import numpy as np
 import torch
@@ -29,6 +30,9 @@ def _stages(nodes):
     for _, grp in itertools.groupby(nodes, key=key):
         runs.append(list(grp))
     return runs
+
+
+_HANDLE = operator.attrgetter("handle")
 
 
 class _NetGraph:
@@ -166,7 +170,9 @@ class QNetwork:
         st = collect(x_calib)
         if keep_stats:
             self.stats["input"] = st
-        self.e_buf["input"] = binding.qscale_exponent(gamma_of(st), self.n_bits)
+        e_input = binding.qscale_exponent(gamma_of(st), self.n_bits)
+        self._forget_plans()                                 # (before the first handle goes: what follows may raise half-way)
+        self.e_buf["input"] = e_input
         binding.qquantize_f32(x_calib, self.e_buf["input"], self.n_bits, out=self.bufs["input"][:n])
         convs = [nd for nd in self.net["nodes"] if nd["op"] == "conv"]
         # the weights depend on nothing that is measured here: converted in the background, a few layers ahead of the
@@ -231,11 +237,10 @@ class QNetwork:
                 hnd.run(self.bufs[nd["src"]], self._conv_dst(nd), self._residual(nd), n_run=n)
             self.e_buf[nd0["dst"]] = e_z
         torch.cuda.synchronize()
-        self._forget_plans()
         return self
 
     def _forget_plans(self):
-        """New layer handles: drop what was made from the old ones."""
+        """Drop what was made from the layer handles, which are about to be replaced or destroyed."""
         self.graph = None
         self._programs = {}
         self._drop_parts()
@@ -244,13 +249,13 @@ class QNetwork:
 
     def load_params(self, params, e_buf):
         """Build the int8 handles from parameters chosen elsewhere (same keys as self.params)."""
+        self._forget_plans()
         self.params = params
         self.e_buf = dict(e_buf)
         for nd in self.net["nodes"]:
             if nd["op"] != "conv":
                 continue
             self.handles[nd["name"]] = self._make_handle(nd)
-        self._forget_plans()
         return self
 
     # ------------------------------------------------------------------ inference
@@ -320,11 +325,17 @@ class QNetwork:
         return binding.Steps(steps)
 
     def _run_program(self, n, address):
-        if n not in self._programs:
+        # a program holds addresses: it serves as long as the handles and buffers they were taken from are the network's
+        # and the handles live (it keeps them from being collected)
+        owners = [*self.handles.values(), *self.bufs.values(), self.x_static]
+        kept, program = self._programs.get(n, ((), None))
+        if len(kept) != len(owners) or not all(map(operator.is_, kept, owners)) or \
+                not all(map(_HANDLE, self.handles.values())):
             if len(self._programs) >= 64:                    # (a list of addresses per batch size: a few KB each)
                 self._programs.clear()
-            self._programs[n] = self._program(slice(0, n))
-        self._programs[n].run(address)
+            program = self._program(slice(0, n))
+            self._programs[n] = owners, program
+        program.run(address)
 
     def _dependencies(self):
         """For every node, the earlier nodes it must follow: writers of what it reads (input or
@@ -586,11 +597,10 @@ class QNetwork:
         return n * (2 if getattr(self, "graph_form", None) == "split2" and self.graph is not None else 1)
 
     def destroy(self):
+        self._forget_plans()
         for h in self.handles.values():
             h.destroy()
         self.handles = {}
-        self._programs = {}
-        self._drop_parts()
 
     def _drop_parts(self):
         for sets in getattr(self, "_parts", {}).values():
