@@ -781,6 +781,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                      d.n_out == 8 &&
                      h->acc_bound + round_room <= 2147483647ll) ? 1 : 0;
   if (hint.fast_epilogue == 0) p.fast_epilogue = 0;
+  // (no other epilogue knows the depthwise operands: create_layer takes the tensor cores only where this one serves)
+  if (dw && !p.fast_epilogue) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: depthwise on the tensor cores without its epilogue");
   if (p.fast_epilogue || d.out_mode != QCONV_OUT_INT8 || np || dw) h->gen_flt = 0;
   p.gen_down = d.rounding != QCONV_ROUND_NEAREST_EVEN ? 1 : 0;
   p.gen_away = d.rounding == QCONV_ROUND_HALF_AWAY && !d.relu ? 1 : 0;
@@ -1611,7 +1613,7 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       // On the tensor cores in rows of 64 or 128 channels, an eighth of padding at most (23 x 49 x 8 x 928, stride 2:
       // 33 -> 8.4 us; a third of it costs: 64 x 56 x 56 x 144 27 -> 34; with rows of 32 the per-tile work outweighs the gain:
       // 112 x 112 x 32 at batch 256 76 -> 96).
-      h->dw_mma = h->flt_epilogue && d.pad_h == 1 && d.pad_w == 1 && d.C % 16 == 0 &&
+      h->dw_mma = h->flt_epilogue && h->hints.fast_epilogue != 0 && d.pad_h == 1 && d.pad_w == 1 && d.C % 16 == 0 &&
                   (h->hints.depthwise_form == 3 || align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8) &&
                   d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && (h->hints.depthwise_form < 0 || h->hints.depthwise_form == 3);
     }

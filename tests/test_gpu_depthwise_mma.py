@@ -46,3 +46,27 @@ def test_less_aligned_tensors_take_the_other_kernels():
         xd.copy_(torch.from_numpy(x))
         conv.run(xd, yd)
         assert conv.status() == 0 and (yd.cpu().numpy() == want).all(), off
+
+
+@pytest.mark.parametrize("case", [(2, 9, 11, 64, 1), (1, 13, 9, 128, 2), (3, 30, 31, 192, 1), (2, 21, 20, 256, 2)])
+def test_plan_hints_never_change_a_depthwise_layer(case):
+    """Every hint of the plan on a layer that the tensor cores take by themselves, and beside the depthwise forms; a hint that
+    takes the fast epilogues away leaves the layer to the CUDA-core kernels."""
+    from paper_1805_07941_b200 import binding
+    N, H, W, C, st = case
+    rng = np.random.default_rng(sum(case))
+    x, w, bias, shift, _, _ = rand_layer(rng, N, H, W, C, C, 3, 3, groups=C, stride=(st, st), pad=(1, 1))
+    shift = (shift - 1).clip(4, 31)
+    kw = dict(R=3, S=3, stride=(st, st), pad=(1, 1), groups=C)
+    want = oracle_conv(x, w, bias, shift, **kw)
+    for form in (-1, 0, 1, 2, 3):
+        for hints in (dict(), dict(fast_epilogue=0), dict(float_rounding=0), dict(uniform_shift=0), dict(halo=0), dict(halo=1),
+                      dict(resident_weights=0), dict(resident_weights=1), dict(tma_store=0), dict(tma_store=1), dict(group_taps=0),
+                      dict(group_taps=1), dict(patch_halo=0), dict(patch_halo=1), dict(bn_max=32), dict(bn_max=256),
+                      dict(ctas_per_sm=1), dict(ctas_per_sm=2), dict(pdl=0), dict(split_k=2), dict(pair_tiles=1), dict(fold=0)):
+            with binding.plan_hints(depthwise_form=form, **hints):
+                got, desc = gpu_conv(x, w, bias, shift, **kw)
+            on_tensor_cores = form in (-1, 3) and "fast_epilogue" not in hints and "float_rounding" not in hints
+            assert ("depthwise3x3/mma" in desc) == on_tensor_cores, (form, hints, desc)
+            assert form != 2 or "tap-packed+tma" in desc, (hints, desc)
+            assert (got == want).all(), (form, hints, desc)
