@@ -229,9 +229,8 @@ int qcalib_collect(const float* d_x, size_t count, int nbins, float range_hi,
  * is the first call into the library on that device, CUDA may load the library's device code --
  * the array with it -- at that moment, so it belongs in start-up); make that first call before any
  * stream capture begins.  All calls on a device share
- * the one array: each call clears the counters it accumulates into before it starts, and two calls
- * whose kernels overlap on the GPU (different streams, or different host threads) race on it and
- * return garbage -- serialise them. */
+ * the one array, whose counters every call finds and leaves at zero; the library serialises the
+ * calls of a device (a call waits until the one before, from whichever thread, has returned). */
 #define QCALIB_STATIC_MAX_BINS 4096
 #define QCALIB_STATIC_MAX_COUNT ((size_t)1 << 40)
 int qcalib_collect_static(const float* d_x, size_t count, int nbins, float range_hi,

@@ -2094,7 +2094,9 @@ static __device__ __align__(256) unsigned char g_calib_static_scratch[sizeof(qc:
 namespace {
 // Device scratch of qcalib_collect and pinned memory its results land in, both made on first use per device and kept.
 struct CalibDevice {
-  std::mutex mu;                                           // one collection at a time on a device's scratch
+  // One collection at a time on each scratch, to its end: a collection relies on the accumulators that the one before left
+  // at zero, so two that overlapped would spoil not only each other but every later one.
+  std::mutex mu, built_in_mu;
   qc::CalibScratch* scratch = nullptr;
   qc::CalibScratch* built_in = nullptr;                    // device address of the array in the library image
   qc::CalibResult* landing = nullptr;
@@ -2110,14 +2112,16 @@ int calib_run(const float* d_x, size_t count, int nbins, float range_hi, qcalib_
   const size_t vecs = (count + 3) / 4;
   CUDA_TRY(launch_chained(qc::calib_pass1_kernel, dim3(grid_for(vecs, 256, 148 * qc::kCalibBlocksPerSm)), dim3(256), 0, st, d_x, count, sc,
                           nbins, vec_ok));
-  CUDA_TRY(launch_chained(qc::calib_hist_kernel, dim3(grid_for(vecs, qc::kCalibHistThreads, 148 * 2)), dim3(qc::kCalibHistThreads),
-                          nbins * sizeof(unsigned int), st, d_x, count, sc, nbins, range_hi, vec_ok, landing));
+  cudaError_t e = launch_chained(qc::calib_hist_kernel, dim3(grid_for(vecs, qc::kCalibHistThreads, 148 * 2)), dim3(qc::kCalibHistThreads),
+                                 nbins * sizeof(unsigned int), st, d_x, count, sc, nbins, range_hi, vec_ok, landing);
   qc::CalibResult pageable;
-  if (!landing) {
-    CUDA_TRY(cudaMemcpyAsync(&pageable, &sc->res, offsetof(qc::CalibResult, hist) + sizeof(uint64_t) * nbins, cudaMemcpyDeviceToHost, st));
+  if (e == cudaSuccess && !landing) {
+    e = cudaMemcpyAsync(&pageable, &sc->res, offsetof(qc::CalibResult, hist) + sizeof(uint64_t) * nbins, cudaMemcpyDeviceToHost, st);
     landing = &pageable;
   }
-  CUDA_TRY(cudaStreamSynchronize(st));
+  const cudaError_t done = cudaStreamSynchronize(st);      // (after a failure too: the scratch is the next call's from here on)
+  CUDA_TRY(e);
+  CUDA_TRY(done);
   const qc::CalibHead head = landing->head;
   std::memcpy(host_out->hist, landing->hist, sizeof(uint64_t) * nbins);
   std::memcpy(&host_out->maxabs, &head.maxabs_bits, sizeof(float));
@@ -2173,16 +2177,14 @@ int qcalib_collect_static(const float* d_x, size_t count, int nbins, float range
   CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(QCONV_ERR_CUDA, "device index %d out of range", dev);
   CalibDevice& d = g_calib[dev];
-  {
+  std::lock_guard<std::mutex> lock(d.built_in_mu);
+  if (!d.built_in) {
     // first call on this device: translate the symbol into this device's address (no allocation)
-    std::lock_guard<std::mutex> lock(d.mu);
-    if (!d.built_in) {
-      void* ptr = nullptr;
-      cudaError_t e = cudaGetSymbolAddress(&ptr, g_calib_static_scratch);
-      if (e != cudaSuccess || !ptr)
-        return fail(QCONV_ERR_CUDA, "cudaGetSymbolAddress(built-in calibration scratch): %s", cudaGetErrorString(e));
-      d.built_in = static_cast<qc::CalibScratch*>(ptr);
-    }
+    void* ptr = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(&ptr, g_calib_static_scratch);
+    if (e != cudaSuccess || !ptr)
+      return fail(QCONV_ERR_CUDA, "cudaGetSymbolAddress(built-in calibration scratch): %s", cudaGetErrorString(e));
+    d.built_in = static_cast<qc::CalibScratch*>(ptr);
   }
   // the array starts out zero with the library image, and every collection leaves its accumulators so
   return calib_run(d_x, count, nbins, range_hi, host_out, static_cast<cudaStream_t>(cuda_stream), d.built_in, nullptr);

@@ -70,3 +70,34 @@ def test_static_scratch_rejects_what_it_cannot_hold():
     assert rc == binding.ERR_BAD_ARG and b"count" in binding.lib().qconv_last_error_string()
     ok = binding.qcalib_collect_static(x, 16)                                      # still usable afterwards
     assert ok["count"] == 1000 and ok["hist"][0] == 1000
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("collect", ["qcalib_collect_static", "qcalib_collect"])
+def test_calls_from_several_threads_and_streams_do_not_meet_in_the_scratch(collect):
+    """The counters in the scratch are carried from call to call: a collection has it to itself, so that neither the calls of
+    other threads nor any later one can come out wrong."""
+    import threading
+    import torch
+    run = getattr(binding, collect)
+    rng = np.random.default_rng(3)
+    xs = [torch.from_numpy((rng.standard_normal(n) * (i + 1)).astype(np.float32)).cuda() for i, n in enumerate((3_000_001, 1000, 500_000, 77))]
+    alone = [run(x, 512 + i) for i, x in enumerate(xs)]
+    torch.cuda.synchronize()
+    wrong = []
+
+    def work(i):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(40):
+                got = run(xs[i], 512 + i)
+                if any(got[k] != alone[i][k] for k in ("maxabs", "count", "nonfinite", "sum", "sumsq")) or (got["hist"] != alone[i]["hist"]).any():
+                    wrong.append(i)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(xs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    for i, x in enumerate(xs):
+        _same(run(x, 512 + i), alone[i])
