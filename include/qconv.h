@@ -128,7 +128,7 @@ int qconv_set_plan_hints(const qconv_plan_hints* hints);
  *   res_lshift_host K left shifts t[k] = e_res - e_x - e_w[k] in [0, 23]; required iff has_residual
  *   acc_exp_host    K exponents e_x + e_w[k] in [-126, 96]; read only by QCONV_OUT_FLOAT; NULL means 0
  * Tables and scratch come from a pool of device memory that keeps up to 256 MB of what destroyed handles gave back,
- * until the last handle of the device is gone.
+ * until the last handle of the device is gone or the library itself finds the device full.
  * Errors: BAD_ARG, UNSUPPORTED_SHAPE, OVERFLOW_RISK when
  *   (R*S*C/groups) * 2^(n_in-1) * 2^(n_w-1) + max|bias| + 2^(7 + max t) > 2^31 - 1,
  * BAD_SHIFT, RESIDUAL_SCALE, ALIGNMENT, CUDA.  On error *out is NULL. */

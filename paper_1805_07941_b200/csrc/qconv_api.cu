@@ -106,7 +106,7 @@ inline bool is_window_mode(int m) { return m == MODE_S2D || m == MODE_WROW; }
 
 // Device memory of the handles' tables and scratch.  A network's calibration builds and destroys two handles per layer;
 // cudaMalloc and cudaFree took two thirds of that time, and at times a hundred milliseconds for one call.  Blocks given back are kept for the next handle, at most kKeep bytes per
-// device, and all of them are freed when the last block in use is given back.  Any thread, any stream: a block is only
+// device, and all of them are freed when the last block in use is given back, or when the device has no memory left.  Any thread, any stream: a block is only
 // given back after the device is idle, so whoever takes it next may overwrite it at once.
 class DevicePool {
  public:
@@ -141,12 +141,21 @@ class DevicePool {
       d.kept -= b->bytes;
       d.free.erase(d.free.begin() + static_cast<long>(best));
     } else {
-      e = cudaMalloc(&b->ptr, bytes);
+      e = allocate(&b->ptr, bytes, d);
       if (e != cudaSuccess) { b->ptr = nullptr; return e; }
       b->bytes = bytes;
     }
     ++d.live;
     return cudaSuccess;
+  }
+  // cudaMalloc for memory that is not the pool's.
+  template <typename T>
+  cudaError_t plain(T** ptr, size_t bytes) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu_);
+    return allocate(reinterpret_cast<void**>(ptr), bytes, per_device_[dev & 63]);
   }
 
  private:
@@ -158,6 +167,16 @@ class DevicePool {
   std::mutex mu_;
   PerDevice per_device_[64];
 
+  // On a full device what is kept for later handles goes first.  (Kept blocks are idle.)
+  cudaError_t allocate(void** ptr, size_t bytes, PerDevice& d) {
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e != cudaErrorMemoryAllocation || d.free.empty()) return e;
+    cudaGetLastError();
+    for (auto& f : d.free) cudaFree(f.first);
+    d.free.clear();
+    d.kept = 0;
+    return cudaMalloc(ptr, bytes);
+  }
   void give(Block& b) {
     int dev = 0;
     const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != b.device && cudaSetDevice(b.device) == cudaSuccess;
@@ -2150,7 +2169,7 @@ int qcalib_collect(const float* d_x, size_t count, int nbins, float range_hi, qc
   if (!d.landing) CUDA_TRY(cudaHostAlloc(&d.landing, sizeof(qc::CalibResult), cudaHostAllocPortable));
   if (!d.scratch) {
     qc::CalibScratch* sc = nullptr;
-    CUDA_TRY(cudaMalloc(&sc, sizeof(qc::CalibScratch)));
+    CUDA_TRY(DevicePool::pool().plain(&sc, sizeof(qc::CalibScratch)));
     const cudaError_t e = cudaMemset(sc, 0, sizeof(qc::CalibScratch));
     if (e != cudaSuccess) {
       cudaFree(sc);
@@ -2465,7 +2484,7 @@ int qconv_np_create(qconv_np_handle** out, const qconv_np_desc* desc, const uint
   if (rc) { free_np(h); return rc; }
   h->c_pad = h->gemm->a_channels / spec.planes;
   const size_t bytes = static_cast<size_t>(d.N) * d.H * d.W * h->gemm->a_channels;
-  cudaError_t e = cudaMalloc(&h->d_planes, bytes);
+  cudaError_t e = DevicePool::pool().plain(&h->d_planes, bytes);
   if (e == cudaSuccess && h->c_pad != d.C) {
     // cleared once: the padding channels stay zero (waited for: the stream of the first run need not wait for this one)
     e = cudaMemsetAsync(h->d_planes, 0, bytes, nullptr);
@@ -2568,7 +2587,7 @@ int qthreshold_search(const uint64_t* hist_host, int nbins, float range_hi, int 
   if (!dv.pinned) CUDA_TRY(cudaHostAlloc(&dv.pinned, off_del + sizeof(qc::ThresholdBest), cudaHostAllocPortable));
   if (!dv.scratch) {
     unsigned char* sc = nullptr;
-    CUDA_TRY(cudaMalloc(&sc, off_ticket + sizeof(unsigned int)));
+    CUDA_TRY(DevicePool::pool().plain(&sc, off_ticket + sizeof(unsigned int)));
     cudaError_t me = cudaMemset(sc, 0, off_ticket + sizeof(unsigned int));
     if (me == cudaSuccess) me = cudaDeviceSynchronize();
     if (me != cudaSuccess) {
@@ -2634,8 +2653,8 @@ int qbench_mma_i8(int bn, int mmas_per_cta, int row_bytes, int commit_every, flo
   CUDA_TRY(cudaFuncSetAttribute(qc::mma_peak_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   unsigned long long* d_cycles = nullptr;
   int* d_status = nullptr;
-  CUDA_TRY(cudaMalloc(&d_cycles, sizeof(unsigned long long) * sms));
-  cudaError_t e = cudaMalloc(&d_status, sizeof(int));
+  CUDA_TRY(DevicePool::pool().plain(&d_cycles, sizeof(unsigned long long) * sms));
+  cudaError_t e = DevicePool::pool().plain(&d_status, sizeof(int));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaMemsetAsync(d_status, 0, sizeof(int), st);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
