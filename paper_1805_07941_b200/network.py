@@ -35,23 +35,27 @@ def _stages(nodes):
 _HANDLE = operator.attrgetter("handle")
 
 
-class _NetGraph:
+class _NetGraph(torch.cuda.CUDAGraph):
     """A captured pass whose input may be any buffer of the input's shape: `replay` reads the network's own x_static,
-    `replay_on` the given address (the graph's input kernels are pointed at it; nothing is copied)."""
+    `replay_on` the given address (the graph's input kernels are pointed at it; nothing is copied).  Made with
+    keep_graph=True, recorded, then given its inputs by `ready`."""
 
-    def __init__(self, graph, inputs):
-        self.graph, self.inputs = graph, inputs
-        self.exec = graph.raw_cuda_graph_exec()
-        self.own = self.at = inputs.x.data_ptr()
+    def ready(self, inputs):
+        self.inputs, self.own = inputs, inputs.x.data_ptr()
+        self.instantiate()
+
+    def instantiate(self):
+        super().instantiate()
+        self.at = self.own                                   # (a new executable graph reads what was recorded)
 
     def takes(self, address):
         return address == self.own or (self.inputs.found and (address ^ self.own) % 16 == 0)
 
     def replay_on(self, address):
         if address != self.at:
-            self.inputs.set(self.exec, address)
+            self.inputs.set(self.raw_cuda_graph_exec(), address)
             self.at = address
-        self.graph.replay()
+        super().replay()
 
     def replay(self):
         self.replay_on(self.own)
@@ -472,12 +476,12 @@ class QNetwork:
             fwd()                                       # warm-up outside capture: tensor maps get cached
         torch.cuda.current_stream().wait_stream(s)
         torch.cuda.synchronize()
-        g = torch.cuda.CUDAGraph(keep_graph=True)           # (its nodes are addressed later, to change the input)
+        g = _NetGraph(keep_graph=True)                      # (its nodes are addressed later, to change the input)
         with binding.GraphInputs(self.x_static) as inputs:
             with torch.cuda.graph(g):
                 fwd()
-        g.instantiate()
-        return _NetGraph(g, inputs)
+        g.ready(inputs)
+        return g
 
     def capture(self, how=None):
         """Record one pass over the full batch into a CUDA graph (launch overhead of the few dozen

@@ -51,6 +51,36 @@ def test_input_is_read_where_it_lies(name):
     qn.destroy()
 
 
+def test_a_capture_is_a_cuda_graph():
+    """What `capture` returns does all that torch's graph does; recorded work and a new executable read x_static."""
+    import torch
+    from paper_1805_07941_b200.network import QNetwork
+    net = NETS["rows"]()
+    w = {nd["name"]: wl.gen_weights(nd, 0) for nd in net["nodes"] if nd["op"] == "conv"}
+    xs = [wl.gen_input(net, seed=s) for s in range(2)]
+    params, e_buf, _, _ = network_ref.calibrate(net, xs[0], w)
+    want = [network_ref.run(net, x, params, e_buf)[next(reversed(net["nodes"]))["dst"]] for x in xs]
+    qn = QNetwork(net, w).load_params(params, e_buf)
+    g = qn.capture("chain")
+    assert isinstance(g, torch.cuda.CUDAGraph) and g is qn.graph and len(g.pool()) == 2
+    qn.x_static.copy_(torch.from_numpy(xs[0]))
+    other = torch.from_numpy(xs[1]).cuda()
+    for again in range(2):
+        assert (qn.run(other).cpu().numpy() == want[1]).all()
+        if again:
+            g.instantiate()
+        g.replay()
+        assert (qn.bufs[qn.last].cpu().numpy() == want[0]).all(), again
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        assert (qn.run(other).cpu().numpy() == want[1]).all()
+    g.reset()
+    with pytest.raises(RuntimeError):
+        g.replay()
+    qn.destroy()
+
+
 def test_step_list_reports_the_first_error():
     steps = binding.Steps([dict(op=binding.NET_MAXPOOL, n=1, H=4, W=4, C=16, R=2, stride=2, pad=0)])
     with pytest.raises(binding.QconvError) as e:
