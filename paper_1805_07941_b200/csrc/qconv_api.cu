@@ -10,9 +10,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <mutex>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -2813,20 +2813,19 @@ int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layo
     return QCONV_OK;
   }
   auto at = [&](int k, size_t j) { return j * K + k; };
-  float gall = 0.0f;
-  std::vector<float> gk(K, 0.0f);
-  for (int k = 0; k < K; ++k) {
+  auto largest = [&](int k) {
     float g = 0.0f;
     for (size_t j = 0; j < per_k; ++j) {
-      float a = std::fabs(w_host[at(k, j)]);
+      const float a = std::fabs(w_host[at(k, j)]);
       if (std::isfinite(a)) g = std::max(g, a);
     }
-    gk[k] = g;
-    gall = std::max(gall, g);
-  }
+    return g;
+  };
+  float gall = 0.0f;
+  for (int k = 0; k < K && !per_channel; ++k) gall = std::max(gall, largest(k));
   for (int k = 0; k < K; ++k) {
     int e;
-    qscale_exponent(per_channel ? gk[k] : gall, n, &e);
+    qscale_exponent(per_channel ? largest(k) : gall, n, &e);
     e_w_host[k] = e;
     for (size_t j = 0; j < per_k; ++j) wq_host[at(k, j)] = qc::host_quantize_one(w_host[at(k, j)], e, n);
   }
@@ -2835,7 +2834,7 @@ int qquantize_weights(const float* w_host, int K, int R, int S, int Cg, int layo
 
 // Layers are independent: the largest first over up to eight threads.  (The conversion reads 5 bytes per value from
 // memory twice; beyond eight threads the memory, not the arithmetic, sets the pace.)
-int qquantize_weights_list(const qweights_job* jobs, int count) {
+int qquantize_weights_list(const qweights_job* jobs, int count) try {
   if (!jobs || count < 0) return fail(QCONV_ERR_BAD_ARG, "NULL jobs or negative count");
   std::vector<int> order(count), rc(count, QCONV_OK);
   for (int i = 0; i < count; ++i) order[i] = i;
@@ -2853,15 +2852,18 @@ int qquantize_weights_list(const qweights_job* jobs, int count) {
   // (a thread costs some 20 us to start: worth it from about 2^18 values each)
   const int want = static_cast<int>(std::min<long long>({8, count, total >> 18, std::max(1u, std::thread::hardware_concurrency())}));
   std::vector<std::thread> threads;
+  threads.reserve(8);                                      // (nothing below may throw past a running thread)
   try {
     for (int t = 1; t < want; ++t) threads.emplace_back(work);
-  } catch (const std::system_error&) {                     // no more threads: the ones there are (this one at least) do it
+  } catch (const std::exception&) {                        // no more threads: the ones there are (this one at least) do it
   }
   work();
   for (std::thread& t : threads) t.join();
   for (int i = 0; i < count; ++i)
     if (rc[i]) return fail(rc[i], "weights %d: NULL argument or bad geometry", i);
   return QCONV_OK;
+} catch (const std::exception& ex) {
+  return fail(QCONV_ERR_BAD_ARG, "%d layers: %s", count, ex.what());
 }
 
 int qquantize_bias(const float* b_host, int K, int e_x, const int32_t* e_w_host, int32_t* bias_q_host) {

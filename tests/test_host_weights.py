@@ -1,5 +1,9 @@
 """Host weight conversion (vector form, several layers at once) against the oracle: counts around the vector width,
 values at the ends of the range, non-finite weights, exponents outside the vector form's range."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -36,3 +40,28 @@ def test_ties_go_to_even():
                  np.float32).reshape(1, 1, 1, 17)
     [(wq, e_w)] = binding.qquantize_weights_list([(w, 1, 1, 1, 17, 1)])
     assert e_w[0] == 0 and (wq.reshape(-1) == np.rint(w.reshape(-1)).astype(np.int8)).all()
+
+
+@pytest.mark.parametrize("n", [2, 8])
+@pytest.mark.parametrize("per_channel", [0, 1])
+def test_channels_last_equals_the_oracle(n, per_channel):
+    w = _weights(np.random.default_rng(n), (3, 2, 17, 40), 0.3)
+    wq, e_w = binding.qquantize_weights(w, 40, 3, 2, 17, layout=1, per_channel=per_channel, n=n)
+    wq_ref, e_ref = ref.quantize_weights(w, K=40, R=3, S=2, Cg=17, layout=1, per_channel=per_channel, n=n)
+    assert (e_w == e_ref).all() and (wq == wq_ref.reshape(wq.shape)).all()
+
+
+def test_a_list_that_host_memory_cannot_hold_is_an_error():
+    """The bookkeeping of 2^31 - 1 layers under a limit on the address space: an error code, not an exception through the C entry."""
+    script = """
+import resource
+from paper_1805_07941_b200 import binding
+jobs, lib = (binding.qweights_job * 1)(), binding.lib()
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (1 << 30), resource.RLIM_INFINITY))
+assert lib.qquantize_weights_list(jobs, 2**31 - 1) == binding.ERR_BAD_ARG, "code"
+assert b"2147483647 layers" in lib.qconv_last_error_string()
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    done = subprocess.run([sys.executable, "-c", script], cwd=root, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, (done.returncode, done.stderr[-2000:])
