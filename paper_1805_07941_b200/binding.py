@@ -341,8 +341,8 @@ class QConvNP:
         return lib().qconv_np_status(self.handle)
 
     def describe(self):
-        buf = ctypes.create_string_buffer(400)
-        _check(lib().qconv_np_describe(self.handle, buf, 400))
+        buf = ctypes.create_string_buffer(512)
+        _check(lib().qconv_np_describe(self.handle, buf, 512))
         return buf.value.decode()
 
     def destroy(self):

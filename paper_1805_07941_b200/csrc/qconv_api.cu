@@ -232,6 +232,7 @@ struct qconv_handle {
   long long acc_bound = 0;       // worst-case |accumulator| (Eq. 9 / Eq. 13 bound)
   int max_shift = 0;
   long walk_grid = -1;             // grid size the tile-walk constants in prm were made for
+  int split = 1;                   // CTAs that shared a tile's contraction in the last run
   int gen_flt = 0;               // 1: the same bound with the rounding mode's half: float rounding in the general epilogue
   int flt_epilogue = 0;          // 1: |wide value| < 2^22 for any input (weight-aware bound): float-rounding epilogue
   int uniform_shift = 0;         // 1: all channels share the right shift and the residual left shift
@@ -1874,6 +1875,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
     const long tiles = static_cast<long>(p.tiles_q) * p.tiles_p * p.tiles_n * p.tiles_k;
     if (tiles <= 0 || tiles > 2147483647l) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "tile count out of range");
     const int ksplit = maxabs ? 1 : choose_ksplit(h, tiles);
+    h->split = ksplit;
     if (ksplit > 1) {
       qc::IgemmParams q = h->prm;
       const int num_kb = p.R * p.S * p.nchunks, own = p.BN / 16 / ksplit;
@@ -2089,6 +2091,8 @@ int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len) {
              h->dw_mma ? "depthwise3x3/mma" : "igemm", names[h->mode], p.tq, p.tp, p.tn, p.BN, p.tiles_k, p.BKC, p.nchunks, p.R, p.S, p.stages,
              h->smem_bytes, h->ctas_per_sm, p.fast_epilogue, h->uniform_shift, h->flt_epilogue && p.fast_epilogue, h->fold,
              p.out_stage_bytes ? p.out_stage_bufs : 0, p.b_resident, p.tap_boxes || h->patch ? 0 : p.halo_s, p.tap_boxes ? p.halo_s : 0, h->pair, h->d.pool, h->patch ? " patch=1" : "");
+    const size_t used = std::strlen(buf);
+    if (h->split > 1) snprintf(buf + used, buf_len - used, " split=%d", h->split);
   } else {
     snprintf(buf, buf_len, "%s", h->algo == QCONV_ALGO_DEPTHWISE ? (h->dw_tma ? "depthwise3x3/tap-packed+tma" : h->dw_tap ? "depthwise3x3/tap-packed" : "depthwise3x3/dp4a")
                                                                   : "direct");
@@ -2517,7 +2521,7 @@ int qconv_np_status(qconv_np_handle* h) {
 
 int qconv_np_describe(const qconv_np_handle* h, char* buf, size_t buf_len) {
   if (!h || !buf || buf_len == 0) return fail(QCONV_ERR_BAD_ARG, "NULL argument");
-  char inner[256];
+  char inner[400];
   qconv_describe(h->gemm, inner, sizeof(inner));
   snprintf(buf, buf_len, "np digits_x=%d digits_w=%d products=%d | %s", h->digits_x, h->digits_w, h->gemm->np_products, inner);
   return QCONV_OK;

@@ -11,7 +11,10 @@ pytestmark = pytest.mark.gpu
 CASES = [  # N, n_run, H, W, C, K, R, stride
     (1, 1, 7, 7, 512, 512, 3, 1), (1, 1, 7, 7, 2048, 512, 1, 1), (2, 1, 14, 14, 256, 256, 3, 1), (1, 1, 14, 14, 1024, 256, 1, 1),
     (1, 1, 9, 5, 640, 80, 1, 1), (1, 1, 14, 14, 512, 1024, 1, 2), (3, 2, 5, 5, 256, 48, 5, 1), (1, 1, 3, 3, 896, 208, 3, 2),
-    (64, 33, 1, 1, 2048, 1008, 1, 1), (1, 1, 28, 28, 128, 128, 3, 1)]
+    (64, 33, 1, 1, 2048, 1008, 1, 1), (1, 1, 28, 28, 128, 128, 3, 1), (1, 1, 40, 30, 1152, 128, 1, 1)]
+# CTAs that share a tile, forced to 2 and 4 and as the launch chooses: 1 where the column groups (3 of them) or the stages (3)
+# do not divide, or where the clusters would fill the chip.
+SPLITS = dict(zip(CASES, [(2, 4, 4), (2, 4, 4), (2, 4, 4), (2, 4, 4), (1, 1, 1), (2, 4, 1), (1, 1, 1), (2, 4, 4), (2, 4, 4), (2, 1, 1), (2, 4, 2)]))
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -43,6 +46,8 @@ def test_split_contraction_matches_the_oracle(case, split):
                 for _ in range(2):
                     conv.run(torch.from_numpy(x).cuda(), y, rd, n_run=n_run)
                 assert conv.status() == 0, conv.describe()
+                ran = dict(zip((2, 4, -1, 0), SPLITS[case] + (1,)))[split]
+                assert ("split=%d" % ran in conv.describe()) if ran > 1 else ("split=" not in conv.describe()), conv.describe()
                 got = y.cpu().numpy()
                 assert (got[:n_run] == want).all() and (got[n_run:] == 77).all(), (conv.describe(), with_res, uniform, small)
                 conv.destroy()
@@ -62,7 +67,7 @@ def test_expired_waits_leave_the_cluster_together():
     y = torch.empty((1, 7, 7, 128), dtype=torch.int8, device="cuda")
     conv.set_wait_limit(0)
     conv.run(xd, y)
-    assert conv.status() == binding.ERR_TIMEOUT
+    assert conv.status() == binding.ERR_TIMEOUT and "split=4" in conv.describe()
     conv.set_wait_limit(1 << 22)
     conv.run(xd, y)
     assert conv.status() == 0
