@@ -266,7 +266,7 @@ int qdequantize_np(const uint8_t* d_code, size_t count, int e, int n, int p, flo
  * Supported types: beta_max below 2^21 (three digit planes: every 8-bit type with p >= 3, all narrower
  * ones with at most 4 exponent bits); C a multiple of 16.  Errors: BAD_ARG, UNSUPPORTED_SHAPE, BAD_SHIFT,
  * OVERFLOW_RISK when R*S*C * beta_max_in * beta_max_w + max|bias| >= 2^62 (Eq. 9 with b = beta_max), CUDA.
- * The handle owns its scratch (digit planes of the input, int32 partial sums); one stream at a time. */
+ * The handle owns its scratch (digit planes of the input); one stream at a time. */
 typedef struct {
   int N, H, W, C, K, R, S;
   int stride_h, stride_w, pad_h, pad_w;

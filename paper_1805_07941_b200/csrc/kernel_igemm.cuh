@@ -56,7 +56,8 @@ struct IgemmParams {
                                    //    2 x 2 max-pool is taken in the epilogue (tile rows q fastest: lane ^ 1 is the horizontal
                                    //    neighbour, lane ^ tq the vertical one)
   int q_step;                      // pixels from one box to the next along q, and the box's columns that are outputs:
-                                   //    tq, except in the halo form (tq - 2: the halo's two accumulator columns are dropped)
+                                   //    tq, except in the halo form (tq - (S - 1): the accumulator columns of the halo are dropped)
+                                   //    and in the patch form (up to 14 of the box's 16)
   int tiles_q, tiles_p, tiles_n;   // number of boxes along each output axis
   int tiles_k;                     // number of output-channel tiles
   int BN;                          // channels per tile = MMA N (multiple of 16, <= 256)

@@ -2,7 +2,8 @@
 // tensor-core GEMM.  The betas of an (n, p) type are integers up to beta_max (Eq. 5: 1984 for (8, 4),
 // 245760 for (8, 3)), so the sum of Eq. 6 is an exact integer sum -- but its terms do not fit the int8
 // operands of the MMA.  Each beta is therefore written in base 128 with balanced digits,
-//   beta = d_0 + 128 d_1 + 128^2 d_2,   d_0, d_1 in [-64, 63], the last digit whatever is left (<= 127),
+//   beta = d_0 + 128 d_1 + 128^2 d_2,   d_0, d_1 in [-64, 63], the last digit whatever is left (up to 127 of a one-digit type; of the
+// types with two and three digits at most 16, so that a sum of any two digits fits an int8),
 // and the product of two betas is taken from products of single digits and of sums of two digits (Karatsuba; see
 // np_products in qconv_api.cu).  The kernel below writes the digit combinations of the input that these products need
 // as planes side by side along the channel axis.  One tensor-core layer (igemm_i8_kernel<EPI_NP>) then accumulates every

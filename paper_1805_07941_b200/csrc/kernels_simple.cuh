@@ -92,14 +92,9 @@ maxpool_i8_vec_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, int 
   }
 }
 
-// Strip form for the common windows (3x3 stride 1 or 2, 2x2 stride 2): one thread owns 16 channels
-// of one output column and walks down a strip of output rows.  The horizontal maximum of an input
-// row is taken once and kept in registers for every output row whose window contains it, so a
-// 3x3 stride-1 pool loads 3 vectors per output instead of 9.  The maxima are taken on pairs of
-// 16-bit lanes with the byte on top (the two-lane integer max the hardware has; a four-lane byte
-// max would be emulated) and the top bytes are put together at the end.
-// Depthwise weights [9][C] as the tensor-core form wants them, [rows][9][32] (rows past C are zero) with the weight at position c % 32 and zeros
-// beside it: 16 bytes a thread.  (Made here: the table is 32 times what has to be copied to the device.)
+// Depthwise weights [9][C] as the tensor-core form wants them, [rows][9][32] (rows past C are zero) with the weight at
+// position c % 32 and zeros beside it: 16 bytes a thread.  (Made here: the table is 32 times what has to be copied to the
+// device.)
 __global__ void __launch_bounds__(256)
 depthwise_blocks_kernel(const int8_t* __restrict__ w, uint4* __restrict__ out, int C, int rows) {
   const int i = blockIdx.x * 256 + threadIdx.x;
@@ -112,6 +107,12 @@ depthwise_blocks_kernel(const int8_t* __restrict__ w, uint4* __restrict__ out, i
   out[i] = make_uint4(v[0], v[1], v[2], v[3]);
 }
 
+// Strip form for the common windows (3x3 stride 1 or 2, 2x2 stride 2): one thread owns 16 channels
+// of one output column and walks down a strip of output rows.  The horizontal maximum of an input
+// row is taken once and kept in registers for every output row whose window contains it, so a
+// 3x3 stride-1 pool loads 3 vectors per output instead of 9.  The maxima are taken on pairs of
+// 16-bit lanes with the byte on top (the two-lane integer max the hardware has; a four-lane byte
+// max would be emulated) and the top bytes are put together at the end.
 struct PoolRow { uint32_t w[8]; };            // 16 channels as 8 words of two 16-bit lanes: bytes 0 and 2 of a word, then 1 and 3
 
 // A word's bytes as 16-bit lanes with the byte on top: the even ones shifted there, the odd ones where they are.  What lies

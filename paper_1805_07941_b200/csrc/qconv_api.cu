@@ -786,9 +786,10 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   }
   if (!halo && !patch && !dw && !is_window_mode(h->mode) && hint.ctas_per_sm == 0 && taps_r * taps_s * p.nchunks >= 9) {
     // Tiles that all run at once, one per SM, as chains of stages: a chain is as fast as its ring is deep (four stages cover
-    // half of the latency of a load), so such a layer's CTAs get the whole shared memory.  Drawn layers of 2 to 128 tiles
-    // and 9 to 175 stages: 0 to 25 % faster, 9 % on average; from 150 tiles on they no longer run at once (1.2 to 1.5
-    // times slower), and with fewer stages the next kernel's set-up beside them is worth more.
+    // half of the latency of a load), so such a layer's CTAs get the whole shared memory.  Random layers
+    // (1 x 1 to 5 x 5 filters, 16 to 1024 channels, 7 to 112 pixels a side) of 2 to 128 tiles and 9 to 175 stages: 0 to
+    // 25 % faster, 9 % on average; from 150 tiles on they no longer run at once (1.2 to 1.5 times slower), and with fewer
+    // stages the next kernel's set-up beside them is worth more.
     int tq, tp, tn;
     choose_box(h->Q, h->P, d.N, &tq, &tp, &tn, d.pool != 0);
     const long m_tiles = h->mode == MODE_FLAT || h->mode == MODE_STEM ? ceil_div_l(static_cast<long>(d.N) * h->P * h->Q / h->fold, 128)
@@ -2377,6 +2378,16 @@ int np_host_decode(int code, int n, int p) {
   }
   return ((code >> (n - 1)) & 1) ? -v : v;
 }
+// Sum of those of beta's balanced digits that the mask names.
+int np_digit_sum(int beta, int digits, int mask) {
+  int sum = 0;
+  for (int j = 0; j < digits; ++j) {
+    const int dig = j + 1 < digits ? ((beta + 64) & 127) - 64 : beta;
+    beta = (beta - dig) >> 7;
+    if ((mask >> j) & 1) sum += dig;
+  }
+  return sum;
+}
 void free_np(qconv_np_handle* h) {
   if (!h) return;
   if (h->gemm) free_handle(h->gemm);
@@ -2388,7 +2399,7 @@ void free_np(qconv_np_handle* h) {
 // (Karatsuba): with P_S = (sum of x_i, i in S) (sum of w_i, i in S) over single digits and pairs,
 //   x_i w_j + x_j w_i = P_ij - P_ii - P_jj,
 // three products for two digits and six for three, where the digit-by-digit schoolbook form takes four and nine.  The
-// balanced digits (-64 ... 63, the last one at most 31) leave room for a sum of two in an int8.  Operands of different
+// balanced digits (-64 ... 63; where there are several, the last one is at most 16) leave room for a sum of two in an int8.  Operands of different
 // lengths are padded with zero digits, and products with a zero factor drop out.
 struct NpProduct { int mask; long long coef; };
 std::vector<NpProduct> np_products(int digits_x, int digits_w) {
@@ -2468,11 +2479,11 @@ int qconv_np_create(qconv_np_handle** out, const qconv_np_desc* desc, const uint
     // one table of 256 patterns per product instead of decoding every weight
     int8_t table[256];
     for (int c = 0; c < 256; ++c) {
-      int beta = np_host_decode(c, d.n_w, d.p_w), sum = 0;
-      for (int j = 0; j < pw; ++j) {
-        const int dig = j + 1 < pw ? ((beta + 64) & 127) - 64 : beta;
-        beta = (beta - dig) >> 7;
-        if ((w_mask >> j) & 1) sum += dig;
+      const int sum = np_digit_sum(np_host_decode(c, d.n_w, d.p_w), pw, w_mask);
+      const int sum_x = np_digit_sum(np_host_decode(c, d.n_in, d.p_in), px, x_mask);
+      if (std::min(sum, sum_x) < -128 || std::max(sum, sum_x) > 127) {        // (no type that np_planes lets through)
+        free_np(h);
+        return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: a sum of digits does not fit an int8");
       }
       table[c] = static_cast<int8_t>(sum);
     }
