@@ -206,7 +206,7 @@ def calib_call(elems, warmup, reps):
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s",
                          "frac": gbs / pk["hbm_gbs"], "frac_of_nominal_8000": gbs / NOMINAL_HBM_GBS,
                          "bytes": "8 per element: two passes of 4 (maximum, then histogram on [0, maximum])"},
-            "note": "whole call: clear, two passes, finalize kernel, two device-to-host copies and the sync",
+            "note": "whole call: two passes, results written to pinned host memory, and the sync",
             "threshold_search": {"gamma": gamma, "delta": delta, "nbins": 2048, "measure": "l1",
                                  "ms_host_to_host": float(np.median(thr[max(1, warmup):]))}}
 
