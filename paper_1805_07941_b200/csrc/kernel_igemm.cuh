@@ -81,7 +81,8 @@ struct IgemmParams {
   uint32_t a_stage_bytes, b_stage_bytes;   // shared-memory footprint per stage (1024-aligned)
   uint32_t out_stage_bytes;        // fast int8 epilogues: one staged output tile (128 rows of BN bytes, 1024-aligned); 0: direct stores
   uint32_t out_swz_mask;           // 16-byte-chunk XOR mask of the staged tile's swizzle (7 / 3 / 1 / 0 for BN = 128 / 64 / 32 / other)
-  int out_stage_bufs;              // staged tiles: 2, or 3 when the residual tile is fetched into them by TMA one tile ahead
+  int out_stage_bufs;              // staged tiles: 2, or 3 when the residual tile is fetched into them by TMA one tile ahead; 0 with
+                                   //    out_stage_bytes set: every CTA has one tile, and stages it in the ring, which is idle by then
   uint32_t res_tx_bytes;           // bytes one residual box delivers (BN * tq * tp * tn)
   uint32_t tx_bytes;               // bytes the TMA boxes of one ring stage deliver (activations + weights, or activations alone)
   int halo_s;                      // 0, or S: one activation stage is a box with a horizontal halo (tq = W + S - 1 pixels
@@ -204,8 +205,6 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // ... all but the most recent one.
 __device__ __forceinline__ void bulk_wait_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-// All of this thread's bulk stores are complete.
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Generic-proxy writes to shared memory become visible to the async proxy (TMA).
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void sts_uint4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
@@ -495,13 +494,12 @@ __device__ __forceinline__ int4 lds_int4(uint32_t addr) {
   return v;
 }
 
-// 16 accumulator columns of one row -> 16 output channels.  cst: shared-memory address of the
-// tile's first channel constant.
+// 16 accumulator columns of one row -> 16 output channels, stored by the thread (epilogue_16).  cst: shared-memory
+// address of the tile's first channel constant.
 // RELU: 0 / 1 fixed at compile time (the float-rounding variants: one predicated instruction less per
 // output), 2 = taken from the parameters at run time.
-// RSTG: 2 in the kernel's template list stands for the pooled epilogue (epilogue_pool_16, never this function);
-// RSTG: 1 when the residual tile has been brought into the staged tile by TMA (read there, overwritten
-// in place by the result).
+// RSTG in the kernel's template list: 1 when the residual tile has been brought into the staged tile by TMA (read there,
+// overwritten in place by the result), 2 the pooled epilogue, 4 the split contraction, 5 depthwise.
 // The fast conversion of 16 accumulator columns to 16 int8 codes (four packed words): bias, residual << t, ReLU,
 // shift with nearest-even rounding, saturation.  cst_g: shared-memory address of the first column's constant;
 // rw: the 16 residual bytes (ignored without).
@@ -630,33 +628,17 @@ __device__ __forceinline__ void convert_16(const uint32_t* acc, uint32_t cst_g, 
   }
 }
 
-template <int EPI, int RELU, int RSTG>
-__device__ __forceinline__ void epilogue_16(const uint32_t (&acc)[16], uint32_t cst, int col, int k,
-                                            size_t pix, const IgemmParams& prm, const EpilogueParams& ep,
-                                            const uint4& res16, void* __restrict__ y, uint32_t stage_row) {
+template <int EPI, int RELU>
+__device__ __forceinline__ void epilogue_16(const uint32_t (&acc)[16], uint32_t cst, int col, int k, size_t pix,
+                                            const IgemmParams& prm, const EpilogueParams& ep, const uint4& res16,
+                                            void* __restrict__ y) {
   static_assert(EpiTraits<EPI>::fast, "16-byte-store variants; the others go through general_tile");
-  uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};           // residual bytes, fetched ahead
-  uint32_t stage_addr = 0;
-  if (prm.out_stage_bytes) {
-    // position of these 16 bytes in the staged tile (row-major, 16-byte chunks swizzled as the tensor
-    // maps of the output and the residual expect)
-    const uint32_t off = stage_row + static_cast<uint32_t>(col);
-    stage_addr = off ^ (((off >> 7) & prm.out_swz_mask) << 4);
-    if (EpiTraits<EPI>::res && RSTG == 1) {
-      // the residual tile was brought there by TMA; the result overwrites it in place
-      const int4 r4 = lds_int4(stage_addr);
-      rw[0] = r4.x; rw[1] = r4.y; rw[2] = r4.z; rw[3] = r4.w;
-    }
-  }
+  const uint32_t rw[4] = {res16.x, res16.y, res16.z, res16.w};     // residual bytes, fetched ahead
   uint32_t wds[4];
   const uint32_t cst_g = cst + static_cast<uint32_t>(col) * EpiTraits<EPI>::cst_bytes;
   convert_16<EPI, RELU>(acc, cst_g, load_ahead<EPI>(cst_g, 0), rw, ep, wds);
-  if (prm.out_stage_bytes) {
-    ptx::sts_uint4(stage_addr, wds[0], wds[1], wds[2], wds[3]);
-  } else {
-    *reinterpret_cast<uint4*>(static_cast<int8_t*>(y) + pix * prm.out_c_pitch + prm.out_c_offset + k) =
-        make_uint4(wds[0], wds[1], wds[2], wds[3]);
-  }
+  *reinterpret_cast<uint4*>(static_cast<int8_t*>(y) + pix * prm.out_c_pitch + prm.out_c_offset + k) =
+      make_uint4(wds[0], wds[1], wds[2], wds[3]);
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -1419,7 +1401,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     // the tile being stored, the tile being computed, the residual of the next).  The thread that issues
     // the stores also issues these loads: it alone knows when a buffer's store has finished reading.
     constexpr bool res_staged = EpiTraits<EPI>::res && EpiTraits<EPI>::fast && RSTG == 1;   // the planner then provides three staged tiles
-    const uint32_t stage0 = ptx::smem_u32(out_stage);
+    // (no staged tiles of their own: the CTA's one tile is staged in the ring)
+    const uint32_t stage0 = ptx::smem_u32(prm.out_stage_bufs == 0 ? tiles : out_stage);
     TileWalker walk_next = walk;
     int sbuf = 0;                              // staged buffer of the current tile
     uint32_t res_pending = 0;                  // bit i: a residual load into buffer i has not been consumed yet
@@ -1430,14 +1413,15 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       ptx::tma_load_4d(stage0, &tmap_r, ptx::smem_u32(&sh->res_full[0]), t0.k0, t0.q0, t0.p0, t0.n0);
       res_pending = 1u;
     }
-    // Lean form of a tile's epilogue, for the shapes the instruction-bound layers have: a staged tile 128 or 64
-    // channels wide, residual (if any) staged too.  Straight-line code: no pixel coordinates (the TMA store clips),
-    // no predicates around the column groups, the swizzled position of this thread's 16-byte chunks from
-    // per-thread constants.  (Chunk c of the staged row r sits at c ^ (r & 7) in a 128-byte row, at c ^ ((r >> 1) & 3)
-    // in a 64-byte row: the 16-byte chunk index XOR bits 7.. of the byte offset, masked to the row's chunks.)
-    constexpr bool kLeanOk = EpiTraits<EPI>::fast && !kPool && GPW == kGroupsPerWarp && (!EpiTraits<EPI>::res || RSTG == 1);
-    const bool lean = kLeanOk && prm.out_stage_bytes != 0 && (prm.BN == 128 || prm.BN == 64);
-    const uint32_t lean_col0 = ew < 4 ? 0u : static_cast<uint32_t>(prm.BN) / 2u;          // this warp's half of the columns
+    // Lean form of a tile's epilogue, for staged tiles: no pixel coordinates (the TMA store clips), no predicates beyond
+    // the warp's number of column groups, the swizzled position of this thread's 16-byte chunks from per-thread constants.
+    // (Chunk c of the staged row r sits at c ^ (r & 7) in a 128-byte row, at c ^ ((r >> 1) & 3) in a 64-byte row: the
+    // 16-byte chunk index XOR bits 7.. of the byte offset, masked to the row's chunks; tiles of other widths are not
+    // swizzled.)  A residual is staged too, or comes in registers.
+    constexpr bool kLeanOk = EpiTraits<EPI>::fast && !kPool && !kSplit && GPW == kGroupsPerWarp;
+    const bool lean = kLeanOk && prm.out_stage_bytes != 0;
+    const int lean_groups = g_end - g_begin;
+    const uint32_t lean_col0 = static_cast<uint32_t>(g_begin) * 16u;
     uint32_t lean_off[4];
     {
       const uint32_t row_off = static_cast<uint32_t>(row) * static_cast<uint32_t>(prm.BN);
@@ -1477,7 +1461,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       }
       bool row_ok = true;
       size_t pix = 0, pooled_pix = 0;
-      if (!lean) {
+      if (!lean || (EpiTraits<EPI>::res && !res_staged)) {
         const int q = tc.q0 + q_i, p = tc.p0 + p_i, n = tc.n0 + n_i;
         row_ok = (n_i < prm.tn) && q_i < prm.q_step && q < prm.Q && p < prm.P && n < prm.Nimg;
         pix = (static_cast<size_t>(n) * prm.P + p) * prm.Q + q;
@@ -1558,7 +1542,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
                   acc[4 * c] += v.x; acc[4 * c + 1] += v.y; acc[4 * c + 2] += v.z; acc[4 * c + 3] += v.w;
                 }
               }
-              if (row_ok) epilogue_16<EPI, RELU, 0>(acc, chan, g * 16, tc.k0 + g * 16, pix, prm, ep, rres[i], y, 0u);
+              if (row_ok) epilogue_16<EPI, RELU>(acc, chan, g * 16, tc.k0 + g * 16, pix, prm, ep, rres[i], y);
             }
           }
         }
@@ -1586,7 +1570,6 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&sh->acc_empty[buf]));
         };
-        const uint32_t stage_row = stage_base + static_cast<uint32_t>(row * prm.BN);
         uint32_t acc_a[16], acc_b[16];
         // general epilogues: group i of this warp; words leave group by group (64 bytes a row), bytes after the last
         [[maybe_unused]] auto gen_group = [&](const uint32_t (&acc)[16], int i) {
@@ -1659,34 +1642,51 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           auto group = [&](const uint32_t (&acc)[16], int i, const CstAhead<EPI>& ahead) {
             const uint32_t addr = stage_base + lean_off[i];
             uint32_t rw[4] = {0u, 0u, 0u, 0u}, wds[4];
-            if (EpiTraits<EPI>::res) {                       // the residual tile was brought there by TMA
+            if (res_staged) {                                // the residual tile was brought there by TMA
               const int4 r4 = lds_int4(addr);
               rw[0] = r4.x; rw[1] = r4.y; rw[2] = r4.z; rw[3] = r4.w;
+            } else if (EpiTraits<EPI>::res) {
+              rw[0] = rres[i].x; rw[1] = rres[i].y; rw[2] = rres[i].z; rw[3] = rres[i].w;
             }
             convert_16<EPI, RELU>(acc, c0 + static_cast<uint32_t>(i) * kGroupCst, ahead, rw, ep, wds);
             ptx::sts_uint4(addr, wds[0], wds[1], wds[2], wds[3]);
           };
-          ptx::tmem_ld_32x16(t0, acc_a);
-          CstAhead<EPI> k0 = load_ahead<EPI>(c0, 0);
-          ptx::tmem_ld_wait();
-          ptx::tmem_ld_32x16(t0 + 16, acc_b);
-          CstAhead<EPI> k1 = load_ahead<EPI>(c0 + kGroupCst, 0);
-          group(acc_a, 0, k0);
-          ptx::tmem_ld_wait();
-          if (prm.BN == 128) {
-            ptx::tmem_ld_32x16(t0 + 32, acc_a);
-            k0 = load_ahead<EPI>(c0 + 2 * kGroupCst, 0);
-            group(acc_b, 1, k1);
+          // (a warp has up to four groups; one of the second four warps has none where the tile is 16 wide)
+          if (lean_groups > 0) {
+            ptx::tmem_ld_32x16(t0, acc_a);
+            CstAhead<EPI> k0 = load_ahead<EPI>(c0, 0), k1 = k0;
             ptx::tmem_ld_wait();
-            ptx::tmem_ld_32x16(t0 + 48, acc_b);
-            k1 = load_ahead<EPI>(c0 + 3 * kGroupCst, 0);
-            group(acc_a, 2, k0);
-            ptx::tmem_ld_wait();
+            if (lean_groups > 1) {
+              ptx::tmem_ld_32x16(t0 + 16, acc_b);
+              k1 = load_ahead<EPI>(c0 + kGroupCst, 0);
+              group(acc_a, 0, k0);
+              ptx::tmem_ld_wait();
+              if (lean_groups > 2) {
+                ptx::tmem_ld_32x16(t0 + 32, acc_a);
+                k0 = load_ahead<EPI>(c0 + 2 * kGroupCst, 0);
+                group(acc_b, 1, k1);
+                ptx::tmem_ld_wait();
+                if (lean_groups > 3) {
+                  ptx::tmem_ld_32x16(t0 + 48, acc_b);
+                  k1 = load_ahead<EPI>(c0 + 3 * kGroupCst, 0);
+                  group(acc_a, 2, k0);
+                  ptx::tmem_ld_wait();
+                  release();
+                  group(acc_b, 3, k1);
+                } else {
+                  release();
+                  group(acc_a, 2, k0);
+                }
+              } else {
+                release();
+                group(acc_b, 1, k1);
+              }
+            } else {
+              release();
+              group(acc_a, 0, k0);
+            }
+          } else {
             release();
-            group(acc_b, 3, k1);
-          } else {                                            // 64 wide: two groups per warp
-            release();
-            group(acc_b, 1, k1);
           }
         } else {
         if (g_begin < g_end) {
@@ -1704,7 +1704,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             } else if constexpr (!EpiTraits<EPI>::fast) {
               gen_group(acc_a, i);
             } else if (row_ok && tc.k0 + g0 * 16 < prm.K)
-              epilogue_16<EPI, RELU, RSTG>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, prm, ep, rres[i & (kGroupsPerWarp - 1)], y, stage_row);
+              epilogue_16<EPI, RELU>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, prm, ep, rres[i & (kGroupsPerWarp - 1)], y);
             if (g1 < g_end) {
               ptx::tmem_ld_wait();
               if (g2 < g_end && i + 2 < GPW) ptx::tmem_ld_32x16(t_addr + g2 * 16, acc_a); else release();
@@ -1714,7 +1714,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
               } else if constexpr (!EpiTraits<EPI>::fast) {
                 gen_group(acc_b, i + 1);
               } else if (row_ok && tc.k0 + g1 * 16 < prm.K)
-                epilogue_16<EPI, RELU, RSTG>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, prm, ep, rres[(i + 1) & (kGroupsPerWarp - 1)], y, stage_row);
+                epilogue_16<EPI, RELU>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, prm, ep, rres[(i + 1) & (kGroupsPerWarp - 1)], y);
               if (g2 < g_end && i + 2 < GPW) ptx::tmem_ld_wait();
             }
           }
@@ -1754,7 +1754,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       flush_maxabs(gen_max, y);
     }
     if (EpiTraits<EPI>::fast && prm.out_stage_bytes && etid == 0) {
-      ptx::bulk_wait_all();
+      // (read, not complete: the grid's completion covers the writes, and whoever depends on them waits for that)
+      ptx::bulk_wait_read_all();
       // after an early exit residual tiles may still be on their way into this CTA's shared memory:
       // let them land (bounded) before the CTA retires
       if (res_staged) {

@@ -307,7 +307,7 @@ igemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             if (tc.k0 + g0 * 16 < prm.K)
               epilogue_pool_16<EPI, RELU>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pooled_pix, row_ok, lane, eprm.pool_bit, eprm, ep, y);
           } else if (row_ok && tc.k0 + g0 * 16 < prm.K)
-            epilogue_16<EPI, RELU, 0>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, eprm, ep, no_res, y, 0u);
+            epilogue_16<EPI, RELU>(acc_a, chan, g0 * 16, tc.k0 + g0 * 16, pix, eprm, ep, no_res, y);
           if (g1 < g_end) {
             ptx::tmem_ld_wait();
             if (g2 < g_end && i + 2 < kGroupsPerWarpWide) ptx::tmem_ld_32x16(t_addr + g2 * 16, acc_a); else release();
@@ -315,7 +315,7 @@ igemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
               if (tc.k0 + g1 * 16 < prm.K)
                 epilogue_pool_16<EPI, RELU>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pooled_pix, row_ok, lane, eprm.pool_bit, eprm, ep, y);
             } else if (row_ok && tc.k0 + g1 * 16 < prm.K)
-              epilogue_16<EPI, RELU, 0>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, eprm, ep, no_res, y, 0u);
+              epilogue_16<EPI, RELU>(acc_b, chan, g1 * 16, tc.k0 + g1 * 16, pix, eprm, ep, no_res, y);
             if (g2 < g_end && i + 2 < kGroupsPerWarpWide) ptx::tmem_ld_wait();
           }
         }

@@ -244,6 +244,9 @@ struct qconv_handle {
   int8_t* d_w_mma = nullptr;     // its weights: [C][9][32]
   uint32_t* d_dw_tap = nullptr;  // tap-packed form: weight rows [3][C], bias + magic [C], 2^-s [C], rounding offset [C] (float bits)
   int dw_tap = 0;
+  uint32_t plan_stage_bytes = 0; // staged output tiles as planned; a run may do without or use the ring (plan_staging)
+  int plan_stage_bufs = 0;
+  bool ring_out_fits = false;    // no staged tiles in the plan, but a CTA with one tile may stage it in its ring
   int patch = 0;                 // 1: patch form (one activation box of 16 x (tp + 2) pixels serves all nine taps)
   int pair = 0;                  // 1: tiles of 256 pixels x 256 channels on pairs of SMs (kernel_igemm_pair.cuh)
   int fold = 1;                  // flat GEMMs with few output channels: this many pixels form one GEMM row
@@ -862,7 +865,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
       }
     }
     if (!placed || !p.fast_epilogue) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "internal: the patch form does not fit");
-    p.store_rows = p.out_stage_bytes ? pt.tp : 0;
+    p.store_rows = may_stage ? pt.tp : 0;
   }
   const int staged_tiles = p.out_stage_bytes ? p.out_stage_bufs : 0;
   h->kg_total = all_taps * p.nchunks * b_row;
@@ -907,6 +910,11 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     }
   }
   p.stages = stages;
+  h->ring_out_fits = p.fast_epilogue && !p.out_stage_bytes && hint.tma_store != 0 && (p.BN == 128 || (p.BN == 64 && h->ctas_per_sm == 2)) && !h->pair && !d.pool &&
+                     !(halo && halo_segs > 1) && !(patch && d.has_residual) &&
+                     static_cast<size_t>(stages) * (p.a_stage_bytes + (p.b_resident ? 0 : p.b_stage_bytes)) >= static_cast<size_t>(out_tile);
+  h->plan_stage_bytes = p.out_stage_bytes;
+  h->plan_stage_bufs = p.out_stage_bufs;
   h->smem_bytes = 1024 + static_cast<size_t>(stages) * (p.a_stage_bytes + (p.b_resident ? 0 : p.b_stage_bytes)) +
                   (p.b_resident ? static_cast<size_t>(num_kb_plan) * p.b_stage_bytes : 0) +
                   static_cast<size_t>(staged_tiles) * p.out_stage_bytes + p.gen_stage_bytes + sizeof(qc::IgemmShared);
@@ -1274,6 +1282,29 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
   h->a_key_ptr = a_ptr;
   h->a_key_n = n_run;
   return QCONV_OK;
+}
+
+// How this run's output tiles leave (fast epilogues).  As planned, beside the ring; or, where the plan has no room for that (long
+// contractions) and every CTA has one tile, staged in the ring, which is idle once the accumulators are complete: staged tiles
+// take the lean epilogue and leave by TMA in whole rows, where 32 lanes storing 16 bytes of 32 rows each touch 32 half sectors per
+// instruction (32 x 28 x 28 x 512 -> 128, 1 x 1: 6.05 -> 5.8 us; 128 x 14 x 14 x 512 -> 128 6.1 -> 5.8).  Up to a third of the SMs'
+// worth of tiles is stored by the threads themselves whatever the plan: there it is the chain of one tile that counts, and
+// barrier, TMA store and its wait lengthen it (us per launch, staged / direct: 14 tiles of 28 x 28 x 512 -> 128, 1 x 1 3.1 / 2.9; 32
+// of 7 x 7 x 512 -> 2048 with residual 3.4 / 3.15; 56 of 28 x 28 x 128 -> 512 2.7 / 2.8; 100 of 56 x 56 x 64 -> 256 2.85 / 3.06;
+// ResNet-50 on one image 195.2 -> 191.7).
+void plan_staging(qconv_handle* h, long tiles) {
+  qc::IgemmParams& p = h->prm;
+  if (!p.fast_epilogue) return;
+  uint32_t bytes = h->plan_stage_bytes;
+  int bufs = h->plan_stage_bufs;
+  if (!bytes && h->ring_out_fits && tiles <= static_cast<long>(h->num_sms) * h->ctas_per_sm) {
+    bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(qc::kTileM) * p.BN, 1024));
+    bufs = 0;
+  }
+  if (tiles * 3 <= h->num_sms && h->hints.tma_store != 1) bytes = 0;
+  if (bytes != p.out_stage_bytes) h->y_key_ptr = h->r_key_ptr = nullptr;
+  p.out_stage_bytes = bytes;
+  p.out_stage_bufs = bufs;
 }
 
 // Output tensor map for the TMA stores of the fast epilogues: the same pixel boxes as the accumulator
@@ -1831,7 +1862,11 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
       h->prm.gen_vec_y = widest(reinterpret_cast<uintptr_t>(d_y) | es * d.out_c_pitch | es * d.out_c_offset | es * d.K);
       h->prm.gen_vec_res = widest(reinterpret_cast<uintptr_t>(d_residual) | static_cast<uintptr_t>(d.K));
     }
-    if (h->prm.out_stage_bytes) {
+    const long tiles = static_cast<long>(h->prm.tiles_q) * h->prm.tiles_p * h->prm.tiles_n * h->prm.tiles_k;
+    const int ksplit = maxabs || h->pair || tiles <= 0 ? 1 : choose_ksplit(h, tiles);
+    h->split = ksplit;
+    if (ksplit == 1) plan_staging(h, tiles);
+    if (h->prm.out_stage_bytes && ksplit == 1) {
       rc = prepare_y_map(h, d_y, n_run);
       if (rc) return rc;
       if (d.has_residual && h->prm.out_stage_bufs == 3) {
@@ -1873,10 +1908,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
       if (le != cudaSuccess) return fail(QCONV_ERR_CUDA, "kernel launch (SM pairs): %s", cudaGetErrorString(le));
       return QCONV_OK;
     }
-    const long tiles = static_cast<long>(p.tiles_q) * p.tiles_p * p.tiles_n * p.tiles_k;
     if (tiles <= 0 || tiles > 2147483647l) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "tile count out of range");
-    const int ksplit = maxabs ? 1 : choose_ksplit(h, tiles);
-    h->split = ksplit;
     if (ksplit > 1) {
       qc::IgemmParams q = h->prm;
       const int num_kb = p.R * p.S * p.nchunks, own = p.BN / 16 / ksplit;
