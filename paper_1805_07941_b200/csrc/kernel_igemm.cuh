@@ -114,6 +114,7 @@ struct IgemmParams {
   int np_coef[kNpMaxProducts];     // weight of its accumulator in the 64-bit sum
   int np_n, np_p;                  // output type
   float np_top;                    // its beta_max
+  int np_low;                      // EPI_NP3: low bits of the sum that the conversion keeps as one sticky bit, minus 7
 };
 
 // Error codes written to the status word.
@@ -428,6 +429,7 @@ struct TileWalker {
 //   GEN, GEN_RES: I8 where the wide value stays below 2^22 as well (see FLT below): any rounding mode by the rounding of the
 //                          fused multiply-add; GEN_RES also serves the mode that needs the sign (half away, no ReLU)
 //   NP: digit products of floating-point operands recombined in 64 bits and converted to the (n, p) output type
+//   NP3: the three products of two-digit operands, recombined and converted in 32 bits (np3_encode)
 //   FAST_I8_U / FAST_I8_RES_U: the same with one shift for all channels (per-layer scales): only the
 //                          bias is per channel, everything else sits in kernel parameters
 //   FLT_I8*:               the four fast variants again for layers whose wide value provably stays below
@@ -440,7 +442,7 @@ struct TileWalker {
 //                          on the bit patterns (positive floats order like integers).
 enum : int { EPI_FAST_I8 = 0, EPI_FAST_I8_RES = 1, EPI_I8 = 2, EPI_I32 = 3, EPI_F32 = 4, EPI_FAST_I8_U = 5,
              EPI_FAST_I8_RES_U = 6, EPI_FLT_I8 = 7, EPI_FLT_I8_RES = 8, EPI_FLT_I8_U = 9, EPI_FLT_I8_RES_U = 10,
-             EPI_MAX = 11, EPI_NP = 12, EPI_GEN = 13, EPI_GEN_RES = 14 };
+             EPI_MAX = 11, EPI_NP = 12, EPI_GEN = 13, EPI_GEN_RES = 14, EPI_NP3 = 15 };
 
 template <int EPI> struct EpiTraits {
   static constexpr bool flt = EPI >= EPI_FLT_I8 && EPI <= EPI_FLT_I8_RES_U;
@@ -452,7 +454,8 @@ template <int EPI> struct EpiTraits {
                               EPI == EPI_FLT_I8_RES_U;
   // shared-memory form of the channel constants: 4 bytes a channel when only the biases differ; for the float rounding
   // without residual 8, two channels side by side as {bias, bias, 2^-s, 2^-s}; else the table's 16
-  static constexpr bool paired = EPI == EPI_FLT_I8 || EPI == EPI_GEN || EPI == EPI_I8 || EPI == EPI_I32 || EPI == EPI_F32 || EPI == EPI_MAX;
+  static constexpr bool paired = EPI == EPI_FLT_I8 || EPI == EPI_GEN || EPI == EPI_I8 || EPI == EPI_I32 || EPI == EPI_F32 || EPI == EPI_MAX || EPI == EPI_NP3;
+  static constexpr bool np = EPI == EPI_NP || EPI == EPI_NP3;
   static constexpr bool gen = EPI == EPI_GEN || EPI == EPI_GEN_RES, bytes = EPI == EPI_I8 || gen;   // general int8
   static constexpr uint32_t cst_bytes = uni ? 4u : paired ? 8u : 16u;
 };
@@ -843,6 +846,37 @@ __device__ __forceinline__ uint32_t np_encode(long long v, int s, const NpEncode
   return code | ((v < 0 && code) ? 1u << f.sign_bit : 0u);
 }
 
+// The same for the three products of two-digit operands, without 64-bit arithmetic.  The sum is
+//   v = P0 + bias + 128 (P01 - P0 - P1) + 128^2 P1 = a + 128 h  with a = P0 + bias, h = P01 - P0 + 127 P1,
+// both int32.  The shift s leaves every number that the conversion compares with (grid points and their midpoints) a multiple of
+// 2^(s-1); so of v's low np_low + 7 <= s - 1 bits only whether they are zero matters: u = 2 floor(v / 2^(np_low+7)) + sticky, below
+// 2^23 in magnitude (the host chose np_low so), is an exact binary32 number, and u 2^(np_low+6-s) lies between the same
+// neighbours as v / 2^s.  scale: 2^(np_low+6-s).  23 instructions an output; with 64-bit sums 45.
+struct Np3Encode {
+  uint32_t ke_min, ke_up, ke_off, low_mask;
+  int low, p, sign_bit;
+  float top;
+};
+template <bool RELU>
+__device__ __forceinline__ uint32_t np3_encode(int32_t p0, int32_t p1, int32_t p01, int32_t bias, float scale, const Np3Encode& f) {
+  const int32_t a = p0 + bias;
+  // (modulo 2^32: x itself is below 2^31)
+  const int32_t x = static_cast<int32_t>(static_cast<uint32_t>(p01) - static_cast<uint32_t>(p0) + 127u * static_cast<uint32_t>(p1)) + (a >> 7);
+  const uint32_t rest = (static_cast<uint32_t>(a) & 127u) | (static_cast<uint32_t>(x) & f.low_mask) << 7;
+  int32_t u = 2 * (x >> f.low) + static_cast<int32_t>(min(rest, 1u));
+  const bool negative = !RELU && u < 0;
+  u = RELU ? max(u, 0) : abs(u);
+  const float m = fminf((__int_as_float(0x4B000000 | u) - 8388608.0f) * scale, f.top);
+  const uint32_t ke = max(__float_as_uint(m) & 0x7F800000u, f.ke_min);
+  const float t = __uint_as_float(ke + f.ke_up) + m;
+  uint32_t code = (ke >> (23 - f.p)) + __float_as_uint(t) - ke - f.ke_off;
+  if (f.p == 0) {                                            // (as in np_encode)
+    const uint32_t fr = __float_as_uint(m) & 0x7FFFFFu, E = (__float_as_uint(m) >> 23) - 126u;
+    code = m >= 1.0f ? E + (fr + (E & 1u) > 0x400000u ? 1u : 0u) : (m > 0.5f ? 1u : 0u);
+  }
+  return code | (negative && code ? 1u << f.sign_bit : 0u);
+}
+
 // v / 2^s rounded in the descriptor's mode, in one pass: (v + z + cond) >> s, with m = 2^s - 1 (odd unless s = 0):
 //   nearest-even: z = m / 2, cond = lowest bit of the truncated quotient;  half away: z = m / 2, cond = v > 0;
 //   half up: z = (m + 1) / 2;  floor: z = 0;  no cond where s = 0.
@@ -1059,7 +1093,7 @@ __device__ __forceinline__ void epilogue_pool_16(const uint32_t (&acc)[16], uint
 // carries twice the tensor work per byte fetched and per instruction of the issuing thread; both
 // accumulator buffers together fill the tensor memory, hence one CTA per SM).
 template <int EPI, int RELU = 2, int RSTG = 0, int GPW = kGroupsPerWarp>
-__global__ void __launch_bounds__(kIgemmThreads, (GPW > kGroupsPerWarp || EPI == EPI_NP) ? 1 : 2)
+__global__ void __launch_bounds__(kIgemmThreads, (GPW > kGroupsPerWarp || EpiTraits<EPI>::np) ? 1 : 2)
 igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                 const __grid_constant__ CUtensorMap tmap_y, const __grid_constant__ CUtensorMap tmap_r,
                 const IgemmParams prm, const EpilogueParams ep, const int4* __restrict__ chan_table,
@@ -1151,7 +1185,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       const uint32_t a_dst = tiles_addr + static_cast<uint32_t>(slot) * stage_bytes;
       const int w0 = tc.q0 * prm.stride_w - prm.pad_w + sx, h0 = tc.p0 * prm.stride_h - prm.pad_h + r;
       int a_ci = ci;                                         // channel chunk of the activations
-      if (EPI == EPI_NP) {
+      if (EpiTraits<EPI>::np) {
         int in_plane;
         const int product = prm.fd_np_cpp.divmod(ci, &in_plane);
         a_ci = prm.np_a[product] * prm.np_cpp + in_plane;
@@ -1308,8 +1342,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       uint32_t phase = 0;
       bool ok = true;
       for (int tile = first_tile; tile < total_tiles && ok; tile += gridDim.x, ++it) {
-        const int buf = (EPI == EPI_NP && prm.acc_bufs == 1) ? 0 : it & 1;
-        const uint32_t use = static_cast<uint32_t>((EPI == EPI_NP && prm.acc_bufs == 1) ? it : it >> 1);
+        const int buf = (EpiTraits<EPI>::np && prm.acc_bufs == 1) ? 0 : it & 1;
+        const uint32_t use = static_cast<uint32_t>((EpiTraits<EPI>::np && prm.acc_bufs == 1) ? it : it >> 1);
         // the epilogue must have drained this accumulator buffer (two tiles ago)
         ok = wait_bounded<0, kHint>(ptx::smem_u32(&sh->acc_empty[buf]), (use & 1u) ^ 1u, wait_limit, sh, status);
         if (!ok) break;
@@ -1347,7 +1381,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             ptx::mma_commit(empty0 + 8u * stage);             // stage free once these MMAs retire
           }
           accumulate = 1;
-          if (EPI == EPI_NP) {
+          if (EpiTraits<EPI>::np) {
             // the next product starts its own columns, cleared by its first chunk of the first tap
             if (++np_chunk == prm.np_cpp) {
               np_chunk = 0;
@@ -1433,8 +1467,8 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     // it carries `ok == false` to the next barrier, which doubles as a vote, and all leave together.
     for (int tile = first_tile; tile < total_tiles; tile += gridDim.x, ++it, walk.next(prm)) {
       const TileCoord tc = walk.coord(prm);
-      const int buf = (EPI == EPI_NP && prm.acc_bufs == 1) ? 0 : it & 1;
-      const uint32_t use = static_cast<uint32_t>((EPI == EPI_NP && prm.acc_bufs == 1) ? it : it >> 1);
+      const int buf = (EpiTraits<EPI>::np && prm.acc_bufs == 1) ? 0 : it & 1;
+      const uint32_t use = static_cast<uint32_t>((EpiTraits<EPI>::np && prm.acc_bufs == 1) ? it : it >> 1);
       // Slot of the per-tile channel constants: by the tile's parity even where there is one accumulator buffer.  A warp that
       // is done with a tile stages the next one's constants while slower warps still read theirs; past the vote behind the
       // staging every warp is done with the tile before, whose slot the tile after may then overwrite.
@@ -1484,7 +1518,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
       const int gen_k0 = tc.k0 + g_begin * 16;
       const int gen_cols = max(0, min((g_end - g_begin) * 16, prm.K - gen_k0));
       // (int8 results overwrite it in place, group by group; words have rows of their own behind it)
-      const bool gen_res = !EpiTraits<EPI>::fast && EPI != EPI_NP && res != nullptr;
+      const bool gen_res = !EpiTraits<EPI>::fast && !EpiTraits<EPI>::np && res != nullptr;
       uint8_t* gen_out = (EPI == EPI_I32 || EPI == EPI_F32) && gen_res ? gen_stage + kEpilogueWarps * kGenWarpBytes : gen_stage;
       int gen_m = 0;
       if (gen_res) {
@@ -1592,7 +1626,39 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             __syncwarp();
           }
         };
-        if constexpr (EPI == EPI_NP) {
+        if constexpr (EPI == EPI_NP3) {
+          const Np3Encode f = {static_cast<uint32_t>(127 + prm.np_p) << 23, static_cast<uint32_t>(23 - prm.np_p) << 23,
+                               (static_cast<uint32_t>(23 - prm.np_p) << 23) + (static_cast<uint32_t>(127 + prm.np_p) << prm.np_p),
+                               (1u << prm.np_low) - 1u, prm.np_low, prm.np_p, prm.np_n - 1, prm.np_top};
+          const uint32_t t0 = t_addr + static_cast<uint32_t>(g_begin) * 16u, bn = static_cast<uint32_t>(prm.BN);
+          uint32_t acc_c[16];
+          for (int i = 0; i * 16 < gen_cols; ++i) {
+            ptx::tmem_ld_32x16(t0 + 16u * i, acc_a);
+            ptx::tmem_ld_32x16(t0 + bn + 16u * i, acc_b);
+            ptx::tmem_ld_32x16(t0 + 2u * bn + 16u * i, acc_c);
+            ptx::tmem_ld_wait();
+            if ((i + 1) * 16 >= gen_cols) release();
+            const uint32_t cst_g = chan + (static_cast<uint32_t>(g_begin + i) * 16u) * EpiTraits<EPI>::cst_bytes;
+            uint32_t wds[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              const int4 k01 = lds_int4(cst_g + static_cast<uint32_t>(g * 32)), k23 = lds_int4(cst_g + static_cast<uint32_t>(g * 32 + 16));
+              const int32_t bias[4] = {k01.x, k01.y, k23.x, k23.y}, sc[4] = {k01.z, k01.w, k23.z, k23.w};
+              uint32_t o[4];
+#pragma unroll
+              for (int b = 0; b < 4; ++b)
+                o[b] = np3_encode<RELU == 1>(static_cast<int32_t>(acc_a[4 * g + b]), static_cast<int32_t>(acc_b[4 * g + b]),
+                                             static_cast<int32_t>(acc_c[4 * g + b]), bias[b], __int_as_float(sc[b]), f);
+              wds[g] = __byte_perm(__byte_perm(o[0], o[1], 0x0040), __byte_perm(o[2], o[3], 0x0040), 0x5410);
+            }
+            ptx::sts_uint4(ptx::smem_u32(gen_stage) + static_cast<uint32_t>(lane * kGenPitch + i * 16), wds[0], wds[1], wds[2], wds[3]);
+          }
+          if (gen_cols <= 0) release();
+          __syncwarp();
+          gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + prm.out_c_offset + gen_k0,
+                         static_cast<long long>(pix) * prm.out_c_pitch, row_ok, gen_cols, lane);
+          __syncwarp();
+        } else if constexpr (EPI == EPI_NP) {
           const NpEncode f = {static_cast<uint32_t>(127 + prm.np_p) << 23, static_cast<uint32_t>(23 - prm.np_p) << 23,
                               (static_cast<uint32_t>(23 - prm.np_p) << 23) + (static_cast<uint32_t>(127 + prm.np_p) << prm.np_p),
                               prm.np_p, prm.np_n - 1, prm.np_top};

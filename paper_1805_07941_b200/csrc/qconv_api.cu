@@ -207,6 +207,7 @@ struct NpSpec {
   int a_plane[qc::kNpMaxProducts], coef[qc::kNpMaxProducts];
   int n_out, p_out;
   float top;                                               // beta_max of the output type
+  long long largest_sum, largest_bias;                     // Eq. 9 with b = beta_max and the largest bias; that bias
   const int8_t* w[qc::kNpMaxProducts];                     // per product: the weights' digit combination, [K][R][S][C]
 };
 
@@ -221,6 +222,7 @@ struct qconv_handle {
   int a_channels = 0;            // channels of the activation tensor (planes * padded C for floating-point operands)
   const NpSpec* np = nullptr;    // set while the handle is built
   int np_products = 0;
+  bool np3 = false;              // two-digit operands whose sums are recombined and converted in 32 bits
   bool weights_as_is = false;    // those weights lie as the host handed them over ([K][R][S][C])
   int8_t* d_w = nullptr;         // direct: [R][S][Cg][K]; depthwise: [R*S][C]; igemm: [Kpad][Kg_total]
   int32_t* d_bias = nullptr;
@@ -607,6 +609,15 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     h->a_channels = np->planes * p.np_cpp * p.BKC;
     for (int m = 0; m < np->products; ++m) { p.np_a[m] = np->a_plane[m]; p.np_coef[m] = np->coef[m]; }
     p.np_n = np->n_out; p.np_p = np->p_out; p.np_top = np->top;
+    // Two-digit operands: the conversion in 32 bits (np3_encode) where the largest sum and the smallest shift leave room for it:
+    // |v| < 2^(22 + low) and low <= s - 1 for some low >= 7; v / 128 and P0 + bias within an int32.  (Beyond: a sum of 2^33 with
+    // a shift below 13, for instance.)
+    int low = 7, min_shift = 31;
+    while ((np->largest_sum >> low) >= (1ll << 22) - 1) ++low;
+    for (int k = 0; k < d.K; ++k) min_shift = std::min(min_shift, shift_host ? shift_host[k] : 0);
+    h->np3 = np->products == 3 && np->coef[0] == -127 && np->coef[1] == 16384 - 128 && np->coef[2] == 128 && low <= min_shift - 1 &&
+             np->largest_sum < (1ll << 37) && np->largest_bias < (1ll << 30) && hint.float_rounding != 0;
+    p.np_low = low - 7;
   }
   p.R = taps_r; p.S = taps_s;
   int bn_max = std::min(2 * qc::kGroupsPerWarp * 16, std::max(16, (hint.bn_max > 0 ? hint.bn_max : 128) / 16 * 16));
@@ -1023,7 +1034,14 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     const int t = (d.has_residual && res_lshift_host) ? res_lshift_host[k] : 0;
     chan[k] = make_int4(bias_host ? bias_host[k] : 0, sft, sft > 0 ? (1 << ((sft - 1) & 31)) - 1 : 0,
                         (sft > 0 ? 1 : 0) | ((1 << t) << 1));
-    if (np) { chan[k].z = chan[k].w = 0; continue; }         // (shifts up to 40)
+    if (np) {                                                // (shifts up to 40)
+      if (h->np3) {
+        const float scale = std::ldexp(1.0f, p.np_low + 6 - sft);
+        std::memcpy(&chan[k].y, &scale, sizeof(int));
+      }
+      chan[k].z = chan[k].w = 0;
+      continue;
+    }
     if (d.out_mode == QCONV_OUT_INT8 && !p.fast_epilogue && !h->gen_flt) chan[k].y = sft | t << 8;
     if (h->gen_flt) {
       // {magic + bias + half, bits of 2^-s, half - 1 (half away by sign: not in the bias then), 2^t << 1}
@@ -1111,6 +1129,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_F32>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_MAX>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_NP>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_NP3, 0>),
+                          static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_NP3, 1>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_U, 2, 4>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8, 2, 4>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8_RES_U, 2, 4>),
@@ -1149,6 +1169,7 @@ PairKernel pair_kernel_for(const qconv_handle* h) {
 
 IgemmKernel igemm_kernel_for(const qconv_handle* h, bool maxabs) {
   if (maxabs) return qc::igemm_i8_kernel<qc::EPI_MAX>;
+  if (h->np3) return h->d.relu ? qc::igemm_i8_kernel<qc::EPI_NP3, 1> : qc::igemm_i8_kernel<qc::EPI_NP3, 0>;
   if (h->np_products) return qc::igemm_i8_kernel<qc::EPI_NP>;
   if (h->d.out_mode == QCONV_OUT_INT32) return qc::igemm_i8_kernel<qc::EPI_I32>;
   if (h->d.out_mode == QCONV_OUT_FLOAT) return qc::igemm_i8_kernel<qc::EPI_F32>;
@@ -2126,6 +2147,7 @@ int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len) {
              p.out_stage_bytes ? p.out_stage_bufs : 0, p.b_resident, p.tap_boxes || h->patch ? 0 : p.halo_s, p.tap_boxes ? p.halo_s : 0, h->pair, h->d.pool, h->patch ? " patch=1" : "");
     const size_t used = std::strlen(buf);
     if (h->split > 1) snprintf(buf + used, buf_len - used, " split=%d", h->split);
+    else if (h->np3) snprintf(buf + used, buf_len - used, " sums=32");
   } else {
     snprintf(buf, buf_len, "%s", h->algo == QCONV_ALGO_DEPTHWISE ? (h->dw_tma ? "depthwise3x3/tap-packed+tma" : h->dw_tap ? "depthwise3x3/tap-packed" : "depthwise3x3/dp4a")
                                                                   : "direct");
@@ -2499,6 +2521,8 @@ int qconv_np_create(qconv_np_handle** out, const qconv_np_desc* desc, const uint
   NpSpec spec;
   spec.products = static_cast<int>(products.size());
   spec.n_out = d.n_out; spec.p_out = d.p_out; spec.top = static_cast<float>(bmax[2]);
+  spec.largest_sum = static_cast<long long>(d.R) * d.S * d.C * bmax[0] * bmax[1] + max_bias;
+  spec.largest_bias = max_bias;
   for (size_t m = 0; m < products.size(); ++m) {
     // the input's digit combination: one plane for each that differs
     const int x_mask = products[m].mask & ((1 << px) - 1), w_mask = products[m].mask & ((1 << pw) - 1);
