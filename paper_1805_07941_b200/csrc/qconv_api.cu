@@ -714,14 +714,17 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   // -> 128 72 -> 60, x 128 -> 128 with its pool 102 -> 84, 128 x 28 x 28 x 96 -> 128 20.0 -> 14.8, 128 x 14 x 14 x 112 -> 224
   // 14.8 -> 9.1; at one wave of tiles (32 x 28 x 28 x 128 -> 128: 7.2 -> 6.8) it is about even.
   const bool patch_fits = h->mode == MODE_BOX && d.R == 3 && d.S == 3 && d.stride_h == 1 && d.stride_w == 1 && d.pad_h == 1 && d.pad_w == 1 &&
-                          p.nchunks == 1 && p.BKC >= 64 && fast_possible && d.K % 16 == 0 && d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0;
+                          p.nchunks == 1 && fast_possible && d.K % 16 == 0 && d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0;
   bool patch = false;
   if (patch_fits && hint.patch_halo != 0 && hint.bn_max <= 0 && hint.halo != 1 && hint.group_taps != 1 && hint.pair_tiles != 1) {
     const long tiles = static_cast<long>(pt.segs) * pt.rows * d.N * ceil_div(k_eff, 128);
     const double used = static_cast<double>(h->Q) * h->P / (static_cast<double>(pt.segs) * pt.rows * 128);
     // from a wave of tiles on, as long as most accumulator rows are outputs and the activations are read for two channel
     // tiles at most
-    patch = hint.patch_halo == 1 || (tiles >= h->num_sms && used >= 0.75 && k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0);
+    // ... and at up to 32 channels (rows of 32 bytes) also below a wave, where the one box is one wait instead of three: 32 x 32
+    // x 16 -> 16 3.6 -> 3.0 us, 56 x 56 x 32 -> 32 3.3 -> 3.1; with rows of 64 or 128 bytes three boxes are 0.2 us faster there.
+    patch = hint.patch_halo == 1 || (k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0 &&
+                                     ((tiles >= h->num_sms && used >= 0.75) || (p.BKC == 32 && tiles <= h->num_sms)));
   }
   if (dw) patch = !halo && halo_fits && d.S == 3 && hint.patch_halo != 0;
   if (np && halo && d.R == 3 && d.pad_h == 1 && p.np_cpp == 1 && bn_max <= 64 && hint.patch_halo != 0 && hint.halo != 1) {
@@ -740,7 +743,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     wide = false;
     halo = false;
     h->pair = 0;
-    bn_max = dw ? p.BKC : np ? bn_max : 128;
+    bn_max = dw ? p.BKC : np ? bn_max : bn_max <= 64 ? 64 : 128;
     taps_r = taps_s = 1;
     p.R = p.S = 1;
   }
