@@ -2295,18 +2295,19 @@ int qmaxpool_i8(const int8_t* d_x, int N, int H, int W, int C, int R, int S, int
   const bool strip_ok = vec && R == S && ((R == 3 && (stride == 1 || stride == 2)) || (R == 2 && stride == 2));
   if (strip_ok) {
     // strips as long as still leaves every SM several hundred threads
+    const int columns = ceil_div(Q, R == 3 && stride == 1 ? 2 : 1);
     int rows = 16;
-    while (rows > 2 && static_cast<size_t>(N) * ceil_div(P, rows) * Q * (C / 16) < 148u * 1024u) rows /= 2;
+    while (rows > 2 && static_cast<size_t>(N) * ceil_div(P, rows) * columns * (C / 16) < 148u * 1024u) rows /= 2;
     const int strips = ceil_div(P, rows);
-    const size_t threads = static_cast<size_t>(N) * strips * Q * (C / 16);
+    const size_t threads = static_cast<size_t>(N) * strips * columns * (C / 16);
     if (threads > 2147483647ull) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "pooling: tensor too large");
     const dim3 grid(static_cast<unsigned int>((threads + 127) / 128));
     if (R == 3 && stride == 1)
-      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 1>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
+      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 1, 2>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
     else if (R == 3)
-      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 2>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
+      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 2, 1>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
     else
-      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<2, 2, 2>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
+      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<2, 2, 2, 1>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
   } else if (vec)
     CUDA_TRY(launch_chained(qc::maxpool_i8_vec_kernel, dim3(grid_for(pix * (C / 16), 256, 148 * 32)), dim3(256), 0, st,
                             d_x, d_y, N, H, W, C, R, S, stride, pad, P, Q));
