@@ -21,6 +21,7 @@
 #include "graph_inputs.cuh"
 #include "host_weights.cuh"
 #include "kernel_igemm.cuh"
+#include "kernel_dw_mma.cuh"
 #include "kernel_dw_tma.cuh"
 #include "kernel_igemm_pair.cuh"
 #include "kernel_mma_peak.cuh"
@@ -242,6 +243,8 @@ struct qconv_handle {
   int num_sms = 148;
   int ctas_per_sm = 2;
   int use_pdl = 1;
+  int dw_warp = 0;               // depthwise on warp-level matrix instructions (kernel_dw_mma.cuh)
+  qc::DwMmaParams dw_mma_prm = {};
   int dw_mma = 0;                // depthwise on the tensor cores (prm, mode and the maps are then its plan)
   int8_t* d_w_mma = nullptr;     // its weights: [C][9][32]
   uint32_t* d_dw_tap = nullptr;  // tap-packed form: weight rows [3][C], bias + magic [C], 2^-s [C], rounding offset [C] (float bits)
@@ -256,7 +259,7 @@ struct qconv_handle {
   qc::DwTmaParams dw_prm = {};
   CUtensorMap dw_map;
   const void* dw_key_ptr = nullptr;
-  int dw_key_n = -1;
+  int dw_key_n = -1, dw_key_form = 0;
   int8_t* d_pack = nullptr;      // stem: packed patches [N*P*Q][kg_pad]
   int stem_segp = 0;             // stem: bytes per filter-row segment of a packed row (0: taps back to back)
   // stride-2 stem in space-to-depth form: d_pack is [N][s2d_h][s2d_wp] 16-byte block pixels, the image starting
@@ -1404,18 +1407,59 @@ void plan_dw_tma(qconv_handle* h) {
   h->dw_tma = 1;
 }
 
-int prepare_dw_map(qconv_handle* h, const int8_t* x, int n_run) {
-  if (h->dw_key_ptr == x && h->dw_key_n == n_run) return QCONV_OK;
+// Tile of the depthwise kernel on warp-level matrix instructions: eight warps, each 32 channels x two groups of 8 pixels, over
+// 32, 64 or 128 channels; narrow images share a CTA.  The width whose padding (channels, groups, halo columns) costs least.
+void plan_dw_mma(qconv_handle* h) {
+  const qconv_desc& d = h->d;
+  const int st = d.stride_h;
+  double best = 0.0;
+  qc::DwMmaParams bp = {};
+  for (int cb : {128, 64, 32}) {
+    qc::DwMmaParams p = {};
+    p.cb = cb;
+    p.swz_mask = cb / 16 - 1;
+    const int wc = cb / 32, all = ceil_div(h->Q, 8);
+    int most = 2 * (qc::kDwMmaWarps / wc);
+    while (most * 8 * st + 3 - st > 256) --most;           // (a copy's box spans at most 256 pixels)
+    p.q_blocks = ceil_div(all, most);
+    p.groups = ceil_div(all, p.q_blocks);
+    p.images = p.q_blocks > 1 ? 1 : std::max(1, std::min(d.N, most / p.groups));
+    p.pix = p.groups * 8 * st + 3 - st;
+    p.warps = ceil_div(p.groups * p.images, 2) * wc;
+    p.row_bytes = p.images * p.pix * cb;
+    p.stage_bytes = static_cast<int>(align_up(p.row_bytes, 1024));
+    const double channels = static_cast<double>(align_up(d.C, cb)) / d.C;
+    const double pixels = static_cast<double>(p.q_blocks) * (p.warps / wc) * 16 / (static_cast<double>(h->Q) * p.images);
+    const double halo = static_cast<double>(p.pix) / (p.groups * 8 * st);
+    const double cost = channels * pixels * (0.7 + 0.3 * halo);
+    if (bp.cb == 0 || cost < best * 0.999) { best = cost; bp = p; }
+  }
+  while ((32 << bp.wc_log2) < bp.cb) ++bp.wc_log2;
+  bp.fd_q_blocks = make_fastdiv(bp.q_blocks);
+  bp.fd_groups = make_fastdiv(bp.groups);
+  bp.lo = d.relu ? 0 : h->lo;
+  const float c1 = h->uni_s <= 22 ? std::ldexp(1.0f, -h->uni_s) : 0.0f;
+  bp.c1 = c1;
+  bp.c2 = static_cast<float>(12582912.0 * (1.0 - static_cast<double>(c1)));
+  h->dw_mma_prm = bp;
+  h->dw_warp = 1;
+}
+
+// Box of the depthwise kernels' row copies: `channels` x `pixels` x one row x `images`.
+int prepare_dw_map(qconv_handle* h, const int8_t* x, int n_run, int channels, int pixels, int images, int swizzle) {
+  const int form = channels + 1024 * swizzle;
+  if (h->dw_key_ptr == x && h->dw_key_n == n_run && h->dw_key_form == form) return QCONV_OK;
   const qconv_desc& d = h->d;
   cuuint64_t dims[4] = {static_cast<cuuint64_t>(d.C), static_cast<cuuint64_t>(d.W), static_cast<cuuint64_t>(d.H),
                         static_cast<cuuint64_t>(n_run)};
   cuuint64_t strides[3] = {static_cast<cuuint64_t>(d.C), static_cast<cuuint64_t>(d.W) * d.C,
                            static_cast<cuuint64_t>(d.H) * d.W * d.C};
-  cuuint32_t box[4] = {static_cast<cuuint32_t>(h->dw_prm.cwb_box * 4), static_cast<cuuint32_t>(h->dw_prm.pix), 1, 1};
-  int rc = encode_map(&h->dw_map, x, 4, dims, strides, box, 0);
+  cuuint32_t box[4] = {static_cast<cuuint32_t>(channels), static_cast<cuuint32_t>(pixels), 1, static_cast<cuuint32_t>(images)};
+  int rc = encode_map(&h->dw_map, x, 4, dims, strides, box, swizzle);
   if (rc) return rc;
   h->dw_key_ptr = x;
   h->dw_key_n = n_run;
+  h->dw_key_form = form;
   return QCONV_OK;
 }
 
@@ -1686,12 +1730,19 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       parts.add(&h->d_dw_tap, t.data(), t.size() * 4);
       h->dw_tap = 1;
       if (d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
-      // On the tensor cores in rows of 64 or 128 channels, an eighth of padding at most (23 x 49 x 8 x 928, stride 2:
-      // 33 -> 8.4 us; a third of it costs: 64 x 56 x 56 x 144 27 -> 34; with rows of 32 the per-tile work outweighs the gain:
-      // 112 x 112 x 32 at batch 256 76 -> 96).
-      h->dw_mma = h->flt_epilogue && h->hints.fast_epilogue != 0 && d.pad_h == 1 && d.pad_w == 1 && d.C % 16 == 0 &&
-                  (h->hints.depthwise_form == 3 || align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8) &&
-                  d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && (h->hints.depthwise_form < 0 || h->hints.depthwise_form == 3);
+      // On the tensor cores by warp-level instructions (kernel_dw_mma.cuh) where the channels fill its groups of 32, and for
+      // small layers whatever they do; else by tcgen05 in rows of 64 or 128 channels with an eighth of padding at most; else dp4a.
+      // us per launch, warp level / tcgen05 / dp4a: 256 x 112 x 112 x 32 67 / 138 / 73, 256 x 56 x 56 x 128 stride 2 27.6 / 28.4 /
+      // 29.9, 256 x 28 x 28 x 256 41 / 37 / 39, 256 x 14 x 14 x 512 22.8 / 22.2 / 22.6, 32 x 56 x 56 x 96 8.4 / 12.8 / 14.6, 64 x 56 x 56 x
+      // 144 26.3 / 34 / 25.4, 13 x 13 x 13 x 1008 4.6 / 5.4 / 5.6; one image of those 2.8 to 3.2 / 3.3 to 4.0 / 3.9 to 4.2.  Alone it is
+      // no faster at batch 256, but its many short CTAs leave no tail: the MobileNet-v1 stack with it throughout 784 us, 818 before.
+      const long long outputs = static_cast<long long>(d.N) * P * Q * d.C;
+      const bool tensor_cores = h->flt_epilogue && h->hints.fast_epilogue != 0 && d.C % 16 == 0;
+      if (tensor_cores && d.out_c_pitch % 8 == 0 && d.out_c_offset % 8 == 0 &&
+          (h->hints.depthwise_form == 3 || (h->hints.depthwise_form < 0 && (d.C % 32 == 0 || outputs <= (4ll << 20)))))
+        plan_dw_mma(h);
+      h->dw_mma = tensor_cores && !h->dw_warp && d.pad_h == 1 && d.pad_w == 1 && align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8 &&
+                  d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && h->hints.depthwise_form < 0;
     }
     if (!rc && h->dw_mma) {
       h->mode = MODE_BOX;
@@ -1732,6 +1783,46 @@ cudaError_t launch_row_pack(const qconv_handle* h, const void* src, bool f32, in
   }
 }
 
+int run_dw_mma(qconv_handle* h, const int8_t* x, int8_t* y, int n_run, const qc::ConvGeom& g, const qc::DwTapParams& tp, cudaStream_t st) {
+  qc::DwMmaParams p = h->dw_mma_prm;
+  int rc = prepare_dw_map(h, x, n_run, p.cb, p.pix, p.images, p.cb);
+  if (rc) return rc;
+  // Rows per strip: a CTA's fixed cost is about six rows' worth (set-up, filling its ring), its halo two rows; two CTAs run on
+  // an SM.  The strip length whose rounds of CTAs take the fewest rows in all.
+  const long columns = static_cast<long>(ceil_div(g.C, p.cb)) * p.q_blocks * ceil_div(n_run, p.images), slots = 2l * h->num_sms;
+  long best = -1;
+  for (int strips = 1; strips <= std::max(1, h->P / 2); ++strips) {
+    const int rows = ceil_div(h->P, strips);
+    if (ceil_div(h->P, rows) != strips) continue;
+    const long cost = ceil_div_l(columns * strips, slots) * ((rows - 1) * g.stride_h + 3 + 6);
+    if (best < 0 || cost < best) { best = cost; p.rows_per_cta = rows; }
+  }
+  const dim3 grid(ceil_div(g.C, p.cb) * p.q_blocks, ceil_div(h->P, p.rows_per_cta), ceil_div(n_run, p.images));
+  const size_t smem = 1024 + static_cast<size_t>(qc::kDwMmaStages) * p.stage_bytes + sizeof(qc::DwMmaShared);
+  const bool uni = h->uniform_shift && h->hints.uniform_shift != 0;
+  using Kernel = decltype(&qc::depthwise3x3_mma_kernel<1, true, true>);
+  static constexpr Kernel kernels[2][2][2] = {
+      {{qc::depthwise3x3_mma_kernel<1, false, false>, qc::depthwise3x3_mma_kernel<1, false, true>},
+       {qc::depthwise3x3_mma_kernel<1, true, false>, qc::depthwise3x3_mma_kernel<1, true, true>}},
+      {{qc::depthwise3x3_mma_kernel<2, false, false>, qc::depthwise3x3_mma_kernel<2, false, true>},
+       {qc::depthwise3x3_mma_kernel<2, true, false>, qc::depthwise3x3_mma_kernel<2, true, true>}}};
+  const Kernel kernel = kernels[g.stride_h - 1][uni][h->d.relu != 0];
+  static std::once_flag attr_once[64];                       // (the attribute belongs to the current device)
+  static cudaError_t attr_err = cudaSuccess;
+  std::call_once(attr_once[h->device & 63], [] {
+    for (const auto& by_stride : kernels)
+      for (const auto& by_scale : by_stride)
+        for (Kernel k : by_scale) {
+          const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+          if (e != cudaSuccess) attr_err = e;
+        }
+  });
+  CUDA_TRY(attr_err);
+  const int8_t* weights = h->d_w;
+  CUDA_TRY(launch_chained(kernel, grid, dim3(p.warps * 32), smem, st, h->dw_map, weights, y, g, tp, p, h->d_status, h->wait_limit));
+  return QCONV_OK;
+}
+
 // One layer launch.  input_is_packed: d_x is the handle's own space-to-depth scratch, already filled
 // (qconv_run_f32 converts and packs in one kernel).  maxabs: d_y is the word of a running maximum (float bits of the
 // largest |float output|) and nothing else is written.
@@ -1761,11 +1852,15 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
          reinterpret_cast<uintptr_t>(d_residual)) & 3)
       return fail(QCONV_ERR_ALIGNMENT, "depthwise kernel needs 4-byte aligned tensors");
     constexpr int TW = 4;
+    const bool mma_aligned = (reinterpret_cast<uintptr_t>(d_x) & 15) == 0 && (reinterpret_cast<uintptr_t>(d_y) & 7) == 0;
     if (h->dw_tap && n_run <= 65535) {
       const qc::DwTapParams tp{h->d_dw_tap, reinterpret_cast<const int32_t*>(h->d_dw_tap + static_cast<size_t>(3) * d.C),
                                reinterpret_cast<const float*>(h->d_dw_tap + static_cast<size_t>(4) * d.C),
                                reinterpret_cast<const float*>(h->d_dw_tap + static_cast<size_t>(5) * d.C),
                                12582912.0f + static_cast<float>(d.relu ? 0 : h->lo), 12582912.0f + static_cast<float>(h->hi)};
+      // (A run that is granted no polls has to report that; this kernel would find rows that landed in time.  The next one
+      // counts its first probe as a poll.)
+      if (h->dw_warp && mma_aligned && h->wait_limit != 0) return run_dw_mma(h, d_x, static_cast<int8_t*>(d_y), n_run, g, tp, st);
       const int per_row = ceil_div(h->Q, TW) * (d.C / 4);
       // rows per thread: long strips amortise the per-thread tables, but the grid must still fill the GPU
       int rows = 16;
@@ -1773,7 +1868,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
       rows = std::min(rows, h->P);
       dim3 grid(ceil_div(per_row, 256), ceil_div(h->P, rows), n_run);
       if (h->dw_tma && (reinterpret_cast<uintptr_t>(d_x) & 15) == 0) {
-        int rc = prepare_dw_map(h, d_x, n_run);
+        int rc = prepare_dw_map(h, d_x, n_run, h->dw_prm.cwb_box * 4, h->dw_prm.pix, 1, 0);
         if (rc) return rc;
         qc::DwTmaParams prm = h->dw_prm;
         const int ctas_row = (d.C / 4 / prm.cwb) * prm.q_blocks;
@@ -2152,7 +2247,7 @@ int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len) {
     if (h->split > 1) snprintf(buf + used, buf_len - used, " split=%d", h->split);
     else if (h->np3) snprintf(buf + used, buf_len - used, " sums=32");
   } else {
-    snprintf(buf, buf_len, "%s", h->algo == QCONV_ALGO_DEPTHWISE ? (h->dw_tma ? "depthwise3x3/tap-packed+tma" : h->dw_tap ? "depthwise3x3/tap-packed" : "depthwise3x3/dp4a")
+    snprintf(buf, buf_len, "%s", h->algo == QCONV_ALGO_DEPTHWISE ? (h->dw_warp ? "depthwise3x3/mma+tma" : h->dw_tma ? "depthwise3x3/tap-packed+tma" : h->dw_tap ? "depthwise3x3/tap-packed" : "depthwise3x3/dp4a")
                                                                   : "direct");
   }
   return QCONV_OK;
