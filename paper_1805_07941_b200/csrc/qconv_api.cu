@@ -1407,9 +1407,22 @@ void plan_dw_tma(qconv_handle* h) {
   h->dw_tma = 1;
 }
 
+size_t dw_mma_smem(const qc::DwMmaParams& p) {
+  return 1024 + static_cast<size_t>(qc::kDwMmaStages) * p.stage_bytes + sizeof(qc::DwMmaShared);
+}
+
+// CTAs of that kernel on an SM: 16 warps at 128 registers a thread, 227 KB of shared memory.  (Five warps: three.  Strips chosen for
+// two: 128 x 72 x 72 x 32 24.0 -> 17.1 us, 64 x 75 x 75 x 96 34.2 -> 25.9, 64 x 33 x 65 x 128 22.3 -> 17.6.)
+int dw_mma_ctas_per_sm(const qc::DwMmaParams& p) {
+  return static_cast<int>(std::max<size_t>(1, std::min<size_t>(16 / p.warps, 227 * 1024 / (dw_mma_smem(p) + 1024))));
+}
+
 // Tile of the depthwise kernel on warp-level matrix instructions: eight warps, each 32 channels x two groups of 8 pixels, over
 // 32, 64 or 128 channels; narrow images share a CTA.  The width whose padding (channels, groups, halo columns) costs least.
-void plan_dw_mma(qconv_handle* h) {
+// Unless `whatever_it_costs`, none where a third of the work would be padding and rows are narrow: 64 x 33 x 33 x 512 stride 2 14.4 us
+// against tcgen05's 11.8, 128 x 36 x 36 x 128 stride 2 8.4 against 7.7 (128 channels wide it is faster all the same: 128 x 9 x 9 x 512 at
+// a cost of 1.84 7.8 against 8.3).
+void plan_dw_mma(qconv_handle* h, bool whatever_it_costs) {
   const qconv_desc& d = h->d;
   const int st = d.stride_h;
   double best = 0.0;
@@ -1434,6 +1447,7 @@ void plan_dw_mma(qconv_handle* h) {
     const double cost = channels * pixels * (0.7 + 0.3 * halo);
     if (bp.cb == 0 || cost < best * 0.999) { best = cost; bp = p; }
   }
+  if (!whatever_it_costs && bp.cb < 128 && best > 1.3) return;
   while ((32 << bp.wc_log2) < bp.cb) ++bp.wc_log2;
   bp.fd_q_blocks = make_fastdiv(bp.q_blocks);
   bp.fd_groups = make_fastdiv(bp.groups);
@@ -1733,14 +1747,14 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       // On the tensor cores by warp-level instructions (kernel_dw_mma.cuh) where the channels fill its groups of 32, and for
       // small layers whatever they do; else by tcgen05 in rows of 64 or 128 channels with an eighth of padding at most; else dp4a.
       // us per launch, warp level / tcgen05 / dp4a: 256 x 112 x 112 x 32 67 / 138 / 73, 256 x 56 x 56 x 128 stride 2 27.6 / 28.4 /
-      // 29.9, 256 x 28 x 28 x 256 41 / 37 / 39, 256 x 14 x 14 x 512 22.8 / 22.2 / 22.6, 32 x 56 x 56 x 96 8.4 / 12.8 / 14.6, 64 x 56 x 56 x
+      // 29.9, 256 x 28 x 28 x 256 40 / 37 / 39, 256 x 14 x 14 x 512 21.6 / 22.2 / 22.6, 32 x 56 x 56 x 96 8.1 / 12.8 / 14.6, 64 x 56 x 56 x
       // 144 26.3 / 34 / 25.4, 13 x 13 x 13 x 1008 4.6 / 5.4 / 5.6; one image of those 2.8 to 3.2 / 3.3 to 4.0 / 3.9 to 4.2.  Alone it is
-      // no faster at batch 256, but its many short CTAs leave no tail: the MobileNet-v1 stack with it throughout 784 us, 818 before.
+      // no faster at batch 256, but its many short CTAs leave no tail: the MobileNet-v1 stack with it throughout 771 us, 818 before.
       const long long outputs = static_cast<long long>(d.N) * P * Q * d.C;
       const bool tensor_cores = h->flt_epilogue && h->hints.fast_epilogue != 0 && d.C % 16 == 0;
       if (tensor_cores && d.out_c_pitch % 8 == 0 && d.out_c_offset % 8 == 0 &&
           (h->hints.depthwise_form == 3 || (h->hints.depthwise_form < 0 && (d.C % 32 == 0 || outputs <= (4ll << 20)))))
-        plan_dw_mma(h);
+        plan_dw_mma(h, h->hints.depthwise_form == 3 || outputs <= (4ll << 20) || align_up(d.C, 64) != static_cast<size_t>(d.C));
       h->dw_mma = tensor_cores && !h->dw_warp && d.pad_h == 1 && d.pad_w == 1 && align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8 &&
                   d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && h->hints.depthwise_form < 0;
     }
@@ -1787,9 +1801,10 @@ int run_dw_mma(qconv_handle* h, const int8_t* x, int8_t* y, int n_run, const qc:
   qc::DwMmaParams p = h->dw_mma_prm;
   int rc = prepare_dw_map(h, x, n_run, p.cb, p.pix, p.images, p.cb);
   if (rc) return rc;
-  // Rows per strip: a CTA's fixed cost is about six rows' worth (set-up, filling its ring), its halo two rows; two CTAs run on
-  // an SM.  The strip length whose rounds of CTAs take the fewest rows in all.
-  const long columns = static_cast<long>(ceil_div(g.C, p.cb)) * p.q_blocks * ceil_div(n_run, p.images), slots = 2l * h->num_sms;
+  // Rows per strip: a CTA's fixed cost is about six rows' worth (set-up, filling its ring), its halo two rows.  The strip
+  // length whose rounds of CTAs take the fewest rows in all.
+  const long columns = static_cast<long>(ceil_div(g.C, p.cb)) * p.q_blocks * ceil_div(n_run, p.images);
+  const long slots = static_cast<long>(dw_mma_ctas_per_sm(p)) * h->num_sms;
   long best = -1;
   for (int strips = 1; strips <= std::max(1, h->P / 2); ++strips) {
     const int rows = ceil_div(h->P, strips);
@@ -1798,7 +1813,7 @@ int run_dw_mma(qconv_handle* h, const int8_t* x, int8_t* y, int n_run, const qc:
     if (best < 0 || cost < best) { best = cost; p.rows_per_cta = rows; }
   }
   const dim3 grid(ceil_div(g.C, p.cb) * p.q_blocks, ceil_div(h->P, p.rows_per_cta), ceil_div(n_run, p.images));
-  const size_t smem = 1024 + static_cast<size_t>(qc::kDwMmaStages) * p.stage_bytes + sizeof(qc::DwMmaShared);
+  const size_t smem = dw_mma_smem(p);
   const bool uni = h->uniform_shift && h->hints.uniform_shift != 0;
   using Kernel = decltype(&qc::depthwise3x3_mma_kernel<1, true, true>);
   static constexpr Kernel kernels[2][2][2] = {
