@@ -20,8 +20,8 @@
 // -> 771 us; one image's layers 3.3-4.2 -> 2.8-3.2 us each.  Registers decide its speed: per-channel scales held in them instead of
 // shared memory 782 us, a few more spilled 807-848.
 //
-// Every wait is bounded: on expiry the CTA raises the status word and everybody leaves; the issuing lane stays until its
-// copies have landed.
+// Every wait is bounded, its first probe counted as a poll: on expiry the CTA raises the status word and everybody leaves; the
+// issuing lane stays until its copies have landed.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -58,7 +58,7 @@ struct DwMmaShared {
 };
 
 __device__ __forceinline__ bool dw_mma_wait(uint32_t bar, uint32_t parity, unsigned int limit, DwMmaShared* sh, int* status) {
-  for (unsigned int it = 0; it < limit; ++it) {
+  for (unsigned int it = 1; it < limit; ++it) {               // (the caller has probed once)
     if (ptx::mbar_try_wait(bar, parity)) return true;
     if (*reinterpret_cast<volatile int*>(&sh->abort_flag)) return false;
   }
@@ -222,7 +222,7 @@ depthwise3x3_mma_kernel(const __grid_constant__ CUtensorMap tmap_x, const int8_t
     }
   };
   // One input row against filter rows: FIRST starts slot s0 (filter row 0), MID adds row 1 to s1, LAST row 2 to s2.
-  bool go = true;
+  bool go = wait_limit != 0;                                  // (no polls granted: every warp gives up here)
   int stage = 0, taken = 0;
   uint32_t parity = 0;
   auto take = [&](auto first, auto mid, auto last, int32_t (&s0)[4][4], int32_t (&s1)[4][4], int32_t (&s2)[4][4]) {
@@ -300,6 +300,7 @@ depthwise3x3_mma_kernel(const __grid_constant__ CUtensorMap tmap_x, const int8_t
   // After a wait that expired, copies already on their way must land before this CTA's shared memory goes away, whatever the
   // caller's wait limit.  (A strip that was walked to its end has used every row.)
   if (issuer && !go) {
+    if (wait_limit == 0) atomicExch(status, kStatusTimeout);
     for (int i = issued > kDwMmaStages ? issued - kDwMmaStages : 0; i < issued; ++i) {
       const uint32_t par = static_cast<uint32_t>(i / kDwMmaStages) & 1u;
       for (unsigned int it = 0; it < kDrainPolls; ++it)

@@ -1873,9 +1873,7 @@ int run_layer(qconv_handle* h, const int8_t* d_x, const int8_t* d_residual, void
                                reinterpret_cast<const float*>(h->d_dw_tap + static_cast<size_t>(4) * d.C),
                                reinterpret_cast<const float*>(h->d_dw_tap + static_cast<size_t>(5) * d.C),
                                12582912.0f + static_cast<float>(d.relu ? 0 : h->lo), 12582912.0f + static_cast<float>(h->hi)};
-      // (A run that is granted no polls has to report that; this kernel would find rows that landed in time.  The next one
-      // counts its first probe as a poll.)
-      if (h->dw_warp && mma_aligned && h->wait_limit != 0) return run_dw_mma(h, d_x, static_cast<int8_t*>(d_y), n_run, g, tp, st);
+      if (h->dw_warp && mma_aligned) return run_dw_mma(h, d_x, static_cast<int8_t*>(d_y), n_run, g, tp, st);
       const int per_row = ceil_div(h->Q, TW) * (d.C / 4);
       // rows per thread: long strips amortise the per-thread tables, but the grid must still fill the GPU
       int rows = 16;

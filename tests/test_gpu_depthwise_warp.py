@@ -46,16 +46,22 @@ def test_depthwise_on_warp_instructions_matches_the_oracle(case, uniform):
     conv.destroy()
 
 
-def test_an_expired_wait_is_reported_and_the_next_run_is_right():
+@pytest.mark.parametrize("C,stride", [(64, 1), (16, 1), (112, 1), (240, 2), (1008, 1)])
+def test_an_expired_wait_is_reported_and_the_next_run_is_right(C, stride):
+    """No polls granted: every warp leaves, the copies in flight land, the status says so.  (Also where 32 does not divide the
+    channels and no other kernel for the layer has waits.)"""
     from paper_1805_07941_b200 import binding
     rng = np.random.default_rng(1)
-    x, w, bias, shift, _, _ = rand_layer(rng, 2, 40, 30, 64, 64, 3, 3, groups=64, pad=(1, 1))
+    x, w, bias, shift, _, _ = rand_layer(rng, 2, 40, 30, C, C, 3, 3, groups=C, stride=(stride, stride), pad=(1, 1))
     shift = (shift - 1).clip(4, 31)
-    conv = binding.QConv(w, bias, shift, N=2, H=40, W=30, C=64, K=64, R=3, S=3, pad_h=1, pad_w=1, groups=64)
-    xd, y = torch.from_numpy(x).cuda(), torch.empty((2, 40, 30, 64), dtype=torch.int8, device="cuda")
-    conv.set_wait_limit(0)
-    conv.run(xd, y)
-    assert conv.status() == binding.ERR_TIMEOUT
-    conv.set_wait_limit(1 << 22)
-    conv.run(xd, y)
-    assert conv.status() == 0 and (y.cpu().numpy() == oracle_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1), groups=64)).all()
+    conv = binding.QConv(w, bias, shift, N=2, H=40, W=30, C=C, K=C, R=3, S=3, stride_h=stride, stride_w=stride, pad_h=1, pad_w=1, groups=C)
+    assert "depthwise3x3/mma+tma" in conv.describe()
+    xd, y = torch.from_numpy(x).cuda(), torch.empty((2, conv.P, conv.Q, C), dtype=torch.int8, device="cuda")
+    want = oracle_conv(x, w, bias, shift, R=3, S=3, stride=(stride, stride), pad=(1, 1), groups=C)
+    for _ in range(2):
+        conv.set_wait_limit(0)
+        conv.run(xd, y)
+        assert conv.status() == binding.ERR_TIMEOUT
+        conv.set_wait_limit(1 << 22)
+        conv.run(xd, y)
+        assert conv.status() == 0 and (y.cpu().numpy() == want).all()
