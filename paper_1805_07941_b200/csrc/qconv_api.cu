@@ -30,6 +30,7 @@
 #include "kernels_npconv.cuh"
 #include "kernels_simple.cuh"
 #include "kernels_threshold.cuh"
+#include "per_device.cuh"
 
 static_assert(QCALIB_STATIC_MAX_BINS <= qc::kCalibMaxBins, "built-in scratch holds kCalibMaxBins counters");
 
@@ -1099,9 +1100,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     CUDA_TRY(cudaStreamSynchronize(nullptr));              // (the stream of the first run need not wait for this one)
   }
   // the attribute belongs to the current device: once per device, not once per process
-  static std::once_flag attr_once[64];
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once[h->device & 63], [] {
+  static qc::PerDevice<cudaError_t> attrs;
+  const cudaError_t attr_err = attrs.once(h->device, [] {
     for (IgemmKernel k : {static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FLT_I8, 0>),
@@ -1145,9 +1145,10 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8, 2, 4>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES_U, 2, 4>),
                           static_cast<IgemmKernel>(qc::igemm_i8_kernel<qc::EPI_FAST_I8_RES, 2, 4>)}) {
-      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      if (e != cudaSuccess) attr_err = e;
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      if (e != cudaSuccess) return e;
     }
+    return cudaSuccess;
   });
   if (attr_err != cudaSuccess)
     return fail(QCONV_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(attr_err));
@@ -1415,6 +1416,28 @@ size_t dw_mma_smem(const qc::DwMmaParams& p) {
 // two: 128 x 72 x 72 x 32 24.0 -> 17.1 us, 64 x 75 x 75 x 96 34.2 -> 25.9, 64 x 33 x 65 x 128 22.3 -> 17.6.)
 int dw_mma_ctas_per_sm(const qc::DwMmaParams& p) {
   return static_cast<int>(std::max<size_t>(1, std::min<size_t>(16 / p.warps, 227 * 1024 / (dw_mma_smem(p) + 1024))));
+}
+
+using DwMmaKernel = decltype(&qc::depthwise3x3_mma_kernel<1, true, true>);
+constexpr DwMmaKernel kDwMmaKernels[2][2][2] = {             // [stride - 1][one scale for all channels][ReLU]
+    {{qc::depthwise3x3_mma_kernel<1, false, false>, qc::depthwise3x3_mma_kernel<1, false, true>},
+     {qc::depthwise3x3_mma_kernel<1, true, false>, qc::depthwise3x3_mma_kernel<1, true, true>}},
+    {{qc::depthwise3x3_mma_kernel<2, false, false>, qc::depthwise3x3_mma_kernel<2, false, true>},
+     {qc::depthwise3x3_mma_kernel<2, true, false>, qc::depthwise3x3_mma_kernel<2, true, true>}}};
+
+// Their shared memory, at creation: the attribute belongs to the current device, which then is the handle's.
+int allow_dw_mma_smem(int device) {
+  static qc::PerDevice<cudaError_t> attrs;
+  CUDA_TRY(attrs.once(device, [] {
+    for (const auto& by_stride : kDwMmaKernels)
+      for (const auto& by_scale : by_stride)
+        for (DwMmaKernel k : by_scale) {
+          const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+          if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+  }));
+  return QCONV_OK;
 }
 
 // Tile of the depthwise kernel on warp-level matrix instructions: eight warps, each 32 channels x two groups of 8 pixels, over
@@ -1758,6 +1781,7 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       h->dw_mma = tensor_cores && !h->dw_warp && d.pad_h == 1 && d.pad_w == 1 && align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8 &&
                   d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && h->hints.depthwise_form < 0;
     }
+    if (!rc && h->dw_warp) rc = allow_dw_mma_smem(h->device);
     if (!rc && h->dw_mma) {
       h->mode = MODE_BOX;
       rc = plan_igemm(h, parts, nullptr, w_krsc, bias_host, shift_host, nullptr, nullptr);
@@ -1815,24 +1839,7 @@ int run_dw_mma(qconv_handle* h, const int8_t* x, int8_t* y, int n_run, const qc:
   const dim3 grid(ceil_div(g.C, p.cb) * p.q_blocks, ceil_div(h->P, p.rows_per_cta), ceil_div(n_run, p.images));
   const size_t smem = dw_mma_smem(p);
   const bool uni = h->uniform_shift && h->hints.uniform_shift != 0;
-  using Kernel = decltype(&qc::depthwise3x3_mma_kernel<1, true, true>);
-  static constexpr Kernel kernels[2][2][2] = {
-      {{qc::depthwise3x3_mma_kernel<1, false, false>, qc::depthwise3x3_mma_kernel<1, false, true>},
-       {qc::depthwise3x3_mma_kernel<1, true, false>, qc::depthwise3x3_mma_kernel<1, true, true>}},
-      {{qc::depthwise3x3_mma_kernel<2, false, false>, qc::depthwise3x3_mma_kernel<2, false, true>},
-       {qc::depthwise3x3_mma_kernel<2, true, false>, qc::depthwise3x3_mma_kernel<2, true, true>}}};
-  const Kernel kernel = kernels[g.stride_h - 1][uni][h->d.relu != 0];
-  static std::once_flag attr_once[64];                       // (the attribute belongs to the current device)
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once[h->device & 63], [] {
-    for (const auto& by_stride : kernels)
-      for (const auto& by_scale : by_stride)
-        for (Kernel k : by_scale) {
-          const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
-          if (e != cudaSuccess) attr_err = e;
-        }
-  });
-  CUDA_TRY(attr_err);
+  const DwMmaKernel kernel = kDwMmaKernels[g.stride_h - 1][uni][h->d.relu != 0];
   const int8_t* weights = h->d_w;
   CUDA_TRY(launch_chained(kernel, grid, dim3(p.warps * 32), smem, st, h->dw_map, weights, y, g, tp, p, h->d_status, h->wait_limit));
   return QCONV_OK;
