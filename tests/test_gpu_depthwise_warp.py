@@ -2,6 +2,8 @@
 16 of a warp, channel counts around its 32 and the staged 32 / 64 / 128, images that share a CTA, strips around the rows in
 flight, both strides, windows of a wider tensor, partial batches, unpadded layers, little-aligned outputs, and a wait that
 expires."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -65,3 +67,32 @@ def test_an_expired_wait_is_reported_and_the_next_run_is_right(C, stride):
         conv.set_wait_limit(1 << 22)
         conv.run(xd, y)
         assert conv.status() == 0 and (y.cpu().numpy() == want).all()
+
+
+def test_a_tall_layers_call_costs_the_host_no_more_than_a_short_ones():
+    """How a batch is cut into strips is found once, not on every call; each batch size has its own cut."""
+    from paper_1805_07941_b200 import binding
+    rng = np.random.default_rng(2)
+    per_call = {}
+    for H in (64, 32768):
+        x, w, bias, shift, _, _ = rand_layer(rng, 3, H, 1, 16, 16, 3, 3, groups=16, pad=(1, 1))
+        shift = (shift - 1).clip(4, 31)
+        conv = binding.QConv(w, bias, shift, N=3, H=H, W=1, C=16, K=16, R=3, S=3, pad_h=1, pad_w=1, groups=16)
+        xd = torch.from_numpy(x).cuda()
+        want = oracle_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1), groups=16)
+        for n in (1, 3, 2, 3):
+            y = torch.full((3, H, 1, 16), 77, dtype=torch.int8, device="cuda")
+            conv.run(xd, y, n_run=n)
+            assert conv.status() == 0
+            got = y.cpu().numpy()
+            assert (got[:n] == want[:n]).all() and (got[n:] == 77).all()
+        trials = []
+        for _ in range(5):
+            start = time.perf_counter()
+            for _ in range(200):                             # (queued behind one another: the host's time alone)
+                conv.run(xd, y)
+            trials.append((time.perf_counter() - start) / 200)
+            torch.cuda.synchronize()
+        per_call[H] = min(trials)
+    # the search took about 50 us at this height
+    assert per_call[32768] < 2 * per_call[64] + 20e-6, per_call
