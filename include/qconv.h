@@ -103,7 +103,8 @@ typedef struct {
   int tma_store;         /* output tiles staged in shared memory and stored by TMA: 0 never, 1 wherever they fit */
   int tma_residual;      /* residual tiles fetched by TMA into the staged tiles: 0 never            */
   int depthwise_form;    /* 0: general dp4a kernel, 1: tap-packed kernel with register loads (no TMA rows),
-                            2: with TMA rows, 3: tensor cores wherever they fit                     */
+                            2: with TMA rows, 3: tcgen05 wherever it fits ("depthwise3x3/mma/..." in
+                            qconv_describe), 4: warp-level matrix instructions ("depthwise3x3/mma+tma") */
   int pdl;               /* programmatic dependent launch: 0 off                                    */
   int group_taps;        /* 3x3-like layers on at most 64 channels, the taps of a filter row sharing
                             one ring stage: 0 never, 1 wherever the shape allows                    */

@@ -489,6 +489,46 @@ PatchTile patch_tile(int Q, int P, bool pool) {
   return t;
 }
 
+// Tile of the halo form: whole image rows with their halo, W + S - 1 accumulator rows per image row (S - 1 of them discarded);
+// an image wider than that leaves room for is cut into equal column segments, each with its own halo.
+int halo_segments(const qconv_desc& d) { return ceil_div(d.W, qc::kTileM - (d.S - 1)); }
+void halo_box(const qconv_handle* h, int* tq, int* tp, int* tn, int* step) {
+  const qconv_desc& d = h->d;
+  const int segs = halo_segments(d);
+  *step = ceil_div(d.W, segs);
+  *tq = *step + d.S - 1;
+  *tp = std::max(1, std::min(h->P, qc::kTileM / *tq));
+  *tn = (segs == 1 && *tp == h->P) ? std::max(1, std::min(d.N, qc::kTileM / (*tq * *tp))) : 1;
+}
+
+// Tiles of a depthwise layer on tcgen05: channels (bytes) of a row, and at stride 1 the form (patch, or a box per filter row)
+// whose tiles waste fewer accumulator rows.
+struct DwTiles { int bkc; bool halo; long tiles; };
+DwTiles dw_tiles(const qconv_handle* h) {
+  const qconv_desc& d = h->d;
+  const qconv_plan_hints& hint = h->hints;
+  DwTiles t = {};
+  // 128 wide unless the last tile would be mostly padding; at stride 2 rows of 64 bytes, the three taps of a filter row sharing
+  // a stage
+  const bool wide_row = d.stride_h == 1 && !(hint.bn_max > 0 && hint.bn_max < 128) && align_up(d.C, 128) * 7 <= align_up(d.C, 64) * 8;
+  t.bkc = wide_row ? 128 : d.C > 32 ? 64 : 32;
+  if (d.stride_h == 1) {
+    const PatchTile pt = patch_tile(h->Q, h->P, false);
+    int tq, tp, tn, step;
+    halo_box(h, &tq, &tp, &tn, &step);
+    const long patches = static_cast<long>(pt.segs) * pt.rows * d.N;
+    const long halos = static_cast<long>(ceil_div(h->Q, step)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
+    t.halo = hint.halo != 0 && halos < patches;
+    t.tiles = t.halo ? halos : patches;
+  } else {
+    int tq, tp, tn;
+    choose_box(h->Q, h->P, d.N, &tq, &tp, &tn);
+    t.tiles = static_cast<long>(ceil_div(h->Q, tq)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
+  }
+  t.tiles *= ceil_div(d.C, t.bkc);
+  return t;
+}
+
 int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_of, const int8_t* w_krsc /* host [K][R][S][Cg] */,
                const int32_t* bias_host, const int32_t* shift_host, const int32_t* res_lshift_host, const int32_t* acc_exp_host) {
   const qconv_desc& d = h->d;
@@ -583,24 +623,12 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
   const bool halo_fits = h->mode == MODE_BOX && d.stride_h == 1 && d.stride_w == 1 && (d.S == 3 || d.S == 5) && d.pad_w == d.S / 2 &&
                          (dw || d.C > 32) && hint.halo != 0 && d.pool == 0;
   bool halo = false;
-  // Its tile: whole image rows with their halo, W + S - 1 accumulator rows per image row (S - 1 of them discarded);
-  // an image wider than that leaves room for is cut into equal column segments, each with its own halo.
-  const int halo_segs = ceil_div(d.W, qc::kTileM - (d.S - 1));
-  auto halo_box = [&](int* tq, int* tp, int* tn, int* step) {
-    *step = ceil_div(d.W, halo_segs);
-    *tq = *step + d.S - 1;
-    *tp = std::max(1, std::min(h->P, qc::kTileM / *tq));
-    *tn = (halo_segs == 1 && *tp == h->P) ? std::max(1, std::min(d.N, qc::kTileM / (*tq * *tp))) : 1;
-  };
+  const int halo_segs = halo_segments(d);
   const PatchTile pt = patch_tile(h->Q, h->P, d.pool != 0);
   p.BKC = choose_bkc(c_eff);
   if (is_window_mode(h->mode)) p.BKC = c_eff <= 32 ? 32 : (c_eff <= 64 ? 64 : 128);   // a row is one chunk (two at most)
-  // (depthwise at stride 2: rows of 64 bytes, the three taps of a filter row sharing a stage)
-  // (128 wide unless the last tile would be mostly padding)
-  if (dw) {
-    const bool wide_row = d.stride_h == 1 && !(hint.bn_max > 0 && hint.bn_max < 128) && align_up(d.C, 128) * 7 <= align_up(d.C, 64) * 8;
-    p.BKC = wide_row ? 128 : d.C > 32 ? 64 : 32;
-  }
+  const DwTiles dwt = dw ? dw_tiles(h) : DwTiles{};
+  if (dw) p.BKC = dwt.bkc;
   p.nchunks = dw ? 1 : ceil_div(c_eff, p.BKC);
   const int b_row = dw ? 32 : p.BKC;                       // bytes of a weight row per chunk
   h->a_channels = d.C;
@@ -690,7 +718,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // ... unless its rows' waste makes many more tiles of it, more than run at once; and five weight chunks per stage only
     // where they are small or the layer's CTAs have an SM each.
     int tq, tp, tn, step, bq, bp, bn;
-    halo_box(&tq, &tp, &tn, &step);
+    halo_box(h, &tq, &tp, &tn, &step);
     choose_box(h->Q, h->P, d.N, &bq, &bp, &bn);
     const int tk = ceil_div(k_eff, std::min(bn_max, 64));
     const long halo_tiles = static_cast<long>(ceil_div(h->Q, step)) * ceil_div(h->P, tp) * ceil_div(d.N, tn) * tk;
@@ -698,12 +726,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     halo = (halo_tiles <= h->num_sms || halo_tiles * 10 <= box_tiles * 13) && (d.S == 3 || k_eff <= 32 || halo_tiles <= h->num_sms);
   }
   if (dw) {
-    // stride 1: the form (patch, or a box per filter row) whose tiles waste fewer accumulator rows
-    int tq, tp, tn, step;
-    halo_box(&tq, &tp, &tn, &step);
-    const long halo_tiles = static_cast<long>(ceil_div(h->Q, step)) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
     bn_max = p.BKC;
-    halo = halo_fits && halo_tiles < static_cast<long>(pt.segs) * pt.rows * d.N;
+    halo = halo_fits && dwt.halo;
   }
   if (halo) {
     wide = false;
@@ -736,7 +760,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // Floating-point operands: a stage of a digit product is a patch and its nine weight chunks.  The layer runs at the rate
     // its operands arrive, so the form with fewer bytes on the busiest SM wins.
     int tq, tp, tn, step;
-    halo_box(&tq, &tp, &tn, &step);
+    halo_box(h, &tq, &tp, &tn, &step);
     auto busiest = [&](long boxes, long activations) {
       return ceil_div_l(boxes * ceil_div(k_eff, bn_max), h->num_sms) * (activations + 9l * bn_max * p.BKC);
     };
@@ -802,7 +826,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // A halo-form layer with no more tiles than SMs runs one CTA per SM at most: give that CTA the whole
     // shared memory (its stages are large, and its one chain of stages is as fast as the ring is deep).
     int tq, tp, tn, step;
-    halo_box(&tq, &tp, &tn, &step);
+    halo_box(h, &tq, &tp, &tn, &step);
     const long m_tiles = static_cast<long>(halo_segs) * ceil_div(h->P, tp) * ceil_div(d.N, tn);
     if (m_tiles * p.tiles_k <= h->num_sms) h->ctas_per_sm = 1;
   }
@@ -951,7 +975,7 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     if (h->win_pb % 16) h->s2d_wp += h->s2d_wp & 1;        // the row pitch in bytes is a multiple of 16 as well
   } else {
     choose_box(h->Q, h->P, d.N, &p.tq, &p.tp, &p.tn, d.pool != 0, static_cast<long>(h->num_sms) * h->ctas_per_sm / p.tiles_k);
-    if (halo) halo_box(&p.tq, &p.tp, &p.tn, &p.q_step);
+    if (halo) halo_box(h, &p.tq, &p.tp, &p.tn, &p.q_step);
     if (patch) { p.tq = 16; p.tp = pt.tp; p.tn = 1; p.q_step = pt.q_step; }
     p.pad_h = d.pad_h; p.pad_w = d.pad_w;
     p.stride_h = d.stride_h; p.stride_w = d.stride_w;
@@ -1441,6 +1465,24 @@ int allow_dw_mma_smem(int device) {
   return QCONV_OK;
 }
 
+// Output rows per strip of that kernel: a CTA's fixed cost is about six rows' worth (set-up, filling its ring), its halo two
+// rows.  The strip length whose rounds of CTAs take the fewest rows in all; it depends on the batch alone and is kept with it (the
+// search takes the host 0.4 us at 112 rows, 22 at 8192).
+void plan_dw_mma_strips(qconv_handle* h, int n_run) {
+  if (h->dw_rows_n == n_run) return;
+  qc::DwMmaParams& p = h->dw_mma_prm;
+  const long columns = static_cast<long>(ceil_div(h->d.C, p.cb)) * p.q_blocks * ceil_div(n_run, p.images);
+  const long slots = static_cast<long>(dw_mma_ctas_per_sm(p)) * h->num_sms;
+  long best = -1;
+  for (int strips = 1; strips <= std::max(1, h->P / 2); ++strips) {
+    const int rows = ceil_div(h->P, strips);
+    if (ceil_div(h->P, rows) != strips) continue;
+    const long cost = ceil_div_l(columns * strips, slots) * ((rows - 1) * h->d.stride_h + 3 + 6);
+    if (best < 0 || cost < best) { best = cost; p.rows_per_cta = rows; }
+  }
+  h->dw_rows_n = n_run;
+}
+
 // Tile of the depthwise kernel on warp-level matrix instructions: eight warps, each 32 channels x two groups of 8 pixels, over
 // 32, 64 or 128 channels; narrow images share a CTA.  The width whose padding (channels, groups, halo columns) costs least.
 // Unless `whatever_it_costs`, none where a third of the work would be padding and rows are narrow: 64 x 33 x 33 x 512 stride 2 14.4 us
@@ -1481,6 +1523,28 @@ void plan_dw_mma(qconv_handle* h, bool whatever_it_costs) {
   bp.c2 = static_cast<float>(12582912.0 * (1.0 - static_cast<double>(c1)));
   h->dw_mma_prm = bp;
   h->dw_warp = 1;
+}
+
+// Whether tcgen05 takes a large layer in clearly less time than the kernel on warp-level instructions, by a model of both in us,
+// fitted to 130 layers of 1 to 115 million outputs (it meets their times within 5 and 7 %).  Warp level: the busiest SM's rows of
+// CTAs at the rate of 16 warps, or the rounds of CTAs at a CTA's own pace where there are fewer warps, and the bytes; tcgen05: its
+// tiles.  Narrow images leave the groups of 8 columns partly empty, few CTAs more than the SMs hold leave most of them idle.
+// us, warp level / tcgen05: 212 x 41 x 9 x 512 stride 2 19.8 / 12.8, 96 x 28 x 28 x 256 18.8 / 15.2, 200 x 10 x 10 x 512 13.7 / 11.0, 128 x 36 x 36 x 128
+// 18.5 / 16.5, 128 x 28 x 28 x 512 38.0 / 32.0; the other way round 64 x 28 x 28 x 576 19.9 / 23.5, 128 x 14 x 14 x 512 11.0 / 12.9.  Stride 1 keeps a
+// margin: between other layers, short CTAs without a tail are worth a few us (MobileNet-v1, batch 256, with its 56 x 56 x 128 or
+// its 14 x 14 x 512 layers on tcgen05: + 6 and + 20 us of 774, where alone these take 71 and 19 there, 69 and 21 here).
+bool dw_tcgen05_wins(qconv_handle* h) {
+  const qconv_desc& d = h->d;
+  plan_dw_mma_strips(h, d.N);
+  const qc::DwMmaParams& p = h->dw_mma_prm;
+  const double mb = 1e-6 * d.N * d.C * (static_cast<double>(d.H) * d.W + static_cast<double>(h->P) * h->Q);
+  const long ctas = static_cast<long>(ceil_div(d.C, p.cb)) * p.q_blocks * ceil_div(d.N, p.images) * ceil_div(h->P, p.rows_per_cta);
+  const double rows = (p.rows_per_cta - 1) * d.stride_h + 3;
+  const double busiest = ceil_div_l(ctas, h->num_sms) * p.warps / 16.0, rounds = ceil_div_l(ctas, static_cast<long>(h->num_sms) * dw_mma_ctas_per_sm(p));
+  const DwTiles t = dw_tiles(h);
+  const double tiles = static_cast<double>(t.tiles) / h->num_sms;
+  if (d.stride_h == 1) return 4.0 + tiles * (t.bkc == 128 ? 1.23 : 0.77) < 0.90 * (0.8 + std::max(0.50 * busiest, 0.45 * rounds) * (rows + 1.3) + 0.065 * mb);
+  return 4.0 + tiles * 1.08 < 0.97 * (1.2 + std::max(0.337 * busiest, 0.308 * rounds) * (rows + 2.3) + 0.05 * mb);
 }
 
 // Box of the depthwise kernels' row copies: `channels` x `pixels` x one row x `images`.
@@ -1769,18 +1833,19 @@ int create_layer(qconv_handle** out, const qconv_desc* desc, const int8_t* w_hos
       h->dw_tap = 1;
       if (d.C % 32 == 0 && h->hints.depthwise_form != 1) plan_dw_tma(h);
       // On the tensor cores by warp-level instructions (kernel_dw_mma.cuh) where the channels fill its groups of 32, and for
-      // small layers whatever they do; else by tcgen05 in rows of 64 or 128 channels with an eighth of padding at most; else dp4a.
-      // us per launch, warp level / tcgen05 / dp4a: 256 x 112 x 112 x 32 67 / 138 / 73, 256 x 56 x 56 x 128 stride 2 27.6 / 28.4 /
-      // 29.9, 256 x 28 x 28 x 256 40 / 37 / 39, 256 x 14 x 14 x 512 21.6 / 22.2 / 22.6, 32 x 56 x 56 x 96 8.1 / 12.8 / 14.6, 64 x 56 x 56 x
-      // 144 26.3 / 34 / 25.4, 13 x 13 x 13 x 1008 4.6 / 5.4 / 5.6; one image of those 2.8 to 3.2 / 3.3 to 4.0 / 3.9 to 4.2.  Alone it is
-      // no faster at batch 256, but its many short CTAs leave no tail: the MobileNet-v1 stack with it throughout 771 us, 818 before.
+      // small layers whatever they do; by tcgen05, in rows of 64 or 128 channels with an eighth of padding at most, where they do
+      // not or where that is faster (dw_tcgen05_wins); else dp4a.  us per launch, warp level / tcgen05 / dp4a: 256 x 112 x 112 x 32
+      // 67 / 91 / 73, 256 x 56 x 56 x 128 stride 2 27.4 / 27.8 / 30.2, 32 x 56 x 56 x 96 8.1 / 12.8 / 14.6, 64 x 56 x 56 x 144 26.3 / 34 / 25.4, 13 x 13 x
+      // 13 x 1008 4.6 / 5.4 / 5.6; one image of those 2.8 to 3.2 / 3.3 to 4.0 / 3.9 to 4.2.  (With both planned, an output that is
+      // 8-byte aligned only still takes the warp level.)
       const long long outputs = static_cast<long long>(d.N) * P * Q * d.C;
+      const int form = h->hints.depthwise_form;
       const bool tensor_cores = h->flt_epilogue && h->hints.fast_epilogue != 0 && d.C % 16 == 0;
       if (tensor_cores && d.out_c_pitch % 8 == 0 && d.out_c_offset % 8 == 0 &&
-          (h->hints.depthwise_form == 3 || (h->hints.depthwise_form < 0 && (d.C % 32 == 0 || outputs <= (4ll << 20)))))
-        plan_dw_mma(h, h->hints.depthwise_form == 3 || outputs <= (4ll << 20) || align_up(d.C, 64) != static_cast<size_t>(d.C));
-      h->dw_mma = tensor_cores && !h->dw_warp && d.pad_h == 1 && d.pad_w == 1 && align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8 &&
-                  d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && h->hints.depthwise_form < 0;
+          (form == 4 || (form < 0 && (d.C % 32 == 0 || outputs <= (4ll << 20)))))
+        plan_dw_mma(h, form == 4 || outputs <= (4ll << 20) || align_up(d.C, 64) != static_cast<size_t>(d.C));
+      h->dw_mma = tensor_cores && d.pad_h == 1 && d.pad_w == 1 && (form == 3 || align_up(d.C, 64) * 7 <= static_cast<size_t>(d.C) * 8) &&
+                  d.out_c_pitch % 16 == 0 && d.out_c_offset % 16 == 0 && (form < 0 || form == 3) && (!h->dw_warp || dw_tcgen05_wins(h));
     }
     if (!rc && h->dw_warp) rc = allow_dw_mma_smem(h->device);
     if (!rc && h->dw_mma) {
@@ -1826,21 +1891,7 @@ int run_dw_mma(qconv_handle* h, const int8_t* x, int8_t* y, int n_run, const qc:
   qc::DwMmaParams& p = h->dw_mma_prm;
   int rc = prepare_dw_map(h, x, n_run, p.cb, p.pix, p.images, p.cb);
   if (rc) return rc;
-  // Rows per strip: a CTA's fixed cost is about six rows' worth (set-up, filling its ring), its halo two rows.  The strip
-  // length whose rounds of CTAs take the fewest rows in all; it depends on the batch alone and is kept with it (the search
-  // takes the host 0.4 us at 112 rows, 22 at 8192).
-  if (h->dw_rows_n != n_run) {
-    const long columns = static_cast<long>(ceil_div(g.C, p.cb)) * p.q_blocks * ceil_div(n_run, p.images);
-    const long slots = static_cast<long>(dw_mma_ctas_per_sm(p)) * h->num_sms;
-    long best = -1;
-    for (int strips = 1; strips <= std::max(1, h->P / 2); ++strips) {
-      const int rows = ceil_div(h->P, strips);
-      if (ceil_div(h->P, rows) != strips) continue;
-      const long cost = ceil_div_l(columns * strips, slots) * ((rows - 1) * g.stride_h + 3 + 6);
-      if (best < 0 || cost < best) { best = cost; p.rows_per_cta = rows; }
-    }
-    h->dw_rows_n = n_run;
-  }
+  plan_dw_mma_strips(h, n_run);
   const dim3 grid(ceil_div(g.C, p.cb) * p.q_blocks, ceil_div(h->P, p.rows_per_cta), ceil_div(n_run, p.images));
   const size_t smem = dw_mma_smem(p);
   const bool uni = h->uniform_shift && h->hints.uniform_shift != 0;

@@ -31,9 +31,9 @@ def test_depthwise_on_warp_instructions_matches_the_oracle(case, uniform):
         kw = dict(R=3, S=3, stride=(st, st), pad=(pad, pad), groups=C, relu=relu, symmetric=uniform)
         win = dict(kw, out_c_offset=8, out_c_pitch=C + 24)
         got, desc = gpu_conv(x, w, bias, shift, **kw)
-        assert "depthwise3x3/mma" in desc and (got == oracle_conv(x, w, bias, shift, **kw)).all(), desc
+        assert "depthwise3x3/mma+tma" in desc and (got == oracle_conv(x, w, bias, shift, **kw)).all(), desc
         got, desc = gpu_conv(x, w, bias, shift, **win)
-        assert "depthwise3x3/mma" in desc and (got == oracle_conv(x, w, bias, shift, **win)).all(), desc
+        assert "depthwise3x3/mma+tma" in desc and (got == oracle_conv(x, w, bias, shift, **win)).all(), desc
     # a partial batch, then the whole one, and an output that is 8-byte aligned only
     want = oracle_conv(x, w, bias, shift, R=3, S=3, stride=(st, st), pad=(pad, pad), groups=C)
     conv = binding.QConv(w, bias, shift, N=N, H=H, W=W, C=C, K=C, R=3, S=3, stride_h=st, stride_w=st, pad_h=pad, pad_w=pad, groups=C)
