@@ -1454,6 +1454,10 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     // swizzled.)  A residual is staged too, or comes in registers.
     constexpr bool kLeanOk = EpiTraits<EPI>::fast && !kPool && !kSplit && GPW == kGroupsPerWarp;
     const bool lean = kLeanOk && prm.out_stage_bytes != 0;
+    // The integer epilogue with a residual and per-channel constants has no registers to spare: with both forms of the tile in
+    // the kernel it spilled 128 bytes (276 read back; one form: 60 and 88), so this form also serves its direct stores.  us, 3 x
+    // 3 with residual: 62 x 31 x 17 x 224 -> 576 58.3 -> 54.7, 35 x 42 x 29 x 160 -> 880 stride 2 33.7 -> 29.3, 2 x 38 x 33 x 240 -> 16 5.6 -> 4.75.
+    constexpr bool kOneForm = kLeanOk && EPI == EPI_FAST_I8_RES;
     const int lean_groups = g_end - g_begin;
     const uint32_t lean_col0 = static_cast<uint32_t>(g_begin) * 16u;
     uint32_t lean_off[4];
@@ -1700,7 +1704,7 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
           gen_copy<true>(prm.gen_vec_y, gen_stage, static_cast<int8_t*>(y) + prm.out_c_offset + gen_k0,
                          static_cast<long long>(pix) * prm.out_c_pitch, row_ok, gen_cols, lane);
           __syncwarp();
-        } else if (kLeanOk && lean) {
+        } else if (kLeanOk && (lean || kOneForm)) {
           // loads one group ahead of the arithmetic, as below, without the bookkeeping
           const uint32_t t0 = t_addr + lean_col0;
           const uint32_t c0 = chan + lean_col0 * EpiTraits<EPI>::cst_bytes;
@@ -1715,7 +1719,11 @@ igemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
               rw[0] = rres[i].x; rw[1] = rres[i].y; rw[2] = rres[i].z; rw[3] = rres[i].w;
             }
             convert_16<EPI, RELU>(acc, c0 + static_cast<uint32_t>(i) * kGroupCst, ahead, rw, ep, wds);
-            ptx::sts_uint4(addr, wds[0], wds[1], wds[2], wds[3]);
+            const int k = tc.k0 + static_cast<int>(lean_col0) + 16 * i;
+            if (!kOneForm || lean)
+              ptx::sts_uint4(addr, wds[0], wds[1], wds[2], wds[3]);
+            else if (row_ok && k < prm.K)
+              *reinterpret_cast<uint4*>(static_cast<int8_t*>(y) + pix * prm.out_c_pitch + prm.out_c_offset + k) = make_uint4(wds[0], wds[1], wds[2], wds[3]);
           };
           // (a warp has up to four groups; one of the second four warps has none where the tile is 16 wide)
           if (lean_groups > 0) {

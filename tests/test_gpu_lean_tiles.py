@@ -21,7 +21,7 @@ def test_staged_tiles_of_any_width_match_the_oracle(case):
     import torch
     from paper_1805_07941_b200 import binding
     N, n_runs, H, W, C, K, R, stride = case
-    for with_res, uniform, small, window in ((0, 0, 1, 0), (0, 1, 1, 1), (1, 0, 1, 0), (1, 1, 0, 0), (0, 1, 0, 0)):
+    for with_res, uniform, small, window in ((0, 0, 1, 0), (0, 1, 1, 1), (1, 0, 1, 0), (1, 1, 0, 0), (0, 1, 0, 0), (1, 0, 0, 0), (1, 0, 0, 1)):
         rng = np.random.default_rng(N + H + K + with_res + 2 * uniform)
         x, w, bias, shift, res, t = rand_layer(rng, N, H, W, C, K, R, R, with_res=bool(with_res), stride=(stride, stride), pad=(R // 2, R // 2),
                                                per_channel_shift=not uniform)
