@@ -112,7 +112,7 @@ typedef struct {
                             0 never, 1 wherever the shape allows                                    */
   int split_k;           /* CTAs of a cluster sharing a tile's contraction when a run has few tiles: 0 never,
                             2 or 4 wherever the shape allows                                        */
-  int patch_halo;        /* 3x3 stride-1 layers on 48 to 128 channels, one activation box serving all nine
+  int patch_halo;        /* 3x3 stride-1 layers on up to 128 channels, one activation box serving all nine
                             taps: 0 never, 1 wherever the shape allows                              */
   int bn_max;            /* 0, or the widest channel tile (multiple of 16): up to 128, or 256 to take
                             256-wide tiles (one CTA per SM) wherever the layer's shape allows them  */

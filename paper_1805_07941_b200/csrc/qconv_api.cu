@@ -772,7 +772,10 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     wide = false;
     halo = false;
     h->pair = 0;
-    bn_max = dw ? p.BKC : np ? bn_max : bn_max <= 64 ? 64 : 128;
+    // (64 wide only below a wave of its own tiles, which are more than the boxes': 20 x 28 x 28 x 64 -> 128 5.6 us 64 wide, 4.9 128;
+    // x 128 -> 128 6.45 / 5.7)
+    const bool below_a_wave = static_cast<long>(pt.segs) * pt.rows * d.N * ceil_div(k_eff, 128) < h->num_sms;
+    bn_max = dw ? p.BKC : np ? bn_max : bn_max <= 64 && below_a_wave ? 64 : 128;
     taps_r = taps_s = 1;
     p.R = p.S = 1;
   }

@@ -11,7 +11,10 @@ pytestmark = pytest.mark.gpu
 
 CASES = [  # N, H, W, C, K
     (2, 8, 14, 64, 64), (1, 7, 13, 64, 128), (3, 9, 15, 128, 128), (2, 16, 28, 48, 64), (1, 17, 29, 96, 208), (2, 5, 3, 128, 256),
-    (1, 1, 1, 64, 16), (2, 20, 43, 112, 80), (40, 28, 28, 64, 64), (30, 30, 30, 128, 128)]
+    (1, 1, 1, 64, 16), (2, 20, 43, 112, 80), (40, 28, 28, 64, 64), (30, 30, 30, 128, 128),
+    # rows of 32 bytes: 16 and 32 channels, one and several channel tiles, images smaller than a tile, several tiles per CTA
+    (1, 8, 14, 16, 16), (2, 7, 13, 32, 48), (3, 16, 28, 16, 208), (2, 6, 10, 32, 256), (5, 9, 15, 32, 112), (1, 1, 1, 32, 16), (2, 18, 30, 16, 128),
+    (40, 28, 28, 32, 64), (24, 30, 30, 16, 32)]
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -45,3 +48,18 @@ def test_patch_form_matches_the_oracle(case, uniform):
                     with binding.plan_hints(patch_halo=1):
                         got, desc = gpu_conv(x, w, bias, shift, pool=2, **kw)
                     assert "patch=1" in desc and (got == ref.maxpool_i8(want, 2, 2, 2, 0)).all(), desc
+
+
+# N, H, W, C, K -> whether the plan takes the patch form by itself (below a wave of tiles only at up to 32 channels), and its width:
+# 64 channels only where 128-wide tiles are fewer than the SMs
+PLANS = [(1, 32, 32, 16, 16, 1, 16), (1, 56, 56, 32, 32, 1, 32), (16, 7, 7, 32, 256, 1, 64), (32, 14, 14, 32, 128, 1, 64), (20, 28, 28, 32, 128, 1, 128),
+         (1, 32, 32, 48, 64, 0, 64), (20, 28, 28, 64, 128, 1, 128), (10, 28, 28, 128, 256, 1, 128), (10, 28, 28, 96, 192, 1, 96)]
+
+
+@pytest.mark.parametrize("N,H,W,C,K,patch,BN", PLANS)
+def test_the_tiles_of_the_patch_form(N, H, W, C, K, patch, BN):
+    rng = np.random.default_rng(N + C)
+    x, w, bias, shift, _, _ = rand_layer(rng, N, H, W, C, K, 3, 3, pad=(1, 1))
+    got, desc = gpu_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1))
+    assert ("patch=1" in desc) == bool(patch) and " BN=%d " % BN in desc, desc
+    assert (got == oracle_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1))).all(), desc
