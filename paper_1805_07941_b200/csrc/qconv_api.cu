@@ -1347,17 +1347,20 @@ int prepare_a_map(qconv_handle* h, const int8_t* a_ptr, int n_run) {
 // worth of tiles is stored by the threads themselves whatever the plan: there it is the chain of one tile that counts, and
 // barrier, TMA store and its wait lengthen it (us per launch, staged / direct: 14 tiles of 28 x 28 x 512 -> 128, 1 x 1 3.1 / 2.9; 32
 // of 7 x 7 x 512 -> 2048 with residual 3.4 / 3.15; 56 of 28 x 28 x 128 -> 512 2.7 / 2.8; 100 of 56 x 56 x 64 -> 256 2.85 / 3.06;
-// ResNet-50 on one image 195.2 -> 191.7).
+// ResNet-50 on one image 195.2 -> 191.7).  The patch form, whose tiles leave by one store per image row, as long as every CTA has one
+// tile: 3 x 3, 32 channels, 64 x 9 x 5 -> 256 4.3 -> 3.9, 110 x 5 x 5 -> 128 4.0 -> 3.5; 20 x 28 x 28 x 64 -> 64 4.3 -> 3.8.
 void plan_staging(qconv_handle* h, long tiles) {
   qc::IgemmParams& p = h->prm;
   if (!p.fast_epilogue) return;
   uint32_t bytes = h->plan_stage_bytes;
   int bufs = h->plan_stage_bufs;
-  if (!bytes && h->ring_out_fits && tiles <= static_cast<long>(h->num_sms) * h->ctas_per_sm) {
+  const long one_each = static_cast<long>(h->num_sms) * h->ctas_per_sm;
+  if (!bytes && h->ring_out_fits && tiles <= one_each) {
     bytes = static_cast<uint32_t>(align_up(static_cast<size_t>(qc::kTileM) * p.BN, 1024));
     bufs = 0;
   }
-  if (tiles * 3 <= h->num_sms && h->hints.tma_store != 1) bytes = 0;
+  const long most = h->patch ? one_each : h->num_sms / 3;
+  if (tiles <= most && h->hints.tma_store != 1) bytes = 0;
   if (bytes != p.out_stage_bytes) h->y_key_ptr = h->r_key_ptr = nullptr;
   p.out_stage_bytes = bytes;
   p.out_stage_bufs = bufs;

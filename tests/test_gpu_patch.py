@@ -63,3 +63,24 @@ def test_the_tiles_of_the_patch_form(N, H, W, C, K, patch, BN):
     got, desc = gpu_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1))
     assert ("patch=1" in desc) == bool(patch) and " BN=%d " % BN in desc, desc
     assert (got == oracle_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1))).all(), desc
+
+
+@pytest.mark.parametrize("N,H,W,C,K", [(64, 9, 5, 32, 256), (110, 5, 5, 32, 128), (33, 9, 9, 16, 64)])
+def test_one_tile_to_a_cta_is_stored_without_staging(N, H, W, C, K):
+    """Tiles leave straight from the registers while every CTA has one, whatever the plan holds for larger batches."""
+    from paper_1805_07941_b200 import binding
+    import torch
+    rng = np.random.default_rng(N + K)
+    x, w, bias, shift, _, _ = rand_layer(rng, N, H, W, C, K, 3, 3, pad=(1, 1))
+    want = oracle_conv(x, w, bias, shift, R=3, S=3, pad=(1, 1))
+    for hints, stores in ((dict(), "tma_store=0"), (dict(tma_store=1), "tma_store=2")):
+        with binding.plan_hints(patch_halo=1, **hints):
+            conv = binding.QConv(w, bias, shift, N=N, H=H, W=W, C=C, K=K, R=3, S=3, pad_h=1, pad_w=1)
+        xd = torch.from_numpy(x).cuda()
+        for n in (N, 3, N):
+            y = torch.full((N, H, W, K), 77, dtype=torch.int8, device="cuda")
+            conv.run(xd, y, n_run=n)
+            assert conv.status() == 0 and "patch=1" in conv.describe() and stores in conv.describe(), conv.describe()
+            got = y.cpu().numpy()
+            assert (got[:n] == want[:n]).all() and (got[n:] == 77).all()
+        conv.destroy()
