@@ -187,7 +187,7 @@ int qconv_status(qconv_handle* h);
 int qconv_set_wait_limit(qconv_handle* h, unsigned int polls);
 
 /* Writes a one-line description of the plan (algorithm, tile shape, stages) into buf; with split=2 or 4 at its end if the last
- * run shared the contraction of its tiles (that depends on n_run). */
+ * run shared the contraction of its tiles, ring=1 if it staged them in the operand ring (these and tma_store depend on n_run). */
 int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len);
 
 int qconv_destroy(qconv_handle* h);

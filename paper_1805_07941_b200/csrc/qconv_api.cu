@@ -956,6 +956,8 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     }
   }
   p.stages = stages;
+  // (of the widths that the store's box swizzles, 64 only with two CTAs on an SM: with one, whose ring is several times as deep,
+  // staging costs 0.2 us: 4 x 28 x 25 x 176 -> 272, 3 x 3 6.2 direct, 6.4 staged; with two 24 x 11 x 28 x 544 -> 128, 1 x 1 4.15 / 3.8)
   h->ring_out_fits = p.fast_epilogue && !p.out_stage_bytes && hint.tma_store != 0 && (p.BN == 128 || (p.BN == 64 && h->ctas_per_sm == 2)) && !h->pair && !d.pool &&
                      !(halo && halo_segs > 1) && !(patch && d.has_residual) &&
                      static_cast<size_t>(stages) * (p.a_stage_bytes + (p.b_resident ? 0 : p.b_stage_bytes)) >= static_cast<size_t>(out_tile);
@@ -2328,6 +2330,7 @@ int qconv_describe(const qconv_handle* h, char* buf, size_t buf_len) {
     const size_t used = std::strlen(buf);
     if (h->split > 1) snprintf(buf + used, buf_len - used, " split=%d", h->split);
     else if (h->np3) snprintf(buf + used, buf_len - used, " sums=32");
+    else if (p.out_stage_bytes && !p.out_stage_bufs) snprintf(buf + used, buf_len - used, " ring=1");
   } else {
     snprintf(buf, buf_len, "%s", h->algo == QCONV_ALGO_DEPTHWISE ? (h->dw_warp ? "depthwise3x3/mma+tma" : h->dw_tma ? "depthwise3x3/tap-packed+tma" : h->dw_tap ? "depthwise3x3/tap-packed" : "depthwise3x3/dp4a")
                                                                   : "direct");

@@ -556,7 +556,7 @@ def test_bounded_wait_reports_timeout_and_context_survives(case):
     want = oracle_conv(x, w, bias, shift, res, t, **kw)
     assert (got == want).all(), conv.describe()
     if dw:
-        assert "tma" in conv.describe()
+        assert "depthwise3x3/mma+tma" in conv.describe()
     xd = torch.from_numpy(x).cuda()
     rd = torch.from_numpy(res).cuda() if res is not None else None
     y = torch.zeros((N, H, W, K), dtype=torch.int8, device="cuda")
