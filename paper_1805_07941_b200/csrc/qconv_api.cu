@@ -2475,14 +2475,20 @@ int qmaxpool_i8(const int8_t* d_x, int N, int H, int W, int C, int R, int S, int
   const bool strip_ok = vec && R == S && ((R == 3 && (stride == 1 || stride == 2)) || (R == 2 && stride == 2));
   if (strip_ok) {
     // strips as long as still leaves every SM several hundred threads
-    const int columns = ceil_div(Q, R == 3 && stride == 1 ? 2 : 1);
+    // 3 x 3 at stride 1: two output columns a thread from about two warps' worth of such threads an SM on, one below, where the
+    // longer chain of a thread counts (us, one / two: 2 x 2 x 39 x 336 1.63 / 1.83, 3 x 70 x 30 x 80 1.84 / 2.03, 16 x 7 x 7 x 832 2.34 / 2.14,
+    // 16 x 28 x 28 x 192 3.8 / 2.3)
+    const bool two = R == 3 && stride == 1 && Q > 1 && static_cast<size_t>(N) * ceil_div(P, 2) * ceil_div(Q, 2) * (C / 16) >= 148u * 72u;
+    const int columns = ceil_div(Q, two ? 2 : 1);
     int rows = 16;
     while (rows > 2 && static_cast<size_t>(N) * ceil_div(P, rows) * columns * (C / 16) < 148u * 1024u) rows /= 2;
     const int strips = ceil_div(P, rows);
     const size_t threads = static_cast<size_t>(N) * strips * columns * (C / 16);
     if (threads > 2147483647ull) return fail(QCONV_ERR_UNSUPPORTED_SHAPE, "pooling: tensor too large");
     const dim3 grid(static_cast<unsigned int>((threads + 127) / 128));
-    if (R == 3 && stride == 1)
+    if (R == 3 && stride == 1 && !two)
+      CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 1, 1>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
+    else if (two)
       CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 1, 2>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
     else if (R == 3)
       CUDA_TRY(launch_chained(qc::maxpool_i8_strip_kernel<3, 3, 2, 1>, grid, dim3(128), 0, st, d_x, d_y, N, H, W, C, pad, P, Q, rows, strips));
