@@ -13,12 +13,13 @@
 // both chunks, and one exchange leaves each lane 8 consecutive channels of a pixel.
 //
 // What it was made against: 128 x 32-byte operands per tcgen05.mma of N = 32 (54 cycles for 1/32 of useful products), and 17
-// instructions an output in the dp4a form.  Here an output takes 12.4 (ncu, 64 x 56 x 56 x 128: issue slots 51 %, ALU pipe 31 %,
-// matrix pipe 24 %, long scoreboard and fixed latencies among the stalls, up to 128 registers and so 16 warps an SM), and alone the
-// kernel is no faster at large sizes (256 x 56 x 56 x 128 69 / 69 / 74 us).  It is where launches follow one another: a third of the
-// set-up, and short CTAs in place of a persistent grid whose two CTAs an SM finish 10 us apart.  MobileNet-v1 stack, batch 256: 818
-// -> 771 us; one image's layers 3.3-4.2 -> 2.8-3.2 us each.  Registers decide its speed: per-channel scales held in them instead of
-// shared memory 782 us, a few more spilled 807-848.
+// instructions an output in the dp4a form.  Here an output takes 12.1 (ncu, 64 x 56 x 56 x 128: issue slots 51 %, ALU pipe 28 %,
+// matrix pipe 25 %, fixed latencies and long scoreboard among the stalls, 122 registers and so 16 warps an SM), and alone the
+// kernel is no faster at large sizes (256 x 56 x 56 x 128 69 us, 71 on tcgen05, 74 with dp4a) and slower where narrow or short images
+// leave its groups or strips partly empty (dw_tcgen05_wins, qconv_api.cu, chooses).  It is where launches follow one another: a
+// third of the set-up, and short CTAs in place of a persistent grid whose two CTAs an SM finish 10 us apart.  MobileNet-v1 stack,
+// batch 256: 818 -> 771 us; one image's layers 3.3-4.2 -> 2.8-3.2 us each.  Registers decide its speed: per-channel scales held in
+// them instead of shared memory 782 us, a few more spilled 807-848.
 //
 // Every wait is bounded, its first probe counted as a poll: on expiry the CTA raises the status word and everybody leaves; the
 // issuing lane stays until its copies have landed.

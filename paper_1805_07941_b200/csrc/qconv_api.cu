@@ -752,6 +752,9 @@ int plan_igemm(qconv_handle* h, DeviceParts& parts, const qconv_handle* weights_
     // tiles at most
     // ... and at up to 32 channels (rows of 32 bytes) also below a wave, where the one box is one wait instead of three: 32 x 32
     // x 16 -> 16 3.6 -> 3.0 us, 56 x 56 x 32 -> 32 3.3 -> 3.1; with rows of 64 or 128 bytes three boxes are 0.2 us faster there.
+    // (Whatever part of a tile the images fill: small ones take a tile each where boxes put several into one, and still gain. us,
+    // boxes / patch, 32 channels: 16 x 7 x 7 -> 256 3.6 / 2.8, 64 x 7 x 7 -> 128 3.7 / 3.3, 64 x 4 x 4 -> 256 3.7 / 3.7; at worst 64 x 9 x 5 -> 128
+    // 3.7 / 3.9.)
     patch = hint.patch_halo == 1 || (k_eff <= 256 && hint.halo != 0 && hint.resident_weights != 0 &&
                                      ((tiles >= h->num_sms && used >= 0.75) || (p.BKC == 32 && tiles <= h->num_sms)));
   }
@@ -1545,14 +1548,17 @@ bool dw_tcgen05_wins(qconv_handle* h) {
   const qconv_desc& d = h->d;
   plan_dw_mma_strips(h, d.N);
   const qc::DwMmaParams& p = h->dw_mma_prm;
+  const bool s1 = d.stride_h == 1;
   const double mb = 1e-6 * d.N * d.C * (static_cast<double>(d.H) * d.W + static_cast<double>(h->P) * h->Q);
   const long ctas = static_cast<long>(ceil_div(d.C, p.cb)) * p.q_blocks * ceil_div(d.N, p.images) * ceil_div(h->P, p.rows_per_cta);
   const double rows = (p.rows_per_cta - 1) * d.stride_h + 3;
   const double busiest = ceil_div_l(ctas, h->num_sms) * p.warps / 16.0, rounds = ceil_div_l(ctas, static_cast<long>(h->num_sms) * dw_mma_ctas_per_sm(p));
+  const double warp_level = s1 ? 0.8 + std::max(0.50 * busiest, 0.45 * rounds) * (rows + 1.3) + 0.065 * mb
+                               : 1.2 + std::max(0.337 * busiest, 0.308 * rounds) * (rows + 2.3) + 0.05 * mb;
+  const double budget = (s1 ? 0.90 : 0.97) * warp_level - 4.0;
+  if (budget <= 0.0) return false;
   const DwTiles t = dw_tiles(h);
-  const double tiles = static_cast<double>(t.tiles) / h->num_sms;
-  if (d.stride_h == 1) return 4.0 + tiles * (t.bkc == 128 ? 1.23 : 0.77) < 0.90 * (0.8 + std::max(0.50 * busiest, 0.45 * rounds) * (rows + 1.3) + 0.065 * mb);
-  return 4.0 + tiles * 1.08 < 0.97 * (1.2 + std::max(0.337 * busiest, 0.308 * rounds) * (rows + 2.3) + 0.05 * mb);
+  return static_cast<double>(t.tiles) / h->num_sms * (!s1 ? 1.08 : t.bkc == 128 ? 1.23 : 0.77) < budget;
 }
 
 // Box of the depthwise kernels' row copies: `channels` x `pixels` x one row x `images`.

@@ -113,3 +113,31 @@ def test_random_layer_matches_the_oracle(seed):
             assert (gp[..., :off] == 77).all() and (gp[..., off + K:] == 77).all()
         assert (gp[n_run:] == 77).all()
         pc.destroy()
+
+
+@pytest.mark.parametrize("seed", range(24))
+def test_random_depthwise_layer_matches_the_oracle(seed):
+    """3x3 depthwise layers of random shapes in the form the plan takes and in each that the matrix instructions have."""
+    import torch
+    from paper_1805_07941_b200 import binding
+    rng = np.random.default_rng(7000 + seed)
+    N, H, W, C = int(rng.integers(1, 40)), int(rng.integers(1, 41)), int(rng.integers(1, 71)), 16 * int(rng.integers(1, 25))
+    st, relu, concat = int(rng.integers(1, 3)), int(rng.integers(0, 2)), bool(rng.integers(0, 2))
+    x, w, bias, shift, _, _ = rand_layer(rng, N, H, W, C, C, 3, 3, groups=C, stride=(st, st), pad=(1, 1), per_channel_shift=bool(rng.integers(0, 2)))
+    shift = (shift - 1).clip(4, 31)
+    off, pitch = (16, C + 48) if concat else (0, 0)
+    kw = dict(R=3, S=3, stride=(st, st), pad=(1, 1), groups=C, relu=relu, out_c_offset=off, out_c_pitch=pitch)
+    want = oracle_conv(x, w, bias, shift, **kw)
+    xd = torch.from_numpy(x).cuda()
+    for form, name in ((-1, "depthwise3x3/"), (3, "depthwise3x3/mma/"), (4, "depthwise3x3/mma+tma")):
+        with binding.plan_hints(depthwise_form=form):
+            conv = binding.QConv(w, bias, shift, None, None, N=N, H=H, W=W, C=C, K=C, R=3, S=3, stride_h=st, stride_w=st, pad_h=1, pad_w=1,
+                                 groups=C, relu=relu, out_c_offset=off, out_c_pitch=pitch)
+        assert conv.describe().startswith(name), conv.describe()
+        for n in (N, max(1, N - 1), N):
+            y = torch.full((N, conv.P, conv.Q, pitch or C), 77, dtype=torch.int8, device="cuda")
+            conv.run(xd, y, n_run=n)
+            assert conv.status() == 0, conv.describe()
+            got = y.cpu().numpy()
+            assert (got[:n] == want[:n]).all() and (got[n:] == 77).all(), (conv.describe(), (N, H, W, C, st, n))
+        conv.destroy()
